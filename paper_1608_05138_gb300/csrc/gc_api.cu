@@ -317,6 +317,7 @@ struct RelabelPlan {
   std::vector<int32_t> mid, longr;  // rows of 33..4096 entries, and longer ones
   std::vector<int64_t> long_off;    // offset of each long row's padded copy
   int64_t tmp_len = 0;
+  int32_t obound[kOBounds] = {};    // first rank of degree >= kOBoundDeg[k]
 };
 
 RelabelPlan plan_relabel(int32_t n, const int32_t* rp) {
@@ -370,6 +371,7 @@ RelabelPlan plan_relabel(int32_t n, const int32_t* rp) {
     base[D] = r;
     S[D] = sl;
   }
+  for (int k = 0; k < kOBounds; ++k) R.obound[k] = base[std::min<size_t>((size_t)kOBoundDeg[k], D)];
   run_threads(nt, [&](int t) {
     int32_t* c = cnt.data() + (size_t)t * D;
     for (int32_t x = chunk(t, nt); x < chunk(t + 1, nt); ++x) {
@@ -570,7 +572,9 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
                          (int32_t)R.mid.size(), d_lists + R.mid.size(), d_loff, (int32_t)R.longr.size(), d_tmp, s);
   drop_temps();
   if (st != GC_OK) return fail(st);
-  st = prepare_graph(n, g->m, g->d_rp, g->d_ci, nullptr, d_eid, d_perm, &g->prep, s);
+  const int32_t zero = 0;
+  const RankInfo rank = {R.rp.data(), 1, &zero, &n, R.obound};
+  st = prepare_graph(n, g->m, g->d_rp, g->d_ci, nullptr, d_eid, d_perm, &rank, &g->prep, s);
   d_eid = nullptr;  // owned by the preparation buffers from here on
   if (st != GC_OK) return fail(st);
   cudaFreeAsync(d_perm, s);
@@ -602,7 +606,7 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
   GC_CHECK(pool_alloc(&g->d_csum, sizeof(unsigned long long) * (13 * 2 + 17 * 2), s), "alloc sums");
   g->d_x = g->d_csum + 13 * 2;
   {
-    gc_status st2 = scratch_init(&g->sc, g->m, n, g->prep.kmax, g->prep.cnx_max, s);
+    gc_status st2 = scratch_init(&g->sc, g->m, n, g->prep.kmax, s);
     if (st2 != GC_OK) return fail(st2);
     scratch_guess_tlist(&g->sc, g->m);
   }
@@ -702,6 +706,9 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
   dg.gm = g->d_gm;
   dg.table_n = g->n;
   dg.ranked = true;
+  dg.hgeom = g->prep.hgeom;
+  dg.hseg = g->prep.hseg;
+  dg.hpos = g->prep.hpos;
   KUnits ku;
   ku.units = g->prep.kunits;
   ku.cunits = g->prep.cunits;

@@ -278,11 +278,11 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
     k_globalize<<<blocks, 256, 0, s>>>(n, d_rp, d_vgid, d_desc, d_ci);
     GB_TRY(cudaGetLastError(), "k_globalize");
   }
-  if ((st = prepare_graph(n, m, d_rp, d_ci, d_vgid, nullptr, nullptr, &prep, s)) != GC_OK) {
+  if ((st = prepare_graph(n, m, d_rp, d_ci, d_vgid, nullptr, nullptr, nullptr, &prep, s)) != GC_OK) {
     L->error = gc_last_error();
     goto out;
   }
-  if ((st = scratch_init(&sc, m, table_n, prep.kmax, prep.cnx_max, s)) != GC_OK) {
+  if ((st = scratch_init(&sc, m, table_n, prep.kmax, s)) != GC_OK) {
     L->error = gc_last_error();
     goto out;
   }
@@ -306,6 +306,9 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
     dg.gm = d_gm;
     dg.table_n = table_n;
     dg.ranked = false;
+    dg.hgeom = nullptr;
+    dg.hseg = nullptr;
+    dg.hpos = nullptr;
     KUnits ku;
     ku.units = prep.kunits;
     ku.cunits = prep.cunits;

@@ -333,49 +333,46 @@ __global__ void __launch_bounds__(kBlock) k_pass_c(DevGraph g, CountArgs a) {
 // (a few thousand hubs carry almost all of them on power-law graphs) would
 // otherwise hit a vertex-indexed table in DRAM at random. Ids are ranks, so
 // the lower-rank neighbours X of h are a prefix of Gamma(h) and, for x in X,
-// the o < h are a prefix of Gamma(x), ascending. The o-range [0, h) is swept
-// in blocks of a.hub_tab words: cnt_h(o) for the block is built in shared
-// memory from each x's run of o in the block (a per-x cursor walks Gamma(x)
-// once over all blocks; the end of the run is found by galloping search),
-// then the wedges of the block are attributed with the block's counts.
+// the o < h are a prefix of Gamma(x), ascending. The o-range is swept in
+// blocks of a.hub_tab words of shared-memory counters: cnt_h(o) for the block
+// from each x's run of o in it, then the wedges of the block are attributed
+// with the block's counts.
+// Counter widths: cnt_h(o) <= d_o and ids ascend by degree, so the o-range has
+// fixed segments of 2- to 32-bit counters (HubSeg), several to a block; o of
+// degree 1 close no cycle and are skipped. On R-MAT scale 22 the id range of
+// 4.2M takes 8 blocks and 12 segments where blocks of one 10-, 16- or 32-bit
+// width took 31 to 94, so that a run has 100 entries instead of 16 (sweeps of
+// (x, block) 2.2e9 -> 4.4e8), and the segments' bounds in every longer row
+// are looked up in a table made once per graph instead of searched. The
+// whole kernel: 180 -> 128 ms there; 8.5 -> 6.4 ms on Chung-Lu 1M, where
+// about a quarter of the warps' time is still the barrier between a block's
+// two phases, and the shared-memory pipe, with three-way bank conflicts of
+// random counters, is busy half of the time.
 // In both phases a warp works on a chunk of up to 32 x's: for a hub of more
 // than 1024 x's it takes chunks from a shared counter, heaviest first; for a
-// smaller hub each warp keeps one chunk, x = w, w + 32, ..., with its cursors
-// in registers, so that the warps carry equal work. Runs of 32 or more
-// entries are taken by the whole warp one
-// at a time, the shorter ones are dealt to its lanes end to end, so that run
-// lengths, however skewed, do not leave lanes idle, and the P atomics of
-// consecutive lanes hit consecutive slots. The per-x sums of the attribution
-// collect in shared memory (warp sums for long runs, shared atomics for
-// short ones). The block fills shared memory: the longer the runs per block,
-// the more wedges take the whole-warp path.
+// smaller hub each warp keeps one chunk, x = w, w + 32, ..., so that the
+// warps carry about equal work. run_chunk orders the loads of a chunk's runs
+// so that consecutive lanes load, and add to, consecutive slots. The block
+// fills shared memory up to the step of the L1 carveout that kHubTabDefault
+// explains: the longer the runs per block, the fewer the sweeps.
 constexpr int kHeavyBlock = 1024;
 constexpr int kHeavyWarps = kHeavyBlock / 32;
 
-// Counters of the block, kCpw to a word: one 32-bit counter; two 16-bit
-// counters when the unit has fewer than 65536 lower neighbours; three 10-bit
-// counters when it has fewer than 1023 (no count exceeds the number of lower
-// neighbours, so no carry crosses into the next field) -- twice or three
-// times the o-range per block.
-template <int kCpw>
-__device__ __forceinline__ void add_count(uint32_t* tab, int32_t slot) {
-  if (kCpw == 3) {
-    const uint32_t w = (uint32_t)slot / 3u;
-    atomicAdd(&tab[w], 1u << (((uint32_t)slot - 3u * w) * 10u));
-  } else if (kCpw == 2) {
-    atomicAdd(&tab[slot >> 1], 1u << ((slot & 1) << 4));
-  } else {
-    atomicAdd(&tab[slot], 1u);
-  }
+// Counters of a segment, 2^lg to a word (no count of the segment reaches its
+// field's size, so no carry crosses into the next field).
+struct Fields {
+  int lg;         // log2 of the counters per word
+  int sh;         // log2 of a counter's bits
+  uint32_t low;   // counters per word - 1
+  uint32_t mask;  // a counter's bits
+  __device__ __forceinline__ explicit Fields(int l)
+      : lg(l), sh(5 - l), low((1u << l) - 1u), mask(l ? (1u << (32 >> l)) - 1u : 0xffffffffu) {}
+};
+__device__ __forceinline__ void add_count(uint32_t* tab, uint32_t slot, const Fields& f) {
+  atomicAdd(&tab[slot >> f.lg], 1u << ((slot & f.low) << f.sh));
 }
-template <int kCpw>
-__device__ __forceinline__ uint32_t read_count(const uint32_t* tab, int32_t slot) {
-  if (kCpw == 3) {
-    const uint32_t w = (uint32_t)slot / 3u;
-    return (tab[w] >> (((uint32_t)slot - 3u * w) * 10u)) & 1023u;
-  }
-  if (kCpw == 2) return (tab[slot >> 1] >> ((slot & 1) << 4)) & 0xffffu;
-  return tab[slot];
+__device__ __forceinline__ uint32_t read_count(const uint32_t* tab, uint32_t slot, const Fields& f) {
+  return (tab[slot >> f.lg] >> ((slot & f.low) << f.sh)) & f.mask;
 }
 
 // first index in [p, e) with a[index] >= key; a ascending
@@ -436,221 +433,158 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// The counts of one chunk's runs: lane l's run is [st, st + L) of Gamma(x)
-// for its x (L = 0 for none); runs of 32 or more entries are taken by the
-// whole warp one at a time, the shorter ones dealt to the lanes end to end.
-template <int kCpw>
-__device__ __forceinline__ void count_chunk(const DevGraph& g, uint32_t* tab, int32_t* comp, int32_t st, int32_t L,
-                                            int32_t lo_id, int lane) {
-  // runs of 32 or more entries (most of the wedges): the whole warp,
-  // one run at a time, consecutive entries over the lanes
-  unsigned lm = __ballot_sync(0xffffffffu, L >= 32);
+// The runs of one chunk, in one segment: lane l's run is [st, st + L) of
+// Gamma(x) for its x (L = 0 for none), all its o in the segment that starts at
+// lo_id and whose counters start at tab. kAttr = false counts each o; true
+// attributes each wedge: cnt_h(o) - 1 to the slot (x, o), and the sum over the
+// run to `acc` of the run's lane (the slot (h, x)). Entries are loaded 32
+// consecutive ones to a window, in three steps by what the run has left, so
+// that no window is issued for nothing and several loads are in flight:
+// whole blocks of eight windows, one run at a time; the other whole windows,
+// of all runs end to end; and the last < 32 entries of every run, dealt to the
+// lanes end to end. (One step of eight windows for any run of 32 entries or
+// more, as before, left more than half of the windows of runs of about 100
+// entries empty: 75 instructions per 32 wedges on R-MAT scale 18.) Sums over
+// the distinct o of a run stay in 32 bits: cnt_h(o) <= d_o, and all degrees
+// sum to 2m < 2^31.
+template <bool kAttr>
+__device__ __forceinline__ void run_chunk(const DevGraph& g, const CountArgs& a, uint32_t* tab, uint32_t* sx32,
+                                          int32_t* comp, int32_t st, int32_t L, int32_t lo_id, const Fields& f,
+                                          int lane, unsigned long long& acc) {
+  // one window's entry o at slot q; returns its count for the sum
+  auto one = [&](int32_t o, int32_t q) -> uint32_t {
+    const uint32_t slot = (uint32_t)(o - lo_id);
+    if (!kAttr) {
+      add_count(tab, slot, f);
+      return 0u;
+    }
+    const uint32_t cnt = read_count(tab, slot, f) - 1u;
+    if (cnt) atomicAdd(&a.P[q], (unsigned long long)cnt);
+    return cnt;
+  };
+  unsigned lm = __ballot_sync(0xffffffffu, L >= 256);
   while (lm) {
     const int src = __ffs(lm) - 1;
     lm &= lm - 1;
-    const int32_t s0 = __shfl_sync(0xffffffffu, st, src);
-    const int32_t n0 = __shfl_sync(0xffffffffu, L, src);
-    for (int32_t k0 = 0; k0 < n0; k0 += 256) {  // eight windows of loads in flight
+    const int32_t* s0 = g.ci + __shfl_sync(0xffffffffu, st, src);
+    const int32_t n0 = __shfl_sync(0xffffffffu, L, src) & ~255;
+    for (int32_t k = lane; k < n0; k += 256) {
       int32_t o[8];
+      uint32_t sum = 0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int32_t kk = k0 + 32 * j + lane;
-        o[j] = kk < n0 ? g.ci[s0 + kk] : -1;
+      for (int j = 0; j < 8; ++j) o[j] = s0[k + 32 * j];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) sum += one(o[j], (int32_t)(s0 - g.ci) + k + 32 * j);
+      if (kAttr) {
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == src) acc += sum;
       }
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (o[j] >= 0) add_count<kCpw>(tab, o[j] - lo_id);
     }
   }
-  // shorter runs dealt to the lanes end to end
-  const int32_t Ls = L < 32 ? L : 0;
-  const Deal d = deal_setup(Ls, comp, lane);
-  const int32_t sb = st - d.excl;  // slot of position kk of this lane's run: sb + kk
-  int before = 0;
-  for (int32_t k0 = 0; k0 < d.total; k0 += 128) {
-    int32_t q[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int ol = deal_owner(d, Ls, k0 + 32 * j, comp, lane, before);
-      const int32_t kk = k0 + 32 * j + lane;
-      const int32_t bj = __shfl_sync(0xffffffffu, sb, ol);
-      q[j] = kk < d.total ? bj + kk : -1;
+  // whole windows left: at most seven a run
+  st += L & ~255;
+  L &= 255;
+  {
+    int32_t incl = L >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
     }
-    int32_t o[4];
+    const int32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    const int32_t base = st - 32 * (incl - (L >> 5));  // window w of this run starts at base + 32 w
+    for (int32_t w0 = 0; w0 < total; w0 += 4) {
+      int32_t q[4], o[4], own[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) o[j] = q[j] >= 0 ? g.ci[q[j]] : lo_id;
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (q[j] >= 0) add_count<kCpw>(tab, o[j] - lo_id);
-  }
-}
-
-// The attribution of one chunk's wedges (runs as in count_chunk; lane l's x
-// is the i-th lower neighbour, i < nx): cnt_h(o) - 1 to the slot (x, o) of
-// each wedge, and the sum over the run to the slot (h, x).
-template <int kCpw>
-__device__ __forceinline__ void attr_chunk(const DevGraph& g, const CountArgs& a, uint32_t* tab,
-                                           unsigned long long* sx, uint32_t* sx32, int32_t* comp, int32_t st,
-                                           int32_t L, int32_t i, int32_t nx, int32_t hb, int32_t lo_id, int lane) {
-  sx[lane] = 0ull;  // per x of the chunk: sum of its wedges' counts
-  sx32[lane] = 0u;
-  __syncwarp();
-  // runs of 32 or more entries: the whole warp, one run at a time
-  unsigned lm = __ballot_sync(0xffffffffu, L >= 32);
-  while (lm) {
-    const int src = __ffs(lm) - 1;
-    lm &= lm - 1;
-    const int32_t s0 = __shfl_sync(0xffffffffu, st, src);
-    const int32_t n0 = __shfl_sync(0xffffffffu, L, src);
-    unsigned long long acc = 0ull;
-    for (int32_t k0 = 0; k0 < n0; k0 += 256) {  // eight windows of loads in flight
-      int32_t o[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int32_t kk = k0 + 32 * j + lane;
-        o[j] = kk < n0 ? g.ci[s0 + kk] : -1;
+      for (int j = 0; j < 4; ++j) {
+        own[j] = __popc(__ballot_sync(0xffffffffu, incl <= w0 + j)) & 31;  // & 31: past the last window
+        q[j] = __shfl_sync(0xffffffffu, base, own[j]) + 32 * (w0 + j) + lane;
+        o[j] = w0 + j < total ? g.ci[q[j]] : -1;
       }
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (o[j] < 0) continue;
-        const uint32_t cnt = read_count<kCpw>(tab, o[j] - lo_id) - 1u;
-        if (cnt) {
-          atomicAdd(&a.P[s0 + k0 + 32 * j + lane], (unsigned long long)cnt);  // slot (x, o)
-          acc += cnt;
+      for (int j = 0; j < 4; ++j) {
+        if (w0 + j >= total) break;  // warp-uniform
+        uint32_t cnt = one(o[j], q[j]);
+        if (kAttr) {
+          cnt = __reduce_add_sync(0xffffffffu, cnt);
+          if (lane == own[j]) acc += cnt;
         }
       }
     }
-    for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == src) sx[lane] += acc;
   }
-  __syncwarp();
-  // shorter runs dealt to the lanes end to end
-  const int32_t Ls = L < 32 ? L : 0;
-  const Deal d = deal_setup(Ls, comp, lane);
+  // the last entries of every run, dealt to the lanes end to end
+  st += L & ~31;
+  L &= 31;
+  if (kAttr) {
+    sx32[lane] = 0u;
+    __syncwarp();
+  }
+  const Deal d = deal_setup(L, comp, lane);
   const int32_t sb = st - d.excl;  // slot of position kk of this lane's run: sb + kk
   int before = 0;
   for (int32_t k0 = 0; k0 < d.total; k0 += 128) {
-    int32_t q[4], ol[4];
+    int32_t q[4], ol[4], o[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      ol[j] = deal_owner(d, Ls, k0 + 32 * j, comp, lane, before);
+      ol[j] = deal_owner(d, L, k0 + 32 * j, comp, lane, before);
       const int32_t kk = k0 + 32 * j + lane;
       const int32_t bj = __shfl_sync(0xffffffffu, sb, ol[j]);
       q[j] = kk < d.total ? bj + kk : -1;
     }
-    int32_t o[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) o[j] = q[j] >= 0 ? g.ci[q[j]] : lo_id;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      if (q[j] >= 0) {
-        const uint32_t cnt = read_count<kCpw>(tab, o[j] - lo_id) - 1u;
-        if (cnt) {
-          atomicAdd(&a.P[q[j]], (unsigned long long)cnt);  // slot (x, o)
-          atomicAdd(&sx32[ol[j]], cnt);                    // the owner's sum
-        }
-      }
+      if (q[j] < 0) continue;
+      const uint32_t cnt = one(o[j], q[j]);
+      if (kAttr && cnt) atomicAdd(&sx32[ol[j]], cnt);  // the owner's sum
     }
   }
   __syncwarp();
-  if (i < nx) {
-    const unsigned long long sum = sx[lane] + sx32[lane];
-    if (sum) atomicAdd(&a.P[hb + i], sum);  // slot (h, x)
-  }
-}
-
-// One block [lo_id, r1) of a hub job: the counts of the block from each
-// x's run in it (found by galloping search from the x's cursor), then the
-// attribution of the block's wedges, for a hub of more than 1024 lower
-// neighbours: chunks of 32 consecutive x's taken heaviest first (X ascends
-// by degree), their cursors in the CTA's buffers (a smaller hub runs
-// hub_block_small). Called by the whole CTA after the table is zeroed and
-// the chunk counters reset (and a barrier).
-template <int kCpw>
-__device__ __forceinline__ void hub_block(const DevGraph& g, const CountArgs& a, uint32_t* tab, int32_t* s_chunk,
-                                          unsigned long long* sx, uint32_t* sx32, int32_t* comp, int32_t* beg,
-                                          int32_t* cur, const int32_t* endp, int32_t nx, int32_t nchunks,
-                                          int32_t hb, int32_t lo_id, int32_t r1, int lane) {
-  // counts of the block
-  for (;;) {
-    int32_t c = 0;
-    if (lane == 0) c = atomicAdd(&s_chunk[0], 1);
-    c = __shfl_sync(0xffffffffu, c, 0);
-    if (c >= nchunks) break;
-    const int32_t i = (nchunks - 1 - c) * 32 + lane;
-    int32_t st = 0, L = 0;
-    if (i < nx) {
-      st = cur[i];
-      const int32_t en = gallop_lower_bound(g.ci, st, endp[i], r1);
-      L = en - st;
-      beg[i] = st;
-      cur[i] = en;
-    }
-    count_chunk<kCpw>(g, tab, comp, st, L, lo_id, lane);
-    __syncwarp();
-  }
-  __syncthreads();
-  // attribution of the block's wedges
-  for (;;) {
-    int32_t c = 0;
-    if (lane == 0) c = atomicAdd(&s_chunk[1], 1);
-    c = __shfl_sync(0xffffffffu, c, 0);
-    if (c >= nchunks) break;
-    const int32_t i = (nchunks - 1 - c) * 32 + lane;
-    int32_t st = 0, L = 0;
-    if (i < nx) {
-      st = beg[i];
-      L = cur[i] - st;
-    }
-    attr_chunk<kCpw>(g, a, tab, sx, sx32, comp, st, L, i, nx, hb, lo_id, lane);
+  if (kAttr) {
+    acc += sx32[lane];
     __syncwarp();
   }
 }
 
-// One block of a hub of at most 1024 lower neighbours: warp w always takes
-// the chunk x = w, w + 32, ..., so each thread keeps its x's cursor (cur) and
-// run in registers across the two phases and the blocks of the job. Called
-// by the whole CTA after the table is zeroed (and a barrier).
-template <int kCpw>
-__device__ __forceinline__ void hub_block_small(const DevGraph& g, const CountArgs& a, uint32_t* tab,
-                                                unsigned long long* sx, uint32_t* sx32, int32_t* comp,
-                                                int32_t& cur, int32_t endx, int32_t i, int32_t nx, int32_t hb,
-                                                int32_t lo_id, int32_t r1, int lane) {
-  int32_t st = 0, L = 0, en = cur;
-  if (i < nx) {
-    st = cur;
-    en = gallop_lower_bound(g.ci, st, endx, r1);
-    L = en - st;
+// The run {o in Gamma(x) : o in the segment, in the job's o-range [jlo, jhi),
+// o < h} of a lower neighbour x of h: [st, st + L). `k` is the segment's place
+// in its graph; rend the slot of (x, h). Rows with a position table read the
+// segment's bounds there; the others (at most max(31, segments) entries) are
+// searched; a job that starts or ends inside the segment is searched too.
+__device__ __forceinline__ void hub_run(const DevGraph& g, const HubGeom& ge, const HubSeg& sg, int32_t k, int32_t x,
+                                        int32_t rend, int32_t jlo, int32_t jhi, int32_t& st, int32_t& L) {
+  int32_t en;
+  if (x >= ge.xmin) {
+    const int32_t* pp = g.hpos + ge.pos + (int64_t)(x - ge.xmin) * (ge.nseg + 1) + k;
+    st = pp[0];
+    en = min(pp[1], rend);
+    if (jlo > sg.lo) st = gallop_lower_bound(g.ci, st, en, jlo);
+  } else {
+    st = gallop_lower_bound(g.ci, g.rp[x], rend, max(jlo, sg.lo));
+    en = gallop_lower_bound(g.ci, st, rend, sg.hi);
   }
-  count_chunk<kCpw>(g, tab, comp, st, L, lo_id, lane);
-  __syncwarp();
-  __syncthreads();
-  attr_chunk<kCpw>(g, a, tab, sx, sx32, comp, st, L, i, nx, hb, lo_id, lane);
-  __syncwarp();
-  cur = en;
+  if (jhi < sg.hi) en = gallop_lower_bound(g.ci, st, en, jhi);
+  L = max(en - st, 0);
 }
 
 __global__ void __launch_bounds__(kHeavyBlock, 1) k_pass_c_heavy(DevGraph g, CountArgs a) {
   extern __shared__ uint32_t tab[];  // a.hub_tab words of counters
   __shared__ int32_t s_unit, s_nx, s_chunk[2];
   const unsigned long long t_start = global_ns();
-  __shared__ unsigned long long s_sx[kHeavyWarps][32];
   __shared__ uint32_t s_sx32[kHeavyWarps][32];  // the short runs' part (< 32 entries x counts < 2^26)
   __shared__ int32_t s_comp[kHeavyWarps][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int32_t* beg = a.cbuf + (size_t)blockIdx.x * 3 * (size_t)a.cbuf_nx;
-  int32_t* cur = beg + a.cbuf_nx;
-  int32_t* endp = cur + a.cbuf_nx;
   int32_t* comp = s_comp[warp];
-  long long w_wedge = 0, w_blocks = 0, w_jobs = 0;
+  long long w_wedge = 0, w_sweeps = 0, w_jobs = 0;
   for (;;) {
     __syncthreads();
     if (threadIdx.x == 0) s_unit = atomicAdd(a.cursor + 8, 1);
     __syncthreads();
     const int32_t jb = s_unit;
     if (jb >= a.n_cjobs) break;
-    const int4 job = a.cjobs[jb];  // hub (index into cunits), first block, blocks
+    const int4 job = a.cjobs[jb];  // hub (index into cunits), its o-range [y, z), 2 x segment of y + first
     const int32_t h = a.cunits[job.x];
+    const HubGeom ge = g.hgeom[g.vgid ? g.vgid[h] : 0];
     const int32_t hb = g.rp[h], he = g.rp[h + 1];
     if (threadIdx.x == 0) {
       int32_t lo = hb, hi = he;  // first slot of Gamma(h) with id >= h
@@ -662,67 +596,74 @@ __global__ void __launch_bounds__(kHeavyBlock, 1) k_pass_c_heavy(DevGraph g, Cou
     }
     __syncthreads();
     const int32_t nx = s_nx;
-    if (nx > a.cbuf_nx) {  // cannot happen: the buffers are sized for the largest hub
-      if (threadIdx.x == 0) atomicOr(a.status, (int32_t)kSpillOverflow);
-      continue;
-    }
-    // more than 1024 lower neighbours: chunks of 32 consecutive x's (32 of
-    // them at 1024 too, the same in both readings); fewer: one per warp
-    const int32_t nchunks = nx > kHeavyBlock ? (nx + 31) >> 5 : kHeavyWarps;
-    const int cpw = hub_cpw(nx);
-    const int32_t span = cpw * a.hub_tab;
-    const int64_t job_lo = (int64_t)job.y * span;                       // the job's o-range
-    const int64_t job_hi = min((int64_t)h, job_lo + (int64_t)job.z * span);
-    // at most 1024 lower neighbours: this thread's x (chunk = warp) and its
-    // cursor in registers; otherwise the cursors of all x in the CTA's buffers
-    const bool small = nchunks == kHeavyWarps;
-    const int32_t ix = warp + kHeavyWarps * lane;
-    int32_t rcur = 0, rend = 0;
-    if (small) {
-      if (ix < nx) {
-        const int32_t x = g.ci[hb + ix];
-        const int32_t xb = g.rp[x];
-        rend = min(max(g.rev[hb + ix], xb), g.rp[x + 1]);  // Gamma(x) below the slot of (x, h) is < h
-        rcur = job.y == 0 ? xb : gallop_lower_bound(g.ci, xb, rend, (int32_t)job_lo);
-        if (job.y == 0) w_wedge += rend - xb;  // the hub's wedges, counted by its first job
-      }
-    } else {
+    // chunks of 32 x's: of consecutive ones, taken heaviest first (X ascends
+    // by degree) from a shared counter, when there are more than a CTA's
+    // threads; otherwise one chunk per warp, x = warp, warp + 32, ...
+    const bool small = nx <= kHeavyBlock;
+    const int32_t nchunks = small ? kHeavyWarps : (nx + 31) >> 5;
+    if (job.w & 1) {  // the hub's wedges, counted by its first job
       for (int32_t i = threadIdx.x; i < nx; i += kHeavyBlock) {
-        const int32_t x = g.ci[hb + i];
-        const int32_t xb = g.rp[x];
-        const int32_t lo = min(max(g.rev[hb + i], xb), g.rp[x + 1]);  // Gamma(x) below the slot of (x, h) is < h
-        cur[i] = job.y == 0 ? xb : gallop_lower_bound(g.ci, xb, lo, (int32_t)job_lo);
-        endp[i] = lo;
-        if (job.y == 0) w_wedge += lo - xb;  // the hub's wedges, counted by its first job
+        const int32_t xb = g.rp[g.ci[hb + i]];
+        w_wedge += max(g.rev[hb + i], xb) - xb;  // Gamma(x) below the slot of (x, h) is < h
       }
     }
     if (threadIdx.x == 0) ++w_jobs;
-    for (int64_t lo64 = job_lo; lo64 < job_hi; lo64 += span) {
-      const int32_t lo_id = (int32_t)lo64;
-      const int32_t r1 = (int32_t)min(lo64 + span, job_hi);
-      const int32_t words = (r1 - lo_id + cpw - 1) / cpw;
+    const int32_t jlo = job.y, jhi = job.z, seg_end = ge.seg + ge.nseg;
+    const int32_t jcut = jhi == h ? 0x7fffffff : jhi;  // runs end below h by themselves
+    // this thread's x when its chunk is fixed
+    int32_t rx = 0, rrend = 0;
+    const int32_t ri = warp + kHeavyWarps * lane;
+    if (small && ri < nx) {
+      rx = g.ci[hb + ri];
+      rrend = min(max(g.rev[hb + ri], g.rp[rx]), g.rp[rx + 1]);
+    }
+    for (int32_t s0 = job.w >> 1, s1; s0 < seg_end && g.hseg[s0].lo < jhi; s0 = s1) {
+      // one block: segments [s0, s1)
+      int32_t words = 0;
+      const int32_t w0 = g.hseg[s0].word;
+      for (s1 = s0; s1 < seg_end;) {
+        const HubSeg sg = g.hseg[s1];
+        if (sg.lo >= jhi) break;
+        words = sg.word - w0 + ((min(sg.hi, jhi) - sg.lo + (1 << sg.lg) - 1) >> sg.lg);
+        ++s1;
+        if (sg.last) break;
+      }
       for (int32_t i = threadIdx.x; i < words; i += kHeavyBlock) tab[i] = 0u;
       if (threadIdx.x == 0) {
-        w_blocks += nx;
+        w_sweeps += (long long)nx * (s1 - s0);
         s_chunk[0] = 0;
         s_chunk[1] = 0;
       }
       __syncthreads();
-      if (small) {
-        if (cpw == 3)
-          hub_block_small<3>(g, a, tab, s_sx[warp], s_sx32[warp], comp, rcur, rend, ix, nx, hb, lo_id, r1, lane);
-        else
-          hub_block_small<2>(g, a, tab, s_sx[warp], s_sx32[warp], comp, rcur, rend, ix, nx, hb, lo_id, r1, lane);
-      } else if (cpw == 3)
-        hub_block<3>(g, a, tab, s_chunk, s_sx[warp], s_sx32[warp], comp, beg, cur, endp, nx, nchunks, hb, lo_id, r1,
-                     lane);
-      else if (cpw == 2)
-        hub_block<2>(g, a, tab, s_chunk, s_sx[warp], s_sx32[warp], comp, beg, cur, endp, nx, nchunks, hb, lo_id, r1,
-                     lane);
-      else
-        hub_block<1>(g, a, tab, s_chunk, s_sx[warp], s_sx32[warp], comp, beg, cur, endp, nx, nchunks, hb, lo_id, r1,
-                     lane);
-      __syncthreads();
+      for (int phase = 0; phase < 2; ++phase) {  // the block's counts, then the attribution of its wedges
+        for (int32_t c = 0;;) {
+          if (!small) {
+            if (lane == 0) c = atomicAdd(&s_chunk[phase], 1);
+            c = __shfl_sync(0xffffffffu, c, 0);
+            if (c >= nchunks) break;
+          }
+          const int32_t i = small ? ri : (nchunks - 1 - c) * 32 + lane;
+          int32_t x = rx, rend = rrend;
+          if (!small && i < nx) {
+            x = g.ci[hb + i];
+            rend = min(max(g.rev[hb + i], g.rp[x]), g.rp[x + 1]);
+          }
+          unsigned long long acc = 0;  // this x's wedges' counts
+          for (int32_t s = s0; s < s1; ++s) {
+            const HubSeg sg = g.hseg[s];
+            const Fields f(sg.lg);
+            int32_t st = 0, L = 0;
+            if (i < nx) hub_run(g, ge, sg, s - ge.seg, x, rend, jlo, jcut, st, L);
+            if (phase == 0)
+              run_chunk<false>(g, a, tab + (sg.word - w0), s_sx32[warp], comp, st, L, sg.lo, f, lane, acc);
+            else
+              run_chunk<true>(g, a, tab + (sg.word - w0), s_sx32[warp], comp, st, L, sg.lo, f, lane, acc);
+          }
+          if (acc) atomicAdd(&a.P[hb + i], acc);  // slot (h, x); only runs of x in [0, nx) add to acc
+          if (small) break;
+        }
+        __syncthreads();
+      }
     }
   }
   for (int o = 16; o; o >>= 1) w_wedge += __shfl_xor_sync(0xffffffffu, w_wedge, o);
@@ -731,7 +672,7 @@ __global__ void __launch_bounds__(kHeavyBlock, 1) k_pass_c_heavy(DevGraph g, Cou
     atomicAdd(a.work + kWorkCHeavyWedge, (unsigned long long)w_wedge);
   }
   if (threadIdx.x == 0) {
-    if (w_blocks) atomicAdd(a.work + kWorkCBlocks, (unsigned long long)w_blocks);
+    if (w_sweeps) atomicAdd(a.work + kWorkCBlocks, (unsigned long long)w_sweeps);
     if (w_jobs) atomicAdd(a.work + kWorkCHubJobs, (unsigned long long)w_jobs);
     const unsigned long long life = global_ns() - t_start;
     atomicAdd(a.work + kWorkCHubCtas, 1ull);
@@ -1071,7 +1012,7 @@ gc_status run_pass_c(const DevGraph& g, const CountArgs& a, cudaStream_t s) {
 }
 
 gc_status run_pass_c_heavy(const DevGraph& g, const CountArgs& a, cudaStream_t s) {
-  if (a.n_cheavy <= 0) return GC_OK;
+  if (a.n_cheavy <= 0 || !g.hgeom) return GC_OK;
   const size_t smem = sizeof(uint32_t) * (size_t)a.hub_tab;
   cudaError_t e = cudaFuncSetAttribute(k_pass_c_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return cuda_fail(e, "k_pass_c_heavy");

@@ -12,6 +12,27 @@ namespace gc {
 
 typedef unsigned __int128 u128;
 
+// The o-range of the hub kernel of pass C, laid out once per ranked graph: a
+// vertex of degree 1 closes no 4-cycle, and a count of o never exceeds d_o, so
+// ids, which ascend by degree, split at these degrees into classes of 2-, 4-,
+// 8-, 16- and 32-bit counters (kOBoundDeg[k] is where class k starts).
+constexpr int kOBounds = 5;
+constexpr int kOBoundDeg[kOBounds] = {2, 4, 16, 256, 65536};
+// One segment: ids [lo, hi), 2^lg counters to a 32-bit word, from word `word`
+// of the count block. Consecutive segments share a block until one is `last`.
+struct HubSeg {
+  int32_t lo, hi, word;
+  int16_t lg, last;
+};
+// Segments of one graph, and the places of its segment bounds in the rows:
+// row x >= xmin (the rows of at least 32 entries and of more entries than
+// bounds) has, for its k-th segment, its first slot of id >= lo, and the slot
+// past the last segment: hpos[pos + (x - xmin) * (nseg + 1) + k].
+struct HubGeom {
+  int32_t seg, nseg, xmin, end;
+  int64_t pos;
+};
+
 // Device view of a (possibly multi-graph) CSR. A batch of graphs is counted
 // as their disjoint union: vertices of graph g occupy the global id range
 // [gbase[g], gbase[g] + gn[g]); per-edge x3/x7/x10 of a disjoint union equal
@@ -36,6 +57,9 @@ struct DevGraph {
   const int64_t* gm;       // [G] edges of each graph
   int32_t table_n;         // max gn[g]: size of one Psi table
   bool ranked;             // ids are the (degree, id) ranks and rows ascend
+  const HubGeom* hgeom;    // ranked: [G] (nullptr when the graph has no hub units)
+  const HubSeg* hseg;
+  const int32_t* hpos;
 };
 
 // Pass K (4-cliques and cross terms by lowest vertex) runs in tiers by the
@@ -57,11 +81,9 @@ struct CountArgs {
   int32_t n_chash_big;     // hashed units of more than kHashSmallW wedges (the first of them)
   int32_t n_chash2;        // units of the packed-key hash tier, after the hashed units
   int32_t n_chash2_big;    // of them, units of more than kHash2HalfMaxW wedges (the first)
-  const int4* cjobs;       // pass C hub kernel: jobs (hub index into cunits, first o-range block, blocks),
-                           // heaviest first
+  const int4* cjobs;       // pass C hub kernel: jobs (hub index into cunits, o-range [y, z), twice the
+                           // segment of y, + 1 for the hub's first job), heaviest first
   int32_t n_cjobs;
-  int32_t* cbuf;           // pass C hub kernel: per-CTA cursors (cbuf_ctas x 3 x cbuf_nx ints)
-  int32_t cbuf_nx;
   int32_t hub_tab;         // pass C hub kernel: words of the count block (hub_tab_words())
   const int32_t* kunits;   // pass K: lowest vertices a with |out(a)| >= 2, tiers in KTier order
   int32_t ktier_off[kNumTiers + 1];  // tier t = kunits[ktier_off[t] .. ktier_off[t + 1])
@@ -141,8 +163,6 @@ struct Scratch {
   unsigned long long* P = nullptr;   // [2m]
   unsigned long long* xc = nullptr;  // [m][2]
   int32_t* misc = nullptr;           // [32] cursors, status
-  int32_t* cbuf = nullptr;           // pass C hub cursors
-  int32_t cbuf_nx = 0;
   uint32_t* tables = nullptr;        // count_grid_size() x table_n
   size_t tables_n = 0;
   unsigned char* kbuf = nullptr;     // pass K global tier
@@ -166,7 +186,7 @@ struct Scratch {
 };
 // Allocates the scratch of a graph with m edges, Psi tables of table_n
 // vertices and largest out-degree kmax (stream-ordered).
-gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, int32_t cnx_max, cudaStream_t s);
+gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, cudaStream_t s);
 void scratch_free(Scratch* sc, cudaStream_t s);
 // Size of pass T's edge lists for the first count of a whole graph with m
 // edges: 32 m entries within the list budget (units past it scan again).
@@ -255,7 +275,18 @@ struct PrepBuffers {
   int32_t n_chash2 = 0;        // units of the packed-key hash tier
   int32_t n_chash2_big = 0;    // of them, units of more than kHash2HalfMaxW wedges
   int32_t n_cunits = 0;
-  int32_t cnx_max = 0;      // most lower neighbours of a hub unit
+  HubGeom* hgeom = nullptr;    // layout of the hub kernel's o-range (owns hseg's block)
+  HubSeg* hseg = nullptr;
+  int32_t* hpos = nullptr;
+};
+// What the host knows of a ranked graph (ids = ranks, rows ascending) when it
+// is prepared.
+struct RankInfo {
+  const int32_t* rp;      // [n + 1] internal row pointers
+  int32_t G;              // graphs, each a range of ids
+  const int32_t* gbase;   // [G] first id of each, ascending
+  const int32_t* gn;      // [G] vertices of each
+  const int32_t* obound;  // [G][kOBounds] first id of degree >= kOBoundDeg[k] (the graph's end if none)
 };
 // Builds degrees, edge ids, the edge list, degree-oriented out-lists and the
 // binned unit list on `stream`. vgid may be nullptr (single graph).
@@ -264,13 +295,13 @@ struct PrepBuffers {
 // vertex id, used to write the edge list in the caller's labels.
 gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t* d_ci,
                         const int32_t* d_vgid, int32_t* d_eid_given, const int32_t* d_perm,
-                        PrepBuffers* out, cudaStream_t stream);
+                        const RankInfo* rank, PrepBuffers* out, cudaStream_t stream);
 // Splits the pass-C units of a ranked graph (ids = ranks, rows ascending)
 // into hub units for the blocked kernel, units of at most kHashMaxW wedges
 // for the hashed kernel and the rest, leaving out units without wedges
-// (fills cunits, n_cheavy, chash_w, n_chash, n_cunits, cnx_max; otherwise
+// (fills cunits, n_cheavy, chash_w, n_chash, n_cunits; otherwise
 // cunits is a copy of units).
-gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, bool ranked, PrepBuffers* p,
+gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, const RankInfo* rank, PrepBuffers* p,
                            cudaStream_t stream);
 void free_prep(PrepBuffers* p, cudaStream_t s);
 // Smallest slot p with rev[p] == p (no reverse: the input is not symmetric),
@@ -324,10 +355,10 @@ constexpr int kHeavyTab = 53248;  // largest o-range block of the hub kernel of 
 // 45056, 213.3 at 39936, 226.7 at 32768).
 constexpr int kHubTabDefault = 45056;
 int hub_tab_words();
-// Counters per word of the hub kernel for a unit of nx lower neighbours
-// (count fields of 32, 16 or 10 bits; no count exceeds nx): one block of
-// its o-range spans hub_cpw(nx) * hub_tab_words() ids.
-__host__ __device__ __forceinline__ int hub_cpw(int64_t nx) { return nx < 1023 ? 3 : nx < 65536 ? 2 : 1; }
+// Counters per word that a unit of nx lower neighbours could use over its
+// whole o-range by nx alone; the rule that picks the hub units estimates
+// their blocks with it.
+inline int hub_cpw(int64_t nx) { return nx < 1023 ? 3 : nx < 65536 ? 2 : 1; }
 // Units of pass C with at most kHashMaxW wedges count in a shared-memory
 // hash of 2 kHashMaxW keys (at most half full: a unit has no more distinct
 // o than wedges).

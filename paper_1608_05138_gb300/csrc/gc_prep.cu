@@ -267,6 +267,17 @@ __global__ void k_cwork(int32_t n_units, const int32_t* __restrict__ units, cons
   }
 }
 
+// DevGraph::hpos of the rows of one graph: thread per (row, bound).
+__global__ void k_hub_pos(HubGeom ge, const HubSeg* __restrict__ seg, const int32_t* __restrict__ rp,
+                          const int32_t* __restrict__ ci, int32_t* __restrict__ pos) {
+  const int64_t per = ge.nseg + 1, total = (int64_t)(ge.end - ge.xmin) * per;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t x = ge.xmin + (int32_t)(t / per), k = (int32_t)(t % per);
+    const int32_t id = k < ge.nseg ? seg[ge.seg + k].lo : seg[ge.seg + k - 1].hi;
+    pos[ge.pos + t] = lower_bound_i32(ci, rp[x], rp[x + 1], id);
+  }
+}
+
 // Smallest slot whose reverse was not found (rev[p] == p): the input is not
 // symmetric exactly when there is one.
 __global__ void k_first_unreversed(int64_t nnz, const int32_t* __restrict__ rev, int32_t* __restrict__ first) {
@@ -447,7 +458,7 @@ static void sort_by_wedges_desc(std::vector<int32_t>* v, const std::vector<long 
   v->swap(out);
 }
 
-gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, bool ranked, PrepBuffers* p,
+gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, const RankInfo* rank, PrepBuffers* p,
                            cudaStream_t s) {
   const int32_t nu = p->n_units;
   cudaError_t e = pool_alloc(&p->cunits, sizeof(int32_t) * (nu > 0 ? nu : 1), s);
@@ -459,8 +470,7 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
   p->n_chash2 = 0;
   p->n_chash2_big = 0;
   p->n_cunits = nu;
-  p->cnx_max = 0;
-  if (!ranked || n <= kSmemTableMax || nu == 0) {
+  if (!rank || n <= kSmemTableMax || nu == 0) {
     e = nu > 0 ? cudaMemcpyAsync(p->cunits, p->units, sizeof(int32_t) * nu, cudaMemcpyDeviceToDevice, s) : cudaSuccess;
     return e == cudaSuccess ? GC_OK : cuda_fail(e, "copy cunits");
   }
@@ -522,10 +532,7 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
   out.reserve(heavy.size() + hashed.size() + hashed2.size() + rest.size());
   std::vector<int32_t> hw;
   hw.reserve(hashed.size() + hashed2.size());
-  for (int32_t k : heavy) {
-    out.push_back(U[k]);
-    if (NX[k] > p->cnx_max) p->cnx_max = NX[k];
-  }
+  for (int32_t k : heavy) out.push_back(U[k]);
   for (int32_t k : hashed) {
     out.push_back(U[k]);
     hw.push_back((int32_t)W[k]);
@@ -545,41 +552,112 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
   p->n_chash2_big = 0;  // heaviest first too
   while (p->n_chash2_big < p->n_chash2 && W[hashed2[(size_t)p->n_chash2_big]] > kHash2HalfMaxW) ++p->n_chash2_big;
   p->n_cunits = (int32_t)out.size();
-  // Hub units cut into jobs of consecutive o-range blocks (the finer
-  // granularity of Sec. 4.4: one hub's work spread over several CTAs), so
-  // that the heaviest hubs do not end as one SM's serial tail. A unit's cost
-  // is estimated as its wedges plus kSweepCost per (lower neighbour, block)
-  // sweep; a unit is cut into about cost / target jobs, target = total cost
-  // over jobs_per_cta x the hub kernel's CTAs (GC_HUB_JOBS_PER_CTA, default 1;
-  // 0: one job per hub). Jobs are taken heaviest first.
+  // The hub kernel's o-range (see HubSeg): per graph, each degree class in
+  // order, cut where a count block is full.
+  std::vector<HubSeg> segs;
+  std::vector<HubGeom> geom;
+  int64_t n_pos = 0;
+  if (!heavy.empty()) {
+    for (int32_t gi = 0; gi < rank->G; ++gi) {
+      const int32_t* ob = rank->obound + (size_t)gi * kOBounds;
+      const int32_t end = rank->gbase[gi] + rank->gn[gi];
+      HubGeom ge = {(int32_t)segs.size(), 0, end, end, n_pos};
+      int32_t word = 0;
+      for (int c = 0; c < kOBounds; ++c) {
+        const int lg = kOBounds - 1 - c;
+        const int32_t ce = c + 1 < kOBounds ? ob[c + 1] : end;
+        for (int32_t lo = ob[c]; lo < ce;) {
+          const int32_t hi = (int32_t)std::min<int64_t>(ce, lo + ((tab - word) << lg));
+          segs.push_back({lo, hi, word, (int16_t)lg, 0});
+          word += (hi - lo + (1 << lg) - 1) >> lg;
+          if (word >= tab || hi == end) {
+            segs.back().last = 1;
+            word = 0;
+          }
+          lo = hi;
+        }
+      }
+      ge.nseg = (int32_t)segs.size() - ge.seg;
+      if (ge.nseg > 0) {
+        // rows of at least max(32, bounds) entries: the last ids
+        const int32_t least = std::max(32, ge.nseg + 1);
+        int32_t a = rank->gbase[gi], b = end;
+        while (a < b) {
+          const int32_t mid = a + (b - a) / 2;
+          if (rank->rp[mid + 1] - rank->rp[mid] < least) a = mid + 1; else b = mid;
+        }
+        ge.xmin = a;
+        n_pos += (int64_t)(end - a) * (ge.nseg + 1);
+      }
+      geom.push_back(ge);
+    }
+  }
+  // Hub units cut into jobs of consecutive o-ranges (the finer granularity of
+  // Sec. 4.4: one hub's work spread over several CTAs), so that the heaviest
+  // hubs do not end as one SM's serial tail. A unit's cost is estimated as
+  // its wedges plus kSweepCost per (lower neighbour, segment) sweep; a unit is
+  // cut into about cost / target jobs, target = total cost over jobs_per_cta
+  // x the hub kernel's CTAs (GC_HUB_JOBS_PER_CTA, default 1; 0: one job per
+  // hub), at ids that split the entries of its o-range's rows evenly (an o
+  // is met about in proportion to its degree). A job looks at every lower
+  // neighbour, so it keeps at least kJobWedges wedges and eight for each of
+  // them. Jobs are taken heaviest first.
   std::vector<int4> jobs;
-  {
+  if (!heavy.empty()) {
     constexpr double kSweepCost = 4.0;
+    constexpr long long kJobWedges = 8192;
     const int per_cta = hub_jobs_per_cta();
+    auto geom_of = [&](int32_t h) -> const HubGeom& {
+      return geom[(size_t)(std::upper_bound(rank->gbase, rank->gbase + rank->G, h) - rank->gbase) - 1];
+    };
+    auto seg_of = [&](const HubGeom& ge, int32_t id) {  // the segment holding id (the last one past the end)
+      int32_t k = ge.seg;
+      while (k + 1 < ge.seg + ge.nseg && segs[(size_t)k].hi <= id) ++k;
+      return k;
+    };
     std::vector<double> cost(heavy.size());
-    std::vector<long long> nblk(heavy.size());
     double total = 0;
     for (size_t i = 0; i < heavy.size(); ++i) {
       const int32_t k = heavy[i];
-      const long long span = (long long)hub_cpw(NX[k]) * hub_tab_words();
-      nblk[i] = ((long long)U[k] + span - 1) / span;
-      cost[i] = (double)W[k] + kSweepCost * (double)NX[k] * (double)nblk[i];
+      const HubGeom& ge = geom_of(U[k]);
+      cost[i] = (double)W[k] + kSweepCost * (double)NX[k] * (double)(seg_of(ge, U[k]) - ge.seg + 1);
       total += cost[i];
     }
     const double target = per_cta > 0 ? total / ((double)(count_grid_size() / kCtasPerSm) * per_cta) : 0.0;
     std::vector<std::pair<double, int4>> cj;
     for (size_t i = 0; i < heavy.size(); ++i) {
+      const int32_t h = U[heavy[i]];
+      const HubGeom& ge = geom_of(h);
+      const int32_t lo = ge.nseg > 0 ? std::min(segs[(size_t)ge.seg].lo, h) : h;
       long long J = target > 0 ? (long long)std::ceil(cost[i] / target) : 1;
-      J = std::max(1LL, std::min(J, nblk[i]));
-      const long long nb = (nblk[i] + J - 1) / J;
-      for (long long b0 = 0; b0 < nblk[i]; b0 += nb) {
-        const long long len = std::min(nb, nblk[i] - b0);
-        cj.push_back({cost[i] * (double)len / (double)nblk[i], make_int4((int)i, (int)b0, (int)len, 0)});
+      J = std::max(1LL, std::min(J, W[heavy[i]] / std::max(kJobWedges, 8LL * NX[heavy[i]])));
+      int32_t from = lo;
+      for (long long j = 1; j <= J; ++j) {
+        const long long upto = rank->rp[lo] + (long long)(rank->rp[h] - rank->rp[lo]) * j / J;
+        const int32_t to =
+            j == J ? h : (int32_t)(std::upper_bound(rank->rp + lo, rank->rp + h, (int32_t)upto) - rank->rp) - 1;
+        if (to <= from && (j < J || from > lo)) continue;  // nothing in this share (a hub keeps at least one job)
+        cj.push_back({cost[i] / (double)J, make_int4((int)i, from, to, 2 * seg_of(ge, from) + (from == lo))});
+        from = to;
       }
     }
     std::stable_sort(cj.begin(), cj.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
     jobs.reserve(cj.size());
     for (auto& c : cj) jobs.push_back(c.second);
+    // device copies: the geometry and the segments in one block, and the rows' positions
+    const size_t gb = sizeof(HubGeom) * geom.size(), sb = sizeof(HubSeg) * segs.size();
+    e = pool_alloc(&p->hgeom, gb + sb + sizeof(HubSeg), s);
+    if (e == cudaSuccess) p->hseg = reinterpret_cast<HubSeg*>(p->hgeom + geom.size());
+    if (e == cudaSuccess) e = cudaMemcpyAsync(p->hgeom, geom.data(), gb, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && sb) e = cudaMemcpyAsync(p->hseg, segs.data(), sb, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = pool_alloc(&p->hpos, sizeof(int32_t) * (size_t)(n_pos > 0 ? n_pos : 1), s);
+    for (const HubGeom& ge : geom) {
+      const int64_t work = (int64_t)(ge.end - ge.xmin) * (ge.nseg + 1);
+      if (e != cudaSuccess || ge.nseg == 0 || work == 0) continue;
+      k_hub_pos<<<grid_for(work, 256), 256, 0, s>>>(ge, p->hseg, d_rp, d_ci, p->hpos);
+      e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "hub layout");
   }
   p->n_cjobs = (int32_t)jobs.size();
   if (!jobs.empty()) {
@@ -631,12 +709,14 @@ void free_prep(PrepBuffers* p, cudaStream_t s) {
   if (p->cunits) cudaFreeAsync(p->cunits, s);
   if (p->cjobs) cudaFreeAsync(p->cjobs, s);
   if (p->chash_w) cudaFreeAsync(p->chash_w, s);
+  if (p->hgeom) cudaFreeAsync(p->hgeom, s);
+  if (p->hpos) cudaFreeAsync(p->hpos, s);
   *p = PrepBuffers();
 }
 
 gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t* d_ci,
                         const int32_t* d_vgid, int32_t* d_eid_given, const int32_t* d_perm,
-                        PrepBuffers* out, cudaStream_t s) {
+                        const RankInfo* rank, PrepBuffers* out, cudaStream_t s) {
   (void)d_vgid;
   PrepBuffers P;
   P.eid = d_eid_given;
@@ -733,7 +813,7 @@ gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t
   } else {
     GC_TRY(cudaMemsetAsync(P.out_ptr, 0, sizeof(int32_t), s), "memset out_ptr");
   }
-  if ((st = classify_c_units(n, d_rp, d_ci, d_perm != nullptr, &P, s)) != GC_OK) goto fail;
+  if ((st = classify_c_units(n, d_rp, d_ci, rank, &P, s)) != GC_OK) goto fail;
   cudaFreeAsync(up, s);
   cudaFreeAsync(upoff, s);
   cudaFreeAsync(out_cnt, s);

@@ -48,14 +48,14 @@ long long t_list_cap_knob() {
 
 void scratch_free(Scratch* sc, cudaStream_t s) {
   for (void* p : {(void*)sc->trio, (void*)sc->P, (void*)sc->xc, (void*)sc->misc,
-                  (void*)sc->cbuf, (void*)sc->tables, (void*)sc->kbuf, (void*)sc->hitbuf, (void*)sc->work,
+                  (void*)sc->tables, (void*)sc->kbuf, (void*)sc->hitbuf, (void*)sc->work,
                   (void*)sc->tlist, (void*)sc->tl_off, (void*)sc->tl_cnt, (void*)sc->tl_fill, (void*)sc->dsum,
                   (void*)sc->vsum})
     if (p) cudaFreeAsync(p, s);
   *sc = Scratch();
 }
 
-gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, int32_t cnx_max, cudaStream_t s) {
+gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
 #define GS_TRY(call)                                \
   do {                                              \
@@ -72,10 +72,6 @@ gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, in
     sc->tables_n = (size_t)count_grid_size() * (size_t)table_n;
     GS_TRY(pool_alloc(&sc->tables, sizeof(uint32_t) * sc->tables_n, s));
     GS_TRY(cudaMemsetAsync(sc->tables, 0, sizeof(uint32_t) * sc->tables_n, s));
-  }
-  if (cnx_max > 0) {
-    sc->cbuf_nx = cnx_max;
-    GS_TRY(pool_alloc(&sc->cbuf, sizeof(int32_t) * 3 * (size_t)cnx_max * (size_t)(count_grid_size() / kCtasPerSm), s));
   }
   {  // pass K: each CTA records the edges of its current H_a (at most C(kmax, 2))
     const long long full = (long long)kmax * (kmax - 1) / 2;
@@ -131,8 +127,6 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
   a.n_chash_mid = ku.n_chash_mid;
   a.n_chash2_big = ku.n_chash2_big;
   a.n_chash2 = ku.n_chash2;
-  a.cbuf = sc->cbuf;
-  a.cbuf_nx = sc->cbuf_nx;
   a.hub_tab = hub_tab_words();
   for (int t = 0; t <= kNumTiers; ++t) a.ktier_off[t] = ku.tier_off[t];
   a.cursor = sc->misc;  // [0] pass C, [2 + tier] pass K, [8] pass C hubs, [9] pass C hashed, [10 + tier] pass T,

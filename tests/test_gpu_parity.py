@@ -232,6 +232,26 @@ def test_hub_counts_near_the_10_bit_field_limit():
     assert w["c_heavy_wedges"] >= 54000 and w["c_wedges"] == W.sum()
 
 
+@pytest.mark.parametrize("nx,per", [(1100, 40), (900, 100)])
+def test_hub_counts_at_the_counter_field_limits(nx, per):
+    # h joined to nx vertices x (in registers up to 1024 of them, in the CTA's
+    # cursor buffers above); o of degree 15, 16, 255 and 256, all of whose
+    # neighbours are x, so that cnt_h(o) = d_o: the largest counts of the 4-
+    # and 8-bit fields and the smallest of the next ones
+    rng = np.random.default_rng(nx)
+    E = [(0, x) for x in range(1, nx + 1)]
+    o = nx + 1
+    for d in (15, 16, 255, 256):
+        for _ in range(per):
+            E += [(o, int(x)) for x in rng.choice(nx, d, replace=False) + 1]
+            o += 1
+    rp, ci = graphs.csr_large(20_000, E)
+    W, nb = wedges_by_highest_vertex(rp, ci)
+    w = _count_with_work(rp, ci)
+    assert W[0] == per * (15 + 16 + 255 + 256) and nb[0] == nx
+    assert w["c_heavy_wedges"] >= W[0] and w["c_wedges"] == W.sum()
+
+
 def test_hub_over_a_skewed_o_range():
     # 3M vertices, almost all isolated (the lowest ranks): h has 620 lower
     # neighbours, 600 of them with 150 o each, drawn with weights 1/(i + 100)

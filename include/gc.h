@@ -320,8 +320,8 @@ gc_status gc_batch_last_stats(gc_batch b, double* out);
  * allocator callback, a budget that forbids growth). The
  * paper has no counterpart: it is a variant of the triangle step that reads
  * the caller's device CSR in place and uses, as its only scratch, a 32 MiB
- * file-scope device array (256 bitmaps of 2^20 bits) that every GPU loading
- * libgc.so holds until the process exits.
+ * file-scope device array that every GPU loading libgc.so holds until the
+ * process exits.
  *   n        vertices, 0 <= n <= 1,048,576; larger n returns GC_ERR_OVERFLOW
  *   row_ptr  device pointer, n + 1 int32 (same CSR rules as gc_graph_upload;
  *            not validated here: a column index outside [0, n) is skipped,
@@ -335,9 +335,8 @@ gc_status gc_batch_last_stats(gc_batch b, double* out);
  * (cudaGetSymbolAddress) -- make that first call before any stream capture.
  * The address is kept per device ordinal for the life of the process: it
  * assumes the runtime's primary context and no cudaDeviceReset afterwards.
- * All calls share the array and each call clears it first: calls whose
- * kernels overlap on the GPU (other streams, other threads) race and give
- * wrong results.
+ * All calls share the array: calls whose kernels overlap on the GPU (other
+ * streams, other threads) race and give wrong results.
  */
 gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr, const int32_t* col_idx, int32_t* tri_out,
                                     void* stream);

@@ -3,15 +3,32 @@
 // Callers that own a fixed memory arena, or that run where a device
 // allocation may not happen at all (inside another allocator's callback,
 // under a hard budget that forbids growth), cannot use gc_graph_upload: it
-// allocates the CSR copy, the preparation arrays and the per-CTA tables. This entry point is a variant
-// of the triangle step (Alg. 1: a Psi bitmap of Gamma(x), probed with the
-// neighbours of each neighbour) that works directly on the caller's device
-// CSR and writes the caller's device output. Its only scratch -- one bitmap
-// per CTA marking Gamma(x) -- lives in a file-scope __device__ array that
-// every GPU loading the library holds until the process exits:
-//   kNoAllocCtas bitmaps x kNoAllocMaxN bits = 256 x 1,048,576 bits = 32 MiB.
-// Graphs with more than kNoAllocMaxN vertices are rejected. A column index
-// outside [0, n) is skipped (it would otherwise touch another CTA's bitmap).
+// allocates the CSR copy, the preparation arrays and the per-CTA tables. This
+// entry point is a variant of the triangle step (Alg. 1) that works directly
+// on the caller's device CSR and writes the caller's device output. Its only
+// scratch lives in a file-scope __device__ array of 32 MiB that every GPU
+// loading the library holds until the process exits. Graphs with more than
+// kNoAllocMaxN vertices are rejected.
+//
+// tri[p] of the slot p = (x, y) is the number of entries of row y that are in
+// row x. In a simple symmetric graph the slots of both directions agree, so
+// each edge is counted once, at its end of higher (degree, id): the entries of
+// the shorter row are looked up in a set of the longer one. That is
+// sum min(d_x, d_y) lookups over the edges, where looking up row y in a bitmap
+// of row x for every slot, in global memory, took sum d^2 (Chung-Lu, 100 003
+// vertices, 1 000 003 edges, exponent 2.3: 2.2e9 lookups and 7.9 ms for a
+// pass, 0.60 ms now: 38 us k_rows, 226 k_tri_long, 224 k_tri_short, 66
+// k_tri_reverse, all waiting on chains of dependent loads).
+//   k_rows   marks the rows that break the CSR rules (not strictly ascending,
+//            a column out of range, a self-loop) and lists the long rows
+//   k_tri_long, k_tri_short   the slots (x, y), y below x in (degree, id): a CTA
+//            per part of a long row with a bitmap of the vertices in shared
+//            memory, a warp per other row with a hash of at most 128 entries
+//   k_tri_reverse   the other slots, from the reverse slot (a binary search);
+//            slots without one, or with an end whose row breaks the rules, are
+//            marked
+//   k_tri_marked    the marked slots by the definition, with a bitmap per CTA in
+//            the scratch array (nothing to do for a valid graph)
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -23,11 +40,28 @@ namespace gc {
 namespace {
 
 constexpr int32_t kNoAllocMaxN = 1 << 20;              // vertices
-constexpr int kNoAllocCtas = 256;                      // CTAs, one bitmap each
-constexpr int kNoAllocWords = kNoAllocMaxN / 32;       // 32-bit words per bitmap
+constexpr int kNoAllocWords = kNoAllocMaxN / 32;       // 32-bit words of a bitmap of the vertices
+constexpr int kNoAllocCtas = 192;                      // CTAs of k_tri_marked, one bitmap each
 constexpr int kNoAllocBlock = 512;
+// Scratch layout, in 32-bit words: counters, a bit per row that breaks the
+// CSR rules, the list of long rows, the bitmaps of k_tri_marked.
+enum { kCurLong = 0, kNumLong, kCurShort, kNumMarked, kNumCounters };
+constexpr size_t kOffBad = 32;
+constexpr size_t kOffLong = kOffBad + kNoAllocWords;
+constexpr size_t kOffMaps = (size_t)2 * kNoAllocMaxN;
+constexpr size_t kScratchWords = kOffMaps + (size_t)kNoAllocCtas * kNoAllocWords;  // 32 MiB
+static_assert(kScratchWords * 4 == (size_t)32 << 20, "scratch size");
 
-static __device__ __align__(256) uint32_t g_noalloc_scratch[(size_t)kNoAllocCtas * kNoAllocWords];
+// Rows of at most this many entries are a warp's; a longer one is a CTA's.
+constexpr int kShortRow = 128;
+constexpr int kShortSlots = 2 * kShortRow;  // hash of a short row, at most half full
+constexpr int kTriBlock = 256;
+constexpr int kPart = 512;       // slots of a long row that one CTA takes
+constexpr int kHeavyRun = 512;   // a lower neighbour's row of this many entries is all warps' together
+constexpr uint32_t kMaxParts = (uint32_t)(kOffMaps - kOffLong);  // list entries: x (20 bits) and the part above
+constexpr uint32_t kNoPart = 0xffffffffu;
+
+static __device__ __align__(256) uint32_t g_noalloc_scratch[kScratchWords];
 
 // Device address of g_noalloc_scratch, looked up once per device ordinal and
 // kept for the life of the process: this assumes the device's primary context
@@ -37,39 +71,320 @@ constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mu;
 uint32_t* g_noalloc_ptr[kMaxDevices] = {};
 
-// tri[p] = |Gamma(x) ∩ Gamma(ci[p])| for every slot p of row x. Rows are dealt
-// round-robin to CTAs; each CTA marks Gamma(x) in its bitmap, counts marked
-// neighbours of every y in Gamma(x) (one warp per y), then unmarks Gamma(x).
-__global__ void __launch_bounds__(kNoAllocBlock) k_triangles_noalloc(int32_t n, const int32_t* __restrict__ rp,
-                                                                     const int32_t* __restrict__ ci,
-                                                                     int32_t* __restrict__ tri,
-                                                                     uint32_t* __restrict__ scratch) {
-  uint32_t* bm = scratch + (size_t)blockIdx.x * kNoAllocWords;
+__device__ __forceinline__ bool row_bad(const uint32_t* scratch, int32_t x) {
+  return (scratch[kOffBad + (x >> 5)] >> (x & 31)) & 1u;
+}
+
+// The row of slot p, one of 32 consecutive slots of a warp, p0 the first (the
+// whole warp calls): the warp's first and last rows by two searches of rp, the
+// lane's between them.
+__device__ __forceinline__ int32_t row_of_slot(int32_t n, const int32_t* __restrict__ rp, int32_t p0, int32_t p,
+                                               int32_t p_last) {
+  auto search = [&](int32_t lo, int32_t hi, int32_t q) {  // last row in [lo, hi] that starts at or before q
+    while (lo < hi) {
+      const int32_t mid = lo + ((hi - lo + 1) >> 1);
+      if (rp[mid] <= q) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+  };
+  const int32_t x0 = search(0, n - 1, p0);
+  return search(x0, search(x0, n - 1, p_last), p);
+}
+
+// Thread per slot: rows with a column out of range, a self-loop or two entries
+// out of order; thread per row: the long rows, in parts of kPart slots. (A warp
+// per row would walk the longest rows alone: 0.4 ms for one of 25 000 entries.)
+__global__ void __launch_bounds__(kTriBlock) k_rows(int32_t n, const int32_t* __restrict__ rp,
+                                                    const int32_t* __restrict__ ci, uint32_t* __restrict__ scratch) {
+  const int lane = threadIdx.x & 31;
+  const int64_t t0 = (int64_t)blockIdx.x * kTriBlock + threadIdx.x, threads = (int64_t)gridDim.x * kTriBlock;
+  for (int64_t x = t0; x < n; x += threads) {
+    const int32_t d = rp[x + 1] - rp[x];
+    if (d <= kShortRow) continue;
+    if (d > n) {  // more entries than vertices
+      atomicOr(scratch + kOffBad + (x >> 5), 1u << (x & 31));
+      continue;
+    }
+    const uint32_t parts = (uint32_t)((d + kPart - 1) / kPart);
+    const uint32_t at = atomicAdd(scratch + kNumLong, parts);
+    const bool fits = at + parts <= kMaxParts;  // else (only beyond 2^29 entries) by k_tri_marked
+    if (!fits) atomicOr(scratch + kOffBad + (x >> 5), 1u << (x & 31));
+    for (uint32_t k = 0; k < parts && at + k < kMaxParts; ++k)
+      scratch[kOffLong + at + k] = fits ? (uint32_t)x | (k << 20) : kNoPart;
+  }
+  const int64_t nnz = rp[n];
+  for (int64_t p = t0; p - lane < nnz; p += threads) {
+    const int32_t p0 = (int32_t)(p - lane), p_last = (int32_t)min((int64_t)p0 + 31, nnz - 1);
+    const int32_t q = (int32_t)min(p, nnz - 1);
+    const int32_t x = row_of_slot(n, rp, p0, q, p_last);
+    const int32_t y = ci[q];
+    if ((uint32_t)y >= (uint32_t)n || y == x || (q > rp[x] && ci[q - 1] >= y))
+      atomicOr(scratch + kOffBad + (x >> 5), 1u << (x & 31));
+  }
+}
+
+// The lower neighbours of x in one window of 32 slots of its row: lane l's
+// slot p, and whether it is counted here (both rows follow the rules, and y is
+// below x in (degree, id)); its row [yb, yb + L).
+__device__ __forceinline__ void lower_slot(int32_t n, const int32_t* rp, const int32_t* ci, const uint32_t* scratch,
+                                           int32_t x, int32_t dx, int32_t p, int32_t e, int32_t& yb, int32_t& L,
+                                           bool& mine) {
+  yb = L = 0;
+  mine = false;
+  if (p >= e) return;
+  const int32_t y = ci[p];
+  if ((uint32_t)y >= (uint32_t)n || row_bad(scratch, y)) return;
+  yb = rp[y];
+  const int32_t dy = rp[y + 1] - yb;
+  mine = dy < dx || (dy == dx && y < x);
+  L = mine ? dy : 0;
+}
+
+// Counts, for 32 runs laid end to end over the lanes (lane l's run is [yb, yb +
+// L)), the entries for which `in` holds, per run in cnt[32] (the warp's).
+template <class In>
+__device__ __forceinline__ void count_runs(const int32_t* __restrict__ ci, int32_t yb, int32_t L, int32_t* cnt, int lane,
+                                           In in) {
+  int32_t incl = L;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  const int32_t total = __shfl_sync(0xffffffffu, incl, 31), base = yb - (incl - L);
+  for (int32_t k0 = 0; k0 < total; k0 += 128) {  // four windows of loads in flight
+    int32_t w[4], own[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int32_t k = k0 + 32 * j + lane;
+      int r = 0;  // the run of position k: how many runs end at or before it
+#pragma unroll
+      for (int step = 16; step; step >>= 1)
+        if (__shfl_sync(0xffffffffu, incl, r + step - 1) <= k) r += step;
+      own[j] = r;
+      const int32_t b = __shfl_sync(0xffffffffu, base, r);
+      w[j] = k < total ? ci[b + k] : -1;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (w[j] >= 0 && in(w[j])) atomicAdd(&cnt[own[j]], 1);
+  }
+}
+
+// Warp per row of 2 .. kShortRow entries: its entries in an open-addressing
+// hash (twice the slots), behind a filter of 32 bits a slot word.
+__global__ void __launch_bounds__(kTriBlock) k_tri_short(int32_t n, const int32_t* __restrict__ rp,
+                                                         const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
+                                                         uint32_t* __restrict__ scratch) {
+  constexpr int kW = kTriBlock / 32;
+  __shared__ int32_t s_key[kW][kShortSlots];
+  __shared__ uint32_t s_filt[kW][kShortRow];
+  __shared__ int32_t s_cnt[kW][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int32_t *key = s_key[warp], *cnt = s_cnt[warp];
+  uint32_t* filt = s_filt[warp];
+  for (;;) {
+    int32_t x0 = 0;  // eight rows at a time
+    if (lane == 0) x0 = (int32_t)atomicAdd(scratch + kCurShort, 8u);
+    x0 = __shfl_sync(0xffffffffu, x0, 0);
+    if (x0 >= n) break;
+    for (int32_t x = x0; x < min(x0 + 8, n); ++x) {
+      const int32_t b = rp[x], e = rp[x + 1], d = e - b;
+      if (d > kShortRow || d == 0 || row_bad(scratch, x)) continue;  // warp-uniform
+      int bits = 5;
+      while ((1 << bits) < 2 * d) ++bits;  // at most log2(kShortSlots)
+      const uint32_t mask = (1u << bits) - 1u;
+      const int fbits = bits + 4;  // 16 filter bits per hash slot
+      for (int i = lane; i <= (int)mask; i += 32) key[i] = -1;
+      for (int i = lane; i < (1 << fbits) / 32; i += 32) filt[i] = 0u;
+      __syncwarp();
+      for (int32_t p = b + lane; p < e; p += 32) {
+        const int32_t y = ci[p];
+        const uint32_t hy = (uint32_t)y * 0x9E3779B1u;
+        uint32_t s = hy >> (32 - bits);
+        while (atomicCAS(&key[s], -1, y) != -1) s = (s + 1) & mask;  // rows ascend: no y twice, half full
+        const uint32_t f = ((uint32_t)y * 0x85EBCA6Bu) >> (32 - fbits);
+        atomicOr(&filt[f >> 5], 1u << (f & 31));
+      }
+      __syncwarp();
+      for (int32_t p0 = b; p0 < e; p0 += 32) {
+        int32_t yb, L;
+        bool mine;
+        lower_slot(n, rp, ci, scratch, x, d, p0 + lane, e, yb, L, mine);
+        cnt[lane] = 0;
+        __syncwarp();
+        count_runs(ci, yb, L, cnt, lane, [&](int32_t w) -> bool {
+          const uint32_t f = ((uint32_t)w * 0x85EBCA6Bu) >> (32 - fbits);
+          if (!((filt[f >> 5] >> (f & 31)) & 1u)) return false;
+          uint32_t s = ((uint32_t)w * 0x9E3779B1u) >> (32 - bits);
+          for (;;) {
+            const int32_t k = key[s];
+            if (k == w) return true;
+            if (k == -1) return false;
+            s = (s + 1) & mask;
+          }
+        });
+        __syncwarp();
+        if (mine) tri[p0 + lane] = cnt[lane];
+        __syncwarp();
+      }
+    }
+  }
+}
+
+// CTA per part of a long row: a bitmap of the n vertices in shared memory with
+// the whole row; the warps take windows of 32 slots of the part, and leave the
+// long rows of lower neighbours to a list that all warps then read together
+// (the heaviest neighbours are often next to each other, and one warp alone
+// took 0.9 ms for them).
+__global__ void __launch_bounds__(kNoAllocBlock) k_tri_long(int32_t n, const int32_t* __restrict__ rp,
+                                                            const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
+                                                            uint32_t* __restrict__ scratch) {
+  extern __shared__ uint32_t bm[];  // (n + 31) / 32 words
+  __shared__ uint32_t s_x;
+  __shared__ int32_t s_next, s_heavy, s_cnt[kNoAllocBlock / 32][32];
+  __shared__ int32_t s_hp[kPart], s_hb[kPart], s_he[kPart], s_hc[kPart];  // the listed slots, their rows, their counts
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int32_t* cnt = s_cnt[warp];
+  const uint32_t n_long = min(scratch[kNumLong], kMaxParts);
+  auto in = [&](int32_t w) -> bool { return (bm[w >> 5] >> (w & 31)) & 1u; };
+  for (int32_t i = threadIdx.x; i < (n + 31) / 32; i += kNoAllocBlock) bm[i] = 0u;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t k, v;
+      do {
+        k = atomicAdd(scratch + kCurLong, 1u);
+        v = k < n_long ? scratch[kOffLong + k] : kNoPart;
+      } while (k < n_long && v == kNoPart);
+      s_x = v;
+    }
+    __syncthreads();
+    if (s_x == kNoPart) break;
+    const int32_t x = (int32_t)(s_x & 0xfffffu), part = (int32_t)(s_x >> 20);
+    if (row_bad(scratch, x)) continue;
+    const int32_t b = rp[x], e = rp[x + 1];
+    const int32_t pe = min(e, b + (part + 1) * kPart);
+    if (threadIdx.x == 0) {
+      s_next = b + part * kPart;
+      s_heavy = 0;
+    }
+    for (int32_t p = b + threadIdx.x; p < e; p += kNoAllocBlock) {
+      const int32_t y = ci[p];
+      atomicOr(&bm[y >> 5], 1u << (y & 31));
+    }
+    __syncthreads();
+    for (;;) {
+      int32_t p0 = 0;
+      if (lane == 0) p0 = atomicAdd(&s_next, 32);
+      p0 = __shfl_sync(0xffffffffu, p0, 0);
+      if (p0 >= pe) break;
+      int32_t yb, L;
+      bool mine;
+      lower_slot(n, rp, ci, scratch, x, e - b, p0 + lane, pe, yb, L, mine);
+      if (L >= kHeavyRun) {
+        const int32_t k = atomicAdd(&s_heavy, 1);
+        s_hp[k] = p0 + lane;
+        s_hb[k] = yb;
+        s_he[k] = yb + L;
+        s_hc[k] = 0;
+        L = 0;
+        mine = false;
+      }
+      cnt[lane] = 0;
+      __syncwarp();
+      count_runs(ci, yb, L, cnt, lane, in);
+      __syncwarp();
+      if (mine) tri[p0 + lane] = cnt[lane];
+      __syncwarp();
+    }
+    __syncthreads();
+    const int32_t heavy = s_heavy;
+    for (int32_t k = 0; k < heavy; ++k) {
+      const int32_t yb = s_hb[k], ye = s_he[k];
+      int32_t c = 0;
+      for (int32_t q0 = yb + 128 * warp; q0 < ye; q0 += 128 * (kNoAllocBlock / 32)) {
+        int32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = q0 + 32 * j + lane < ye ? ci[q0 + 32 * j + lane] : -1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) c += w[j] >= 0 && in(w[j]);
+      }
+      c = (int32_t)__reduce_add_sync(0xffffffffu, (unsigned)c);
+      if (lane == 0 && c) atomicAdd(&s_hc[k], c);
+    }
+    __syncthreads();
+    for (int32_t k = threadIdx.x; k < heavy; k += kNoAllocBlock) tri[s_hp[k]] = s_hc[k];
+    for (int32_t p = b + threadIdx.x; p < e; p += kNoAllocBlock) bm[ci[p] >> 5] = 0u;
+  }
+}
+
+// The slots (x, y) with y above x: the value of the reverse slot. Thread per
+// slot.
+__global__ void __launch_bounds__(kTriBlock) k_tri_reverse(int32_t n, const int32_t* __restrict__ rp,
+                                                           const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
+                                                           uint32_t* __restrict__ scratch) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nnz = rp[n], threads = (int64_t)gridDim.x * kTriBlock;
+  bool marked = false;
+  for (int64_t p = (int64_t)blockIdx.x * kTriBlock + threadIdx.x; p - lane < nnz; p += threads) {
+    const int32_t p0 = (int32_t)(p - lane), p_last = (int32_t)min((int64_t)p0 + 31, nnz - 1);
+    const int32_t q = (int32_t)min(p, nnz - 1);
+    const int32_t x = row_of_slot(n, rp, p0, q, p_last);
+    if (p >= nnz) continue;
+    const int32_t y = ci[q], dx = rp[x + 1] - rp[x];
+    bool found = false;
+    if (!row_bad(scratch, x) && !row_bad(scratch, y)) {  // a row that follows the rules has its columns in range
+      const int32_t yb = rp[y], ye = rp[y + 1], dy = ye - yb;
+      if (dy < dx || (dy == dx && y < x)) continue;  // counted at this slot
+      int32_t lo = yb, hi = ye;
+      while (lo < hi) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (ci[mid] < x) lo = mid + 1; else hi = mid;
+      }
+      found = lo < ye && ci[lo] == x;
+      if (found) tri[q] = tri[lo];
+    }
+    if (!found) {
+      tri[q] = -1;
+      marked = true;
+    }
+  }
+  if (marked) atomicAdd(scratch + kNumMarked, 1u);
+}
+
+// The marked slots, by the definition: the row's columns marked in the CTA's
+// bitmap, the row of each marked slot's column looked up in it by one warp, the
+// bitmap cleared again. A column outside [0, n) is skipped; its own slot gets 0.
+__global__ void __launch_bounds__(kNoAllocBlock) k_tri_marked(int32_t n, const int32_t* __restrict__ rp,
+                                                              const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
+                                                              uint32_t* __restrict__ scratch) {
+  if (scratch[kNumMarked] == 0u) return;
+  uint32_t* bm = scratch + kOffMaps + (size_t)blockIdx.x * kNoAllocWords;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int warps = kNoAllocBlock / 32;
-  // the array keeps the previous call's contents: start from zero
-  const int32_t words = (n + 31) / 32;
+  const int32_t words = (n + 31) / 32;  // the array keeps the previous call's contents: start from zero
   for (int32_t i = threadIdx.x; i < words; i += kNoAllocBlock) bm[i] = 0u;
   __syncthreads();
   for (int32_t x = blockIdx.x; x < n; x += gridDim.x) {
     const int32_t xb = rp[x], xe = rp[x + 1];
+    bool any = false;
+    for (int32_t p = xb + threadIdx.x; p < xe; p += kNoAllocBlock) any |= tri[p] == -1;
+    if (!__syncthreads_or(any)) continue;
     for (int32_t p = xb + threadIdx.x; p < xe; p += kNoAllocBlock) {
       const int32_t w = ci[p];
       if ((uint32_t)w < (uint32_t)n) atomicOr(&bm[w >> 5], 1u << (w & 31));
     }
     __syncthreads();
     for (int32_t p = xb + warp; p < xe; p += warps) {
+      if (tri[p] != -1) continue;
       const int32_t y = ci[p];
       int c = 0;
-      if ((uint32_t)y >= (uint32_t)n) {  // not a vertex: no row to scan
-        if (lane == 0) tri[p] = 0;
-        continue;
-      }
-      for (int32_t q = rp[y] + lane; q < rp[y + 1]; q += 32) {
-        const int32_t w = ci[q];
-        if ((uint32_t)w < (uint32_t)n) c += (bm[w >> 5] >> (w & 31)) & 1u;
-      }
-      for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      if ((uint32_t)y < (uint32_t)n)
+        for (int32_t q = rp[y] + lane; q < rp[y + 1]; q += 32) {
+          const int32_t w = ci[q];
+          if ((uint32_t)w < (uint32_t)n) c += (bm[w >> 5] >> (w & 31)) & 1u;
+        }
+      c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
       if (lane == 0) tri[p] = c;
     }
     __syncthreads();
@@ -118,8 +433,24 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
     }
     scratch = g_noalloc_ptr[dev];
   }
-  k_triangles_noalloc<<<kNoAllocCtas, kNoAllocBlock, 0, (cudaStream_t)stream>>>(n, row_ptr, col_idx, tri_out,
-                                                                                  scratch);
+  cudaStream_t s = (cudaStream_t)stream;
+  int sms = 0, per_sm = 0;
+  const size_t smem = sizeof(uint32_t) * (size_t)((n + 31) / 32);
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return cuda_fail(e, "cudaDeviceGetAttribute");
+  if ((e = cudaFuncSetAttribute(k_tri_long, cudaFuncAttributeMaxDynamicSharedMemorySize, kNoAllocWords * 4)) !=
+          cudaSuccess ||
+      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tri_long, kNoAllocBlock, smem)) != cudaSuccess)
+    return cuda_fail(e, "k_tri_long");
+  // counters and the bad-row bits
+  if ((e = cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * (kOffBad + (size_t)((n + 31) / 32)), s)) != cudaSuccess)
+    return cuda_fail(e, "zero counters");
+  const int grid = sms * 8;  // 2048 threads an SM; the number of slots is on the device only
+  k_rows<<<grid, kTriBlock, 0, s>>>(n, row_ptr, col_idx, scratch);
+  k_tri_long<<<sms * (per_sm > 0 ? per_sm : 1), kNoAllocBlock, smem, s>>>(n, row_ptr, col_idx, tri_out, scratch);
+  k_tri_short<<<grid, kTriBlock, 0, s>>>(n, row_ptr, col_idx, tri_out, scratch);
+  k_tri_reverse<<<grid, kTriBlock, 0, s>>>(n, row_ptr, col_idx, tri_out, scratch);
+  k_tri_marked<<<kNoAllocCtas, kNoAllocBlock, 0, s>>>(n, row_ptr, col_idx, tri_out, scratch);
   e = cudaGetLastError();
-  return e == cudaSuccess ? GC_OK : cuda_fail(e, "k_triangles_noalloc");
+  return e == cudaSuccess ? GC_OK : cuda_fail(e, "gc_edge_triangles_noalloc");
 }

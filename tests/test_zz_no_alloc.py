@@ -72,6 +72,57 @@ def test_noalloc_matches_regular_entry_point_twice(make):
         np.testing.assert_array_equal(out.cpu().numpy(), expect)
 
 
+@pytest.mark.parametrize("make", [
+    lambda: graphs.complete(128),          # rows of 127 entries: the longest a warp takes
+    lambda: graphs.complete(131),          # rows of 130: a CTA's
+    lambda: graphgen.chung_lu(1 << 20, 300000, 2.1, 600000.0, 3000.0, 64),  # the largest bitmap
+    lambda: graphs.csr(70, [(3, 40)]),     # one edge, a partial bitmap word
+])
+def test_noalloc_row_lengths(make):
+    import torch
+    rp, ci = make()
+    d_rp, d_ci = torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda()
+    out = torch.full((len(ci),), -1, dtype=torch.int32, device="cuda")
+    gcb.gc_edge_triangles_noalloc(d_rp, d_ci, out)
+    np.testing.assert_array_equal(out.cpu().numpy(), _oracle_per_slot(rp, ci))
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_noalloc_rows_that_break_the_rules(seed):
+    # not validated, but safe and by the definition: tri[p] of (x, y) is the
+    # number of entries of row y in [0, n) that are in row x; 0 for y outside
+    import torch
+    rng = np.random.default_rng(seed)
+    n = 300
+    rp, ci = graphgen.chung_lu(n, 4000, 2.3, 8000.0, 200.0, 70 + seed)
+    ci = ci.copy()
+    for x in rng.choice(n, 40, replace=False):
+        row = ci[rp[x]:rp[x + 1]]
+        if len(row) < 3:
+            continue
+        kind = rng.integers(0, 5)
+        if kind == 0:
+            rng.shuffle(row)                              # unsorted
+        elif kind == 1:
+            row[0] = row[-1]                              # a neighbour twice, one reverse missing
+        elif kind == 2:
+            row[rng.integers(0, len(row))] = rng.choice([-1, n, 2**31 - 1, -2**31])
+        elif kind == 3:
+            row[rng.integers(0, len(row))] = x            # self-loop
+        else:
+            free = np.setdiff1d(np.arange(n), np.append(row, x))
+            if len(free):
+                row[0] = free[0]                          # sorted or not, asymmetric
+                row.sort()
+    rows = [ci[rp[x]:rp[x + 1]] for x in range(n)]
+    sets = [set(r.tolist()) for r in rows]
+    expect = [sum(0 <= w < n and w in sets[x] for w in rows[y].tolist()) if 0 <= y < n else 0
+              for x in range(n) for y in rows[x].tolist()]
+    out = torch.full((len(ci),), -7, dtype=torch.int32, device="cuda")
+    gcb.gc_edge_triangles_noalloc(torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda(), out)
+    np.testing.assert_array_equal(out.cpu().numpy(), np.array(expect, np.int32))
+
+
 def test_noalloc_rejects_graphs_above_its_limit():
     import torch
     n = (1 << 20) + 1

@@ -122,7 +122,7 @@ struct Result {
 // Timers of one launch (CUDA events on its stream): the size classes of the
 // small-graph kernels (eager launches only), the whole small-graph sequence
 // (copies in, kernels, derive, copy out) and the larger graphs' passes.
-enum { kEvSmall0 = 0, kEvSmallSeq0 = kSmallClasses + 1, kEvSmallSeq1, kEvUnion0, kEvUnion1, kNumLaunchEv };
+enum { kEvSmall0 = 0, kEvSmallSeq0 = 2 * kSmallClasses, kEvSmallSeq1, kEvUnion0, kEvUnion1, kNumLaunchEv };
 
 struct Launch {
   std::vector<uint64_t> tickets;
@@ -146,26 +146,34 @@ struct Launch {
 // captured and replayed as a CUDA graph. `busy` marks the end of the slot's
 // last sequence: the host waits on it before it refills or regrows them.
 struct SmallBufs {
-  size_t cap_rows = 0, cap_nnz = 0, cap_g = 0;
-  int32_t *d_rp = nullptr, *d_ci = nullptr, *d_order = nullptr, *d_gn = nullptr, *d_misc = nullptr;
+  size_t cap_rows = 0, cap_nnz = 0, cap_g = 0, cap_units = 0;
+  int32_t *d_rp = nullptr, *d_ci = nullptr, *d_gn = nullptr, *d_misc = nullptr;
+  int2 *d_units = nullptr, *h_units = nullptr;
   int64_t *d_voff = nullptr, *d_eoff = nullptr, *d_gm = nullptr;
-  unsigned long long *d_csum = nullptr, *d_x = nullptr;
-  int32_t *h_rp = nullptr, *h_ci = nullptr, *h_order = nullptr, *h_gn = nullptr;
+  unsigned long long *d_sums = nullptr, *d_csum = nullptr, *d_x = nullptr;
+  int32_t *h_rp = nullptr, *h_ci = nullptr, *h_gn = nullptr;
   int64_t *h_voff = nullptr, *h_eoff = nullptr, *h_gm = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t busy = nullptr;
+  SmallFork fork;
 };
 
 void free_small_bufs(SmallBufs* b) {
   if (b->busy) cudaEventSynchronize(b->busy);
-  for (void* p : {(void*)b->d_rp, (void*)b->d_ci, (void*)b->d_order, (void*)b->d_gn, (void*)b->d_misc,
-                  (void*)b->d_voff, (void*)b->d_eoff, (void*)b->d_gm, (void*)b->d_csum, (void*)b->d_x})
+  for (void* p : {(void*)b->d_rp, (void*)b->d_ci, (void*)b->d_units, (void*)b->d_gn, (void*)b->d_misc,
+                  (void*)b->d_voff, (void*)b->d_eoff, (void*)b->d_gm, (void*)b->d_sums, (void*)b->d_csum,
+                  (void*)b->d_x})
     if (p) cudaFree(p);
-  for (void* p : {(void*)b->h_rp, (void*)b->h_ci, (void*)b->h_order, (void*)b->h_gn, (void*)b->h_voff,
+  for (void* p : {(void*)b->h_rp, (void*)b->h_ci, (void*)b->h_units, (void*)b->h_gn, (void*)b->h_voff,
                   (void*)b->h_eoff, (void*)b->h_gm})
     if (p) cudaFreeHost(p);
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->busy) cudaEventDestroy(b->busy);
+  if (b->fork.start) cudaEventDestroy(b->fork.start);
+  for (auto& e : b->fork.done)
+    if (e) cudaEventDestroy(e);
+  for (auto& t : b->fork.stream)
+    if (t) cudaStreamDestroy(t);
   *b = SmallBufs();
 }
 
@@ -398,7 +406,7 @@ gc_status run_small(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
       c1 = 0; GS_TRY(grow_pair(&sb->d_eoff, &sb->h_eoff, &c1, need), "small buffers");
       c1 = 0; GS_TRY(grow_pair(&sb->d_gm, &sb->h_gm, &c1, need), "small buffers");
       c1 = 0; GS_TRY(grow_pair(&sb->d_gn, &sb->h_gn, &c1, need), "small buffers");
-      c1 = 0; GS_TRY(grow_pair(&sb->d_order, &sb->h_order, &c1, need), "small buffers");
+      c1 = 0; GS_TRY(grow_pair<unsigned long long>(&sb->d_sums, nullptr, &c1, kSmallSums * need), "small buffers");
       c1 = 0; GS_TRY(grow_pair<unsigned long long>(&sb->d_csum, nullptr, &c1, 26 * need), "small buffers");
       c1 = 0; GS_TRY(grow_pair<unsigned long long>(&sb->d_x, nullptr, &c1, 34 * need), "small buffers");
       if (!sb->d_misc) GS_TRY(cudaMalloc(&sb->d_misc, sizeof(int32_t) * (kSmallClasses + 1)), "small buffers");
@@ -408,20 +416,25 @@ gc_status run_small(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
     sb->cap_nnz = cn;
     sb->cap_g = cg;
   }
-  // order: graphs binned by size class, largest m first within a class
   int32_t class_off[kSmallClasses + 1] = {0};
+  std::vector<int2> units;
   {
-    std::vector<int32_t> cls((size_t)G);
+    std::vector<int32_t> gn((size_t)G);
+    std::vector<int64_t> gm((size_t)G);
     for (int32_t gi = 0; gi < G; ++gi) {
-      cls[gi] = small_class_of(graphs[gi]->n);
-      ++class_off[cls[gi] + 1];
+      gn[(size_t)gi] = graphs[gi]->n;
+      gm[(size_t)gi] = graphs[gi]->m;
     }
-    for (int c = 0; c < kSmallClasses; ++c) class_off[c + 1] += class_off[c];
-    std::vector<int32_t> pos(class_off, class_off + kSmallClasses);
-    for (int32_t gi = 0; gi < G; ++gi) sb->h_order[pos[cls[gi]]++] = gi;
-    for (int c = 0; c < kSmallClasses; ++c)
-      std::sort(sb->h_order + class_off[c], sb->h_order + class_off[c + 1],
-                [&](int32_t a, int32_t b) { return graphs[a]->m > graphs[b]->m; });
+    small_units(gn, gm, &units, class_off);
+    GS_TRY(grow_pair(&sb->d_units, &sb->h_units, &sb->cap_units, units.size()), "small buffers");
+    std::memcpy(sb->h_units, units.data(), sizeof(int2) * units.size());
+  }
+  if (!sb->fork.start) {
+    GS_TRY(cudaEventCreateWithFlags(&sb->fork.start, cudaEventDisableTiming), "small fork");
+    for (int c = 0; c < kSmallClasses; ++c) {
+      GS_TRY(cudaEventCreateWithFlags(&sb->fork.done[c], cudaEventDisableTiming), "small fork");
+      GS_TRY(cudaStreamCreateWithFlags(&sb->fork.stream[c], cudaStreamNonBlocking), "small fork");
+    }
   }
   std::memcpy(sb->h_voff, voff.data(), sizeof(int64_t) * voff.size());
   std::memcpy(sb->h_eoff, eoff.data(), sizeof(int64_t) * eoff.size());
@@ -458,13 +471,16 @@ gc_status run_small(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
     if (r == cudaSuccess) r = cudaMemcpyAsync(sb->d_eoff, sb->h_eoff, b8 * (G + 1), cudaMemcpyHostToDevice, s);
     if (r == cudaSuccess) r = cudaMemcpyAsync(sb->d_gn, sb->h_gn, b4 * G, cudaMemcpyHostToDevice, s);
     if (r == cudaSuccess) r = cudaMemcpyAsync(sb->d_gm, sb->h_gm, b8 * G, cudaMemcpyHostToDevice, s);
-    if (r == cudaSuccess) r = cudaMemcpyAsync(sb->d_order, sb->h_order, b4 * G, cudaMemcpyHostToDevice, s);
+    if (r == cudaSuccess)
+      r = cudaMemcpyAsync(sb->d_units, sb->h_units, sizeof(int2) * units.size(), cudaMemcpyHostToDevice, s);
     if (r == cudaSuccess) r = cudaMemsetAsync(sb->d_misc, 0, b4 * (kSmallClasses + 1), s);
-    if (r == cudaSuccess) r = cudaMemsetAsync(sb->d_csum, 0, sizeof(unsigned long long) * 26 * (size_t)G, s);
+    if (r == cudaSuccess) r = cudaMemsetAsync(sb->d_sums, 0, sizeof(unsigned long long) * kSmallSums * (size_t)G, s);
     if (r != cudaSuccess) return r;
-    if (run_small_graphs(sb->d_rp, sb->d_voff, sb->d_ci, sb->d_eoff, sb->d_order, class_off, sb->d_misc,
-                         sb->d_misc + kSmallClasses, sb->d_csum, cfg, graph_mode ? nullptr : L->ev + kEvSmall0,
-                         s) != GC_OK)
+    const SmallGraphs sg = {G,           sb->d_rp,    sb->d_ci,   sb->d_gn,   sb->d_voff, sb->d_eoff, sb->d_gm,
+                            sb->d_units, sb->d_misc, sb->d_misc + kSmallClasses, sb->d_sums, sb->d_csum};
+    // eager launches time each class, one after the other
+    if (run_small_graphs(sg, class_off, cfg, graph_mode ? nullptr : L->ev + kEvSmall0,
+                         graph_mode ? &sb->fork : nullptr, s) != GC_OK)
       return cudaErrorLaunchFailure;
     DevGraph dg = DevGraph();
     dg.G = G;
@@ -579,7 +595,7 @@ void retire_locked(gc_batch b) {
         return cudaEventElapsedTime(&f, L->ev[a], L->ev[z]) == cudaSuccess ? (double)f : 0.0;
       };
       for (int c = 0; c < kSmallClasses; ++c)
-        b->last_stats[c] = L->timed_classes ? ms(kEvSmall0 + c, kEvSmall0 + c + 1) : 0.0;
+        b->last_stats[c] = L->timed_classes ? ms(kEvSmall0 + 2 * c, kEvSmall0 + 2 * c + 1) : 0.0;
       b->last_stats[kSmallClasses] = L->timed_small ? ms(kEvSmallSeq0, kEvSmallSeq1) : 0.0;
       b->last_stats[kSmallClasses + 1] = L->timed_union ? ms(kEvUnion0, kEvUnion1) : 0.0;
       b->last_stats[kSmallClasses + 2] = L->replayed ? 1.0 : 0.0;

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <vector>
 
 #include "../../include/gc.h"
 
@@ -330,15 +331,33 @@ bool load_tuned_config(BatchConfig* cfg, std::string* source);
 // Raises the dynamic shared-memory limit of every instantiation (once per
 // device, before any launch or capture).
 gc_status small_graphs_setup();
-// rp/voff: concatenated local row pointers and their offsets; ci/eoff:
-// concatenated local columns; class c counts the graphs
-// order[class_off[c] .. class_off[c + 1]) (largest first within a class);
-// cursor: kSmallClasses zeroed device ints; status: device status word;
-// csum [*][13][2] zeroed. ev (optional): kSmallClasses + 1 events recorded
-// before each class's launch and after the last.
-gc_status run_small_graphs(const int32_t* rp, const int64_t* voff, const int32_t* ci, const int64_t* eoff,
-                           const int32_t* order, const int32_t* class_off, int32_t* cursor, int32_t* status,
-                           unsigned long long* csum, const BatchConfig& cfg, cudaEvent_t* ev, cudaStream_t s);
+// The units of a launch of small graphs (n, m per graph): unit = (graph, part |
+// parts << 16), class c's units[class_off[c] .. class_off[c + 1]), most work
+// first within a class.
+void small_units(const std::vector<int32_t>& n, const std::vector<int64_t>& m, std::vector<int2>* units,
+                 int32_t* class_off);
+constexpr int kSmallSums = 8;  // sums of a graph that the kernels leave in SmallGraphs::sums
+// Device arrays of one launch: rp/voff: concatenated local row pointers and
+// their offsets; ci/eoff: concatenated local columns; gn/gm: vertices and edges
+// per graph; cursor: kSmallClasses zeroed ints; status: device status word;
+// sums [G][kSmallSums] zeroed; csum [G][13][2] receives the unrestricted sums.
+struct SmallGraphs {
+  int32_t G;
+  const int32_t *rp, *ci, *gn;
+  const int64_t *voff, *eoff, *gm;
+  const int2* units;
+  int32_t *cursor, *status;
+  unsigned long long *sums, *csum;
+};
+// Streams on which the size classes of one launch run side by side.
+struct SmallFork {
+  cudaEvent_t start = nullptr, done[kSmallClasses] = {};
+  cudaStream_t stream[kSmallClasses] = {};
+};
+// ev (optional): 2 kSmallClasses events, recorded before and after each class's
+// kernel; fork (optional): the classes run on its streams, joined into s.
+gc_status run_small_graphs(const SmallGraphs& b, const int32_t* class_off, const BatchConfig& cfg, cudaEvent_t* ev,
+                           const SmallFork* fork, cudaStream_t s);
 
 // ---- counting (gc_count.cu: pass C, finish, derive; gc_clique.cu: passes T and K) ----
 int count_grid_size();

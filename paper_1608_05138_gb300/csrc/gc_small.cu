@@ -10,89 +10,59 @@
 // follow per edge as in Sec. 4.5. The batched form returns only the global
 // counts, so the per-edge summands of C_3 .. C_16 are needed only as sums
 // over the edges: they are polynomials in |T|, d_u and d_v, and the kernel
-// sums per edge only |T|, |T|^2 and |T| (d_u + d_v), per vertex d^2 and d^3,
-// per entry d_x d_y, from which the columns follow in closed form
-// (graph_column). Of the two per-edge scans of Alg. 5/6:
-//   C_7  = sum_e x7  = 6 #K4: every 4-clique {a < b < c < d} is met once, at
-//          its edge (a, b), as an edge inside T' = the common neighbours of
-//          a and b above b (sum over T' of popc(row(w) & T') counts it twice);
+// sums per edge only |T|, |T|^2, |T| (d_u + d_v) and d_u d_v, per vertex d^2
+// and d^3, from which the columns follow in closed form (graph_column). Of the
+// two per-edge scans of Alg. 5/6:
 //   C_10 = sum_e x10 = 4 X_10 = 4 C4 - 4 C_8 + 2 C_7, with C4 the 4-cycles as
 //          subgraphs, (1/2) sum over vertex pairs {u, w} of C(c_uw, 2) (c_uw
 //          common neighbours; each cycle is met from both of its diagonals),
-//          X_10 = C4 - X_8 - 3 X_7 and X_8 = C_8 - C_7 (Sec. 4.6).
-// That is a popcount over the n^2 / 2 pairs instead of one over S_u x S_v
-// per edge -- several times less work on the dense graphs of a batch -- and
-// exact: the derivation of Sec. 4.6 then runs unchanged.
-// One lane holds one 32-bit word of each mask; rows are stored at an odd
-// word stride, so that 32 lanes reading one word index of 32 rows hit 32
-// banks. One CTA per graph (work stealing over the graphs, largest first).
+//          X_10 = C4 - X_8 - 3 X_7 and X_8 = C_8 - C_7 (Sec. 4.6). One pass over
+//          the n^2 / 2 pairs, a lane per pair, gives c_uw and, where u ~ w,
+//          |T| of the edge: no reduction over lanes per edge.
+//   C_7  = sum_e x7  = 6 #K4: the 4-cliques with lowest vertex u are the
+//          triangles of H_u, the subgraph induced on the k neighbours above u.
+//          H_u is packed to k bits a row (a ballot per row and word) and its
+//          triangles counted as sum over its edges (i, j), i < j, of the common
+//          neighbours above j: k / 32 words a row instead of n / 32, and no
+//          list of members per edge. A warp per u up to 128 neighbours above
+//          it, the CTA together beyond.
+// Rows are stored at an odd word stride, so that 32 lanes reading one word
+// index of 32 rows hit 32 banks. What bounds it: popc (16 lanes a clock an SM)
+// and shared-memory reads, two each per 32 pairs and word. (Before, each edge
+// listed its common neighbours and took one of their rows at a time over the
+// lanes: the graphs of n <= 512 in a launch of 48 took 5.3 ms, one CTA each;
+// now 0.24 ms, in 256 parts.)
 //
 // Graphs are binned by vertex count into size classes (n <= 64, 128, 256,
-// 512, 1024); each class runs its own instantiation, whose bitmatrix and
-// member lists are sized for the class, so that small graphs take little
-// shared memory and many CTAs fit on an SM. The block size of each class is
-// a tuning parameter (BatchConfig).
+// 512, 1024); each class runs its own instantiation, whose shared memory is
+// sized for the class, so that small graphs take little and many CTAs fit on
+// an SM. The block size of each class is a tuning parameter (BatchConfig). A
+// CTA takes one unit at a time from the class's list, most work first: a
+// graph, or, when a launch has too few graphs to fill the GPU, a part of one
+// (every parts-th vertex u); each part loads the graph's bit rows, and the
+// sums of a graph meet in global memory.
 #include <cuda_runtime.h>
+
+#include <algorithm>
+#include <utility>
+#include <vector>
 
 #include "gc_internal.h"
 
 namespace gc {
 namespace {
 
-__device__ __forceinline__ void add_u128(unsigned long long* p, u128 v) {
-  unsigned long long lo = (unsigned long long)v;
-  unsigned long long hi = (unsigned long long)(v >> 64);
-  unsigned long long old = atomicAdd(p, lo);
-  if (old + lo < old) hi += 1ull;
-  if (hi) atomicAdd(p + 1, hi);
-}
-
 constexpr unsigned kFull = 0xffffffffu;
 
 // Sums of one graph from which its unrestricted sums follow in closed form
-// (graph_columns): per edge (u, v) with t = |T| and a = d_u + d_v, the sums
-// of t, t^2, t a and the 4-clique term; per vertex, d^2 and d^3; per
-// directed entry (x, y), d_x d_y.
-enum { kQt, kQtt, kQta, kQk, kQd2, kQd3, kQdd, kQn };
+// (graph_column): per edge (u, v) with t = |T| and a = d_u + d_v, the sums of
+// t, t^2, t a and d_u d_v; per vertex, d^2 and d^3; over vertex pairs,
+// C(c_uw, 2); and the 4-cliques.
+enum { kQt, kQtt, kQta, kQdd, kQd2, kQd3, kQc4, kQk4, kQn };
+static_assert(kQn == kSmallSums, "sums of a small graph");
 
-// sum over the members b of `mask` (word w in lane w; the words below w0 and
-// from W on are 0) of popc(row(b) & mask), this lane's part. The members are
-// listed in `list` (the warp's shared buffer), then each lane takes one
-// (member, word) pair over the words [w0, W): Wq = the power of two >= W - w0
-// lanes per member, 32 / Wq members per step. kS: the row stride of the size
-// class, in words.
-template <int kS>
-__device__ __forceinline__ uint32_t masked_row_popc(const uint32_t* __restrict__ bm, uint32_t mask, int lane, int w0,
-                                                    int W, int16_t* list) {
-  const int span = W - w0;
-  const int c = __popc(mask);
-  int incl = c;
-  for (int o = 1; o < span; o <<= 1) {  // lanes w0 .. W-1 carry the members
-    const int y = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += y;
-  }
-  const int total = __shfl_sync(kFull, incl, W - 1);
-  int pos = incl - c;
-  uint32_t word = mask;
-  while (word) {
-    const int b = __ffs(word) - 1;
-    word &= word - 1;
-    list[pos++] = (int16_t)(lane * 32 + b);
-  }
-  __syncwarp();
-  const int lg = span <= 1 ? 0 : 32 - __clz(span - 1);
-  const int w = w0 + (lane & ((1 << lg) - 1));
-  const bool wv = w < W;
-  const uint32_t ow = __shfl_sync(kFull, mask, w & 31);  // word w of the mask
-  uint32_t acc = 0;
-  for (int i = lane >> lg; i < total; i += 32 >> lg)
-    if (wv) acc += __popc(bm[list[i] * kS + w] & ow);
-  __syncwarp();
-  return acc;
-}
-
-// The unrestricted sums of one graph (n vertices, m edges) from the sums
-// q and the sum c4 over vertex pairs of C(c_uw, 2), in the column order
+// The unrestricted sums of one graph (n vertices, m edges) from the sums q,
+// in the column order
 // C_3 C_4 C_5 C_7 C_8 C_9 C_10 C_11 C_12 C_13 C_14 C_15 C_16. Per edge
 // |S_u| = d_u - 1 - t and |S_v| = d_v - 1 - t (Sec. 4.5), so s = a - 2 - 2t
 // and D = n - 2 - t - s, and with A1 = sum a = sum_v d^2,
@@ -105,27 +75,26 @@ __device__ __forceinline__ uint32_t masked_row_popc(const uint32_t* __restrict__
 //   C_14 = m^2 + m - A1,                    C_15 = (n-2) C_4 - C_9 - sum s^2,
 //   C_16 = (sum D^2 - C_5) / 2, sum D^2 = (n-2)^2 m - 2 (n-2)(sum t + C_4)
 //          + sum t^2 + 2 C_9 + sum s^2,
-// C_7 = 6 #K4 = 3 q_k (each 4-clique met twice), C_10 = 4 C4 - 4 C_8 + 2 C_7.
+// C_7 = 6 #K4, C_10 = 4 C4 - 4 C_8 + 2 C_7 with 2 C4 = sum over pairs of C(c_uw, 2).
 // Column k of the graph, k in 0 .. 12. Unsigned arithmetic: every result is a nonnegative count below 2^64, so
 // the wrap-around of the intermediate terms cancels.
-__device__ __forceinline__ unsigned long long graph_column(int k, const unsigned long long* q, unsigned long long c4,
-                                                         int32_t n, int64_t m) {
+__device__ __forceinline__ unsigned long long graph_column(int k, const unsigned long long* q, int32_t n, int64_t m) {
   typedef unsigned long long U;
   const U N2 = (U)(long long)(n - 2), M = (U)m;
   const U St = q[kQt], Stt = q[kQtt], Sta = q[kQta], A1 = q[kQd2];
   const U C4 = A1 - 2ull * M - 2ull * St;
   const U C9 = Sta - 2ull * St - 2ull * Stt;
-  const U C12 = q[kQdd] / 2ull - A1 + M - Sta + 2ull * St + Stt;
-  const U Sss = q[kQd3] + q[kQdd] - 4ull * A1 + 4ull * M - 4ull * (Sta - 2ull * St) + 4ull * Stt;
+  const U C12 = q[kQdd] - A1 + M - Sta + 2ull * St + Stt;
+  const U Sss = q[kQd3] + 2ull * q[kQdd] - 4ull * A1 + 4ull * M - 4ull * (Sta - 2ull * St) + 4ull * Stt;
   const U C5 = N2 * M - St - C4;
   switch (k) {
     case 0: return St;
     case 1: return C4;
     case 2: return C5;
-    case 3: return 3ull * q[kQk];
+    case 3: return 6ull * q[kQk4];
     case 4: return (Stt - St) / 2ull;
     case 5: return C9;
-    case 6: return 2ull * c4 - 2ull * (Stt - St) + 6ull * q[kQk];
+    case 6: return 2ull * q[kQc4] - 2ull * (Stt - St) + 12ull * q[kQk4];
     case 7: return (Sss - 2ull * C12 - C4) / 2ull;
     case 8: return C12;
     case 9: return N2 * St - Stt - C9;
@@ -138,10 +107,30 @@ __device__ __forceinline__ unsigned long long graph_column(int k, const unsigned
 // Row stride of a size class: the words of a row, made odd.
 __host__ __device__ constexpr int small_stride(int kN) { return (kN / 32) | 1; }
 
-// Shared memory of a size class: the bitmatrix (kN rows at the odd stride)
-// and one member list of kN entries per warp.
+// H_u of up to 32 kWords members, packed: block b of 32 rows keeps the words
+// b .. kWords - 1 of its rows (row i: the members j > i), at an odd stride.
+__host__ __device__ constexpr int h_stride(int words, int b) { return (words - b) | 1; }
+__host__ __device__ constexpr int h_words(int words) {
+  int t = 0;
+  for (int b = 0; b < words; ++b) t += 32 * h_stride(words, b);
+  return t;
+}
+// Most members a warp takes alone.
+__host__ __device__ constexpr int warp_members(int kN) { return kN < 128 ? kN : 128; }
+
+// Shared memory of a size class, in bytes: the bitmatrix (kN rows at the odd
+// stride), the H_u of every warp or the CTA's, the member lists of the same,
+// the degrees, and the neighbours above each vertex.
+__host__ __device__ constexpr size_t small_max(size_t a, size_t b) { return a > b ? a : b; }
+__host__ __device__ constexpr size_t small_bm(int kN) { return (size_t)kN * (size_t)small_stride(kN) * 4; }
+__host__ __device__ constexpr size_t small_h(int kN, int kBlock) {
+  return 4 * small_max((size_t)(kBlock / 32) * h_words(warp_members(kN) / 32), h_words(kN / 32));
+}
+__host__ __device__ constexpr size_t small_list(int kN, int kBlock) {
+  return 2 * small_max((size_t)(kBlock / 32) * warp_members(kN), (size_t)kN);
+}
 __host__ __device__ constexpr size_t small_smem(int kN, int kBlock) {
-  return (size_t)kN * (size_t)small_stride(kN) * 4 + (size_t)(kBlock / 32) * (size_t)kN * 2;
+  return small_bm(kN) + small_h(kN, kBlock) + small_list(kN, kBlock) + 4 * (size_t)kN;
 }
 
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long x) {
@@ -149,34 +138,106 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long x) {
   return x;
 }
 
+// Packs H_u (members m[0 .. k), ascending) into h from the bit rows bm, row
+// stride kS; warp wi of nw takes every nw-th (row block, word).
+template <int kS>
+__device__ __forceinline__ void pack_h(const uint32_t* __restrict__ bm, const uint16_t* m, int k, uint32_t* h, int wi,
+                                       int nw, int lane) {
+  const int W = (k + 31) >> 5;
+  int task = 0;
+  for (int b = 0; b < W; ++b) {  // word b: members j = 32 b + lane
+    const int j = 32 * b + lane;
+    const int mj = j < k ? m[j] : 0;
+    const int wj = mj >> 5, sj = 31 - (mj & 31);
+    const uint32_t valid = k - 32 * b >= 32 ? kFull : (1u << (k - 32 * b)) - 1u;
+    int off = 0;
+    for (int rb = 0; rb <= b; ++rb, ++task) {  // rows i = 32 rb + r
+      const int stride = h_stride(W, rb);
+      if (task % nw == wi) {
+        const int mi = 32 * rb + lane < k ? m[32 * rb + lane] : 0;
+        const int rows = min(32, k - 32 * rb);
+        uint32_t val = 0;
+        for (int r = 0; r < rows; ++r) {
+          const uint32_t word = bm[__shfl_sync(kFull, mi, r) * kS + wj];
+          const uint32_t bits = __ballot_sync(kFull, (int32_t)(word << sj) < 0);
+          if (lane == r) val = bits;
+        }
+        val &= valid;
+        if (rb == b) val &= lane == 31 ? 0u : kFull << (lane + 1);  // members above the row's
+        h[off + lane * stride + (b - rb)] = val;
+      }
+      off += 32 * stride;
+    }
+  }
+}
+
+// This lane's part of the triangles of the packed H_u: for every pair (i, j),
+// j = 32 b + lane, with bit j of row i set, the common members above j.
+__device__ __forceinline__ uint32_t count_h(const uint32_t* h, int k, int wi, int nw, int lane) {
+  const int W = (k + 31) >> 5;
+  uint32_t acc = 0;
+  int task = 0, offb = 0;
+  for (int b = 0; b < W; ++b) {
+    const uint32_t* hj = h + offb + lane * h_stride(W, b);  // words b .. W - 1 of row j
+    int off = 0;
+    for (int rb = 0; rb <= b; ++rb, ++task) {
+      const int stride = h_stride(W, rb);
+      if (task % nw == wi) {
+        const uint32_t* hi0 = h + off + (b - rb);  // word b of row 32 rb
+        const int rows = min(32, k - 32 * rb);
+        for (int w = b; w < W; w += 4) {
+          uint32_t x[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) x[q] = w + q < W ? hj[w - b + q] : 0u;
+          const uint32_t* hi = hi0;
+          for (int r = 0; r < rows; ++r, hi += stride) {
+            const uint32_t on = 0u - ((hi[0] >> lane) & 1u);  // all ones when i ~ j
+            uint32_t c = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (w + q < W) c += __popc(hi[w - b + q] & x[q]);  // warp-uniform
+            acc += c & on;
+          }
+        }
+      }
+      off += 32 * stride;
+    }
+    offb += 32 * h_stride(W, b);
+  }
+  return acc;
+}
+
 // at least 1536 threads resident per SM (at most 42 registers a thread): the
-// kernel is bound by instruction issue and shared-memory latency, and the
-// more warps an SM holds, the more of its cycles issue
+// kernel waits on shared memory and popc, and the more warps an SM holds, the
+// more of its cycles issue
 template <int kN, int kBlock>
 __global__ void __launch_bounds__(kBlock, 1536 / kBlock) k_small_graphs(const int32_t* __restrict__ rp,
                                                          const int64_t* __restrict__ voff,
                                                          const int32_t* __restrict__ ci,
                                                          const int64_t* __restrict__ eoff,
-                                                         const int32_t* __restrict__ order, int32_t G,
+                                                         const int2* __restrict__ units, int32_t n_units,
                                                          int32_t* __restrict__ cursor, int32_t* __restrict__ status,
-                                                         unsigned long long* __restrict__ csum) {
+                                                         unsigned long long* __restrict__ sums) {
   constexpr int kS = small_stride(kN);  // words per bit row, odd
   constexpr int kWarps = kBlock / 32;
+  constexpr int kWarpK = warp_members(kN);
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t* bm = reinterpret_cast<uint32_t*>(smem);
-  int16_t* s_list = reinterpret_cast<int16_t*>(smem + (size_t)kN * kS * 4);
-  __shared__ int32_t s_g;
-  // per graph: the per-edge sums and the sum over pairs of C(c_uw, 2)
-  __shared__ unsigned long long s_q[kQn], s_c4;
+  uint32_t* s_h = reinterpret_cast<uint32_t*>(smem + small_bm(kN));
+  uint16_t* s_m = reinterpret_cast<uint16_t*>(smem + small_bm(kN) + small_h(kN, kBlock));
+  uint16_t* s_deg = reinterpret_cast<uint16_t*>(smem + small_bm(kN) + small_h(kN, kBlock) + small_list(kN, kBlock));
+  uint16_t* s_up = s_deg + kN;
+  __shared__ int32_t s_unit;
+  __shared__ unsigned long long s_q[kQn];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (;;) {
     __syncthreads();
-    if (threadIdx.x == 0) s_g = atomicAdd(cursor, 1);
+    if (threadIdx.x == 0) s_unit = atomicAdd(cursor, 1);
     if (threadIdx.x < kQn) s_q[threadIdx.x] = 0ull;
-    if (threadIdx.x == kQn) s_c4 = 0ull;
     __syncthreads();
-    if (s_g >= G) break;
-    const int32_t g = order[s_g];
+    if (s_unit >= n_units) break;
+    const int2 unit = units[s_unit];  // graph, part | parts << 16
+    const int32_t g = unit.x, part = unit.y & 0xffff, parts = unit.y >> 16;
     const int32_t* grp = rp + voff[g];
     const int32_t* gci = ci + eoff[g];
     const int32_t n = (int32_t)(voff[g + 1] - voff[g]) - 1;
@@ -187,101 +248,117 @@ __global__ void __launch_bounds__(kBlock, 1536 / kBlock) k_small_graphs(const in
     const int W = (n + 31) / 32;
     for (int32_t i = threadIdx.x; i < n * kS; i += kBlock) bm[i] = 0u;
     __syncthreads();
-    // the bit rows, and the degree sums: lane 0 d^2 and d^3 per vertex, every
-    // lane d_x d_y per entry
-    unsigned long long d2 = 0, d3 = 0, dd = 0;
+    // the bit rows, the degrees, and the neighbours above each vertex
     for (int32_t x = warp; x < n; x += kWarps) {
       const int32_t xb = grp[x], xe = grp[x + 1];
-      const uint32_t dx = (uint32_t)(xe - xb);
+      int up = 0;
+      for (int32_t p0 = xb; p0 < xe; p0 += 32) {
+        const int32_t y = p0 + lane < xe ? gci[p0 + lane] : -1;
+        if (y >= 0) atomicOr(&bm[x * kS + (y >> 5)], 1u << (y & 31));
+        up += __popc(__ballot_sync(kFull, y > x));
+      }
       if (lane == 0) {
-        d2 += dx * dx;
-        d3 += (unsigned long long)(dx * dx) * dx;
+        s_deg[x] = (uint16_t)(xe - xb);
+        s_up[x] = (uint16_t)up;
       }
-      for (int32_t p = xb + lane; p < xe; p += 32) {
-        const int32_t y = gci[p];
-        atomicOr(&bm[x * kS + (y >> 5)], 1u << (y & 31));
-        dd += dx * (uint32_t)(grp[y + 1] - grp[y]);
-      }
-    }
-    dd = warp_sum(dd);
-    if (lane == 0) {
-      if (d2) atomicAdd(&s_q[kQd2], d2);
-      if (d3) atomicAdd(&s_q[kQd3], d3);
-      if (dd) atomicAdd(&s_q[kQdd], dd);
     }
     __syncthreads();
-    int16_t* list = s_list + warp * kN;
-    for (int32_t u = warp; u < n; u += kWarps) {
-      const int32_t ub = grp[u], ue = grp[u + 1];
-      const uint32_t ru = lane < W ? bm[u * kS + lane] : 0u;
-      // each edge once, from its smaller endpoint: the neighbours above u
-      // follow the popc(row(u) below u) ones below it in the sorted row
-      const int uw = u >> 5;
-      const uint32_t below = lane < uw ? ru : (lane == uw ? ru & ((1u << (u & 31)) - 1u) : 0u);
-      const int32_t p1 = ub + (int32_t)__reduce_add_sync(kFull, (unsigned)__popc(below));
-      // sums over the edges of u, each below 2^31 (fewer than 1024 edges,
-      // every term below 2^20)
-      uint32_t a_t = 0, a_tt = 0, a_tdv = 0, a_k = 0;
-      for (int32_t p0 = p1; p0 < ue; p0 += 32) {
-        // 32 neighbours v at a time, each with d_v (both below 2^16)
-        uint32_t vd = 0;
-        if (p0 + lane < ue) {
-          const int32_t y = gci[p0 + lane];
-          vd = (uint32_t)y | ((uint32_t)(grp[y + 1] - grp[y]) << 16);
-        }
-        for (int j = 0; j < 32 && p0 + j < ue; ++j) {
-          const uint32_t vdj = __shfl_sync(kFull, vd, j);
-          const int32_t v = (int32_t)(vdj & 0xffffu);
-          const uint32_t dv = vdj >> 16;
-          const uint32_t rv = lane < W ? bm[v * kS + lane] : 0u;
-          const uint32_t T = ru & rv;
-          const uint32_t t = __reduce_add_sync(kFull, (unsigned)__popc(T));
-          a_t += t;
-          a_tt += t * t;
-          a_tdv += t * dv;
-          if (t > 1u) {
-            // T' = the common neighbours above v; the edges inside T' (each
-            // met from both ends) are the 4-cliques with lowest edge (u, v)
-            const int vb = (v + 1) >> 5;
-            const uint32_t above = lane > vb ? 0xffffffffu : (lane == vb ? 0xffffffffu << ((v + 1) & 31) : 0u);
-            const uint32_t Tp = T & above;
-            const uint32_t ct = __reduce_add_sync(kFull, (unsigned)__popc(Tp));
-            if (ct > 1u) a_k += __reduce_add_sync(kFull, masked_row_popc<kS>(bm, Tp, lane, vb, W, list));
+    // this unit's vertices u: part, part + parts, ..., one per warp in turn.
+    // Pairs (u, w), w > u. Sums over one u stay in 32 bits (a lane has at most
+    // 32 pairs, every term below 2^21).
+    auto add_sum = [&](int i, unsigned long long v) {
+      v = warp_sum(v);
+      if (lane == 0 && v) atomicAdd(&s_q[i], v);
+    };
+    {
+      unsigned long long q_t = 0, q_tt = 0, q_ta = 0, q_dd = 0, q_c4 = 0, d2 = 0, d3 = 0;
+      for (int32_t u = part + parts * warp; u < n; u += parts * kWarps) {
+        const uint32_t* rowu = bm + u * kS;
+        const uint32_t du = s_deg[u];
+        uint32_t a_t = 0, a_tt = 0, a_ta = 0, a_dd = 0, a_c4 = 0;
+        for (int32_t w0 = u + 1; w0 < n; w0 += 32) {
+          const int32_t w = w0 + lane;
+          if (w < n) {
+            const uint32_t* roww = bm + w * kS;
+            uint32_t c = 0;
+  #pragma unroll 4
+            for (int k = 0; k < W; ++k) c += __popc(rowu[k] & roww[k]);
+            a_c4 += c * (c - 1u) / 2u;  // 0 for c = 0: the product is 0
+            if ((rowu[w >> 5] >> (w & 31)) & 1u) {
+              const uint32_t dw = s_deg[w];
+              a_t += c;
+              a_tt += c * c;
+              a_ta += c * (du + dw);
+              a_dd += du * dw;
+            }
           }
         }
-      }
-      // sum over the edges of u of t (d_u + d_v) = d_u sum t + sum t d_v
-      const unsigned long long ta = (unsigned long long)(ue - ub) * a_t + a_tdv;
-      const unsigned long long mine = lane == kQt ? (unsigned long long)a_t
-                                      : lane == kQtt ? (unsigned long long)a_tt
-                                                     : lane == kQta ? ta : (unsigned long long)a_k;
-      if (lane < kQd2 && mine) atomicAdd(&s_q[lane], mine);
-    }
-    // the 4-cycles as subgraphs: C(c_uw, 2) over every pair u < w
-    unsigned long long c4 = 0;
-    for (int32_t u = warp; u < n; u += kWarps) {
-      const uint32_t* rowu = bm + u * kS;
-      for (int32_t w0 = u + 1; w0 < n; w0 += 32) {
-        const int32_t w = w0 + lane;
-        if (w < n) {
-          const uint32_t* roww = bm + w * kS;
-          unsigned c = 0;
-          for (int k = 0; k < W; ++k) c += __popc(rowu[k] & roww[k]);
-          c4 += (unsigned long long)c * (c - 1) / 2;
+        q_t += a_t;
+        q_tt += a_tt;
+        q_ta += a_ta;
+        q_dd += a_dd;
+        q_c4 += a_c4;
+        if (lane == 0) {
+          d2 += du * du;
+          d3 += (unsigned long long)(du * du) * du;
         }
       }
+      add_sum(kQt, q_t);
+      add_sum(kQtt, q_tt);
+      add_sum(kQta, q_ta);
+      add_sum(kQdd, q_dd);
+      add_sum(kQc4, q_c4);
+      add_sum(kQd2, d2);
+      add_sum(kQd3, d3);
     }
-    c4 = warp_sum(c4);
-    if (lane == 0 && c4) atomicAdd(&s_c4, c4);
+    // the 4-cliques with lowest vertex u: the triangles of H_u
+    unsigned long long q_k4 = 0;
+    {
+      uint32_t* h = s_h + warp * h_words(kWarpK / 32);
+      uint16_t* m = s_m + warp * kWarpK;
+      for (int32_t u = part + parts * warp; u < n; u += parts * kWarps) {
+        const int k = s_up[u];
+        if (k < 3 || k > kWarpK) continue;  // warp-uniform
+        const int32_t p1 = grp[u + 1] - k;  // the neighbours above u end its ascending row
+        for (int i = lane; i < k; i += 32) m[i] = (uint16_t)gci[p1 + i];
+        __syncwarp();
+        pack_h<kS>(bm, m, k, h, 0, 1, lane);
+        __syncwarp();
+        q_k4 += count_h(h, k, 0, 1, lane);
+        __syncwarp();
+      }
+    }
+    if (kN > kWarpK) {
+      for (int32_t u = part; u < n; u += parts) {
+        const int k = s_up[u];
+        if (k <= kWarpK) continue;  // CTA-uniform
+        __syncthreads();
+        const int32_t p1 = grp[u + 1] - k;
+        for (int i = threadIdx.x; i < k; i += kBlock) s_m[i] = (uint16_t)gci[p1 + i];
+        __syncthreads();
+        pack_h<kS>(bm, s_m, k, s_h, warp, kWarps, lane);
+        __syncthreads();
+        q_k4 += count_h(s_h, k, warp, kWarps, lane);
+      }
+    }
+    add_sum(kQk4, q_k4);
     __syncthreads();
-    if (threadIdx.x < 13) {  // thread k: the graph's unrestricted sum k
-      const unsigned long long c = graph_column(threadIdx.x, s_q, s_c4, n, (eoff[g + 1] - eoff[g]) / 2);
-      if (c) add_u128(csum + ((size_t)g * 13 + threadIdx.x) * 2, (u128)c);
-    }
+    if (threadIdx.x < kQn && s_q[threadIdx.x])
+      atomicAdd(&sums[(size_t)g * kQn + threadIdx.x], s_q[threadIdx.x]);
   }
 }
 
-typedef void (*SmallKernel)(const int32_t*, const int64_t*, const int32_t*, const int64_t*, const int32_t*, int32_t,
+// The unrestricted sums of every graph: thread per (graph, column).
+__global__ void k_small_columns(int32_t G, const int32_t* __restrict__ gn, const int64_t* __restrict__ gm,
+                                const unsigned long long* __restrict__ sums, unsigned long long* __restrict__ csum) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (int64_t)G * 13) return;
+  const int32_t g = (int32_t)(t / 13), k = (int32_t)(t % 13);
+  csum[2 * t] = graph_column(k, sums + (size_t)g * kQn, gn[g], gm[g]);
+  csum[2 * t + 1] = 0ull;
+}
+
+typedef void (*SmallKernel)(const int32_t*, const int64_t*, const int32_t*, const int64_t*, const int2*, int32_t,
                             int32_t*, int32_t*, unsigned long long*);
 
 // kSmallBlocks[j] threads per CTA for tuning choice j.
@@ -332,11 +409,48 @@ static int block_index(int block) {
   return 2;
 }
 
-// Grid of one size class: resident CTAs, at most one CTA per graph.
-static int small_grid(int cls, int block, int32_t graphs) {
+// Grid of one size class: resident CTAs, at most one CTA per unit.
+static int small_grid(int cls, int block, int32_t units) {
   int grid = g_small_ctas[cls][block_index(block)];
   if (grid < 1) grid = 1;
-  return grid > graphs ? graphs : grid;
+  return grid > units ? units : grid;
+}
+
+// Cost of a graph in SM cycles, roughly (n = 500 at density 0.275 measures
+// about 4e5): two cycles per 32 vertex pairs and word; H_u for k neighbours
+// above u, k spread evenly over [0, 2 m / n], at k^2 / 64 ballots and k^3 /
+// 6144 words of 32 pairs; and the bit rows.
+static double small_cost(int32_t n, int64_t m) {
+  const double W = (n + 31) / 32, k = n > 0 ? (double)m / n : 0.0;
+  return (double)n * n * W / 32 + n * (k * k / 18 + k * k * k / 750 + 20) + (double)m / 4;
+}
+
+void small_units(const std::vector<int32_t>& n, const std::vector<int64_t>& m, std::vector<int2>* units,
+                 int32_t* class_off) {
+  const int32_t G = (int32_t)n.size();
+  std::vector<double> cost((size_t)G);
+  double total = 0;
+  for (int32_t g = 0; g < G; ++g) total += cost[(size_t)g] = small_cost(n[(size_t)g], m[(size_t)g]);
+  // A graph is cut into parts when it would be a long single tail, or when
+  // the launch has too few graphs for the GPU: parts of about an eighth of an
+  // SM's share, but no smaller than kLeast, since each part loads all bit rows
+  // again. 48 graphs of n in [20, 500]: 5.9 ms uncut.
+  constexpr double kLeast = 25000;
+  const double target = std::max(kLeast, total / (8.0 * (count_grid_size() / kCtasPerSm)));
+  std::vector<std::pair<double, int2>> per_class[kSmallClasses];
+  for (int32_t g = 0; g < G; ++g) {
+    const double c = cost[(size_t)g];
+    const int parts = c > 2 * target ? (int)std::min(32.0, c / target) : 1;
+    for (int p = 0; p < parts; ++p)
+      per_class[small_class_of(n[(size_t)g])].push_back({c / parts, make_int2(g, p | (parts << 16))});
+  }
+  units->clear();
+  for (int c = 0; c < kSmallClasses; ++c) {
+    std::sort(per_class[c].begin(), per_class[c].end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+    class_off[c] = (int32_t)units->size();
+    for (auto& u : per_class[c]) units->push_back(u.second);
+  }
+  class_off[kSmallClasses] = (int32_t)units->size();
 }
 
 gc_status small_graphs_setup() {
@@ -357,28 +471,36 @@ gc_status small_graphs_setup() {
   return GC_OK;
 }
 
-gc_status run_small_graphs(const int32_t* rp, const int64_t* voff, const int32_t* ci, const int64_t* eoff,
-                           const int32_t* order, const int32_t* class_off, int32_t* cursor, int32_t* status,
-                           unsigned long long* csum, const BatchConfig& cfg, cudaEvent_t* ev, cudaStream_t s) {
-  for (int c = 0; c < kSmallClasses; ++c) {
-    const int32_t G = class_off[c + 1] - class_off[c];
-    if (ev) {
-      cudaError_t e = cudaEventRecord(ev[c], s);
-      if (e != cudaSuccess) return cuda_fail(e, "small event");
+gc_status run_small_graphs(const SmallGraphs& b, const int32_t* class_off, const BatchConfig& cfg, cudaEvent_t* ev,
+                           const SmallFork* fork, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  if (fork && (e = cudaEventRecord(fork->start, s)) != cudaSuccess) return cuda_fail(e, "small fork");
+  for (int c = kSmallClasses - 1; c >= 0; --c) {  // the largest graphs first
+    const int32_t units = class_off[c + 1] - class_off[c];
+    if (ev && (e = cudaEventRecord(ev[2 * c], s)) != cudaSuccess) return cuda_fail(e, "small event");
+    if (units > 0) {
+      cudaStream_t sc = s;
+      if (fork) {
+        sc = fork->stream[c];
+        if ((e = cudaStreamWaitEvent(sc, fork->start, 0)) != cudaSuccess) return cuda_fail(e, "small fork");
+      }
+      const int block = valid_block(cfg.class_block[c]);
+      const int grid = small_grid(c, block, units);
+      small_kernel(c, block)<<<grid, block, small_smem(kSmallClassN[c], block), sc>>>(
+          b.rp, b.voff, b.ci, b.eoff, b.units + class_off[c], units, b.cursor + c, b.status, b.sums);
+      if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "k_small_graphs");
+      if (fork) {
+        if ((e = cudaEventRecord(fork->done[c], sc)) != cudaSuccess ||
+            (e = cudaStreamWaitEvent(s, fork->done[c], 0)) != cudaSuccess)
+          return cuda_fail(e, "small join");
+      }
     }
-    if (G <= 0) continue;
-    const int block = valid_block(cfg.class_block[c]);
-    const int grid = small_grid(c, block, G);
-    small_kernel(c, block)<<<grid, block, small_smem(kSmallClassN[c], block), s>>>(
-        rp, voff, ci, eoff, order + class_off[c], G, cursor + c, status, csum);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "k_small_graphs");
+    if (ev && (e = cudaEventRecord(ev[2 * c + 1], s)) != cudaSuccess) return cuda_fail(e, "small event");
   }
-  if (ev) {
-    cudaError_t e = cudaEventRecord(ev[kSmallClasses], s);
-    if (e != cudaSuccess) return cuda_fail(e, "small event");
-  }
-  return GC_OK;
+  const int64_t cols = (int64_t)b.G * 13;
+  if (cols > 0) k_small_columns<<<(int)((cols + 255) / 256), 256, 0, s>>>(b.G, b.gn, b.gm, b.sums, b.csum);
+  e = cudaGetLastError();
+  return e == cudaSuccess ? GC_OK : cuda_fail(e, "k_small_columns");
 }
 
 }  // namespace gc

@@ -252,6 +252,35 @@ def test_hub_counts_at_the_counter_field_limits(nx, per):
     assert w["c_heavy_wedges"] >= W[0] and w["c_wedges"] == W.sum()
 
 
+@pytest.mark.parametrize("n,k", [(33, 32), (64, 63), (130, 128), (131, 129), (512, 510), (1024, 1022), (600, 161)])
+@pytest.mark.parametrize("copies", [1, 700])
+def test_batch_four_cliques_of_wide_neighbourhoods(n, k, copies):
+    # vertex 0 joined to vertices 1 .. k, which form a dense random graph: H_0
+    # has k members -- a warp's (up to 128) and the CTA's, partial and whole
+    # words, up to the largest of a size class; alone (a launch of few graphs
+    # is cut into parts) and among others (it is not)
+    rng = np.random.default_rng(n)
+    adj = np.zeros((n, n), bool)
+    adj[0, 1:k + 1] = True
+    adj[1:k + 1, 1:k + 1] = np.triu(rng.random((k, k)) < 0.3, 1)
+    adj |= adj.T
+    rp = np.concatenate([[0], np.cumsum(adj.sum(1))]).astype(np.int32)
+    ci = np.nonzero(adj)[1].astype(np.int32)
+    path = graphs.csr(40, [(i, i + 1) for i in range(39)])
+    all_g = [(rp, ci)] + [path] * (copies - 1)
+    b = gcb.gc_batch_create(8 << 30, gcb.GC_BATCH_MANUAL)
+    try:
+        gcb.gc_batch_set_param(b, gcb.GC_PARAM_SMALL_N_MAX, 1024)
+        t = [gcb.gc_batch_submit(b, *g) for g in all_g]
+        gcb.gc_batch_flush(b)
+        X = [gcb.gc_batch_poll(b, k_) for k_ in t]
+    finally:
+        gcb.gc_batch_destroy(b)
+    assert X[0] == oracle.count(rp, ci)["X"]
+    ref = oracle.count(*path)["X"]
+    assert all(x == ref for x in X[1:])
+
+
 def test_hub_over_a_skewed_o_range():
     # 3M vertices, almost all isolated (the lowest ranks): h has 620 lower
     # neighbours, 600 of them with 150 o each, drawn with weights 1/(i + 100)

@@ -173,7 +173,9 @@ gc_status gc_count_edge_induced(gc_graph g, uint64_t* induced_out, uint64_t* per
 gc_status gc_graph_csums(gc_graph g, uint64_t* lo, uint64_t* hi);
 
 /* Device time of each phase of the last gc_count_edge_graphlets, measured
- * with CUDA events on the graph's stream. ms: host array of
+ * with CUDA events (in graphs of fewer than 2^22 edges the cycles phase runs
+ * beside the triangle and clique phases, so that they add up to more than the
+ * count takes). ms: host array of
  * gc_phase_count() doubles. Phases, in order: "pass_t_triangles" (Alg. 1),
  * "pass_c_cycles" (4-cycles through each edge, Alg. 4/6), "pass_k_cliques"
  * (4-cliques and cross terms, Alg. 3/5), "finish_columns" (Sec. 4.5 columns

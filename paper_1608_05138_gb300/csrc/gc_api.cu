@@ -65,6 +65,84 @@ cudaMemPool_t lib_pool() {
 }
 
 namespace {
+std::mutex g_fork_mu;
+std::vector<ForkSet*> g_forks;          // idle sets, of any device
+constexpr size_t kForksKept = 16;
+
+void fork_destroy(ForkSet* f) {
+  for (auto& t : f->stream)
+    if (t) cudaStreamDestroy(t);
+  for (cudaEvent_t e : f->done)
+    if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : f->begin)
+    if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : f->end)
+    if (e) cudaEventDestroy(e);
+  if (f->start) cudaEventDestroy(f->start);
+  if (f->pinned) cudaFreeHost(f->pinned);
+  delete f;
+}
+}  // namespace
+
+ForkSet* fork_acquire() {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) {
+    cuda_fail(e, "cudaGetDevice");
+    return nullptr;
+  }
+  {
+    std::lock_guard<std::mutex> lk(g_fork_mu);
+    for (size_t i = 0; i < g_forks.size(); ++i)
+      if (g_forks[i]->device == dev) {
+        ForkSet* f = g_forks[i];
+        g_forks.erase(g_forks.begin() + (long)i);
+        return f;
+      }
+  }
+  ForkSet* f = new (std::nothrow) ForkSet();
+  if (!f) {
+    set_error("host allocation failed");
+    return nullptr;
+  }
+  f->device = dev;
+  for (auto& t : f->stream)
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);
+  for (auto& d : f->done)
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&d, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f->start, cudaEventDisableTiming);
+  for (int k = 0; k < kNumPhases; ++k) {
+    if (e == cudaSuccess) e = cudaEventCreate(&f->begin[k]);
+    if (e == cudaSuccess) e = cudaEventCreate(&f->end[k]);
+  }
+  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&f->pinned), kPinnedBytes);
+  if (e != cudaSuccess) {
+    cuda_fail(e, "side streams");
+    fork_destroy(f);
+    return nullptr;
+  }
+  return f;
+}
+
+void fork_drain(ForkSet* f) {
+  if (!f) return;
+  for (auto& t : f->stream) cudaStreamSynchronize(t);
+  cudaGetLastError();
+}
+
+void fork_release(ForkSet* f) {
+  if (!f) return;
+  {
+    std::lock_guard<std::mutex> lk(g_fork_mu);
+    if (g_forks.size() < kForksKept) {
+      g_forks.push_back(f);
+      return;
+    }
+  }
+  fork_destroy(f);
+}
+
+namespace {
 
 int host_threads() {
   const unsigned hw = std::thread::hardware_concurrency();
@@ -420,11 +498,9 @@ struct gc_graph_s {
   int64_t* d_gm = nullptr;     // [1] m
   // counting scratch
   Scratch sc;
-  unsigned long long* d_csum = nullptr;  // [13][2]
-  unsigned long long* d_x = nullptr;     // [17][2]
   uint64_t* d_pe_tmp = nullptr;          // device staging for a host per-edge buffer
   uint64_t* d_ind_tmp = nullptr;         // device staging for a host per-edge induced buffer
-  cudaEvent_t ev[kNumPhases + 1] = {};
+  ForkSet* fs = nullptr;                 // side streams, events and the pinned results
   bool counted = false;
   uint64_t csum_lo[13] = {0}, csum_hi[13] = {0};
   uint64_t work[kNumWork] = {0};
@@ -452,14 +528,13 @@ static void graph_release(gc_graph g) {
   // stream-ordered frees into the library pool (after the graph's queued
   // work), then one synchronisation
   const cudaStream_t s = g->stream;
-  for (void* p : {(void*)g->d_rp, (void*)g->d_ci, (void*)g->d_gbase, (void*)g->d_csum, (void*)g->d_pe_tmp,
+  for (void* p : {(void*)g->d_rp, (void*)g->d_ci, (void*)g->d_gbase, (void*)g->d_pe_tmp,
                   (void*)g->d_ind_tmp})
     if (p) cudaFreeAsync(p, s);
   free_prep(&g->prep, s);
   scratch_free(&g->sc, s);
   cudaStreamSynchronize(s);
-  for (auto& e : g->ev)
-    if (e) cudaEventDestroy(e);
+  fork_release(g->fs);
   delete g;
 }
 
@@ -603,14 +678,12 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
     g->d_gn = g->d_gbase + 1;
     g->d_gm = reinterpret_cast<int64_t*>(reinterpret_cast<char*>(g->d_gbase) + 16);
   }
-  GC_CHECK(pool_alloc(&g->d_csum, sizeof(unsigned long long) * (13 * 2 + 17 * 2), s), "alloc sums");
-  g->d_x = g->d_csum + 13 * 2;
   {
-    gc_status st2 = scratch_init(&g->sc, g->m, n, g->prep.kmax, s);
+    gc_status st2 = scratch_init(&g->sc, g->m, n, g->prep.kmax, g->prep.ktier_off, 1, s);
     if (st2 != GC_OK) return fail(st2);
     scratch_guess_tlist(&g->sc, g->m);
   }
-  for (auto& ev : g->ev) GC_CHECK(cudaEventCreate(&ev), "event create");
+  if (!(g->fs = fork_acquire())) return fail(GC_ERR_CUDA);
   GC_CHECK(cudaStreamSynchronize(s), "sync upload");
 #undef GC_CHECK
   *out = g;
@@ -723,16 +796,13 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
   ku.n_chash2_big = g->prep.n_chash2_big;
   ku.n_cunits = g->prep.n_cunits;
   for (int t = 0; t <= kNumTiers; ++t) ku.tier_off[t] = g->prep.ktier_off[t];
-  if ((st = run_count(dg, g->prep.units, g->prep.n_units, ku, pe_dev, g->d_csum, g->d_x, &g->sc, s, g->ev, pe_host,
-                      ind_dev, ind_host)) != GC_OK)
+  if ((st = run_count(dg, g->prep.units, g->prep.n_units, ku, pe_dev, &g->sc, s, g->fs, pe_host, ind_dev, ind_host)) != GC_OK) {
+    fork_drain(g->fs);
     return st;
-  unsigned long long hx[17 * 2 + 13 * 2];
-  int32_t hstatus = 0;
-  GC_CHECK(cudaMemcpyAsync(hx, g->d_x, sizeof(unsigned long long) * 17 * 2, cudaMemcpyDeviceToHost, s), "copy X");
-  GC_CHECK(cudaMemcpyAsync(hx + 34, g->d_csum, sizeof(unsigned long long) * 13 * 2, cudaMemcpyDeviceToHost, s),
-           "copy C");
-  GC_CHECK(cudaMemcpyAsync(&hstatus, g->sc.misc + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "copy status");
-  GC_CHECK(cudaMemcpyAsync(g->work, g->sc.work, sizeof(g->work), cudaMemcpyDeviceToHost, s), "copy work");
+  }
+  // the results' head of the scratch in one copy: status, work, sums, X
+  if (g->sc.head_bytes > kPinnedBytes) { set_error("internal: results do not fit"); return GC_ERR_CUDA; }
+  GC_CHECK(cudaMemcpyAsync(g->fs->pinned, g->sc.zero, g->sc.head_bytes, cudaMemcpyDeviceToHost, s), "copy results");
   if (staged)
     GC_CHECK(cudaMemcpyAsync(per_edge_out, pe_dev, sizeof(uint64_t) * 13 * (size_t)g->m, cudaMemcpyDeviceToHost, s),
              "copy per-edge");
@@ -740,8 +810,13 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
     GC_CHECK(cudaMemcpyAsync(induced_out, ind_dev, sizeof(uint64_t) * GC_INDUCED_COLS * (size_t)g->m,
                              cudaMemcpyDeviceToHost, s),
              "copy induced");
-  GC_CHECK(cudaEventRecord(g->ev[kNumPhases], s), "event");
+  GC_CHECK(cudaEventRecord(g->fs->end[kPhaseCopy], s), "event");
   GC_CHECK(cudaStreamSynchronize(s), "sync count");
+  auto host_of = [&](const void* d) { return g->fs->pinned + (static_cast<const unsigned char*>(d) - g->sc.zero); };
+  const int32_t hstatus = reinterpret_cast<const int32_t*>(host_of(g->sc.misc))[1];
+  std::memcpy(g->work, host_of(g->sc.work), sizeof(g->work));
+  const uint64_t* hx = reinterpret_cast<const uint64_t*>(host_of(g->sc.x));
+  const uint64_t* hc = reinterpret_cast<const uint64_t*>(host_of(g->sc.csum));
   g->sc.tlist_want = (long long)g->work[kWorkTTriangles];  // the next count keeps pass T's edge lists
 #undef GC_CHECK
   if (hstatus & kSpillOverflow) {
@@ -759,8 +834,8 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
     if (hx[2 * i + 1]) need_hi = true;
   }
   for (int k = 0; k < 13; ++k) {
-    g->csum_lo[k] = hx[34 + 2 * k];
-    g->csum_hi[k] = hx[34 + 2 * k + 1];
+    g->csum_lo[k] = hc[2 * k];
+    g->csum_hi[k] = hc[2 * k + 1];
   }
   g->counted = true;
   if (need_hi && !global_hi) {
@@ -813,7 +888,7 @@ gc_status gc_graph_phase_ms(gc_graph g, double* ms) {
   if (!g->counted) { set_error("graph not counted yet"); return GC_ERR_ARG; }
   for (int i = 0; i < kNumPhases; ++i) {
     float f = 0.f;
-    cudaError_t e = cudaEventElapsedTime(&f, g->ev[i], g->ev[i + 1]);
+    cudaError_t e = cudaEventElapsedTime(&f, g->fs->begin[i], g->fs->end[i]);
     if (e != cudaSuccess) return cuda_fail(e, "event elapsed");
     ms[i] = f;
   }

@@ -193,6 +193,7 @@ struct gc_batch_s {
   uint32_t flags = 0;
   BatchConfig cfg;
   SmallBufs small[kMaxInflight];        // per stream slot
+  ForkSet* forks[kMaxInflight] = {};    // per stream slot, of the larger graphs' launches
   double last_stats[GC_BATCH_STATS] = {};  // of the last retired launch
   int64_t in_use = 0;
   std::mutex mu;
@@ -218,8 +219,8 @@ namespace {
 // The graphs too large for the bitmatrix kernel, as one disjoint union
 // through the general passes. Results go to h_x_dst ([G][17][2], pinned) and
 // the launch status word to *h_status_dst.
-gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* L, unsigned long long* h_x_dst,
-                    int32_t* h_status_dst) {
+gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet* fs, Launch* L,
+                    unsigned long long* h_x_dst, int32_t* h_status_dst) {
   const int32_t G = (int32_t)graphs.size();
   int64_t n_total = 0, nnz_total = 0;
   int32_t table_n = 0;
@@ -252,7 +253,6 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
   }
   int32_t *d_rp = nullptr, *d_ci = nullptr, *d_vgid = nullptr, *d_desc = nullptr;
   int64_t* d_gm = nullptr;
-  unsigned long long *d_csum = nullptr, *d_x = nullptr;
   PrepBuffers prep;
   Scratch sc;
   cudaError_t e = cudaSuccess;
@@ -274,8 +274,6 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
   GB_TRY(pool_alloc(&d_vgid, sizeof(int32_t) * h_vgid.size(), s), "batch alloc");
   GB_TRY(pool_alloc(&d_desc, sizeof(int32_t) * h_desc.size(), s), "batch alloc");
   GB_TRY(pool_alloc(&d_gm, sizeof(int64_t) * G, s), "batch alloc");
-  GB_TRY(pool_alloc(&d_csum, sizeof(unsigned long long) * (size_t)G * 26, s), "batch alloc");
-  GB_TRY(pool_alloc(&d_x, sizeof(unsigned long long) * (size_t)G * 34, s), "batch alloc");
   GB_TRY(cudaMemcpyAsync(d_rp, h_rp.data(), sizeof(int32_t) * h_rp.size(), cudaMemcpyHostToDevice, s), "batch copy");
   GB_TRY(cudaMemcpyAsync(d_ci, h_ci.data(), sizeof(int32_t) * h_ci.size(), cudaMemcpyHostToDevice, s), "batch copy");
   GB_TRY(cudaMemcpyAsync(d_vgid, h_vgid.data(), sizeof(int32_t) * h_vgid.size(), cudaMemcpyHostToDevice, s), "batch copy");
@@ -290,7 +288,7 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
     L->error = gc_last_error();
     goto out;
   }
-  if ((st = scratch_init(&sc, m, table_n, prep.kmax, s)) != GC_OK) {
+  if ((st = scratch_init(&sc, m, table_n, prep.kmax, prep.ktier_off, G, s)) != GC_OK) {
     L->error = gc_last_error();
     goto out;
   }
@@ -331,11 +329,12 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
     ku.n_chash2_big = prep.n_chash2_big;
     ku.n_cunits = prep.n_cunits;
     for (int t = 0; t <= kNumTiers; ++t) ku.tier_off[t] = prep.ktier_off[t];
-    if ((st = run_count(dg, prep.units, prep.n_units, ku, nullptr, d_csum, d_x, &sc, s, nullptr)) != GC_OK) {
+    if ((st = run_count(dg, prep.units, prep.n_units, ku, nullptr, &sc, s, fs)) != GC_OK) {
+      fork_drain(fs);
       L->error = gc_last_error();
       goto out;
     }
-    GB_TRY(cudaMemcpyAsync(h_x_dst, d_x, sizeof(unsigned long long) * (size_t)G * 34, cudaMemcpyDeviceToHost, s),
+    GB_TRY(cudaMemcpyAsync(h_x_dst, sc.x, sizeof(unsigned long long) * (size_t)G * 34, cudaMemcpyDeviceToHost, s),
            "batch copy out");
     GB_TRY(cudaMemcpyAsync(h_status_dst, sc.misc + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "batch copy out");
   }
@@ -343,7 +342,7 @@ out:
 #undef GB_TRY
   free_prep(&prep, s);
   scratch_free(&sc, s);
-  for (void* p : {(void*)d_rp, (void*)d_ci, (void*)d_vgid, (void*)d_desc, (void*)d_gm, (void*)d_csum, (void*)d_x})
+  for (void* p : {(void*)d_rp, (void*)d_ci, (void*)d_vgid, (void*)d_desc, (void*)d_gm})
     if (p) cudaFreeAsync(p, s);
   return st;
 }
@@ -559,7 +558,14 @@ void run_launch(gc_batch b, std::vector<PendingGraph>& graphs, cudaStream_t s, L
   if (!small.empty()) st = run_small(small, s, L, L->h_x, &b->small[L->stream_slot], cfg);
   if (st == GC_OK && !large.empty()) {
     cudaEventRecord(L->ev[kEvUnion0], s);
-    st = run_union(large, s, L, L->h_x + 34 * small.size(), L->h_status + 1);
+    ForkSet*& fs = b->forks[L->stream_slot];
+    if (!fs) fs = fork_acquire();
+    if (!fs) {
+      st = GC_ERR_CUDA;
+      L->error = gc_last_error();
+    } else {
+      st = run_union(large, s, fs, L, L->h_x + 34 * small.size(), L->h_status + 1);
+    }
     cudaEventRecord(L->ev[kEvUnion1], s);
     L->timed_union = st == GC_OK;
   }
@@ -1022,6 +1028,7 @@ gc_status gc_batch_destroy(gc_batch b) {
     retire_locked(b);
   }
   for (auto& sb : b->small) free_small_bufs(&sb);
+  for (auto* f : b->forks) fork_release(f);
   for (auto& s : b->streams) cudaStreamDestroy(s);
   delete b;
   return GC_OK;

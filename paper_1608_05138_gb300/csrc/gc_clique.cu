@@ -100,8 +100,9 @@ struct KLayout {
 // triangle also adds the degree of its third vertex to each of its edges,
 // so that a.dsum[e] = sum_{w in T_e} d_w (for the per-edge induced counts).
 template <int kCap, int kThreads, bool kTri, bool kDeg = false>
-__global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThreads * 64)) k_pass_k(DevGraph g, CountArgs a, int tier) {
+__global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThreads * 64)) k_pass_k(DevGraph g, CountArgs a) {
   constexpr int kW = kThreads / 32;
+  constexpr int tier = kCap == 0 ? kTierGlobal : kCap == 1024 ? kTier1024 : kCap == 512 ? kTier512 : kTier256;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int32_t s_unit, s_cur1, s_cur2, s_nhit;
   __shared__ long long s_loff;
@@ -127,7 +128,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
   int32_t* qq = s_qq[warp];
   // phase-1 hits (i, j, out-slot): pass K's phase 2 needs no rescan, and
   // pass T hands them on to pass K
-  int32_t* hits = (kTri && !a.tlist) ? nullptr : a.hitbuf + (size_t)blockIdx.x * 2 * (size_t)a.hitcap;
+  int2* hits = (kTri && !a.tlist) ? nullptr : a.hitbuf + a.hit_off[tier] + (int64_t)blockIdx.x * a.hit_cap[tier];
 
   const int32_t u0 = a.ktier_off[tier], u1 = a.ktier_off[tier + 1];
   int32_t* cursor = a.cursor + (kTri ? 10 : 2) + tier;
@@ -289,8 +290,8 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
             if (lane == 0) base_h = atomicAdd(&s_nhit, __popc(hit));
             base_h = __shfl_sync(kFull, base_h, 0);
             const int32_t slot = base_h + __popc(hit & ((1u << lane) - 1u));
-            if (j >= 0 && slot < a.hitcap)
-              reinterpret_cast<int2*>(hits)[slot] = make_int2((int32_t)(((uint32_t)i << 16) | (uint32_t)j), q);
+            if (j >= 0 && slot < a.hit_cap[tier])
+              hits[slot] = make_int2((int32_t)(((uint32_t)i << 16) | (uint32_t)j), q);
           }
           pend -= take;
           __syncwarp();  // the entries are read before the buffer is refilled
@@ -349,8 +350,8 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
               atomicOr(&rows[i * S + (j >> 5)], 1u << (j & 31));
               atomicOr(&rows[j * S + (i >> 5)], 1u << (i & 31));
               const int32_t slot = base_h + __popc(hit & ((1u << lane) - 1u));
-              if (slot < a.hitcap)  // read only when k <= 65535
-                reinterpret_cast<int2*>(hits)[slot] = make_int2((int32_t)(((uint32_t)i << 16) | (uint32_t)j), q);
+              if (slot < a.hit_cap[tier])  // read only when k <= 65535
+                hits[slot] = make_int2((int32_t)(((uint32_t)i << 16) | (uint32_t)j), q);
             }
           }
         }
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
         const int32_t nh = s_nhit;
         if (threadIdx.x == 0) {
           long long off = -1;
-          if (nh <= a.hitcap && k <= 65535) {
+          if (nh <= a.hit_cap[tier] && k <= 65535) {
             const unsigned long long o = atomicAdd(a.tlist_fill, (unsigned long long)nh);
             if ((long long)o + nh <= a.tlist_cap) off = (long long)o;
           }
@@ -382,18 +383,18 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
         const long long off = s_loff;
         if (off >= 0)
           for (int32_t e = threadIdx.x; e < nh; e += kThreads)
-            a.tlist[off + e] = reinterpret_cast<const int2*>(hits)[e];
+            a.tlist[off + e] = hits[e];
       }
       continue;
     }
     const int32_t nhit = s_nhit;
 
-    if (nhit <= a.hitcap && k <= 65535) {  // (i, j) packed in 16 bits each
+    if (nhit <= a.hit_cap[tier] && k <= 65535) {  // (i, j) packed in 16 bits each
       // Phase 2 over the recorded edges of H_a: lane per edge.
       for (int32_t e0 = warp * 32; e0 < nhit; e0 += kThreads) {
         const int32_t e = e0 + lane;
         if (e < nhit) {
-          const int2 en = reinterpret_cast<const int2*>(hits)[e];
+          const int2 en = hits[e];
           const int32_t ij = en.x, q = en.y;
           const int32_t i = (int32_t)((uint32_t)ij >> 16), j = ij & 0xffff;
           const uint32_t* ri = rows + i * S;
@@ -524,7 +525,8 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x)
 }
 
 template <bool kTri, bool kDeg = false>
-__global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a, int tier) {
+__global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a) {
+  constexpr int tier = kTier32;
   __shared__ int32_t s_q[kWWarps][32 * 32];  // out-slot of edge (i, j) found from member i
   __shared__ uint32_t s_rowf[kWWarps][64];    // rows and found masks rebuilt from pass T's list
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -707,7 +709,7 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
 }
 
 template <int kCap, int kThreads, bool kTri, bool kDeg = false>
-gc_status launch_tier(const DevGraph& g, const CountArgs& a, int tier, cudaStream_t s, int* launches) {
+gc_status launch_tier(const DevGraph& g, const CountArgs& a, int tier, Fork* fork, int* launches) {
   const int32_t units = a.ktier_off[tier + 1] - a.ktier_off[tier];
   if (units <= 0) return GC_OK;
   const size_t smem = kCap ? KLayout(kCap, !kTri).total : 0;
@@ -723,28 +725,28 @@ gc_status launch_tier(const DevGraph& g, const CountArgs& a, int tier, cudaStrea
   } else {
     grid = a.kbuf_ctas;
   }
-  if (grid > a.hitbuf_ctas) grid = a.hitbuf_ctas;  // one hit buffer per CTA
+  if (grid > a.hit_ctas[tier]) grid = a.hit_ctas[tier];  // one hit list per CTA
   if (grid > units) grid = units;
   if (grid < 1) return GC_OK;
-  kern<<<grid, kThreads, smem, s>>>(g, a, tier);
+  kern<<<grid, kThreads, smem, fork->next()>>>(g, a);
   ++*launches;
   e = cudaGetLastError();
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "k_pass_k");
 }
 
 template <bool kTri, bool kDeg = false>
-gc_status run_tiers(const DevGraph& g, const CountArgs& a, cudaStream_t s, int* launches) {
+gc_status run_tiers(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches) {
   gc_status st;
   if (a.ktier_off[kTierGlobal + 1] > a.ktier_off[kTierGlobal]) {
     if (!a.kbuf || a.kbuf_ctas < 1) {
       set_error("internal: pass K global buffers missing");
       return GC_ERR_CUDA;
     }
-    if ((st = launch_tier<0, 1024, kTri, kDeg>(g, a, kTierGlobal, s, launches)) != GC_OK) return st;
+    if ((st = launch_tier<0, 1024, kTri, kDeg>(g, a, kTierGlobal, fork, launches)) != GC_OK) return st;
   }
-  if ((st = launch_tier<1024, kTri ? 512 : 1024, kTri, kDeg>(g, a, kTier1024, s, launches)) != GC_OK) return st;
-  if ((st = launch_tier<512, 512, kTri, kDeg>(g, a, kTier512, s, launches)) != GC_OK) return st;
-  if ((st = launch_tier<256, 512, kTri, kDeg>(g, a, kTier256, s, launches)) != GC_OK) return st;
+  if ((st = launch_tier<1024, kTri ? 512 : 1024, kTri, kDeg>(g, a, kTier1024, fork, launches)) != GC_OK) return st;
+  if ((st = launch_tier<512, 512, kTri, kDeg>(g, a, kTier512, fork, launches)) != GC_OK) return st;
+  if ((st = launch_tier<256, 512, kTri, kDeg>(g, a, kTier256, fork, launches)) != GC_OK) return st;
   const int32_t units = a.ktier_off[kTier32 + 1] - a.ktier_off[kTier32];
   if (units > 0) {
     int per_sm = 0;
@@ -753,7 +755,7 @@ gc_status run_tiers(const DevGraph& g, const CountArgs& a, cudaStream_t s, int* 
     int grid = (per_sm > 0 ? per_sm : 1) * (count_grid_size() / kCtasPerSm);
     const int need = (units + kWWarps - 1) / kWWarps;
     if (grid > need) grid = need;
-    k_pass_k_warp<kTri, kDeg><<<grid, kWBlock, 0, s>>>(g, a, kTier32);
+    k_pass_k_warp<kTri, kDeg><<<grid, kWBlock, 0, fork->next()>>>(g, a);
     ++*launches;
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "k_pass_k_warp");
@@ -765,12 +767,12 @@ gc_status run_tiers(const DevGraph& g, const CountArgs& a, cudaStream_t s, int* 
 
 size_t kbuf_bytes(int32_t cap) { return cap > 0 ? KLayout(cap).total : 0; }
 
-gc_status run_pass_k(const DevGraph& g, const CountArgs& a, cudaStream_t s, int* launches) {
-  return run_tiers<false>(g, a, s, launches);
+gc_status run_pass_k(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches) {
+  return run_tiers<false>(g, a, fork, launches);
 }
 
-gc_status run_pass_t(const DevGraph& g, const CountArgs& a, cudaStream_t s, int* launches) {
-  return a.dsum ? run_tiers<true, true>(g, a, s, launches) : run_tiers<true>(g, a, s, launches);
+gc_status run_pass_t(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches) {
+  return a.dsum ? run_tiers<true, true>(g, a, fork, launches) : run_tiers<true>(g, a, fork, launches);
 }
 
 }  // namespace gc

@@ -1026,7 +1026,7 @@ gc_status run_pass_c_heavy(const DevGraph& g, const CountArgs& a, cudaStream_t s
 
 template <int kThreads, int kMaxW>
 static gc_status launch_hash(const DevGraph& g, const CountArgs& a, int32_t k0, int32_t k1, int32_t* cursor,
-                             cudaStream_t s) {
+                             Fork* fork, int* launches) {
   if (k1 <= k0) return GC_OK;
   auto kern = k_pass_c_hash<kThreads, kMaxW>;
   const size_t smem = sizeof(int32_t) * 2 * kMaxW + sizeof(uint32_t) * kMaxW;
@@ -1037,23 +1037,24 @@ static gc_status launch_hash(const DevGraph& g, const CountArgs& a, int32_t k0, 
   if (e != cudaSuccess) return cuda_fail(e, "k_pass_c_hash occupancy");
   int grid = (per_sm > 0 ? per_sm : 1) * (count_grid_size() / kCtasPerSm);
   if (grid > k1 - k0) grid = k1 - k0;
-  kern<<<grid, kThreads, smem, s>>>(g, a, k0, k1, cursor);
+  kern<<<grid, kThreads, smem, fork->next()>>>(g, a, k0, k1, cursor);
+  ++*launches;
   e = cudaGetLastError();
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "k_pass_c_hash");
 }
 
-gc_status run_pass_c_hash(const DevGraph& g, const CountArgs& a, cudaStream_t s) {
+gc_status run_pass_c_hash(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches) {
   if (a.n_chash <= 0) return GC_OK;
-  gc_status st = launch_hash<kHashBlock, kHashMaxW>(g, a, 0, a.n_chash_mid, a.cursor + 9, s);
+  gc_status st = launch_hash<kHashBlock, kHashMaxW>(g, a, 0, a.n_chash_mid, a.cursor + 9, fork, launches);
   if (st != GC_OK) return st;
-  st = launch_hash<kHashMidBlock, kHashMidW>(g, a, a.n_chash_mid, a.n_chash_big, a.cursor + 16, s);
+  st = launch_hash<kHashMidBlock, kHashMidW>(g, a, a.n_chash_mid, a.n_chash_big, a.cursor + 16, fork, launches);
   if (st != GC_OK) return st;
-  return launch_hash<kHashSmallBlock, kHashSmallW>(g, a, a.n_chash_big, a.n_chash, a.cursor + 7, s);
+  return launch_hash<kHashSmallBlock, kHashSmallW>(g, a, a.n_chash_big, a.n_chash, a.cursor + 7, fork, launches);
 }
 
 template <int kThreads, int kSlots>
 static gc_status launch_hash2(const DevGraph& g, const CountArgs& a, int32_t k0, int32_t k1, int32_t* cursor,
-                              cudaStream_t s) {
+                              Fork* fork, int* launches) {
   if (k1 <= k0) return GC_OK;
   auto kern = k_pass_c_hash2<kThreads, kSlots>;
   const size_t smem = sizeof(uint32_t) * kSlots;
@@ -1064,16 +1065,17 @@ static gc_status launch_hash2(const DevGraph& g, const CountArgs& a, int32_t k0,
   if (e != cudaSuccess) return cuda_fail(e, "k_pass_c_hash2 occupancy");
   int grid = (per_sm > 0 ? per_sm : 1) * (count_grid_size() / kCtasPerSm);
   if (grid > k1 - k0) grid = k1 - k0;
-  kern<<<grid, kThreads, smem, s>>>(g, a, k0, k1, cursor);
+  kern<<<grid, kThreads, smem, fork->next()>>>(g, a, k0, k1, cursor);
+  ++*launches;
   e = cudaGetLastError();
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "k_pass_c_hash2");
 }
 
-gc_status run_pass_c_hash2(const DevGraph& g, const CountArgs& a, cudaStream_t s) {
+gc_status run_pass_c_hash2(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches) {
   if (a.n_chash2 <= 0) return GC_OK;
-  gc_status st = launch_hash2<kHash2Block, kHash2Slots>(g, a, 0, a.n_chash2_big, a.cursor + 15, s);
+  gc_status st = launch_hash2<kHash2Block, kHash2Slots>(g, a, 0, a.n_chash2_big, a.cursor + 15, fork, launches);
   if (st != GC_OK) return st;
-  return launch_hash2<kHash2Block / 2, kHash2HalfSlots>(g, a, a.n_chash2_big, a.n_chash2, a.cursor + 17, s);
+  return launch_hash2<kHash2Block / 2, kHash2HalfSlots>(g, a, a.n_chash2_big, a.n_chash2, a.cursor + 17, fork, launches);
 }
 
 gc_status run_finish(const DevGraph& g, const CountArgs& a, cudaStream_t s) {

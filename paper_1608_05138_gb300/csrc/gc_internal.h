@@ -100,9 +100,11 @@ struct CountArgs {
   size_t kbuf_stride;
   int32_t kbuf_ctas;
   int32_t kbuf_cap;        // largest k the global tier holds
-  int32_t* hitbuf;         // passes T/K: per-CTA lists of the edges of H_a (hitbuf_ctas x hitcap x 2 ints)
-  int32_t hitcap;
-  int32_t hitbuf_ctas;
+  int2* hitbuf;            // passes T/K: per-CTA lists of the edges of H_a; tier t (tiers run side by side) has
+                           // hit_ctas[t] lists of hit_cap[t] entries from hit_off[t]
+  int64_t hit_off[kNumTiers];
+  int32_t hit_cap[kNumTiers];
+  int32_t hit_ctas[kNumTiers];
   // Edges of every H_a, recorded by pass T for pass K (nullptr: not kept):
   // entry = ((i << 16) | j, out-slot of (b_i, b_j)); unit ui (index into
   // kunits) has tl_cnt[ui] entries from tl_off[ui], or tl_cnt[ui] = -1.
@@ -157,44 +159,103 @@ constexpr int kSmemTableMax = 4096;    // Psi tables up to this many vertices li
 enum Phase { kPhasePassT = 0, kPhasePassC, kPhasePassK, kPhaseFinish, kPhaseInduced, kPhaseDerive, kPhaseCopy,
              kNumPhases };
 
+// Streams and events of one count, kept by the library and lent to one graph
+// handle (or one stream slot of a batch) at a time: kernels of a phase that do
+// not depend on each other run side by side on `stream`, forked from the count's
+// own stream by `start` and joined by `done`; begin/end time the phases;
+// `pinned` receives the results (kPinnedBytes).
+constexpr int kForkStreams = 10;
+constexpr size_t kPinnedBytes = 1024;
+struct ForkSet {
+  cudaStream_t stream[kForkStreams] = {};
+  cudaEvent_t start = nullptr, done[kForkStreams] = {};
+  cudaEvent_t begin[kNumPhases] = {}, end[kNumPhases] = {};
+  unsigned char* pinned = nullptr;
+  int device = 0;
+};
+ForkSet* fork_acquire();         // of the current device; nullptr on failure (message set)
+void fork_release(ForkSet* f);   // its streams must be idle; nullptr is accepted
+void fork_drain(ForkSet* f);     // waits for its streams (after a failed count, whose forks were not joined)
+
+// Side streams of one fork: next() is a stream that starts where the main
+// stream stood at the constructor, join() makes the main stream wait for all
+// of them. Without a set everything stays on the main stream.
+class Fork {
+ public:
+  Fork(cudaStream_t s, ForkSet* f, int first, int count) : s_(s), f_(f), first_(first), count_(count) {
+    if (f_) e_ = cudaEventRecord(f_->start, s_);
+  }
+  cudaStream_t next() {
+    if (!f_ || used_ >= count_ || e_ != cudaSuccess) return s_;
+    cudaStream_t t = f_->stream[first_ + used_++];
+    e_ = cudaStreamWaitEvent(t, f_->start, 0);
+    return t;
+  }
+  cudaError_t join() {
+    for (int k = 0; k < used_ && e_ == cudaSuccess; ++k) {
+      e_ = cudaEventRecord(f_->done[first_ + k], f_->stream[first_ + k]);
+      if (e_ == cudaSuccess) e_ = cudaStreamWaitEvent(s_, f_->done[first_ + k], 0);
+    }
+    used_ = 0;
+    return e_;
+  }
+
+ private:
+  cudaStream_t s_;
+  ForkSet* f_;
+  int first_, count_, used_ = 0;
+  cudaError_t e_ = cudaSuccess;
+};
+
 // Device scratch of one count (lazily grown; owned by a graph handle or by
 // one batch launch).
 struct Scratch {
+  // one block, zeroed before every count: the results' head (misc: cursors and
+  // status, work, fill, csum [G][13][2], x [G][17][2]), then trio, xc and P
+  unsigned char* zero = nullptr;
+  size_t zero_bytes = 0, head_bytes = 0;
+  int32_t* misc = nullptr;             // [32]
+  unsigned long long* work = nullptr;  // [kNumWork]
+  unsigned long long* tl_fill = nullptr;
+  unsigned long long* csum = nullptr;
+  unsigned long long* x = nullptr;
   int32_t* trio = nullptr;           // [m]
-  unsigned long long* P = nullptr;   // [2m]
   unsigned long long* xc = nullptr;  // [m][2]
-  int32_t* misc = nullptr;           // [32] cursors, status
+  unsigned long long* P = nullptr;   // [2m]
   uint32_t* tables = nullptr;        // count_grid_size() x table_n
   size_t tables_n = 0;
   unsigned char* kbuf = nullptr;     // pass K global tier
   size_t kbuf_stride = 0;
   int32_t kbuf_ctas = 0;
   int32_t kbuf_cap = 0;
-  int32_t* hitbuf = nullptr;         // per-CTA H_a edge lists
-  int32_t hitcap = 0;
-  int32_t hitbuf_ctas = 0;
+  int2* hitbuf = nullptr;            // per-CTA H_a edge lists (see CountArgs)
+  int64_t hit_off[kNumTiers] = {};
+  int32_t hit_cap[kNumTiers] = {};
+  int32_t hit_ctas[kNumTiers] = {};
   int2* tlist = nullptr;             // edges of all H_a, from pass T to pass K
   long long tlist_cap = 0;           // entries
   long long tlist_want = 0;          // triangles of the last count (or a first guess): the size to keep
   long long* tl_off = nullptr;       // [units of pass K]
   int32_t* tl_cnt = nullptr;
   int32_t tl_units = 0;
-  unsigned long long* tl_fill = nullptr;
-  unsigned long long* work = nullptr;  // [kNumWork]
   int32_t launches = 0;              // kernels launched by the last run_count
   unsigned long long* dsum = nullptr;  // [m] per-edge induced counts: sum over T of d_w
   unsigned long long* vsum = nullptr;  // [n][2] per-edge induced counts: 2 x triangles, neighbour degrees
 };
-// Allocates the scratch of a graph with m edges, Psi tables of table_n
-// vertices and largest out-degree kmax (stream-ordered).
-gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, cudaStream_t s);
+// Allocates the scratch of a union of G graphs with m edges, Psi tables of
+// table_n vertices, largest out-degree kmax and pass-K tiers tier_off
+// (stream-ordered).
+gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, const int32_t* tier_off, int32_t G,
+                       cudaStream_t s);
 void scratch_free(Scratch* sc, cudaStream_t s);
 // Size of pass T's edge lists for the first count of a whole graph with m
 // edges: 32 m entries within the list budget (units past it scan again).
 void scratch_guess_tlist(Scratch* sc, int64_t m);
-// The whole count: passes T, C, K, finish, derive. csum [G][13][2] and
-// x [G][17][2] are device arrays; ev (optional) receives kNumPhases + 1
-// events. Returns after the derive is queued (no host synchronisation).
+// The whole count: passes T, C, K, finish, derive; the sums and X land in
+// sc->csum and sc->x. Kernels that do not depend on each other run side by
+// side on the set's streams, pass C beside passes T and K in graphs of fewer
+// than kOverlapEdges edges (see run_count). Returns after the derive is queued
+// (no host synchronisation).
 struct KUnits {
   const int32_t* units;
   int32_t tier_off[kNumTiers + 1];
@@ -214,9 +275,8 @@ struct KUnits {
 // (device pointer, or the device view of pinned host memory when
 // induced_host), written after the finish.
 gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, const KUnits& ku,
-                    uint64_t* per_edge, unsigned long long* csum, unsigned long long* x, Scratch* sc,
-                    cudaStream_t s, cudaEvent_t* ev, bool per_edge_host = false, uint64_t* induced = nullptr,
-                    bool induced_host = false);
+                    uint64_t* per_edge, Scratch* sc, cudaStream_t s, ForkSet* fs, bool per_edge_host = false,
+                    uint64_t* induced = nullptr, bool induced_host = false);
 
 // ---- host helpers (gc_api.cu) ----
 void set_error(const std::string& msg);
@@ -384,7 +444,7 @@ inline int hub_cpw(int64_t nx) { return nx < 1023 ? 3 : nx < 65536 ? 2 : 1; }
 constexpr int kHashMaxW = 8192;
 constexpr int kHashSmallW = 512;  // hashed units up to this many wedges run in small CTAs
 constexpr int kHashMidW = 2048;   // and up to this many in middle-sized CTAs
-gc_status run_pass_c_hash(const DevGraph& g, const CountArgs& a, cudaStream_t s);
+gc_status run_pass_c_hash(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches);
 // Units of more than kHashMaxW and at most kHash2MaxW wedges, with fewer than
 // kHash2MaxNx lower neighbours, in graphs of at most 2^22 vertices: a
 // shared-memory hash of kHash2Slots words, each a packed (22-bit vertex,
@@ -397,11 +457,12 @@ constexpr int kHash2MaxNx = 1023;
 constexpr int kHash2HalfSlots = 28672;
 constexpr int kHash2HalfMaxW = 20620;  // (kHash2HalfSlots - 32) * 18 / 25
 constexpr int32_t kHash2MaxN = 1 << 22;
-gc_status run_pass_c_hash2(const DevGraph& g, const CountArgs& a, cudaStream_t s);
+gc_status run_pass_c_hash2(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches);
 gc_status run_derive(const DevGraph& g, const unsigned long long* csum, unsigned long long* x,
                      int32_t* status, cudaStream_t s);
-gc_status run_pass_t(const DevGraph& g, const CountArgs& a, cudaStream_t s, int* launches);
-gc_status run_pass_k(const DevGraph& g, const CountArgs& a, cudaStream_t s, int* launches);
+// The tiers of passes T and K: side by side on the fork's streams.
+gc_status run_pass_t(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches);
+gc_status run_pass_k(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches);
 gc_status run_finish(const DevGraph& g, const CountArgs& a, cudaStream_t s);
 // Per-edge induced counts of H_7..H_16 (needs a.dsum from pass T, and the
 // results of passes C and K); vsum: [n][2] scratch.

@@ -7,10 +7,12 @@
 //   finish  x10, per-edge columns, unrestricted sums             (Sec. 4.5)
 //   derive  X_1..X_17                                            (Sec. 4.6)
 //
-// Everything is queued on one stream with no host synchronisation: the unit
-// lists and their tier boundaries are fixed when the graph is prepared.
+// Everything is queued on the graph's stream, and on side streams forked from
+// it and joined again, with no host synchronisation: the unit lists and their
+// tier boundaries are fixed when the graph is prepared.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdlib>
 
 #include "gc_internal.h"
@@ -20,6 +22,8 @@ namespace gc {
 namespace {
 // Total bytes the pass-K global tier may hold at once.
 constexpr size_t kKbufBudget = size_t(2) << 30;
+// Graphs of fewer edges run pass C beside passes T and K.
+constexpr int32_t kOverlapEdges = 1 << 22;
 // Largest list of the edges of all H_a that pass T keeps for pass K.
 constexpr long long kTListBudget = 24LL << 30;
 // Largest per-CTA list of H_a edges in pass K (units with more edges rescan
@@ -47,15 +51,14 @@ long long t_list_cap_knob() {
 }  // namespace
 
 void scratch_free(Scratch* sc, cudaStream_t s) {
-  for (void* p : {(void*)sc->trio, (void*)sc->P, (void*)sc->xc, (void*)sc->misc,
-                  (void*)sc->tables, (void*)sc->kbuf, (void*)sc->hitbuf, (void*)sc->work,
-                  (void*)sc->tlist, (void*)sc->tl_off, (void*)sc->tl_cnt, (void*)sc->tl_fill, (void*)sc->dsum,
-                  (void*)sc->vsum})
+  for (void* p : {(void*)sc->zero, (void*)sc->tables, (void*)sc->kbuf, (void*)sc->hitbuf, (void*)sc->tlist,
+                  (void*)sc->tl_off, (void*)sc->tl_cnt, (void*)sc->dsum, (void*)sc->vsum})
     if (p) cudaFreeAsync(p, s);
   *sc = Scratch();
 }
 
-gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, cudaStream_t s) {
+gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, const int32_t* tier_off, int32_t G,
+                       cudaStream_t s) {
   cudaError_t e = cudaSuccess;
 #define GS_TRY(call)                                \
   do {                                              \
@@ -63,22 +66,50 @@ gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, cu
     if (e != cudaSuccess) return cuda_fail(e, "scratch alloc"); \
   } while (0)
   const size_t m1 = (size_t)(m > 0 ? m : 1);
-  GS_TRY(pool_alloc(&sc->trio, sizeof(int32_t) * m1, s));
-  GS_TRY(pool_alloc(&sc->P, sizeof(unsigned long long) * 2 * m1, s));
-  GS_TRY(pool_alloc(&sc->xc, sizeof(unsigned long long) * 2 * m1, s));
-  GS_TRY(pool_alloc(&sc->misc, sizeof(int32_t) * 32, s));
-  GS_TRY(pool_alloc(&sc->work, sizeof(unsigned long long) * kNumWork, s));
+  {
+    size_t at = 0;
+    auto take = [&](size_t bytes, size_t align = 16) {
+      at = (at + align - 1) / align * align;
+      const size_t o = at;
+      at += bytes;
+      return o;
+    };
+    const size_t misc = take(sizeof(int32_t) * 32), work = take(sizeof(unsigned long long) * kNumWork),
+                 fill = take(sizeof(unsigned long long)),
+                 csum = take(sizeof(unsigned long long) * 26 * (size_t)G),
+                 x = take(sizeof(unsigned long long) * 34 * (size_t)G);
+    sc->head_bytes = at;
+    const size_t trio = take(sizeof(int32_t) * m1, 256), xc = take(sizeof(unsigned long long) * 2 * m1, 256),
+                 P = take(sizeof(unsigned long long) * 2 * m1, 256);
+    sc->zero_bytes = at;
+    GS_TRY(pool_alloc(&sc->zero, at, s));
+    sc->misc = reinterpret_cast<int32_t*>(sc->zero + misc);
+    sc->work = reinterpret_cast<unsigned long long*>(sc->zero + work);
+    sc->tl_fill = reinterpret_cast<unsigned long long*>(sc->zero + fill);
+    sc->csum = reinterpret_cast<unsigned long long*>(sc->zero + csum);
+    sc->x = reinterpret_cast<unsigned long long*>(sc->zero + x);
+    sc->trio = reinterpret_cast<int32_t*>(sc->zero + trio);
+    sc->xc = reinterpret_cast<unsigned long long*>(sc->zero + xc);
+    sc->P = reinterpret_cast<unsigned long long*>(sc->zero + P);
+  }
   if (table_n > kSmemTableMax) {
     sc->tables_n = (size_t)count_grid_size() * (size_t)table_n;
     GS_TRY(pool_alloc(&sc->tables, sizeof(uint32_t) * sc->tables_n, s));
     GS_TRY(cudaMemsetAsync(sc->tables, 0, sizeof(uint32_t) * sc->tables_n, s));
   }
-  {  // pass K: each CTA records the edges of its current H_a (at most C(kmax, 2))
-    const long long full = (long long)kmax * (kmax - 1) / 2;
-    const long long cap = k_list_cap();
-    sc->hitcap = (int32_t)(full < cap ? (full > 0 ? full : 1) : cap);
-    sc->hitbuf_ctas = 4 * (count_grid_size() / kCtasPerSm);  // up to four CTAs per SM in any tier
-    GS_TRY(pool_alloc(&sc->hitbuf, sizeof(int32_t) * 2 * (size_t)sc->hitcap * (size_t)sc->hitbuf_ctas, s));
+  {  // passes T and K: each CTA records the edges of its current H_a (at most C(k, 2)); up to four CTAs per SM
+    const int32_t ctas = 4 * (count_grid_size() / kCtasPerSm);
+    int64_t at = 0;
+    for (int t = 0; t < kTier32; ++t) {  // the warp tier keeps none
+      const int32_t units = tier_off[t + 1] - tier_off[t];
+      const int64_t k = t == kTierGlobal || kmax < kTierCap[t] ? kmax : kTierCap[t];
+      const int64_t full = k * (k - 1) / 2;
+      sc->hit_cap[t] = (int32_t)std::max<int64_t>(1, std::min<int64_t>(full, k_list_cap()));
+      sc->hit_ctas[t] = std::min(units, ctas);
+      sc->hit_off[t] = at;
+      at += (int64_t)sc->hit_cap[t] * sc->hit_ctas[t];
+    }
+    GS_TRY(pool_alloc(&sc->hitbuf, sizeof(int2) * (size_t)std::max<int64_t>(1, at), s));
   }
   if (kmax > kTierCap[kTier1024]) {
     sc->kbuf_cap = kmax;
@@ -102,8 +133,8 @@ void scratch_guess_tlist(Scratch* sc, int64_t m) {
 static int32_t ku_total(const KUnits& ku) { return ku.tier_off[kNumTiers]; }
 
 gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, const KUnits& ku,
-                    uint64_t* per_edge, unsigned long long* csum, unsigned long long* x, Scratch* sc,
-                    cudaStream_t s, cudaEvent_t* ev, bool per_edge_host, uint64_t* induced, bool induced_host) {
+                    uint64_t* per_edge, Scratch* sc, cudaStream_t s, ForkSet* fs, bool per_edge_host, uint64_t* induced,
+                    bool induced_host) {
   cudaError_t e = cudaSuccess;
   gc_status st = GC_OK;
 #define GR_TRY(call, what)                  \
@@ -111,8 +142,10 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
     e = (call);                             \
     if (e != cudaSuccess) return cuda_fail(e, what); \
   } while (0)
-#define GR_EVENT(i) \
-  if (ev) GR_TRY(cudaEventRecord(ev[i], s), "event")
+#define GR_BEGIN(i, t) \
+  if (fs) GR_TRY(cudaEventRecord(fs->begin[i], t), "event")
+#define GR_END(i, t) \
+  if (fs) GR_TRY(cudaEventRecord(fs->end[i], t), "event")
   CountArgs a;
   a.units = units;
   a.n_units = n_units;
@@ -142,8 +175,11 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
   a.kbuf_ctas = sc->kbuf_ctas;
   a.kbuf_cap = sc->kbuf_cap;
   a.hitbuf = sc->hitbuf;
-  a.hitcap = sc->hitcap;
-  a.hitbuf_ctas = sc->hitbuf_ctas;
+  for (int t = 0; t < kNumTiers; ++t) {
+    a.hit_off[t] = sc->hit_off[t];
+    a.hit_cap[t] = sc->hit_cap[t];
+    a.hit_ctas[t] = sc->hit_ctas[t];
+  }
   // Pass T keeps the edges of the H_a for pass K, in a list sized by the
   // triangles of the previous count of this scratch (or by a first guess);
   // units that do not fit scan their out-lists again in pass K.
@@ -168,7 +204,6 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
         GR_TRY(pool_alloc(&sc->tl_cnt, sizeof(int32_t) * (size_t)nku, s), "alloc list index");
         sc->tl_units = nku;
       }
-      if (!sc->tl_fill) GR_TRY(pool_alloc(&sc->tl_fill, sizeof(unsigned long long), s), "alloc list fill");
     }
   }
   a.tlist = sc->tlist_cap > 0 ? sc->tlist : nullptr;
@@ -176,7 +211,6 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
   a.tlist_fill = sc->tl_fill;
   a.tl_off = sc->tl_off;
   a.tl_cnt = sc->tl_cnt;
-  if (a.tlist) GR_TRY(cudaMemsetAsync(sc->tl_fill, 0, sizeof(unsigned long long), s), "zero list fill");
   a.per_edge = per_edge;
   a.per_edge_host = per_edge != nullptr && per_edge_host;
   a.dsum = nullptr;
@@ -189,62 +223,89 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
     GR_TRY(cudaMemsetAsync(sc->dsum, 0, sizeof(unsigned long long) * (size_t)g.m, s), "zero dsum");
     a.dsum = sc->dsum;
   }
-  a.csum = csum;
+  a.csum = sc->csum;
   a.work = sc->work;
-  const size_t m1 = (size_t)(g.m > 0 ? g.m : 1);
-  GR_TRY(cudaMemsetAsync(sc->misc, 0, sizeof(int32_t) * 32, s), "memset misc");
-  GR_TRY(cudaMemsetAsync(sc->work, 0, sizeof(unsigned long long) * kNumWork, s), "memset work");
-  GR_TRY(cudaMemsetAsync(csum, 0, sizeof(unsigned long long) * 26 * (size_t)g.G, s), "memset sums");
-  GR_TRY(cudaMemsetAsync(sc->P, 0, sizeof(unsigned long long) * 2 * m1, s), "zero P");
-  GR_TRY(cudaMemsetAsync(sc->xc, 0, sizeof(unsigned long long) * 2 * m1, s), "zero x7 and cross");
-  GR_TRY(cudaMemsetAsync(sc->trio, 0, sizeof(int32_t) * m1, s), "zero T");
+  GR_TRY(cudaMemsetAsync(sc->zero, 0, sc->zero_bytes, s), "zero scratch");
   int launches = 0;
-  GR_EVENT(kPhasePassT);
-  int t_launches = 0;
-  if ((st = run_pass_t(g, a, s, &t_launches)) != GC_OK) return st;
-  launches += t_launches;
-  GR_EVENT(kPhasePassC);
-  const int32_t n_cunits = ku.n_cunits;  // pass C units: hubs, hashed units, the others
-  if (n_cunits > 0) {
+  // Pass C needs nothing of passes T and K. In graphs of fewer than
+  // kOverlapEdges edges no pass fills the GPU for long (their kernels end in
+  // tails of single units), so C runs beside T and K; above, the passes follow
+  // each other, so that a pass's time says what it costs, with only the hub and
+  // hash kernels of C side by side (16.8 -> 16.4 ms on Chung-Lu 10M edges; the
+  // tiers of T and K gain nothing there). Chung-Lu, 500 009 edges: 1.06 -> 0.69
+  // ms per count.
+  const bool overlap = fs && g.m < kOverlapEdges;
+  auto pass_c = [&](cudaStream_t t, Fork* fork) -> gc_status {
+    const int32_t n_cunits = ku.n_cunits;  // pass C units: hubs, hashed units, the others
+    if (n_cunits <= 0) return GC_OK;
     if (a.n_cheavy > 0) {
-      if ((st = run_pass_c_heavy(g, a, s)) != GC_OK) return st;
+      if ((st = run_pass_c_heavy(g, a, t)) != GC_OK) return st;
       launches += 1;
     }
-    if (a.n_chash > 0) {
-      if ((st = run_pass_c_hash(g, a, s)) != GC_OK) return st;
-      launches += 1;
-    }
-    if (a.n_chash2 > 0) {
-      if ((st = run_pass_c_hash2(g, a, s)) != GC_OK) return st;
-      launches += 1;
-    }
+    if ((st = run_pass_c_hash2(g, a, fork, &launches)) != GC_OK) return st;
+    if ((st = run_pass_c_hash(g, a, fork, &launches)) != GC_OK) return st;
     const int32_t n_hashed = a.n_cheavy + a.n_chash + a.n_chash2;
     if (n_cunits > n_hashed) {
       CountArgs al = a;  // the remaining units on the vertex-indexed tables
       al.units = a.cunits + n_hashed;
       al.n_units = n_cunits - n_hashed;
-      GR_TRY(cudaMemsetAsync(a.cursor, 0, sizeof(int32_t), s), "reset cursor");
-      if ((st = run_pass_c(g, al, s)) != GC_OK) return st;
+      if ((st = run_pass_c(g, al, t)) != GC_OK) return st;
       launches += 1;
     }
+    return GC_OK;
+  };
+  auto pass_tk = [&](bool tri) -> gc_status {
+    const Phase ph = tri ? kPhasePassT : kPhasePassK;
+    GR_BEGIN(ph, s);
+    Fork tiers(s, overlap ? fs : nullptr, 6, kForkStreams - 6);
+    st = tri ? run_pass_t(g, a, &tiers, &launches) : run_pass_k(g, a, &tiers, &launches);
+    if (st != GC_OK) return st;
+    GR_TRY(tiers.join(), "join");
+    GR_END(ph, s);
+    return GC_OK;
+  };
+  if (overlap) {
+    // pass C on the set's first stream, its kernels forked from there
+    Fork side(s, fs, 0, 1);
+    const cudaStream_t t = side.next();
+    GR_BEGIN(kPhasePassC, t);
+    {
+      Fork units(t, fs, 1, 5);
+      if ((st = pass_c(t, &units)) != GC_OK) return st;
+      GR_TRY(units.join(), "join");
+    }
+    GR_END(kPhasePassC, t);
+    if ((st = pass_tk(true)) != GC_OK) return st;
+    if ((st = pass_tk(false)) != GC_OK) return st;
+    GR_TRY(side.join(), "join");
+  } else {
+    if ((st = pass_tk(true)) != GC_OK) return st;
+    GR_BEGIN(kPhasePassC, s);
+    {
+      Fork units(s, fs, 1, 5);
+      if ((st = pass_c(s, &units)) != GC_OK) return st;
+      GR_TRY(units.join(), "join");
+    }
+    GR_END(kPhasePassC, s);
+    if ((st = pass_tk(false)) != GC_OK) return st;
   }
-  GR_EVENT(kPhasePassK);
-  int k_launches = 0;
-  if ((st = run_pass_k(g, a, s, &k_launches)) != GC_OK) return st;
-  launches += k_launches;
-  GR_EVENT(kPhaseFinish);
+  GR_BEGIN(kPhaseFinish, s);
   if ((st = run_finish(g, a, s)) != GC_OK) return st;
   launches += g.m > 0 ? 1 : 0;
-  GR_EVENT(kPhaseInduced);
+  GR_END(kPhaseFinish, s);
+  GR_BEGIN(kPhaseInduced, s);
   if (want_induced) {
     if ((st = run_induced(g, a, sc->vsum, induced, induced_host, s)) != GC_OK) return st;
     launches += 2;
   }
-  GR_EVENT(kPhaseDerive);
-  if ((st = run_derive(g, csum, x, a.status, s)) != GC_OK) return st;
+  GR_END(kPhaseInduced, s);
+  GR_BEGIN(kPhaseDerive, s);
+  if ((st = run_derive(g, sc->csum, sc->x, a.status, s)) != GC_OK) return st;
   sc->launches = launches + 1;
-  GR_EVENT(kPhaseCopy);
-#undef GR_EVENT
+  GR_END(kPhaseDerive, s);
+  GR_BEGIN(kPhaseCopy, s);
+#undef GR_BEGIN
+#undef GR_END
 #undef GR_TRY
   return GC_OK;
 }

@@ -376,29 +376,7 @@ gc_status validate_csr(int32_t n, const int32_t* rp, const int32_t* ci) {
   return st;
 }
 
-// Host arrays left uninitialised on allocation (every element is written
-// before use).
-template <class T>
-struct HostBuf {
-  std::unique_ptr<T[]> p;
-  T* data() { return p.get(); }
-  T& operator[](size_t i) { return p[i]; }
-  void resize(size_t n) { p.reset(new T[n > 0 ? n : 1]); }
-};
-
-// The host half of preprocessing P1 (Sec. 4.3): vertices ranked by ascending
-// (degree, id) -- a stable counting sort of the degrees -- and what the
-// device relabel needs: internal row pointers, and the internal rows of more
-// than 32 entries listed by the sort that takes them.
-struct RelabelPlan {
-  HostBuf<int32_t> perm, newid, rp;
-  std::vector<int32_t> mid, longr;  // rows of 33..4096 entries, and longer ones
-  std::vector<int64_t> long_off;    // offset of each long row's padded copy
-  int64_t tmp_len = 0;
-  int32_t obound[kOBounds] = {};    // first rank of degree >= kOBoundDeg[k]
-};
-
-RelabelPlan plan_relabel(int32_t n, const int32_t* rp) {
+RelabelPlan plan_relabel(int32_t n, const int32_t* rp, int max_threads) {
   RelabelPlan R;
   R.perm.resize((size_t)n);
   R.newid.resize((size_t)n);
@@ -407,7 +385,7 @@ RelabelPlan plan_relabel(int32_t n, const int32_t* rp) {
   if (n == 0) return R;
   // vertex chunks, one per thread (fewer threads when the per-thread degree
   // histograms would pass 2^24 counters)
-  int nt = n >= (1 << 16) ? host_threads() : 1;
+  int nt = n >= (1 << 16) ? std::min(host_threads(), max_threads) : 1;
   std::vector<int32_t> dmx((size_t)nt, 0);
   auto chunk = [&](int t, int T) { return (int32_t)((int64_t)n * t / T); };
   run_threads(nt, [&](int t) {
@@ -605,7 +583,7 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
     if (e != cudaSuccess) return fail(cuda_fail(e, what)); \
   } while (0)
   try {
-    R = plan_relabel(n, row_ptr);
+    R = plan_relabel(n, row_ptr, host_threads());
   } catch (...) {
     set_error("host allocation failed");
     return fail(GC_ERR_NOMEM);
@@ -643,13 +621,13 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
     GC_CHECK(cudaMemcpyAsync(d_loff, R.long_off.data(), sizeof(int64_t) * R.long_off.size(), cudaMemcpyHostToDevice, s),
              "copy row lists");
   }
-  st = relabel_on_device(n, g->m, d_rp0, d_ci0, d_perm, d_newid, g->d_rp, g->d_ci, d_eid, d_lists,
+  st = relabel_on_device(n, g->m, d_rp0, d_ci0, d_perm, d_newid, g->d_rp, g->d_ci, d_eid, nullptr, nullptr, d_lists,
                          (int32_t)R.mid.size(), d_lists + R.mid.size(), d_loff, (int32_t)R.longr.size(), d_tmp, s);
   drop_temps();
   if (st != GC_OK) return fail(st);
   const int32_t zero = 0;
   const RankInfo rank = {R.rp.data(), 1, &zero, &n, R.obound};
-  st = prepare_graph(n, g->m, g->d_rp, g->d_ci, nullptr, d_eid, d_perm, &rank, &g->prep, s);
+  st = prepare_graph(n, g->m, g->d_rp, g->d_ci, d_eid, d_perm, rank, &g->prep, s);
   d_eid = nullptr;  // owned by the preparation buffers from here on
   if (st != GC_OK) return fail(st);
   cudaFreeAsync(d_perm, s);
@@ -679,7 +657,7 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
     g->d_gm = reinterpret_cast<int64_t*>(reinterpret_cast<char*>(g->d_gbase) + 16);
   }
   {
-    gc_status st2 = scratch_init(&g->sc, g->m, n, g->prep.kmax, g->prep.ktier_off, 1, s);
+    gc_status st2 = scratch_init(&g->sc, g->m, needs_tables(g->prep) ? n : 0, g->prep.kmax, g->prep.ktier_off, 1, s);
     if (st2 != GC_OK) return fail(st2);
     scratch_guess_tlist(&g->sc, g->m);
   }
@@ -778,7 +756,6 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
   dg.gn = g->d_gn;
   dg.gm = g->d_gm;
   dg.table_n = g->n;
-  dg.ranked = true;
   dg.hgeom = g->prep.hgeom;
   dg.hseg = g->prep.hseg;
   dg.hpos = g->prep.hpos;

@@ -17,10 +17,12 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <exception>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -37,16 +39,6 @@ gc_status validate_csr(int32_t n, const int32_t* rp, const int32_t* ci);
 gc_status validate_csr_small(int32_t n, const int32_t* rp, const int32_t* ci, std::vector<int32_t>* fill);
 
 namespace {
-
-__global__ void k_globalize(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ vgid,
-                            const int32_t* __restrict__ gbase, int32_t* __restrict__ ci) {
-  const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int32_t x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += warps) {
-    const int32_t base = gbase[vgid[x]];
-    for (int32_t p = rp[x] + lane; p < rp[x + 1]; p += 32) ci[p] += base;
-  }
-}
 
 // Host buffers for the library's copies of bulk submissions, kept for reuse:
 // a submission takes the smallest kept buffer that holds it, whose pages are
@@ -213,6 +205,30 @@ struct gc_batch_s {
 
 namespace {
 
+// f(0) .. f(count - 1) on the host's cores, at most one thread per call. The
+// first exception is thrown again on the calling thread.
+template <class F>
+void host_parallel(int count, F f) {
+  const unsigned hw = std::thread::hardware_concurrency();
+  const int nt = std::min<int>(count, (int)std::min<unsigned>(hw ? hw : 1, 32));
+  std::atomic<int> next(0);
+  std::exception_ptr err;
+  std::mutex mu;
+  auto work = [&] {
+    try {
+      for (int i; (i = next.fetch_add(1)) < count;) f(i);
+    } catch (...) {
+      std::lock_guard<std::mutex> lk(mu);
+      if (!err) err = std::current_exception();
+    }
+  };
+  std::vector<std::thread> th;
+  for (int t = 1; t < nt; ++t) th.emplace_back(work);
+  work();
+  for (auto& x : th) x.join();
+  if (err) std::rethrow_exception(err);
+}
+
 // Counts `graphs` as one launch on `s`. Fills L (results land in L->h_x when
 // L->done completes). Runs in the dispatcher thread (or the flushing thread
 // in manual mode) without holding the batch lock.
@@ -231,28 +247,62 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
   }
   const int32_t n = (int32_t)n_total;
   const int32_t m = (int32_t)(nnz_total / 2);
-  std::vector<int32_t> h_rp((size_t)n + 1), h_ci((size_t)(nnz_total > 0 ? nnz_total : 1)), h_vgid((size_t)(n > 0 ? n : 1));
-  std::vector<int32_t> h_desc((size_t)2 * G);  // gbase | gn
-  std::vector<int64_t> h_gm((size_t)G);
-  {
-    int64_t vo = 0, eo = 0;
-    for (int32_t gi = 0; gi < G; ++gi) {
-      PendingGraph& pg = *graphs[gi];
-      for (int32_t i = 0; i < pg.n; ++i) {
-        h_rp[vo + i] = (int32_t)(eo + pg.rp[i]);
-        h_vgid[vo + i] = gi;
-      }
-      if (pg.m > 0) std::memcpy(h_ci.data() + eo, pg.ci, sizeof(int32_t) * 2 * pg.m);
-      h_desc[gi] = (int32_t)vo;
-      h_desc[G + gi] = pg.n;
-      h_gm[gi] = pg.m;
-      vo += pg.n;
-      eo += 2 * pg.m;
-    }
-    h_rp[n] = (int32_t)eo;
+  // The union is ranked like a single graph (P1), graph by graph: the ids of
+  // graph g are gbase[g] + the (degree, id) rank in g, so that the hub and hash
+  // kernels of pass C serve it too. (Unranked, with pass C on vertex-indexed
+  // tables in DRAM, 40 Chung-Lu graphs of 1 000 to 2M edges took 29 ms in pass C
+  // alone.) Host arrays, one block: gbase | gn | obound, then per vertex.
+  std::vector<int32_t> gbase((size_t)G + 1), gn((size_t)G), obound((size_t)G * kOBounds);
+  std::vector<int64_t> gm((size_t)G), ebase((size_t)G + 1);
+  gbase[0] = 0;
+  ebase[0] = 0;
+  for (int32_t gi = 0; gi < G; ++gi) {
+    gn[(size_t)gi] = graphs[(size_t)gi]->n;
+    gm[(size_t)gi] = graphs[(size_t)gi]->m;
+    gbase[(size_t)gi + 1] = gbase[(size_t)gi] + graphs[(size_t)gi]->n;
+    ebase[(size_t)gi + 1] = ebase[(size_t)gi] + 2 * graphs[(size_t)gi]->m;
   }
-  int32_t *d_rp = nullptr, *d_ci = nullptr, *d_vgid = nullptr, *d_desc = nullptr;
-  int64_t* d_gm = nullptr;
+  HostBuf<int32_t> h_rp, h_rp0, h_perm, h_newid, h_vgid;
+  std::vector<int32_t> mid, longr;
+  std::vector<int64_t> long_off;
+  int64_t tmp_len = 0;
+  try {
+    for (auto* b : {&h_rp, &h_rp0, &h_perm, &h_newid, &h_vgid}) b->resize((size_t)n + 1);
+    std::vector<RelabelPlan> plans((size_t)G);
+    host_parallel(G, [&](int gi) {
+      const PendingGraph& pg = *graphs[(size_t)gi];
+      RelabelPlan& R = plans[(size_t)gi];
+      R = plan_relabel(pg.n, pg.rp, 1);
+      const int32_t vb = gbase[(size_t)gi], eb = (int32_t)ebase[(size_t)gi];
+      for (int32_t i = 0; i < pg.n; ++i) {
+        h_rp[(size_t)(vb + i)] = eb + R.rp[(size_t)i];
+        h_rp0[(size_t)(vb + i)] = eb + pg.rp[i];
+        h_perm[(size_t)(vb + i)] = vb + R.perm[(size_t)i];
+        h_newid[(size_t)(vb + i)] = vb + R.newid[(size_t)i];
+        h_vgid[(size_t)(vb + i)] = gi;
+      }
+      for (int k = 0; k < kOBounds; ++k) obound[(size_t)gi * kOBounds + (size_t)k] = vb + R.obound[k];
+    });
+    h_rp[(size_t)n] = h_rp0[(size_t)n] = (int32_t)nnz_total;
+    for (int32_t gi = 0; gi < G; ++gi) {
+      const RelabelPlan& R = plans[(size_t)gi];
+      for (int32_t x : R.mid) mid.push_back(gbase[(size_t)gi] + x);
+      for (int32_t x : R.longr) longr.push_back(gbase[(size_t)gi] + x);
+      for (int64_t o : R.long_off) long_off.push_back(tmp_len + o);
+      tmp_len += R.tmp_len;
+    }
+  } catch (...) {
+    set_error("host allocation failed");
+    L->error = gc_last_error();
+    return GC_ERR_NOMEM;
+  }
+  const RankInfo rank = {h_rp.data(), G, gbase.data(), gn.data(), obound.data()};
+  const size_t n1 = (size_t)n + 1, nnz1 = (size_t)(nnz_total > 0 ? nnz_total : 1);
+  const size_t n_lists = mid.size() + longr.size();
+  int32_t *d_rp = nullptr, *d_ci = nullptr, *d_vgid = nullptr, *d_desc = nullptr, *d_rp0 = nullptr, *d_ci0 = nullptr;
+  int32_t *d_perm = nullptr, *d_newid = nullptr, *d_lists = nullptr;
+  int64_t *d_gm = nullptr, *d_loff = nullptr;
+  long long* d_tmp = nullptr;
   PrepBuffers prep;
   Scratch sc;
   cudaError_t e = cudaSuccess;
@@ -260,6 +310,9 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
   auto fail = [&](cudaError_t err, const char* what) {
     st = cuda_fail(err, what);
     L->error = gc_last_error();
+  };
+  auto up = [&](auto* d, const auto* h, size_t count) {
+    return count ? cudaMemcpyAsync(d, h, sizeof(*h) * count, cudaMemcpyHostToDevice, s) : cudaSuccess;
   };
 #define GB_TRY(call, what)  \
   do {                      \
@@ -269,26 +322,48 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
       goto out;             \
     }                       \
   } while (0)
-  GB_TRY(pool_alloc(&d_rp, sizeof(int32_t) * ((size_t)n + 1), s), "batch alloc");
-  GB_TRY(pool_alloc(&d_ci, sizeof(int32_t) * h_ci.size(), s), "batch alloc");
-  GB_TRY(pool_alloc(&d_vgid, sizeof(int32_t) * h_vgid.size(), s), "batch alloc");
-  GB_TRY(pool_alloc(&d_desc, sizeof(int32_t) * h_desc.size(), s), "batch alloc");
-  GB_TRY(pool_alloc(&d_gm, sizeof(int64_t) * G, s), "batch alloc");
-  GB_TRY(cudaMemcpyAsync(d_rp, h_rp.data(), sizeof(int32_t) * h_rp.size(), cudaMemcpyHostToDevice, s), "batch copy");
-  GB_TRY(cudaMemcpyAsync(d_ci, h_ci.data(), sizeof(int32_t) * h_ci.size(), cudaMemcpyHostToDevice, s), "batch copy");
-  GB_TRY(cudaMemcpyAsync(d_vgid, h_vgid.data(), sizeof(int32_t) * h_vgid.size(), cudaMemcpyHostToDevice, s), "batch copy");
-  GB_TRY(cudaMemcpyAsync(d_desc, h_desc.data(), sizeof(int32_t) * h_desc.size(), cudaMemcpyHostToDevice, s), "batch copy");
-  GB_TRY(cudaMemcpyAsync(d_gm, h_gm.data(), sizeof(int64_t) * G, cudaMemcpyHostToDevice, s), "batch copy");
-  if (n > 0) {
-    int blocks = (int)std::min<int64_t>(((int64_t)n * 32 + 255) / 256, 65535LL * 8);
-    k_globalize<<<blocks, 256, 0, s>>>(n, d_rp, d_vgid, d_desc, d_ci);
-    GB_TRY(cudaGetLastError(), "k_globalize");
+  GB_TRY(pool_alloc(&d_rp, sizeof(int32_t) * n1, s), "batch alloc");
+  GB_TRY(pool_alloc(&d_ci, sizeof(int32_t) * nnz1, s), "batch alloc");
+  GB_TRY(pool_alloc(&d_vgid, sizeof(int32_t) * n1, s), "batch alloc");
+  GB_TRY(pool_alloc(&d_desc, sizeof(int32_t) * 2 * (size_t)G, s), "batch alloc");
+  GB_TRY(pool_alloc(&d_gm, sizeof(int64_t) * (size_t)G, s), "batch alloc");
+  GB_TRY(pool_alloc(&d_rp0, sizeof(int32_t) * n1, s), "batch alloc");
+  GB_TRY(pool_alloc(&d_ci0, sizeof(int32_t) * nnz1, s), "batch alloc");
+  GB_TRY(pool_alloc(&d_perm, sizeof(int32_t) * n1, s), "batch alloc");
+  GB_TRY(pool_alloc(&d_newid, sizeof(int32_t) * n1, s), "batch alloc");
+  GB_TRY(pool_alloc(&d_lists, sizeof(int32_t) * (n_lists + 1), s), "batch alloc");
+  GB_TRY(pool_alloc(&d_loff, sizeof(int64_t) * (long_off.size() + 1), s), "batch alloc");
+  GB_TRY(pool_alloc(&d_tmp, sizeof(long long) * (size_t)(tmp_len + 1), s), "batch alloc");
+  for (int32_t gi = 0, gj; gi < G; gi = gj) {  // the columns, graphs that lie next to each other in one copy
+    gj = gi + 1;
+    while (gj < G && graphs[(size_t)gj]->ci == graphs[(size_t)gj - 1]->ci + 2 * gm[(size_t)gj - 1]) ++gj;
+    GB_TRY(up(d_ci0 + ebase[(size_t)gi], graphs[(size_t)gi]->ci, (size_t)(ebase[(size_t)gj] - ebase[(size_t)gi])),
+           "batch copy");
   }
-  if ((st = prepare_graph(n, m, d_rp, d_ci, d_vgid, nullptr, nullptr, nullptr, &prep, s)) != GC_OK) {
+  GB_TRY(up(d_rp, h_rp.data(), n1), "batch copy");
+  GB_TRY(up(d_rp0, h_rp0.data(), n1), "batch copy");
+  GB_TRY(up(d_perm, h_perm.data(), (size_t)n), "batch copy");
+  GB_TRY(up(d_newid, h_newid.data(), (size_t)n), "batch copy");
+  GB_TRY(up(d_vgid, h_vgid.data(), (size_t)n), "batch copy");
+  GB_TRY(up(d_desc, gbase.data(), (size_t)G), "batch copy");
+  GB_TRY(up(d_desc + G, gn.data(), (size_t)G), "batch copy");
+  GB_TRY(up(d_gm, gm.data(), (size_t)G), "batch copy");
+  GB_TRY(up(d_lists, mid.data(), mid.size()), "batch copy");
+  GB_TRY(up(d_lists + mid.size(), longr.data(), longr.size()), "batch copy");
+  GB_TRY(up(d_loff, long_off.data(), long_off.size()), "batch copy");
+  if ((st = relabel_on_device(n, m, d_rp0, d_ci0, d_perm, d_newid, d_rp, d_ci, nullptr, d_vgid, d_desc, d_lists,
+                              (int32_t)mid.size(), d_lists + mid.size(), d_loff, (int32_t)longr.size(), d_tmp, s)) !=
+          GC_OK ||
+      (st = prepare_graph(n, m, d_rp, d_ci, nullptr, nullptr, rank, &prep, s)) != GC_OK) {
     L->error = gc_last_error();
     goto out;
   }
-  if ((st = scratch_init(&sc, m, table_n, prep.kmax, prep.ktier_off, G, s)) != GC_OK) {
+  for (void* p : {(void*)d_rp0, (void*)d_ci0, (void*)d_perm, (void*)d_newid, (void*)d_lists, (void*)d_loff, (void*)d_tmp})
+    cudaFreeAsync(p, s);
+  d_rp0 = d_ci0 = d_perm = d_newid = d_lists = nullptr;
+  d_loff = nullptr;
+  d_tmp = nullptr;
+  if ((st = scratch_init(&sc, m, needs_tables(prep) ? table_n : 0, prep.kmax, prep.ktier_off, G, s)) != GC_OK) {
     L->error = gc_last_error();
     goto out;
   }
@@ -311,10 +386,9 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
     dg.gn = d_desc + G;
     dg.gm = d_gm;
     dg.table_n = table_n;
-    dg.ranked = false;
-    dg.hgeom = nullptr;
-    dg.hseg = nullptr;
-    dg.hpos = nullptr;
+    dg.hgeom = prep.hgeom;
+    dg.hseg = prep.hseg;
+    dg.hpos = prep.hpos;
     KUnits ku;
     ku.units = prep.kunits;
     ku.cunits = prep.cunits;
@@ -342,7 +416,8 @@ out:
 #undef GB_TRY
   free_prep(&prep, s);
   scratch_free(&sc, s);
-  for (void* p : {(void*)d_rp, (void*)d_ci, (void*)d_vgid, (void*)d_desc, (void*)d_gm})
+  for (void* p : {(void*)d_rp, (void*)d_ci, (void*)d_vgid, (void*)d_desc, (void*)d_gm, (void*)d_rp0, (void*)d_ci0,
+                  (void*)d_perm, (void*)d_newid, (void*)d_lists, (void*)d_loff, (void*)d_tmp})
     if (p) cudaFreeAsync(p, s);
   return st;
 }

@@ -36,11 +36,6 @@
 namespace gc {
 namespace {
 
-__device__ __forceinline__ bool rank_less(const int32_t* __restrict__ deg, int32_t a, int32_t b) {
-  int32_t da = deg[a], db = deg[b];
-  return da < db || (da == db && a < b);
-}
-
 __device__ __forceinline__ void atomic_add_u128(unsigned long long* p, u128 v) {
   unsigned long long lo = (unsigned long long)v;
   unsigned long long hi = (unsigned long long)(v >> 64);
@@ -110,7 +105,7 @@ __global__ void __launch_bounds__(kFinBlock) k_finish(DevGraph g, CountArgs a) {
       int32_t o = kByEdge ? g.e2o[i0] : (int32_t)i0;
       if ((uint32_t)o >= (uint32_t)g.m) o = 0;  // only for invalid input
       const int32_t p = g.ocsr[o];
-      if (!kByEdge) eid = g.eid[p];
+      if (!kByEdge && a.per_edge) eid = g.eid[p];
       const int32_t r = g.rev[p];
       const int32_t u = g.ci[r], v = g.ci[p];
       gid = g.vgid ? g.vgid[u] : 0;
@@ -286,7 +281,7 @@ __global__ void __launch_bounds__(kBlock) k_pass_c(DevGraph g, CountArgs a) {
     if (threadIdx.x < 3) s_next[threadIdx.x] = hb;
     __syncthreads();
     // x runs over the lower-rank neighbours of h; o over those of x's
-    // neighbours that rank below h (a prefix of Gamma(x) when ids are ranks).
+    // neighbours that rank below h (a prefix of Gamma(x): ids are ranks).
     for (int pass = 0; pass < (zero_all ? 2 : 3); ++pass) {
       for (;;) {
         int32_t p = 0;
@@ -294,15 +289,13 @@ __global__ void __launch_bounds__(kBlock) k_pass_c(DevGraph g, CountArgs a) {
         p = __shfl_sync(0xffffffffu, p, 0);
         if (p >= he) break;
         const int32_t x = g.ci[p];
-        if (!rank_less(g.deg, x, h)) continue;
+        if (x >= h) break;  // the lower neighbours are a prefix of Gamma(h)
         const int32_t xb = g.rp[x];
-        int32_t xe = g.rp[x + 1];
-        if (g.ranked) xe = min(max(g.rev[p], xb), xe);  // Gamma(x) below the slot of (x, h) is < h
+        const int32_t xe = min(max(g.rev[p], xb), g.rp[x + 1]);  // Gamma(x) below the slot of (x, h) is < h
         unsigned long long s = 0;
         if (pass == 0 && lane == 0) w_wedge += xe - xb;
         for (int32_t q = xb + lane; q < xe; q += 32) {
           const int32_t o = g.ci[q];
-          if (!g.ranked && !rank_less(g.deg, o, h)) continue;
           if (pass == 0) {
             atomicAdd(&tab[o - base], 1u);
           } else if (pass == 1) {
@@ -809,7 +802,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == kHashBlock ? kCtasPerSm 
 // ---------------- pass C for units of at most kHash2MaxW wedges ----------------
 // The same counting and attribution as k_pass_c_hash, for the units whose
 // wedges do not fit that hash: each slot is one 32-bit word holding the
-// vertex o (22 bits; graphs of at most 2^22 vertices) and cnt_h(o) (10 bits;
+// vertex o (22 bits, from its graph's first; graphs of at most 2^22 vertices) and cnt_h(o) (10 bits;
 // units of fewer than 1023 lower neighbours, so a count never reaches 1023
 // and a word is never all ones, the empty mark). kHash2Slots words fill the
 // shared memory of one 1024-thread CTA per SM; a unit uses the first
@@ -870,6 +863,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == kHash2Block ? 1 : 2)
     if (k >= k1) break;
     const int32_t h = a.cunits[first + k];
     const int32_t wk = min(a.chash_w[a.n_chash + k], (int32_t)kHash2MaxW);
+    const int32_t base = g.gbase[g.vgid ? g.vgid[h] : 0];
     const uint32_t size = min((uint32_t)kSlots, (uint32_t)(((long long)wk * 25 + 17) / 18) + 32u);
     const int32_t hb = g.rp[h], he = g.rp[h + 1];
     for (uint32_t i = threadIdx.x; i < size; i += kThreads) htab[i] = kHash2Empty;
@@ -900,9 +894,9 @@ __global__ void __launch_bounds__(kThreads, kThreads == kHash2Block ? 1 : 2)
           for (int j = 0; j < 4; ++j) {
             if (o[j] < 0) continue;
             if (pass == 0) {
-              if (!h2_insert(htab, o[j], size)) atomicOr(a.status, (int32_t)kSpillOverflow);
+              if (!h2_insert(htab, o[j] - base, size)) atomicOr(a.status, (int32_t)kSpillOverflow);
             } else {
-              const uint32_t c = h2_count(htab, o[j], size) - 1u;
+              const uint32_t c = h2_count(htab, o[j] - base, size) - 1u;
               if (c && c < 1023u) {
                 atomicAdd(&a.P[q0 + 32 * j + lane], (unsigned long long)c);  // slot (x, o)
                 sx += c;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -57,7 +58,6 @@ struct DevGraph {
   const int32_t* gn;       // [G] vertices of each graph
   const int64_t* gm;       // [G] edges of each graph
   int32_t table_n;         // max gn[g]: size of one Psi table
-  bool ranked;             // ids are the (degree, id) ranks and rows ascend
   const HubGeom* hgeom;    // ranked: [G] (nullptr when the graph has no hub units)
   const HubSeg* hseg;
   const int32_t* hpos;
@@ -297,14 +297,39 @@ inline cudaError_t pool_alloc(T** p, size_t bytes, cudaStream_t s) {
   return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, pool, s);
 }
 
+// ---- relabelling P1: the host half (gc_api.cu) ----
+// Host arrays left uninitialised on allocation (every element is written
+// before use).
+template <class T>
+struct HostBuf {
+  std::unique_ptr<T[]> p;
+  T* data() { return p.get(); }
+  T& operator[](size_t i) { return p[i]; }
+  void resize(size_t n) { p.reset(new T[n > 0 ? n : 1]); }
+};
+// Vertices ranked by ascending (degree, id) -- a stable counting sort of the
+// degrees -- and what the device relabel needs: internal row pointers, and the
+// internal rows of more than 32 entries listed by the sort that takes them.
+struct RelabelPlan {
+  HostBuf<int32_t> perm, newid, rp;
+  std::vector<int32_t> mid, longr;  // rows of 33..4096 entries, and longer ones
+  std::vector<int64_t> long_off;    // offset of each long row's padded copy
+  int64_t tmp_len = 0;
+  int32_t obound[kOBounds] = {};    // first rank of degree >= kOBoundDeg[k]
+};
+// On at most max_threads host threads. Throws std::bad_alloc.
+RelabelPlan plan_relabel(int32_t n, const int32_t* rp, int max_threads);
+
 // ---- relabelling P1 on the device (gc_relabel.cu) ----
 // Internal row i = caller row perm[i] in internal ids (newid), sorted; eid:
-// caller's edge id of every internal slot. rp: internal row pointers (device);
+// caller's edge id of every internal slot, or nullptr (not wanted). A union of
+// graphs (vgid, gbase: of the internal ids) has caller columns local to their
+// graph, and every other id global. rp: internal row pointers (device);
 // mid_rows / long_rows: internal rows of 33..4096 and of more entries; the
 // long rows are sorted in padded copies at tmp + long_off[k].
 gc_status relabel_on_device(int32_t n, int32_t m, const int32_t* d_rp0, const int32_t* d_ci0,
                             const int32_t* d_perm, const int32_t* d_newid, const int32_t* d_rp, int32_t* d_ci,
-                            int32_t* d_eid, const int32_t* d_mid_rows, int32_t n_mid, const int32_t* d_long_rows,
+                            int32_t* d_eid, const int32_t* d_vgid, const int32_t* d_gbase, const int32_t* d_mid_rows, int32_t n_mid, const int32_t* d_long_rows,
                             const int64_t* d_long_off, int32_t n_long, long long* d_tmp, cudaStream_t s);
 
 // ---- preprocessing (gc_prep.cu) ----
@@ -317,7 +342,6 @@ struct PrepBuffers {
   int32_t* units = nullptr;
   int32_t n_units = 0;
   int32_t dmax = 0;
-  long long* S = nullptr;  // [n] sum of neighbour degrees (Psi build cost of a v-group)
   int32_t* rev = nullptr;  // [2m] slot of the reverse direction of every slot
   int32_t* ocsr = nullptr;  // [m] out-slot -> CSR slot
   int32_t* e2o = nullptr;   // [m] edge id -> out-slot
@@ -349,20 +373,21 @@ struct RankInfo {
   const int32_t* gn;      // [G] vertices of each
   const int32_t* obound;  // [G][kOBounds] first id of degree >= kOBoundDeg[k] (the graph's end if none)
 };
-// Builds degrees, edge ids, the edge list, degree-oriented out-lists and the
-// binned unit list on `stream`. vgid may be nullptr (single graph).
-// d_eid_given (optional): slot -> edge id computed by the caller (ownership
-// passes to PrepBuffers); d_perm (optional, with it): internal -> caller
-// vertex id, used to write the edge list in the caller's labels.
-gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t* d_ci,
-                        const int32_t* d_vgid, int32_t* d_eid_given, const int32_t* d_perm,
-                        const RankInfo* rank, PrepBuffers* out, cudaStream_t stream);
+// Whether some pass-C units are left for the vertex-indexed tables.
+inline bool needs_tables(const PrepBuffers& p) { return p.n_cunits > p.n_cheavy + p.n_chash + p.n_chash2; }
+// Builds degrees, the degree-oriented out-lists, the reverse-slot map and the
+// binned unit lists of a ranked graph on `stream`. d_eid (optional): slot ->
+// edge id from the relabel (ownership passes to PrepBuffers); with it, and
+// d_perm (internal -> caller vertex id), the edge list in the caller's labels
+// and the edge id -> out-slot map are made too.
+gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t* d_ci, int32_t* d_eid,
+                        const int32_t* d_perm, const RankInfo& rank, PrepBuffers* out, cudaStream_t stream);
 // Splits the pass-C units of a ranked graph (ids = ranks, rows ascending)
 // into hub units for the blocked kernel, units of at most kHashMaxW wedges
 // for the hashed kernel and the rest, leaving out units without wedges
 // (fills cunits, n_cheavy, chash_w, n_chash, n_cunits; otherwise
 // cunits is a copy of units).
-gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, const RankInfo* rank, PrepBuffers* p,
+gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, const RankInfo& rank, PrepBuffers* p,
                            cudaStream_t stream);
 void free_prep(PrepBuffers* p, cudaStream_t s);
 // Smallest slot p with rev[p] == p (no reverse: the input is not symmetric),

@@ -3,18 +3,17 @@
 //   * degrees d_x and the P3 orientation of every edge (Sec. 4.3): the "low"
 //     endpoint u has the smaller (degree, id) pair, the "high" endpoint v the
 //     larger, so d_v >= d_u;
-//   * edge ids (rank of (u, v), u < v, in row-major upper-triangle order) and
-//     the slot -> edge id map of both CSR directions;
+//   * the slot -> edge id map of both CSR directions (edge id: rank of (u, v),
+//     u < v, in row-major upper-triangle order of the caller's labels);
 //   * degree-oriented out-lists: out(x) = neighbours of higher (degree, id)
-//     rank, ascending ids. Each pair {a, b} of adjacent vertices appears in
+//     rank, ascending ids, the end of row x since ids are ranks. Each pair {a, b} of adjacent vertices appears in
 //     exactly one out-list; the 4-clique step uses this to count each pair
 //     of T once (the role of the Psi reset in Alg. 5);
 //   * the work units of the counting passes: every vertex v that is the high
 //     endpoint of at least one edge forms one "v-group" (its low neighbours);
 //     groups are binned by floor(log2(estimated work)) and listed heaviest
 //     bin first -- the difficulty-ordered edge queue Pi of Sec. 4.4 at group
-//     granularity, with d_v + sum_{r in Gamma(v)} d_r as the work estimate
-//     (a vertex analogue of the vol ordering of Table 4).
+//     granularity -- and split into the kernels of pass C by their wedges.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -31,11 +30,6 @@ namespace {
 
 constexpr int kScanTile = 2048;  // elements per scan tile (256 threads x 8)
 
-__device__ __forceinline__ bool rank_less(const int32_t* deg, int32_t a, int32_t b) {
-  int32_t da = deg[a], db = deg[b];
-  return da < db || (da == db && a < b);
-}
-
 // first index in [lo, hi) with a[i] >= key
 __device__ __forceinline__ int32_t lower_bound_i32(const int32_t* a, int32_t lo, int32_t hi,
                                                    int32_t key) {
@@ -46,111 +40,74 @@ __device__ __forceinline__ int32_t lower_bound_i32(const int32_t* a, int32_t lo,
   return lo;
 }
 
-__global__ void k_deg_up(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                         int32_t* __restrict__ deg, int32_t* __restrict__ up) {
+// Degrees, out-degrees (ids are ranks, so the higher-rank neighbours of x are
+// the entries above x), and the largest of both.
+__global__ void __launch_bounds__(256) k_deg_out(int32_t n, const int32_t* __restrict__ rp,
+                                                 const int32_t* __restrict__ ci, int32_t* __restrict__ deg,
+                                                 int32_t* __restrict__ out_cnt, int32_t* __restrict__ dmax,
+                                                 int32_t* __restrict__ kmax) {
+  int32_t dm = 0, km = 0;
   for (int32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
-    int32_t b = rp[x], e = rp[x + 1];
-    deg[x] = e - b;
-    up[x] = e - lower_bound_i32(ci, b, e, x + 1);
-  }
-}
-
-// Warp per vertex: number of higher-rank neighbours, sum of neighbour degrees,
-// maximum degree.
-__global__ void k_out_cnt(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                          const int32_t* __restrict__ deg, int32_t* __restrict__ out_cnt,
-                          long long* __restrict__ S, int32_t* __restrict__ dmax, int32_t* __restrict__ kmax) {
-  const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int32_t x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += warps) {
-    int32_t b = rp[x], e = rp[x + 1];
-    int32_t c = 0;
-    long long s = 0;
-    for (int32_t p = b + lane; p < e; p += 32) {
-      int32_t y = ci[p];
-      c += rank_less(deg, x, y) ? 1 : 0;
-      s += deg[y];
-    }
-    for (int o = 16; o; o >>= 1) {
-      c += __shfl_xor_sync(0xffffffffu, c, o);
-      s += __shfl_xor_sync(0xffffffffu, s, o);
-    }
-    if (lane == 0) {
-      out_cnt[x] = c;
-      S[x] = s;
-      if (e - b > 0) atomicMax(dmax, e - b);
-      if (c > 0) atomicMax(kmax, c);
-    }
-  }
-}
-
-// Warp per vertex: edge ids of every slot, edge list, out-lists, and the
-// out-slot of every edge id.
-__global__ void k_edges(int32_t n, int32_t m, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                        const int32_t* __restrict__ deg, const int32_t* __restrict__ up,
-                        const int32_t* __restrict__ upoff, const int32_t* __restrict__ out_ptr,
-                        int32_t* __restrict__ eid, int32_t* __restrict__ uv,
-                        int32_t* __restrict__ out_idx, int32_t* __restrict__ ocsr, int32_t* __restrict__ rev,
-                        int32_t* __restrict__ e2o, bool write_ids, const int32_t* __restrict__ perm) {
-  const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int32_t x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += warps) {
     const int32_t b = rp[x], e = rp[x + 1];
-    const int32_t first_up = e - up[x];
-    int32_t o = out_ptr[x];
-    for (int32_t base = b; base < e; base += 32) {
-      int32_t p = base + lane;
-      bool valid = p < e;
-      int32_t y = valid ? ci[p] : 0;
-      bool is_out = valid && rank_less(deg, x, y);
-      int32_t qr = -1;  // ids given: the reverse slot, once found
-      if (valid && write_ids) {  // the slot of (y, x); the ids below take the same search
-        const int32_t yb = rp[y], ye = rp[y + 1];
-        const int32_t q = lower_bound_i32(ci, yb, ye, x);
-        rev[p] = (q < ye && ci[q] == x) ? q : p;  // p itself only for invalid input
-      } else if (valid && y > x) {  // ids given: one search per edge, from its lower end, sets both
-        const int32_t yb = rp[y], ye = rp[y + 1];
-        const int32_t q = lower_bound_i32(ci, yb, ye, x);
-        if (q < ye && ci[q] == x) {
-          rev[p] = q;
-          rev[q] = p;
-          qr = q;
-        }  // else both keep rev = self (k_rev_init): no reverse, invalid input
+    const int32_t k = e - lower_bound_i32(ci, b, e, x + 1);
+    deg[x] = e - b;
+    out_cnt[x] = k;
+    dm = max(dm, e - b);
+    km = max(km, k);
+  }
+  // one atomic a block and maximum: one a vertex on the same word took 0.8 ms
+  // of the preparation of R-MAT scale 20
+  __shared__ int32_t s_m[2];
+  if (threadIdx.x < 2) s_m[threadIdx.x] = 0;
+  __syncthreads();
+  dm = __reduce_max_sync(0xffffffffu, dm);
+  km = __reduce_max_sync(0xffffffffu, km);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&s_m[0], dm);
+    atomicMax(&s_m[1], km);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (s_m[0]) atomicMax(dmax, s_m[0]);
+    if (s_m[1]) atomicMax(kmax, s_m[1]);
+  }
+}
+
+// Warp per vertex x: the out-list, and the reverse slot of both directions of
+// each of its edges, by one search in the higher end's row. eid (optional):
+// the relabel wrote the id of the slot whose caller labels (perm) ascend; the
+// other slot of the edge takes it here, and e2o the edge's out-slot.
+__global__ void k_edges(int32_t n, int32_t m, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                        const int32_t* __restrict__ out_ptr, int32_t* __restrict__ eid,
+                        int32_t* __restrict__ out_idx, int32_t* __restrict__ ocsr, int32_t* __restrict__ rev,
+                        int32_t* __restrict__ e2o, const int32_t* __restrict__ perm) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t xw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; xw < n; xw += warps) {
+    const int32_t x = (int32_t)xw;
+    const int32_t e = rp[x + 1], o0 = out_ptr[x], k = out_ptr[x + 1] - o0;
+    for (int32_t i = lane; i < k; i += 32) {
+      const int32_t p = e - k + i, os = o0 + i;  // the entries above x end its row
+      const int32_t y = ci[p];
+      out_idx[os] = y;
+      ocsr[os] = p;
+      const int32_t yb = rp[y], ye = rp[y + 1];
+      const int32_t q = lower_bound_i32(ci, yb, ye, x);
+      const bool found = q < ye && ci[q] == x;
+      if (found) {
+        rev[p] = q;
+        rev[q] = p;
+      }  // else both keep rev = self (k_rev_init): no reverse, invalid input
+      if (!eid) continue;
+      int32_t ide;
+      if (found && perm[x] > perm[y]) {
+        ide = eid[q];
+        eid[p] = ide;
+      } else {
+        ide = eid[p];
+        if (found) eid[q] = ide;
       }
-      int32_t id = 0;
-      if (valid && write_ids) {
-        if (y > x) {
-          id = upoff[x] + (p - first_up);
-          uv[2 * (int64_t)id] = x;
-          uv[2 * (int64_t)id + 1] = y;
-        } else {
-          int32_t yb = rp[y], ye = rp[y + 1];
-          int32_t q = lower_bound_i32(ci, yb, ye, x);  // x is in row y (symmetry)
-          id = (q < ye && ci[q] == x) ? upoff[y] + (q - (ye - up[y])) : 0;  // 0 only for invalid input
-        }
-        eid[p] = id;
-      }
-      unsigned mask = __ballot_sync(0xffffffffu, is_out);
-      if (is_out) {
-        const int32_t os = o + __popc(mask & ((1u << lane) - 1u));
-        out_idx[os] = y;
-        ocsr[os] = p;
-        // ids given (ids are ranks, so an out-slot is the slot searched from):
-        // the relabel wrote the id of the slot whose caller labels ascend;
-        // the other slot of the edge takes it here
-        int32_t ide = id;
-        if (!write_ids) {
-          if (qr >= 0 && perm[x] > perm[y]) {
-            ide = eid[qr];
-            eid[p] = ide;
-          } else {
-            ide = eid[p];
-            if (qr >= 0) eid[qr] = ide;
-          }
-        }
-        if ((uint32_t)ide < (uint32_t)m) e2o[ide] = os;  // out of range only for invalid input
-      }
-      o += __popc(mask);
+      if ((uint32_t)ide < (uint32_t)m) e2o[ide] = os;  // out of range only for invalid input
     }
   }
 }
@@ -185,34 +142,40 @@ __device__ __forceinline__ int bin_of(long long cost) {
   return cost <= 1 ? 0 : 63 - __clzll(cost);
 }
 
-// Bin key of a v-group under the chosen ordering (0 vol, 1 degree, 2 none).
-__device__ __forceinline__ int unit_bin(int key, long long S, int32_t d) {
-  return key == 0 ? bin_of(S + d) : (key == 1 ? bin_of(d) : 0);
+// Bin key of a v-group under the chosen ordering (0 volume, 1 degree, 2 none).
+// Only the order of the units on the vertex-indexed tables depends on it (hub
+// and hashed units are sorted by their wedges): the volume is taken as d^2.
+__device__ __forceinline__ int unit_bin(int key, int32_t d) {
+  return key == 0 ? bin_of((long long)d * d) : (key == 1 ? bin_of(d) : 0);
 }
 
-__global__ void k_bin_hist(int32_t n, const int32_t* __restrict__ deg,
-                           const int32_t* __restrict__ out_cnt, const long long* __restrict__ S,
-                           int32_t* __restrict__ hist, int key) {
-  __shared__ int32_t h[64];
-  if (threadIdx.x < 64) h[threadIdx.x] = 0;
-  __syncthreads();
-  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    if (deg[v] - out_cnt[v] > 0) atomicAdd(&h[unit_bin(key, S[v], deg[v])], 1);
+// Counts, or (kScatter) lists by bin from cursor[], the v-groups: one atomic a
+// block and bin.
+template <int kBins, bool kScatter, class Bin>
+__device__ __forceinline__ void bin_vertices(int32_t n, int32_t* __restrict__ cursor, int32_t* __restrict__ list, Bin bin) {
+  __shared__ int32_t h[kBins], base[kBins];
+  for (int32_t v0 = blockIdx.x * blockDim.x; v0 < n; v0 += gridDim.x * blockDim.x) {
+    for (int i = threadIdx.x; i < kBins; i += blockDim.x) h[i] = 0;
+    __syncthreads();
+    const int32_t v = v0 + threadIdx.x;
+    const int b = v < n ? bin(v) : -1;
+    int at = 0;
+    if (b >= 0) at = atomicAdd(&h[b], 1);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kBins; i += blockDim.x)
+      if (h[i]) base[i] = atomicAdd(&cursor[i], h[i]);
+    __syncthreads();
+    if (kScatter && b >= 0) list[base[b] + at] = v;
+    __syncthreads();
   }
-  __syncthreads();
-  if (threadIdx.x < 64 && h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], h[threadIdx.x]);
 }
-
-__global__ void k_bin_scatter(int32_t n, const int32_t* __restrict__ deg,
-                              const int32_t* __restrict__ out_cnt,
-                              const long long* __restrict__ S, int32_t* __restrict__ cursor,
-                              int32_t* __restrict__ units, int key) {
-  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    if (deg[v] - out_cnt[v] > 0) {
-      int32_t pos = atomicAdd(&cursor[unit_bin(key, S[v], deg[v])], 1);
-      units[pos] = v;
-    }
-  }
+template <bool kScatter>
+__global__ void __launch_bounds__(1024) k_bin_units(int32_t n, const int32_t* __restrict__ deg,
+                                                    const int32_t* __restrict__ out_cnt, int32_t* __restrict__ cursor,
+                                                    int32_t* __restrict__ units, int key) {
+  bin_vertices<64, kScatter>(n, cursor, units, [&](int32_t v) {
+    return deg[v] - out_cnt[v] > 0 ? unit_bin(key, deg[v]) : -1;
+  });
 }
 
 // Pass K units: every vertex a with |out(a)| = k >= 2 (a triangle needs two
@@ -221,20 +184,10 @@ __global__ void k_bin_scatter(int32_t n, const int32_t* __restrict__ deg,
 // <= 32) are contiguous ranges of the list.
 __device__ __forceinline__ int kbin_of(int32_t k) { return 32 - __clz(k - 1); }
 
-__global__ void k_kbin_hist(int32_t n, const int32_t* __restrict__ out_cnt, int32_t* __restrict__ hist) {
-  __shared__ int32_t h[32];
-  if (threadIdx.x < 32) h[threadIdx.x] = 0;
-  __syncthreads();
-  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
-    if (out_cnt[v] >= 2) atomicAdd(&h[kbin_of(out_cnt[v])], 1);
-  __syncthreads();
-  if (threadIdx.x < 32 && h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], h[threadIdx.x]);
-}
-
-__global__ void k_kbin_scatter(int32_t n, const int32_t* __restrict__ out_cnt, int32_t* __restrict__ cursor,
-                               int32_t* __restrict__ units) {
-  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
-    if (out_cnt[v] >= 2) units[atomicAdd(&cursor[kbin_of(out_cnt[v])], 1)] = v;
+template <bool kScatter>
+__global__ void __launch_bounds__(1024) k_bin_kunits(int32_t n, const int32_t* __restrict__ out_cnt,
+                                                     int32_t* __restrict__ cursor, int32_t* __restrict__ units) {
+  bin_vertices<32, kScatter>(n, cursor, units, [&](int32_t v) { return out_cnt[v] >= 2 ? kbin_of(out_cnt[v]) : -1; });
 }
 
 // Wedges of every pass-C unit h of a ranked graph: W_h = sum over the
@@ -458,7 +411,7 @@ static void sort_by_wedges_desc(std::vector<int32_t>* v, const std::vector<long 
   v->swap(out);
 }
 
-gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, const RankInfo* rank, PrepBuffers* p,
+gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, const RankInfo& rank, PrepBuffers* p,
                            cudaStream_t s) {
   const int32_t nu = p->n_units;
   cudaError_t e = pool_alloc(&p->cunits, sizeof(int32_t) * (nu > 0 ? nu : 1), s);
@@ -470,7 +423,12 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
   p->n_chash2 = 0;
   p->n_chash2_big = 0;
   p->n_cunits = nu;
-  if (!rank || n <= kSmemTableMax || nu == 0) {
+  int32_t largest = 0;
+  for (int32_t gi = 0; gi < rank.G; ++gi) largest = std::max(largest, rank.gn[gi]);
+  auto graph_of = [&](int32_t h) {
+    return (size_t)(std::upper_bound(rank.gbase, rank.gbase + rank.G, h) - rank.gbase) - 1;
+  };
+  if (largest <= kSmemTableMax || nu == 0) {
     e = nu > 0 ? cudaMemcpyAsync(p->cunits, p->units, sizeof(int32_t) * nu, cudaMemcpyDeviceToDevice, s) : cudaSuccess;
     return e == cudaSuccess ? GC_OK : cuda_fail(e, "copy cunits");
   }
@@ -509,13 +467,13 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
       hashed.push_back(k);
       continue;
     }
-    if (w <= kHash2MaxW && NX[k] < kHash2MaxNx && n <= kHash2MaxN) {
+    if (w <= kHash2MaxW && NX[k] < kHash2MaxNx && largest <= kHash2MaxN) {
       hashed2.push_back(k);
       continue;
     }
     if (w >= 16384 && NX[k] < (1 << 26)) {
       const long long span = (long long)hub_cpw(NX[k]) * tab;
-      const long long blocks = ((long long)U[k] + span - 1) / span;
+      const long long blocks = ((long long)(U[k] - rank.gbase[graph_of(U[k])]) + span - 1) / span;
       const long long per_block = NX[k] > 1024 ? NX[k] : 1024;
       if (w >= blocks * per_block) {
         heavy.push_back(k);
@@ -558,9 +516,9 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
   std::vector<HubGeom> geom;
   int64_t n_pos = 0;
   if (!heavy.empty()) {
-    for (int32_t gi = 0; gi < rank->G; ++gi) {
-      const int32_t* ob = rank->obound + (size_t)gi * kOBounds;
-      const int32_t end = rank->gbase[gi] + rank->gn[gi];
+    for (int32_t gi = 0; gi < rank.G; ++gi) {
+      const int32_t* ob = rank.obound + (size_t)gi * kOBounds;
+      const int32_t end = rank.gbase[gi] + rank.gn[gi];
       HubGeom ge = {(int32_t)segs.size(), 0, end, end, n_pos};
       int32_t word = 0;
       for (int c = 0; c < kOBounds; ++c) {
@@ -581,10 +539,10 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
       if (ge.nseg > 0) {
         // rows of at least max(32, bounds) entries: the last ids
         const int32_t least = std::max(32, ge.nseg + 1);
-        int32_t a = rank->gbase[gi], b = end;
+        int32_t a = rank.gbase[gi], b = end;
         while (a < b) {
           const int32_t mid = a + (b - a) / 2;
-          if (rank->rp[mid + 1] - rank->rp[mid] < least) a = mid + 1; else b = mid;
+          if (rank.rp[mid + 1] - rank.rp[mid] < least) a = mid + 1; else b = mid;
         }
         ge.xmin = a;
         n_pos += (int64_t)(end - a) * (ge.nseg + 1);
@@ -608,7 +566,7 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
     constexpr long long kJobWedges = 8192;
     const int per_cta = hub_jobs_per_cta();
     auto geom_of = [&](int32_t h) -> const HubGeom& {
-      return geom[(size_t)(std::upper_bound(rank->gbase, rank->gbase + rank->G, h) - rank->gbase) - 1];
+      return geom[graph_of(h)];
     };
     auto seg_of = [&](const HubGeom& ge, int32_t id) {  // the segment holding id (the last one past the end)
       int32_t k = ge.seg;
@@ -633,9 +591,9 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
       J = std::max(1LL, std::min(J, W[heavy[i]] / std::max(kJobWedges, 8LL * NX[heavy[i]])));
       int32_t from = lo;
       for (long long j = 1; j <= J; ++j) {
-        const long long upto = rank->rp[lo] + (long long)(rank->rp[h] - rank->rp[lo]) * j / J;
+        const long long upto = rank.rp[lo] + (long long)(rank.rp[h] - rank.rp[lo]) * j / J;
         const int32_t to =
-            j == J ? h : (int32_t)(std::upper_bound(rank->rp + lo, rank->rp + h, (int32_t)upto) - rank->rp) - 1;
+            j == J ? h : (int32_t)(std::upper_bound(rank.rp + lo, rank.rp + h, (int32_t)upto) - rank.rp) - 1;
         if (to <= from && (j < J || from > lo)) continue;  // nothing in this share (a hub keeps at least one job)
         cj.push_back({cost[i] / (double)J, make_int4((int)i, from, to, 2 * seg_of(ge, from) + (from == lo))});
         from = to;
@@ -701,7 +659,6 @@ void free_prep(PrepBuffers* p, cudaStream_t s) {
   if (p->out_ptr) cudaFreeAsync(p->out_ptr, s);
   if (p->out_idx) cudaFreeAsync(p->out_idx, s);
   if (p->units) cudaFreeAsync(p->units, s);
-  if (p->S) cudaFreeAsync(p->S, s);
   if (p->rev) cudaFreeAsync(p->rev, s);
   if (p->ocsr) cudaFreeAsync(p->ocsr, s);
   if (p->e2o) cudaFreeAsync(p->e2o, s);
@@ -714,14 +671,11 @@ void free_prep(PrepBuffers* p, cudaStream_t s) {
   *p = PrepBuffers();
 }
 
-gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t* d_ci,
-                        const int32_t* d_vgid, int32_t* d_eid_given, const int32_t* d_perm,
-                        const RankInfo* rank, PrepBuffers* out, cudaStream_t s) {
-  (void)d_vgid;
+gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t* d_ci, int32_t* d_eid,
+                        const int32_t* d_perm, const RankInfo& rank, PrepBuffers* out, cudaStream_t s) {
   PrepBuffers P;
-  P.eid = d_eid_given;
-  int32_t *up = nullptr, *upoff = nullptr, *out_cnt = nullptr, *dmax = nullptr, *hist = nullptr;
-  long long* S = nullptr;
+  P.eid = d_eid;
+  int32_t *out_cnt = nullptr, *dmax = nullptr, *hist = nullptr;
   gc_status st = GC_OK;
   cudaError_t e = cudaSuccess;
   const int64_t nnz = 2 * (int64_t)m;
@@ -734,48 +688,41 @@ gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t
     }                                      \
   } while (0)
   GC_TRY(pool_alloc(&P.deg, sizeof(int32_t) * (n > 0 ? n : 1), s), "alloc deg");
-  if (!P.eid) GC_TRY(pool_alloc(&P.eid, sizeof(int32_t) * (nnz > 0 ? nnz : 1), s), "alloc eid");
   GC_TRY(pool_alloc(&P.rev, sizeof(int32_t) * (nnz > 0 ? nnz : 1), s), "alloc rev");
-  GC_TRY(pool_alloc(&P.uv, sizeof(int32_t) * (nnz > 0 ? nnz : 1), s), "alloc uv");
   GC_TRY(pool_alloc(&P.out_ptr, sizeof(int32_t) * ((int64_t)n + 1), s), "alloc out_ptr");
   GC_TRY(pool_alloc(&P.out_idx, sizeof(int32_t) * (m > 0 ? m : 1), s), "alloc out_idx");
   GC_TRY(pool_alloc(&P.units, sizeof(int32_t) * (n > 0 ? n : 1), s), "alloc units");
   GC_TRY(pool_alloc(&P.ocsr, sizeof(int32_t) * (m > 0 ? m : 1), s), "alloc ocsr");
-  GC_TRY(pool_alloc(&P.e2o, sizeof(int32_t) * (m > 0 ? m : 1), s), "alloc e2o");
-  GC_TRY(cudaMemsetAsync(P.e2o, 0, sizeof(int32_t) * (m > 0 ? m : 1), s), "memset e2o");  // in range whatever the input
+  if (d_eid) {
+    GC_TRY(pool_alloc(&P.uv, sizeof(int32_t) * (nnz > 0 ? nnz : 1), s), "alloc uv");
+    GC_TRY(pool_alloc(&P.e2o, sizeof(int32_t) * (m > 0 ? m : 1), s), "alloc e2o");
+    GC_TRY(cudaMemsetAsync(P.e2o, 0, sizeof(int32_t) * (m > 0 ? m : 1), s), "memset e2o");  // in range whatever the input
+  }
   GC_TRY(pool_alloc(&P.kunits, sizeof(int32_t) * (n > 0 ? n : 1), s), "alloc kunits");
-  GC_TRY(pool_alloc(&up, sizeof(int32_t) * (n > 0 ? n : 1), s), "alloc up");
-  GC_TRY(pool_alloc(&upoff, sizeof(int32_t) * ((int64_t)n + 1), s), "alloc upoff");
   GC_TRY(pool_alloc(&out_cnt, sizeof(int32_t) * (n > 0 ? n : 1), s), "alloc out_cnt");
-  GC_TRY(pool_alloc(&P.S, sizeof(long long) * (n > 0 ? n : 1), s), "alloc S");
-  S = P.S;
   // [0] max degree, [1..64] v-group bins, [65] max out-degree, [66..97] pass-K bins
   GC_TRY(pool_alloc(&dmax, sizeof(int32_t) * 98, s), "alloc dmax");
   hist = dmax + 1;
   GC_TRY(cudaMemsetAsync(dmax, 0, sizeof(int32_t) * 98, s), "memset");
   if (n > 0) {
-    k_deg_up<<<grid_for(n, 256), 256, 0, s>>>(n, d_rp, d_ci, P.deg, up);
-    GC_TRY(cudaGetLastError(), "k_deg_up");
-    if ((st = exclusive_scan(n, up, upoff, s)) != GC_OK) goto fail;
-    k_out_cnt<<<grid_for((int64_t)n * 32, 256), 256, 0, s>>>(n, d_rp, d_ci, P.deg, out_cnt, S, dmax, dmax + 65);
-    GC_TRY(cudaGetLastError(), "k_out_cnt");
+    const int blocks = std::min(grid_for(n, 256), 8 * (count_grid_size() / kCtasPerSm));
+    const int bin_blocks = std::min(grid_for(n, 1024), 2 * (count_grid_size() / kCtasPerSm));
+    k_deg_out<<<blocks, 256, 0, s>>>(n, d_rp, d_ci, P.deg, out_cnt, dmax, dmax + 65);
+    GC_TRY(cudaGetLastError(), "k_deg_out");
     if ((st = exclusive_scan(n, out_cnt, P.out_ptr, s)) != GC_OK) goto fail;
-    if (d_eid_given) {
-      k_rev_init<<<grid_for(nnz, 256), 256, 0, s>>>(nnz, P.rev);
-      GC_TRY(cudaGetLastError(), "k_rev_init");
-    }
-    k_edges<<<grid_for((int64_t)n * 32, 256), 256, 0, s>>>(n, m, d_rp, d_ci, P.deg, up, upoff,
-                                                            P.out_ptr, P.eid, P.uv, P.out_idx, P.ocsr, P.rev,
-                                                            P.e2o, d_eid_given == nullptr, d_perm);
+    k_rev_init<<<grid_for(nnz, 256), 256, 0, s>>>(nnz, P.rev);
+    GC_TRY(cudaGetLastError(), "k_rev_init");
+    k_edges<<<grid_for((int64_t)n * 32, 256), 256, 0, s>>>(n, m, d_rp, d_ci, P.out_ptr, P.eid, P.out_idx, P.ocsr,
+                                                            P.rev, P.e2o, d_perm);
     GC_TRY(cudaGetLastError(), "k_edges");
-    if (d_eid_given) {
+    if (d_eid) {
       k_uv_perm<<<grid_for((int64_t)n * 32, 256), 256, 0, s>>>(n, d_rp, d_ci, P.eid, d_perm, P.uv);
       GC_TRY(cudaGetLastError(), "k_uv_perm");
     }
-    k_bin_hist<<<grid_for(n, 256), 256, 0, s>>>(n, P.deg, out_cnt, S, hist, order_key());
-    GC_TRY(cudaGetLastError(), "k_bin_hist");
-    k_kbin_hist<<<grid_for(n, 256), 256, 0, s>>>(n, out_cnt, dmax + 66);
-    GC_TRY(cudaGetLastError(), "k_kbin_hist");
+    k_bin_units<false><<<bin_blocks, 1024, 0, s>>>(n, P.deg, out_cnt, hist, nullptr, order_key());
+    GC_TRY(cudaGetLastError(), "k_bin_units");
+    k_bin_kunits<false><<<bin_blocks, 1024, 0, s>>>(n, out_cnt, dmax + 66, nullptr);
+    GC_TRY(cudaGetLastError(), "k_bin_kunits");
     {
       int32_t h[98];
       GC_TRY(cudaMemcpyAsync(h, dmax, sizeof(h), cudaMemcpyDeviceToHost, s), "copy hist");
@@ -796,8 +743,8 @@ gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t
         P.ktier_off[kTierGlobal] = 0;
         P.ktier_off[kNumTiers] = acc;
         GC_TRY(cudaMemcpyAsync(dmax + 66, kc, sizeof(kc), cudaMemcpyHostToDevice, s), "copy k cursors");
-        k_kbin_scatter<<<grid_for(n, 256), 256, 0, s>>>(n, out_cnt, dmax + 66, P.kunits);
-        GC_TRY(cudaGetLastError(), "k_kbin_scatter");
+        k_bin_kunits<true><<<bin_blocks, 1024, 0, s>>>(n, out_cnt, dmax + 66, P.kunits);
+        GC_TRY(cudaGetLastError(), "k_bin_kunits");
       }
       int32_t cur[64];
       int32_t acc = 0;
@@ -807,23 +754,19 @@ gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t
       }
       P.n_units = acc;
       GC_TRY(cudaMemcpyAsync(hist, cur, sizeof(cur), cudaMemcpyHostToDevice, s), "copy cursors");
-      k_bin_scatter<<<grid_for(n, 256), 256, 0, s>>>(n, P.deg, out_cnt, S, hist, P.units, order_key());
-      GC_TRY(cudaGetLastError(), "k_bin_scatter");
+      k_bin_units<true><<<bin_blocks, 1024, 0, s>>>(n, P.deg, out_cnt, hist, P.units, order_key());
+      GC_TRY(cudaGetLastError(), "k_bin_units");
     }
   } else {
     GC_TRY(cudaMemsetAsync(P.out_ptr, 0, sizeof(int32_t), s), "memset out_ptr");
   }
   if ((st = classify_c_units(n, d_rp, d_ci, rank, &P, s)) != GC_OK) goto fail;
-  cudaFreeAsync(up, s);
-  cudaFreeAsync(upoff, s);
   cudaFreeAsync(out_cnt, s);
   cudaFreeAsync(dmax, s);
   *out = P;
   return GC_OK;
 fail:
   cudaStreamSynchronize(s);
-  if (up) cudaFreeAsync(up, s);
-  if (upoff) cudaFreeAsync(upoff, s);
   if (out_cnt) cudaFreeAsync(out_cnt, s);
   if (dmax) cudaFreeAsync(dmax, s);
   free_prep(&P, s);

@@ -50,13 +50,15 @@ __device__ __forceinline__ int32_t lower_bound_dev(const int32_t* a, int32_t lo,
 // caller row, unsorted.
 __global__ void k_fill_rows(int32_t n, const int32_t* __restrict__ rp0, const int32_t* __restrict__ ci0,
                             const int32_t* __restrict__ perm, const int32_t* __restrict__ newid,
+                            const int32_t* __restrict__ vgid, const int32_t* __restrict__ gbase,
                             const int32_t* __restrict__ rp, long long* __restrict__ kv) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
     const int32_t x = perm[i];
     const int32_t b0 = rp0[x], len = rp0[x + 1] - b0, b = rp[i];
-    for (int32_t k = lane; k < len; k += 32) kv[b + k] = ((long long)newid[ci0[b0 + k]] << 32) | k;
+    const int32_t* nid = newid + (vgid ? gbase[vgid[i]] : 0);
+    for (int32_t k = lane; k < len; k += 32) kv[b + k] = ((long long)nid[ci0[b0 + k]] << 32) | k;
   }
 }
 
@@ -180,6 +182,12 @@ __global__ void k_split_eid(int32_t n, int32_t m, const int32_t* __restrict__ rp
   }
 }
 
+// The sorted keys' internal ids alone.
+__global__ void k_split(int64_t nnz, const long long* __restrict__ kv, int32_t* __restrict__ ci) {
+  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < nnz; s += (int64_t)gridDim.x * blockDim.x)
+    ci[s] = (int32_t)(kv[s] >> 32);
+}
+
 int blocks_for(int64_t threads, int block) {
   int64_t b = (threads + block - 1) / block;
   if (b < 1) b = 1;
@@ -191,7 +199,7 @@ int blocks_for(int64_t threads, int block) {
 
 gc_status relabel_on_device(int32_t n, int32_t m, const int32_t* d_rp0, const int32_t* d_ci0,
                             const int32_t* d_perm, const int32_t* d_newid, const int32_t* d_rp, int32_t* d_ci,
-                            int32_t* d_eid, const int32_t* d_mid_rows, int32_t n_mid, const int32_t* d_long_rows,
+                            int32_t* d_eid, const int32_t* d_vgid, const int32_t* d_gbase, const int32_t* d_mid_rows, int32_t n_mid, const int32_t* d_long_rows,
                             const int64_t* d_long_off, int32_t n_long, long long* d_tmp, cudaStream_t s) {
   if (n <= 0) return GC_OK;
   cudaError_t e = cudaSuccess;
@@ -208,7 +216,8 @@ gc_status relabel_on_device(int32_t n, int32_t m, const int32_t* d_rp0, const in
     }                                    \
   } while (0)
   RL_TRY(pool_alloc(&kv, sizeof(long long) * (size_t)(nnz > 0 ? nnz : 1), s), "alloc relabel keys");
-  k_fill_rows<<<blocks_for((int64_t)n * 32, 256), 256, 0, s>>>(n, d_rp0, d_ci0, d_perm, d_newid, d_rp, kv);
+  k_fill_rows<<<blocks_for((int64_t)n * 32, 256), 256, 0, s>>>(n, d_rp0, d_ci0, d_perm, d_newid, d_vgid, d_gbase, d_rp,
+                                                                 kv);
   RL_TRY(cudaGetLastError(), "k_fill_rows");
   k_sort_short<<<blocks_for((int64_t)n * 32, 256), 256, 0, s>>>(n, d_rp, kv);
   RL_TRY(cudaGetLastError(), "k_sort_short");
@@ -219,6 +228,11 @@ gc_status relabel_on_device(int32_t n, int32_t m, const int32_t* d_rp0, const in
   if (n_long > 0) {
     k_sort_long<<<n_long, kLongThreads, 0, s>>>(d_long_rows, d_long_off, d_rp, kv, d_tmp);
     RL_TRY(cudaGetLastError(), "k_sort_long");
+  }
+  if (!d_eid) {
+    k_split<<<blocks_for(nnz, 256), 256, 0, s>>>(nnz, kv, d_ci);
+    RL_TRY(cudaGetLastError(), "k_split");
+    goto out;
   }
   RL_TRY(pool_alloc(&first_up, sizeof(int32_t) * (size_t)n, s), "alloc relabel");
   RL_TRY(pool_alloc(&up_cnt, sizeof(int32_t) * (size_t)n, s), "alloc relabel");

@@ -144,10 +144,8 @@ void fork_release(ForkSet* f) {
 
 namespace {
 
-int host_threads() {
-  const unsigned hw = std::thread::hardware_concurrency();
-  return (int)std::min<unsigned>(hw ? hw : 1, 32);
-}
+// Threads for a loop over `work` entries: one per 2^16, at most host_threads().
+int threads_for(int64_t work) { return (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), work >> 16)); }
 
 // Row ranges [b[t], b[t+1]) holding about equal numbers of entries.
 std::vector<int32_t> nnz_chunks(int32_t n, const int32_t* rp, int nt) {
@@ -164,14 +162,6 @@ std::vector<int32_t> nnz_chunks(int32_t n, const int32_t* rp, int nt) {
   return b;
 }
 
-template <class F>
-void run_threads(int nt, F f) {
-  std::vector<std::thread> th;
-  for (int t = 1; t < nt; ++t) th.emplace_back(f, t);
-  f(0);
-  for (auto& x : th) x.join();
-}
-
 // For a graph that passed the linear checks (columns in range, rows
 // ascending) and failed a symmetry check: the message naming the first entry
 // (x, y) in row order whose reverse (y, x) is absent, found by a binary
@@ -180,10 +170,10 @@ void run_threads(int nt, F f) {
 // the next (x1, y) mismatch although (y, x1) exists -- so the failure path
 // looks it up directly.
 std::string first_without_reverse(int32_t n, const int32_t* rp, const int32_t* ci) {
-  const int nt = rp[n] < (1 << 20) ? 1 : host_threads();
+  const int nt = threads_for(rp[n]);
   const std::vector<int32_t> b = nnz_chunks(n, rp, nt);
   std::vector<std::pair<int32_t, int32_t>> hit((size_t)nt, {-1, -1});
-  run_threads(nt, [&](int t) {
+  host_run(nt, [&](int t) {
     for (int32_t x = b[t]; x < b[t + 1]; ++x)
       for (int32_t p = rp[x]; p < rp[x + 1]; ++p) {
         const int32_t y = ci[p];
@@ -234,9 +224,9 @@ gc_status csr_linear_checks(int32_t n, const int32_t* rp, const int32_t* ci) {
   if (n < 0) { set_error("n < 0"); return GC_ERR_ARG; }
   if (rp[0] != 0) { set_error("row_ptr[0] != 0"); return GC_ERR_RANGE; }
   {  // row_ptr ascending: vertex chunks in parallel, the first decrease in row order
-    const int ntv = n < (1 << 20) ? 1 : host_threads();
+    const int ntv = threads_for(n);
     std::vector<int32_t> first((size_t)ntv, -1);
-    run_threads(ntv, [&](int t) {
+    host_run(ntv, [&](int t) {
       const int32_t x1 = (int32_t)((int64_t)n * (t + 1) / ntv);
       for (int32_t x = (int32_t)((int64_t)n * t / ntv); x < x1; ++x)
         if (rp[x + 1] < rp[x]) {
@@ -252,10 +242,10 @@ gc_status csr_linear_checks(int32_t n, const int32_t* rp, const int32_t* ci) {
   }
   if (rp[n] % 2 != 0) { set_error("row_ptr[n] is odd: the graph cannot be symmetric"); return GC_ERR_ASYMMETRIC; }
   const int64_t nnz = rp[n];
-  const int nt = nnz < (1 << 20) ? 1 : host_threads();
+  const int nt = threads_for(nnz);
   const std::vector<int32_t> b = nnz_chunks(n, rp, nt);
   Checks c(nt);
-  run_threads(nt, [&](int t) {
+  host_run(nt, [&](int t) {
     for (int32_t x = b[t]; x < b[t + 1]; ++x) {
       if (row_ok(ci + rp[x], rp[x + 1] - rp[x], x, n)) continue;
       for (int32_t p = rp[x]; p < rp[x + 1]; ++p) {  // the first failing entry of the first failing row
@@ -276,18 +266,48 @@ gc_status csr_linear_checks(int32_t n, const int32_t* rp, const int32_t* ci) {
 // on first use, at the number of entries of row y below the chunk's first
 // row) gives the slot where x must stand in row y, and the entry there is
 // compared with x. Every entry is checked against a slot of row y, so a
-// missing reverse always fails, and a symmetric graph always passes. The
+// missing reverse always fails, and a symmetric graph always passes. Where the
+// counters would outnumber a chunk's entries by a quarter or more (they are
+// cleared per chunk), the reverse of every upper entry (x, y), y > x, is
+// searched instead: distinct upper entries find distinct lower ones, so the
+// graph is symmetric if all are found and half of the entries are upper. The
 // message of a failure, naming the first entry in row order without a
 // reverse, is returned in *msg (the calling thread sets it).
 gc_status csr_symmetry(int32_t n, const int32_t* rp, const int32_t* ci, std::string* msg) {
   const int64_t nnz = rp[n];
-  int nt = nnz < (1 << 20) ? 1 : host_threads();
+  int nt = threads_for(nnz);
   // per-chunk counters: n ints per thread, at most 1 GiB in all
   const int64_t per = 4 * (int64_t)(n > 0 ? n : 1);
   nt = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (int64_t(1) << 30) / per));
   const std::vector<int32_t> b = nnz_chunks(n, rp, nt);
   std::vector<gc_status> st((size_t)nt, GC_OK);
-  run_threads(nt, [&](int t) {
+  if (nt > 1 && 4 * (int64_t)n > nnz / nt) {
+    std::vector<int64_t> upper((size_t)nt, 0);
+    host_run(nt, [&](int t) {
+      int64_t u = 0;
+      for (int32_t x = b[t]; x < b[t + 1]; ++x) {
+        const int32_t* e = ci + rp[x + 1];
+        const int32_t* p = std::upper_bound(ci + rp[x], e, x);
+        u += e - p;
+        for (; p < e; ++p)
+          if (!std::binary_search(ci + rp[*p], ci + rp[*p + 1], x)) {
+            st[(size_t)t] = GC_ERR_ASYMMETRIC;
+            return;
+          }
+      }
+      upper[(size_t)t] = u;
+    });
+    int64_t total = 0;
+    bool ok = true;
+    for (int t = 0; t < nt; ++t) {
+      total += upper[(size_t)t];
+      ok &= st[(size_t)t] == GC_OK;
+    }
+    if (ok && 2 * total == nnz) return GC_OK;
+    *msg = first_without_reverse(n, rp, ci);
+    return GC_ERR_ASYMMETRIC;
+  }
+  host_run(nt, [&](int t) {
     std::vector<int32_t> fill((size_t)(n > 0 ? n : 1), -1);
     const int32_t x0 = b[t];
     for (int32_t x = x0; x < b[t + 1]; ++x)
@@ -368,6 +388,10 @@ gc_status validate_csr_small(int32_t n, const int32_t* rp, const int32_t* ci, st
 }
 
 gc_status validate_csr(int32_t n, const int32_t* rp, const int32_t* ci) {
+  if (n >= 0 && rp[n] >= 0 && rp[n] < (1 << 17)) {
+    std::vector<int32_t> fill;
+    return validate_csr_small(n, rp, ci, &fill);
+  }
   gc_status st = csr_linear_checks(n, rp, ci);
   if (st != GC_OK) return st;
   std::string msg;
@@ -385,10 +409,10 @@ RelabelPlan plan_relabel(int32_t n, const int32_t* rp, int max_threads) {
   if (n == 0) return R;
   // vertex chunks, one per thread (fewer threads when the per-thread degree
   // histograms would pass 2^24 counters)
-  int nt = n >= (1 << 16) ? std::min(host_threads(), max_threads) : 1;
+  int nt = std::min(threads_for(n), max_threads);
   std::vector<int32_t> dmx((size_t)nt, 0);
   auto chunk = [&](int t, int T) { return (int32_t)((int64_t)n * t / T); };
-  run_threads(nt, [&](int t) {
+  host_run(nt, [&](int t) {
     int32_t d = 0;
     for (int32_t x = chunk(t, nt); x < chunk(t + 1, nt); ++x) d = std::max(d, rp[x + 1] - rp[x]);
     dmx[(size_t)t] = d;
@@ -402,7 +426,7 @@ RelabelPlan plan_relabel(int32_t n, const int32_t* rp, int max_threads) {
   // chunk gives its degree-d vertices: ranks ascend by degree, then by chunk,
   // then by id within the chunk -- the (degree, id) order
   std::vector<int32_t> cnt((size_t)nt * D, 0);
-  run_threads(nt, [&](int t) {
+  host_run(nt, [&](int t) {
     int32_t* c = cnt.data() + (size_t)t * D;
     for (int32_t x = chunk(t, nt); x < chunk(t + 1, nt); ++x) c[rp[x + 1] - rp[x]]++;
   });
@@ -428,7 +452,7 @@ RelabelPlan plan_relabel(int32_t n, const int32_t* rp, int max_threads) {
     S[D] = sl;
   }
   for (int k = 0; k < kOBounds; ++k) R.obound[k] = base[std::min<size_t>((size_t)kOBoundDeg[k], D)];
-  run_threads(nt, [&](int t) {
+  host_run(nt, [&](int t) {
     int32_t* c = cnt.data() + (size_t)t * D;
     for (int32_t x = chunk(t, nt); x < chunk(t + 1, nt); ++x) {
       const int32_t i = c[rp[x + 1] - rp[x]]++;
@@ -437,7 +461,7 @@ RelabelPlan plan_relabel(int32_t n, const int32_t* rp, int max_threads) {
     }
   });
   // internal row pointers: every row of a degree bucket has that degree
-  run_threads(nt, [&](int t) {
+  host_run(nt, [&](int t) {
     for (int32_t i = chunk(t, nt); i < chunk(t + 1, nt); ++i) {
       const int32_t x = R.perm[(size_t)i];
       const int32_t d = rp[x + 1] - rp[x];

@@ -17,17 +17,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
 #include <deque>
-#include <exception>
 #include <mutex>
 #include <string>
 #include <thread>
-#include <unordered_map>
-#include <unordered_set>
 #include <memory>
 #include <thread>
 #include <vector>
@@ -40,62 +36,99 @@ gc_status validate_csr_small(int32_t n, const int32_t* rp, const int32_t* ci, st
 
 namespace {
 
-// Host buffers for the library's copies of bulk submissions, kept for reuse:
-// a submission takes the smallest kept buffer that holds it, whose pages are
-// already mapped, instead of a fresh allocation that every submission would
-// fault in again. Buffers are not initialised (the copy that fills a buffer
-// writes every entry it reads). At most kKeep buffers are kept, the smallest
-// dropped first; the cache lives until the batch and its last buffer are gone.
+// The library's host copy of one submission, pinned where possible, so that a
+// launch copies it to the device directly.
+struct HostBlock {
+  int32_t* p = nullptr;
+  size_t cap = 0;
+  bool pinned = false;
+};
+
+void free_block(const HostBlock& h) {
+  if (h.pinned) cudaFreeHost(h.p);
+  else delete[] h.p;
+}
+
+// Host blocks of retired submissions, kept for reuse: a submission takes the
+// smallest kept block that holds it and is not more than twice as large, whose
+// pages are already mapped and pinned, instead of a fresh allocation. Blocks are
+// not initialised (the copy that fills one writes every entry it reads). Kept
+// are at most kLarge blocks of kLargeBytes or more and kSmall others; the cache
+// lives until the batch and its last block are gone.
 struct HostCache {
-  static constexpr int kKeep = 4;
+  static constexpr int kLarge = 4, kSmall = 64;
+  static constexpr size_t kLargeEntries = (size_t)16 << 20;
   std::mutex mu;
-  std::vector<std::pair<size_t, int32_t*>> free;  // (entries, buffer)
+  std::vector<HostBlock> free;
   ~HostCache() {
-    for (auto& f : free) delete[] f.second;
+    for (auto& h : free) free_block(h);
   }
 };
 
-// A buffer of at least `entries` int32 from the cache (or new); it returns to
-// the cache when its last reference goes. Throws std::bad_alloc.
-std::shared_ptr<int32_t> host_buffer(const std::shared_ptr<HostCache>& cache, size_t entries) {
+// A block of at least `entries` int32; it returns to the cache when its last
+// reference goes. Throws std::bad_alloc.
+std::shared_ptr<HostBlock> host_block(const std::shared_ptr<HostCache>& cache, size_t entries) {
   if (entries == 0) entries = 1;
-  int32_t* p = nullptr;
-  size_t cap = 0;
+  if (entries < 4096) {  // not worth pinning
+    HostBlock h;
+    h.p = new int32_t[entries];
+    h.cap = entries;
+    return std::shared_ptr<HostBlock>(new HostBlock(h), [](HostBlock* q) {
+      free_block(*q);
+      delete q;
+    });
+  }
+  HostBlock h;
   {
     std::lock_guard<std::mutex> lk(cache->mu);
     int best = -1;
-    for (int i = 0; i < (int)cache->free.size(); ++i)
-      if (cache->free[i].first >= entries && (best < 0 || cache->free[i].first < cache->free[best].first)) best = i;
+    for (int i = 0; i < (int)cache->free.size(); ++i) {
+      const size_t cap = cache->free[(size_t)i].cap;
+      if (cap >= entries && cap / 2 <= entries && (best < 0 || cap < cache->free[(size_t)best].cap)) best = i;
+    }
     if (best >= 0) {
-      cap = cache->free[best].first;
-      p = cache->free[best].second;
+      h = cache->free[(size_t)best];
       cache->free.erase(cache->free.begin() + best);
     }
   }
-  if (!p) {
-    p = new int32_t[entries];
-    cap = entries;
+  if (!h.p) {
+    h.cap = entries + entries / 8;
+    if (cudaHostAlloc(reinterpret_cast<void**>(&h.p), sizeof(int32_t) * h.cap, cudaHostAllocPortable) == cudaSuccess) {
+      h.pinned = true;
+    } else {
+      cudaGetLastError();
+      h.p = new int32_t[h.cap];
+    }
   }
   std::shared_ptr<HostCache> keep = cache;
-  return std::shared_ptr<int32_t>(p, [keep, cap](int32_t* q) {
-    std::lock_guard<std::mutex> lk(keep->mu);
-    keep->free.emplace_back(cap, q);
-    if ((int)keep->free.size() > HostCache::kKeep) {
-      auto it = std::min_element(keep->free.begin(), keep->free.end(),
-                                 [](const std::pair<size_t, int32_t*>& a, const std::pair<size_t, int32_t*>& b) {
-                                   return a.first < b.first;
-                                 });
-      delete[] it->second;
-      keep->free.erase(it);
+  return std::shared_ptr<HostBlock>(new HostBlock(h), [keep](HostBlock* q) {
+    HostBlock out = *q;
+    delete q;
+    {
+      std::lock_guard<std::mutex> lk(keep->mu);
+      const bool large = out.cap >= HostCache::kLargeEntries;
+      keep->free.push_back(out);
+      out.p = nullptr;
+      int count = 0, least = -1;
+      for (int i = 0; i < (int)keep->free.size(); ++i) {
+        if ((keep->free[(size_t)i].cap >= HostCache::kLargeEntries) != large) continue;
+        ++count;
+        if (least < 0 || keep->free[(size_t)i].cap < keep->free[(size_t)least].cap) least = i;
+      }
+      if (count > (large ? HostCache::kLarge : HostCache::kSmall)) {
+        out = keep->free[(size_t)least];
+        keep->free.erase(keep->free.begin() + least);
+      }
     }
+    if (out.p) free_block(out);
   });
 }
 
 // A graph waiting for a launch. Its CSR is the library's own copy: rp (n + 1
 // entries starting at 0) and ci (2m entries) point into `owner` -- a copy of
 // one graph (gc_batch_submit), or one shared copy of a whole bulk submission
-// (gc_batch_submit_many: one buffer from the batch's host cache and one bulk
-// copy per graph, made while validating).
+// (gc_batch_submit_many: all row pointers, then all columns, copied while
+// validating).
 struct PendingGraph {
   uint64_t ticket;
   int32_t n;
@@ -103,12 +136,18 @@ struct PendingGraph {
   int64_t bytes;
   const int32_t* rp = nullptr;
   const int32_t* ci = nullptr;
-  std::shared_ptr<int32_t> owner;
+  std::shared_ptr<HostBlock> owner;
 };
 
-struct Result {
-  uint64_t x[34];
-  gc_status status;
+// Results of one launch ([G][17][2]), shared by its tickets until they retire.
+typedef std::vector<uint64_t> Results;
+
+struct Ticket {
+  enum State : uint8_t { kRetired = 0, kLive, kDone };
+  State state = kRetired;
+  gc_status status = GC_OK;
+  int32_t slot = 0;  // row in *out
+  std::shared_ptr<Results> out;
 };
 
 // Timers of one launch (CUDA events on its stream): the size classes of the
@@ -126,8 +165,10 @@ struct Launch {
   cudaEvent_t done = nullptr;
   cudaEvent_t ev[kNumLaunchEv] = {};
   bool timed_classes = false, timed_small = false, timed_union = false, replayed = false;
-  unsigned long long* h_x = nullptr;  // pinned [G][17][2]
-  int32_t* h_status = nullptr;        // pinned
+  unsigned long long* h_x = nullptr;  // pinned [G][17][2], cap_x graphs
+  size_t cap_x = 0;
+  int32_t* h_status = nullptr;        // pinned: small graphs, union
+  std::vector<std::shared_ptr<HostBlock>> owners;  // the device copies from them until the launch is done
   gc_status launch_status = GC_OK;
   std::string error;
 };
@@ -138,7 +179,7 @@ struct Launch {
 // captured and replayed as a CUDA graph. `busy` marks the end of the slot's
 // last sequence: the host waits on it before it refills or regrows them.
 struct SmallBufs {
-  size_t cap_rows = 0, cap_nnz = 0, cap_g = 0, cap_units = 0;
+  size_t cap_rows = 0, cap_nnz = 0, cap_hrows = 0, cap_hnnz = 0, cap_g = 0, cap_units = 0;
   int32_t *d_rp = nullptr, *d_ci = nullptr, *d_gn = nullptr, *d_misc = nullptr;
   int2 *d_units = nullptr, *h_units = nullptr;
   int64_t *d_voff = nullptr, *d_eoff = nullptr, *d_gm = nullptr;
@@ -192,42 +233,35 @@ struct gc_batch_s {
   std::condition_variable cv;
   std::deque<PendingGraph> pending;
   std::vector<Launch*> inflight;
-  std::unordered_map<uint64_t, Result> done;
-  std::unordered_set<uint64_t> live;
-  uint64_t next_ticket = 1;
+  std::deque<Ticket> tickets;           // of the numbers first_ticket .. (the oldest one unretired or later)
+  uint64_t first_ticket = 1;
+  std::vector<Launch*> spare;           // retired launches, for their events and pinned results (at most kMaxSpare)
+  Ticket* find(uint64_t t) {            // nullptr: unknown or retired
+    if (t < first_ticket || t - first_ticket >= tickets.size()) return nullptr;
+    Ticket* k = &tickets[(size_t)(t - first_ticket)];
+    return k->state == Ticket::kRetired ? nullptr : k;
+  }
+  uint64_t add_ticket() {
+    tickets.emplace_back();
+    tickets.back().state = Ticket::kLive;
+    return first_ticket + tickets.size() - 1;
+  }
+  void drop_retired() {
+    while (!tickets.empty() && tickets.front().state == Ticket::kRetired) {
+      tickets.pop_front();
+      ++first_ticket;
+    }
+  }
   bool stop = false;
   std::thread dispatcher;
   cudaStream_t streams[kMaxInflight] = {};
   int next_stream = 0;                  // manual mode: round-robin over the slots
   int device = 0;
-  std::shared_ptr<HostCache> host = std::make_shared<HostCache>();  // bulk-submission copies
+  std::shared_ptr<HostCache> host = std::make_shared<HostCache>();  // submissions' copies
 };
+static constexpr size_t kMaxSpare = 8;
 
 namespace {
-
-// f(0) .. f(count - 1) on the host's cores, at most one thread per call. The
-// first exception is thrown again on the calling thread.
-template <class F>
-void host_parallel(int count, F f) {
-  const unsigned hw = std::thread::hardware_concurrency();
-  const int nt = std::min<int>(count, (int)std::min<unsigned>(hw ? hw : 1, 32));
-  std::atomic<int> next(0);
-  std::exception_ptr err;
-  std::mutex mu;
-  auto work = [&] {
-    try {
-      for (int i; (i = next.fetch_add(1)) < count;) f(i);
-    } catch (...) {
-      std::lock_guard<std::mutex> lk(mu);
-      if (!err) err = std::current_exception();
-    }
-  };
-  std::vector<std::thread> th;
-  for (int t = 1; t < nt; ++t) th.emplace_back(work);
-  work();
-  for (auto& x : th) x.join();
-  if (err) std::rethrow_exception(err);
-}
 
 // Counts `graphs` as one launch on `s`. Fills L (results land in L->h_x when
 // L->done completes). Runs in the dispatcher thread (or the flushing thread
@@ -269,7 +303,7 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
   try {
     for (auto* b : {&h_rp, &h_rp0, &h_perm, &h_newid, &h_vgid}) b->resize((size_t)n + 1);
     std::vector<RelabelPlan> plans((size_t)G);
-    host_parallel(G, [&](int gi) {
+    host_run(G, [&](int gi) {
       const PendingGraph& pg = *graphs[(size_t)gi];
       RelabelPlan& R = plans[(size_t)gi];
       R = plan_relabel(pg.n, pg.rp, 1);
@@ -467,12 +501,24 @@ gc_status run_small(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
       return st;                             \
     }                                        \
   } while (0)
+  // Graphs that lie one after another in one pinned block (a whole bulk
+  // submission) are copied to the device from there; others are packed into
+  // pinned staging first.
+  bool direct = graphs[0]->owner && graphs[0]->owner->pinned;
+  for (int32_t gi = 1; gi < G && direct; ++gi) {
+    const PendingGraph &p = *graphs[(size_t)gi - 1], &q = *graphs[(size_t)gi];
+    direct = q.owner == p.owner && q.rp == p.rp + p.n + 1 && q.ci == p.ci + 2 * p.m;
+  }
   if (sb->busy) GS_TRY(cudaEventSynchronize(sb->busy), "small buffers in use");
   else GS_TRY(cudaEventCreateWithFlags(&sb->busy, cudaEventDisableTiming), "small event");
   {
-    size_t cr = sb->cap_rows, cn = sb->cap_nnz, cg = sb->cap_g;
-    GS_TRY(grow_pair(&sb->d_rp, &sb->h_rp, &cr, rows), "small buffers");
-    GS_TRY(grow_pair(&sb->d_ci, &sb->h_ci, &cn, nnz), "small buffers");
+    size_t cg = sb->cap_g;
+    GS_TRY(grow_pair<int32_t>(&sb->d_rp, nullptr, &sb->cap_rows, rows), "small buffers");
+    GS_TRY(grow_pair<int32_t>(&sb->d_ci, nullptr, &sb->cap_nnz, nnz), "small buffers");
+    if (!direct) {
+      GS_TRY(grow_pair<int32_t>(nullptr, &sb->h_rp, &sb->cap_hrows, rows), "small buffers");
+      GS_TRY(grow_pair<int32_t>(nullptr, &sb->h_ci, &sb->cap_hnnz, nnz), "small buffers");
+    }
     if ((size_t)G + 1 > sb->cap_g || !sb->d_voff) {
       size_t c1 = 0;
       const size_t need = (size_t)G + 1;
@@ -486,8 +532,6 @@ gc_status run_small(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
       if (!sb->d_misc) GS_TRY(cudaMalloc(&sb->d_misc, sizeof(int32_t) * (kSmallClasses + 1)), "small buffers");
       cg = c1 / 34;
     }
-    sb->cap_rows = cr;
-    sb->cap_nnz = cn;
     sb->cap_g = cg;
   }
   int32_t class_off[kSmallClasses + 1] = {0};
@@ -516,31 +560,28 @@ gc_status run_small(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
     sb->h_gn[gi] = graphs[gi]->n;
     sb->h_gm[gi] = graphs[gi]->m;
   }
-  {  // CSR packed on the host cores, each thread the graphs whose entries start in its share
-    const unsigned hw = std::thread::hardware_concurrency();
-    const int nt = eoff[G] < (1 << 22) ? 1 : (int)std::min<unsigned>(hw ? hw : 1, 32);
-    auto pack = [&](int t) {
+  if (!direct) {  // CSR packed on the host cores, each thread the graphs whose entries start in its share
+    const int nt = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), eoff[G] >> 16));
+    host_run(nt, [&](int t) {
       const int64_t e0 = eoff[G] * t / nt, e1 = eoff[G] * (t + 1) / nt;
-      int32_t gi = (int32_t)(std::lower_bound(eoff.begin(), eoff.begin() + G, e0) - eoff.begin());
+      int32_t gi = t == 0 ? 0 : (int32_t)(std::lower_bound(eoff.begin(), eoff.begin() + G, e0) - eoff.begin());
       for (; gi < G && (eoff[gi] < e1 || t == nt - 1); ++gi) {
         std::memcpy(sb->h_rp + voff[gi], graphs[gi]->rp, sizeof(int32_t) * (graphs[gi]->n + 1));
         if (graphs[gi]->m > 0)
           std::memcpy(sb->h_ci + eoff[gi], graphs[gi]->ci, sizeof(int32_t) * 2 * graphs[gi]->m);
       }
-    };
-    std::vector<std::thread> th;
-    for (int t = 1; t < nt; ++t) th.emplace_back(pack, t);
-    pack(0);
-    for (auto& x : th) x.join();
+    });
   }
+  const int32_t* src_rp = direct ? graphs[0]->rp : sb->h_rp;
+  const int32_t* src_ci = direct ? graphs[0]->ci : sb->h_ci;
   const bool graph_mode = cfg.use_graph != 0;
   // the sequence; returns the first failure (for a capture, the capture is
   // ended by the caller)
   auto issue = [&]() -> cudaError_t {
     cudaError_t r = cudaSuccess;
     const size_t b4 = sizeof(int32_t), b8 = sizeof(int64_t);
-    r = cudaMemcpyAsync(sb->d_rp, sb->h_rp, b4 * rows, cudaMemcpyHostToDevice, s);
-    if (r == cudaSuccess && eoff[G] > 0) r = cudaMemcpyAsync(sb->d_ci, sb->h_ci, b4 * (size_t)eoff[G], cudaMemcpyHostToDevice, s);
+    r = cudaMemcpyAsync(sb->d_rp, src_rp, b4 * rows, cudaMemcpyHostToDevice, s);
+    if (r == cudaSuccess && eoff[G] > 0) r = cudaMemcpyAsync(sb->d_ci, src_ci, b4 * (size_t)eoff[G], cudaMemcpyHostToDevice, s);
     if (r == cudaSuccess) r = cudaMemcpyAsync(sb->d_voff, sb->h_voff, b8 * (G + 1), cudaMemcpyHostToDevice, s);
     if (r == cudaSuccess) r = cudaMemcpyAsync(sb->d_eoff, sb->h_eoff, b8 * (G + 1), cudaMemcpyHostToDevice, s);
     if (r == cudaSuccess) r = cudaMemcpyAsync(sb->d_gn, sb->h_gn, b4 * G, cudaMemcpyHostToDevice, s);
@@ -624,12 +665,6 @@ void run_launch(gc_batch b, std::vector<PendingGraph>& graphs, cudaStream_t s, L
   gc_status st = GC_OK;
   L->h_status[0] = 0;
   L->h_status[1] = 0;
-  for (auto& ev : L->ev)
-    if (cudaEventCreate(&ev) != cudaSuccess) {
-      L->launch_status = cuda_fail(cudaGetLastError(), "batch event");
-      L->error = gc_last_error();
-      return;
-    }
   if (!small.empty()) st = run_small(small, s, L, L->h_x, &b->small[L->stream_slot], cfg);
   if (st == GC_OK && !large.empty()) {
     cudaEventRecord(L->ev[kEvUnion0], s);
@@ -645,6 +680,7 @@ void run_launch(gc_batch b, std::vector<PendingGraph>& graphs, cudaStream_t s, L
     L->timed_union = st == GC_OK;
   }
   L->launch_status = st;
+  if (st != GC_OK) cudaStreamSynchronize(s);  // copies already queued read the launch's host blocks
   if (st == GC_OK) {
     cudaError_t e = cudaEventRecord(L->done, s);
     if (e != cudaSuccess) {
@@ -652,6 +688,34 @@ void run_launch(gc_batch b, std::vector<PendingGraph>& graphs, cudaStream_t s, L
       L->error = gc_last_error();
     }
   }
+}
+
+void free_launch(Launch* L) {
+  if (L->h_x) cudaFreeHost(L->h_x);
+  if (L->h_status) cudaFreeHost(L->h_status);
+  if (L->done) cudaEventDestroy(L->done);
+  for (auto& ev : L->ev)
+    if (ev) cudaEventDestroy(ev);
+  delete L;
+}
+
+// Events and pinned results of a launch of G graphs (a spare launch keeps its
+// own).
+cudaError_t init_launch(Launch* L, size_t G) {
+  cudaError_t e = cudaSuccess;
+  if (G > L->cap_x) {
+    if (L->h_x) cudaFreeHost(L->h_x);
+    L->h_x = nullptr;
+    L->cap_x = 0;
+    const size_t want = G + G / 4 + 16;
+    e = cudaMallocHost(&L->h_x, sizeof(unsigned long long) * 34 * want);
+    if (e == cudaSuccess) L->cap_x = want;
+  }
+  if (e == cudaSuccess && !L->h_status) e = cudaMallocHost(&L->h_status, 2 * sizeof(int32_t));
+  if (e == cudaSuccess && !L->done) e = cudaEventCreateWithFlags(&L->done, cudaEventDisableTiming);
+  for (auto& ev : L->ev)
+    if (e == cudaSuccess && !ev) e = cudaEventCreate(&ev);
+  return e;
 }
 
 // Must hold b->mu.
@@ -682,25 +746,27 @@ void retire_locked(gc_batch b) {
       b->last_stats[kSmallClasses + 2] = L->replayed ? 1.0 : 0.0;
       cudaGetLastError();
     }
-    for (size_t k = 0; k < L->tickets.size(); ++k) {
-      Result r;
-      if (L->launch_status == GC_OK) {
-        std::memcpy(r.x, L->h_x + 34 * (size_t)L->slot[k], sizeof(r.x));
-        const int32_t dst = L->h_status[0] | L->h_status[1];
-        r.status = dst == 0 ? GC_OK : GC_ERR_CUDA;
-      } else {
-        std::memset(r.x, 0, sizeof(r.x));
-        r.status = L->launch_status;
+    std::shared_ptr<Results> out;
+    gc_status status = L->launch_status;
+    if (status == GC_OK && (L->h_status[0] | L->h_status[1])) status = GC_ERR_CUDA;
+    if (status == GC_OK) {
+      try {
+        out = std::make_shared<Results>(L->h_x, L->h_x + 34 * L->tickets.size());
+      } catch (...) {
+        status = GC_ERR_NOMEM;
       }
-      b->done[L->tickets[k]] = r;
+    }
+    for (size_t k = 0; k < L->tickets.size(); ++k) {
+      Ticket* t = b->find(L->tickets[k]);  // live until polled
+      t->state = Ticket::kDone;
+      t->status = status;
+      t->slot = L->slot.size() > k ? L->slot[k] : 0;
+      t->out = out;
     }
     b->in_use -= L->bytes;
-    cudaFreeHost(L->h_x);
-    cudaFreeHost(L->h_status);
-    cudaEventDestroy(L->done);
-    for (auto& ev : L->ev)
-      if (ev) cudaEventDestroy(ev);
-    delete L;
+    L->owners.clear();
+    if (b->spare.size() < kMaxSpare) b->spare.push_back(L);
+    else free_launch(L);
     b->inflight.erase(b->inflight.begin() + i);
     b->cv.notify_all();
   }
@@ -710,13 +776,22 @@ void retire_locked(gc_batch b) {
 // Called without the lock; returns false if nothing was pending.
 bool launch_pending(gc_batch b) {
   std::vector<PendingGraph> take;
-  Launch* L = new Launch();
+  Launch* L = nullptr;
   {
     std::lock_guard<std::mutex> lk(b->mu);
-    if (b->pending.empty()) {
-      delete L;
-      return false;
+    if (b->pending.empty()) return false;
+    if (!b->spare.empty()) {
+      L = b->spare.back();
+      b->spare.pop_back();
+    } else {
+      L = new Launch();
     }
+    L->tickets.clear();
+    L->slot.clear();
+    L->bytes = 0;
+    L->timed_classes = L->timed_small = L->timed_union = L->replayed = false;
+    L->launch_status = GC_OK;
+    L->error.clear();
     int64_t nnz = 0, nv = 0;
     while (!b->pending.empty()) {
       PendingGraph& pg = b->pending.front();
@@ -725,6 +800,7 @@ bool launch_pending(gc_batch b) {
       nv += pg.n;
       L->tickets.push_back(pg.ticket);
       L->bytes += pg.bytes;
+      if (pg.owner && (L->owners.empty() || L->owners.back() != pg.owner)) L->owners.push_back(pg.owner);
       take.push_back(std::move(pg));
       b->pending.pop_front();
     }
@@ -746,10 +822,8 @@ bool launch_pending(gc_batch b) {
     L->stream = b->streams[slot];
   }
   cudaSetDevice(b->device);
-  cudaError_t e1 = cudaMallocHost(&L->h_x, sizeof(unsigned long long) * 34 * take.size());
-  cudaError_t e2 = cudaMallocHost(&L->h_status, 2 * sizeof(int32_t));  // small graphs, union
-  cudaError_t e3 = cudaEventCreateWithFlags(&L->done, cudaEventDisableTiming);
-  if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
+  if (init_launch(L, take.size()) != cudaSuccess) {
+    cudaGetLastError();
     L->launch_status = GC_ERR_NOMEM;
   } else {
     run_launch(b, take, L->stream, L);
@@ -773,7 +847,22 @@ void dispatcher_main(gc_batch b) {
       lk.lock();
       continue;
     }
-    b->cv.wait_for(lk, std::chrono::microseconds(100));
+    // woken by a submission; launches in flight are looked at now and then
+    if (b->inflight.empty()) b->cv.wait_for(lk, std::chrono::milliseconds(1));
+    else b->cv.wait_for(lk, std::chrono::microseconds(20));
+  }
+}
+
+// One turn of a poll's wait, with b->mu held by lk: the first turns only give
+// way to other threads (a small launch takes a fraction of a millisecond), the
+// later ones sleep.
+void poll_wait(gc_batch b, std::unique_lock<std::mutex>* lk, std::chrono::steady_clock::time_point began) {
+  if (std::chrono::steady_clock::now() - began < std::chrono::microseconds(500)) {
+    lk->unlock();
+    std::this_thread::yield();
+    lk->lock();
+  } else {
+    b->cv.wait_for(*lk, std::chrono::microseconds(50));
   }
 }
 
@@ -872,26 +961,37 @@ gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const i
   pg.n = n;
   pg.m = m;
   pg.bytes = bytes;
+  {  // refused before the copy is made, where it already shows
+    std::lock_guard<std::mutex> lk(b->mu);
+    if (b->in_use + bytes > b->budget) {
+      set_error("device-memory budget is full");
+      return GC_ERR_BUSY;
+    }
+  }
   try {
-    pg.owner = std::shared_ptr<int32_t>(new int32_t[(size_t)n + 1 + 2 * (size_t)m], std::default_delete<int32_t[]>());
+    pg.owner = host_block(b->host, (size_t)n + 1 + 2 * (size_t)m);
+    int32_t* own = pg.owner->p;
+    pg.rp = own;
+    pg.ci = own + n + 1;
+    std::memcpy(own, row_ptr, sizeof(int32_t) * ((size_t)n + 1));
+    const int nt = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), 2 * m >> 18));
+    host_run(nt, [&](int t) {
+      const size_t e0 = 2 * (size_t)m * (size_t)t / (size_t)nt, e1 = 2 * (size_t)m * ((size_t)t + 1) / (size_t)nt;
+      if (e1 > e0) std::memcpy(own + n + 1 + e0, col_idx + e0, sizeof(int32_t) * (e1 - e0));
+    });
   } catch (...) {
     set_error("host allocation failed");
     return GC_ERR_NOMEM;
   }
-  std::memcpy(pg.owner.get(), row_ptr, sizeof(int32_t) * ((size_t)n + 1));
-  if (m > 0) std::memcpy(pg.owner.get() + n + 1, col_idx, sizeof(int32_t) * 2 * (size_t)m);
-  pg.rp = pg.owner.get();
-  pg.ci = pg.owner.get() + n + 1;
   {
     std::lock_guard<std::mutex> lk(b->mu);
     if (b->in_use + bytes > b->budget) {
       set_error("device-memory budget is full");
       return GC_ERR_BUSY;
     }
-    pg.ticket = b->next_ticket++;
+    pg.ticket = b->add_ticket();
     *ticket_out = pg.ticket;
     b->in_use += bytes;
-    b->live.insert(pg.ticket);
     b->pending.push_back(std::move(pg));
   }
   b->cv.notify_all();
@@ -918,26 +1018,25 @@ gc_status gc_batch_submit_many(gc_batch b, int64_t G, const int32_t* nvert, cons
     own_v[g + 1] = own_v[g] + n + 1;
     own_e[g + 1] = own_e[g] + (eoff[g + 1] - eoff[g]);
   }
-  std::shared_ptr<int32_t> owner;
+  std::shared_ptr<HostBlock> owner;
   try {
-    owner = host_buffer(b->host, (size_t)(own_v[G] + own_e[G]));
+    owner = host_block(b->host, (size_t)(own_v[G] + own_e[G]));
   } catch (...) {
     set_error("host allocation failed");
     return GC_ERR_NOMEM;
   }
-  int32_t* own_rp = owner.get();
-  int32_t* own_ci = owner.get() + own_v[G];
+  int32_t* own_rp = owner->p;
+  int32_t* own_ci = owner->p + own_v[G];
   std::vector<PendingGraph> pgs((size_t)G);
-  unsigned hw = std::thread::hardware_concurrency();
-  const int nt = (int)std::min<int64_t>(std::max(1u, std::min(hw, 32u)), G);
+  // shares of about equal entries, at least 2^14 each, four to a thread
+  const int nt = (int)std::max<int64_t>(1, std::min<int64_t>({4 * (int64_t)host_threads(), G, own_e[G] >> 14}));
   std::vector<gc_status> res(nt, GC_OK);
   std::vector<std::string> msg(nt);
   auto work = [&](int t) {  // the graphs whose entries start in this thread's share
     std::vector<int32_t> fill;  // symmetry-walk scratch of this thread
     const int64_t e0 = own_e[G] * t / nt, e1 = own_e[G] * (t + 1) / nt;
-    int64_t g = std::lower_bound(own_e.begin(), own_e.begin() + G, e0) - own_e.begin();
+    int64_t g = t == 0 ? 0 : std::lower_bound(own_e.begin(), own_e.begin() + G, e0) - own_e.begin();
     for (; g < G && (own_e[g] < e1 || t == nt - 1); ++g) {
-      if (t > 0 && own_e[g] < e0) continue;
       const int32_t n = nvert[g];
       const int32_t* rp = row_ptr + voff[g];
       const int32_t* ci = col_idx ? col_idx + eoff[g] : nullptr;
@@ -963,10 +1062,12 @@ gc_status gc_batch_submit_many(gc_batch b, int64_t G, const int32_t* nvert, cons
       pg.owner = owner;
     }
   };
-  std::vector<std::thread> th;
-  for (int t = 1; t < nt; ++t) th.emplace_back(work, t);
-  work(0);
-  for (auto& x : th) x.join();
+  try {
+    host_run(nt, work);
+  } catch (...) {
+    set_error("host allocation failed");
+    return GC_ERR_NOMEM;
+  }
   for (int t = 0; t < nt; ++t)
     if (res[t] != GC_OK) {
       set_error(msg[t]);
@@ -986,9 +1087,8 @@ gc_status gc_batch_submit_many(gc_batch b, int64_t G, const int32_t* nvert, cons
     }
     b->in_use += bytes;
     for (int64_t g = 0; g < G; ++g) {
-      pgs[(size_t)g].ticket = b->next_ticket++;
+      pgs[(size_t)g].ticket = b->add_ticket();
       tickets_out[g] = pgs[(size_t)g].ticket;
-      b->live.insert(pgs[(size_t)g].ticket);
       b->pending.push_back(std::move(pgs[(size_t)g]));
     }
   }
@@ -1010,28 +1110,30 @@ gc_status gc_batch_flush(gc_batch b) {
 gc_status gc_batch_poll(gc_batch b, uint64_t ticket, uint64_t* global_out, uint64_t* global_hi,
                         int32_t timeout_us) {
   if (!b || !global_out) { set_error("NULL argument"); return GC_ERR_ARG; }
-  const auto deadline = std::chrono::steady_clock::now() + std::chrono::microseconds(timeout_us > 0 ? timeout_us : 0);
+  const auto began = std::chrono::steady_clock::now();
+  const auto deadline = began + std::chrono::microseconds(timeout_us > 0 ? timeout_us : 0);
   std::unique_lock<std::mutex> lk(b->mu);
-  if (!b->live.count(ticket)) {
-    set_error("unknown or retired ticket");
-    return GC_ERR_ARG;
-  }
   for (;;) {
+    Ticket* t = b->find(ticket);
+    if (!t) {
+      set_error("unknown or retired ticket");
+      return GC_ERR_ARG;
+    }
     if (b->flags & GC_BATCH_MANUAL) retire_locked(b);
-    auto it = b->done.find(ticket);
-    if (it != b->done.end()) {
-      Result r = it->second;
-      b->done.erase(it);
-      b->live.erase(ticket);
+    if (t->state == Ticket::kDone) {
+      const Ticket r = std::move(*t);
+      *t = Ticket();
+      b->drop_retired();
       if (r.status != GC_OK) {
         set_error("batch launch failed");
         return r.status;
       }
+      const uint64_t* x = r.out->data() + 34 * (size_t)r.slot;
       bool need_hi = false;
       for (int i = 0; i < 17; ++i) {
-        global_out[i] = r.x[2 * i];
-        if (global_hi) global_hi[i] = r.x[2 * i + 1];
-        if (r.x[2 * i + 1]) need_hi = true;
+        global_out[i] = x[2 * i];
+        if (global_hi) global_hi[i] = x[2 * i + 1];
+        if (x[2 * i + 1]) need_hi = true;
       }
       if (need_hi && !global_hi) {
         set_error("a global count exceeds 64 bits and global_hi is NULL");
@@ -1041,46 +1143,63 @@ gc_status gc_batch_poll(gc_batch b, uint64_t ticket, uint64_t* global_out, uint6
     }
     if (timeout_us == 0) return GC_PENDING;
     if (timeout_us > 0 && std::chrono::steady_clock::now() >= deadline) return GC_PENDING;
-    b->cv.wait_for(lk, std::chrono::microseconds(50));
+    poll_wait(b, &lk, began);
   }
 }
 
 gc_status gc_batch_poll_many(gc_batch b, int64_t G, const uint64_t* tickets, uint64_t* global_out,
                              uint64_t* global_hi, int32_t timeout_us) {
   if (!b || G < 0 || (G > 0 && (!tickets || !global_out))) { set_error("bad arguments"); return GC_ERR_ARG; }
-  const auto deadline = std::chrono::steady_clock::now() + std::chrono::microseconds(timeout_us > 0 ? timeout_us : 0);
+  const auto began = std::chrono::steady_clock::now();
+  const auto deadline = began + std::chrono::microseconds(timeout_us > 0 ? timeout_us : 0);
   std::unique_lock<std::mutex> lk(b->mu);
   for (int64_t i = 0; i < G; ++i)
-    if (!b->live.count(tickets[i])) {
+    if (!b->find(tickets[i])) {
       set_error("ticket " + std::to_string(i) + " is unknown or retired");
       return GC_ERR_ARG;
     }
   int64_t ready = 0;  // tickets[0 .. ready) are known to be done
   for (;;) {
     if (b->flags & GC_BATCH_MANUAL) retire_locked(b);
-    while (ready < G && b->done.count(tickets[ready])) ++ready;
+    for (; ready < G; ++ready) {
+      const Ticket* t = b->find(tickets[ready]);
+      if (!t) {  // retired by another thread's poll meanwhile
+        set_error("ticket " + std::to_string(ready) + " is unknown or retired");
+        return GC_ERR_ARG;
+      }
+      if (t->state != Ticket::kDone) break;
+    }
     if (ready == G) break;
     if (timeout_us == 0) return GC_PENDING;
     if (timeout_us > 0 && std::chrono::steady_clock::now() >= deadline) return GC_PENDING;
-    b->cv.wait_for(lk, std::chrono::microseconds(50));
+    poll_wait(b, &lk, began);
   }
   gc_status first = GC_OK;
   bool need_hi = false;
+  static const uint64_t kZero[34] = {0};
   for (int64_t i = 0; i < G; ++i) {
-    auto it = b->done.find(tickets[i]);
-    const Result r = it->second;
-    b->done.erase(it);
-    b->live.erase(tickets[i]);
-    if (r.status != GC_OK && first == GC_OK) {
-      first = r.status;
+    const Ticket* t = b->find(tickets[i]);
+    if (!t) {  // retired while the lock was let go
+      if (first == GC_OK) {
+        first = GC_ERR_ARG;
+        set_error("ticket " + std::to_string(i) + " is unknown or retired");
+      }
+      continue;
+    }
+    if (t->status != GC_OK && first == GC_OK) {
+      first = t->status;
       set_error("the launch of ticket " + std::to_string(i) + " failed");
     }
+    const uint64_t* x = t->out ? t->out->data() + 34 * (size_t)t->slot : kZero;
     for (int k = 0; k < 17; ++k) {
-      global_out[17 * i + k] = r.x[2 * k];
-      if (global_hi) global_hi[17 * i + k] = r.x[2 * k + 1];
-      if (r.x[2 * k + 1]) need_hi = true;
+      global_out[17 * i + k] = x[2 * k];
+      if (global_hi) global_hi[17 * i + k] = x[2 * k + 1];
+      if (x[2 * k + 1]) need_hi = true;
     }
   }
+  for (int64_t i = 0; i < G; ++i)
+    if (Ticket* t = b->find(tickets[i])) *t = Ticket();
+  b->drop_retired();
   if (first != GC_OK) return first;
   if (need_hi && !global_hi) {
     set_error("a global count exceeds 64 bits and global_hi is NULL");
@@ -1104,6 +1223,7 @@ gc_status gc_batch_destroy(gc_batch b) {
   }
   for (auto& sb : b->small) free_small_bufs(&sb);
   for (auto* f : b->forks) fork_release(f);
+  for (Launch* L : b->spare) free_launch(L);
   for (auto& s : b->streams) cudaStreamDestroy(s);
   delete b;
   return GC_OK;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <memory>
 #include <string>
 #include <vector>
@@ -296,6 +297,13 @@ inline cudaError_t pool_alloc(T** p, size_t bytes, cudaStream_t s) {
   if (!pool) return cudaErrorMemoryAllocation;
   return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, pool, s);
 }
+
+// ---- host threads (gc_host.cu) ----
+int host_threads();  // the cores of the host, at most 32
+// f(0) .. f(n - 1) on the library's host threads and the calling thread; the
+// calls of one host_run start in order. The first exception is thrown again
+// here, after all have ended. Any thread may call it.
+void host_run(int n, const std::function<void(int)>& f);
 
 // ---- relabelling P1: the host half (gc_api.cu) ----
 // Host arrays left uninitialised on allocation (every element is written

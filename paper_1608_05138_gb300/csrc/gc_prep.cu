@@ -220,9 +220,11 @@ __global__ void k_cwork(int32_t n_units, const int32_t* __restrict__ units, cons
   }
 }
 
-// DevGraph::hpos of the rows of one graph: thread per (row, bound).
-__global__ void k_hub_pos(HubGeom ge, const HubSeg* __restrict__ seg, const int32_t* __restrict__ rp,
-                          const int32_t* __restrict__ ci, int32_t* __restrict__ pos) {
+// DevGraph::hpos: a row of CTAs per graph, thread per (row, bound).
+__global__ void k_hub_pos(const HubGeom* __restrict__ geom, const HubSeg* __restrict__ seg,
+                          const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, int32_t* __restrict__ pos) {
+  const HubGeom ge = geom[blockIdx.y];
+  if (ge.nseg == 0) return;
   const int64_t per = ge.nseg + 1, total = (int64_t)(ge.end - ge.xmin) * per;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int32_t x = ge.xmin + (int32_t)(t / per), k = (int32_t)(t % per);
@@ -609,10 +611,11 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
     if (e == cudaSuccess) e = cudaMemcpyAsync(p->hgeom, geom.data(), gb, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && sb) e = cudaMemcpyAsync(p->hseg, segs.data(), sb, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = pool_alloc(&p->hpos, sizeof(int32_t) * (size_t)(n_pos > 0 ? n_pos : 1), s);
-    for (const HubGeom& ge : geom) {
-      const int64_t work = (int64_t)(ge.end - ge.xmin) * (ge.nseg + 1);
-      if (e != cudaSuccess || ge.nseg == 0 || work == 0) continue;
-      k_hub_pos<<<grid_for(work, 256), 256, 0, s>>>(ge, p->hseg, d_rp, d_ci, p->hpos);
+    int64_t widest = 0;
+    for (const HubGeom& ge : geom) widest = std::max(widest, (int64_t)(ge.end - ge.xmin) * (ge.nseg + 1));
+    for (size_t g0 = 0; g0 < geom.size() && widest > 0 && e == cudaSuccess; g0 += 32768) {
+      const dim3 grid((unsigned)std::min(grid_for(widest, 256), 4096), (unsigned)std::min<size_t>(32768, geom.size() - g0));
+      k_hub_pos<<<grid, 256, 0, s>>>(p->hgeom + g0, p->hseg, d_rp, d_ci, p->hpos);
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_fail(e, "hub layout");

@@ -44,7 +44,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <utility>
+#include <cmath>
 #include <vector>
 
 #include "gc_internal.h"
@@ -437,20 +437,24 @@ void small_units(const std::vector<int32_t>& n, const std::vector<int64_t>& m, s
   // again. 48 graphs of n in [20, 500]: 5.9 ms uncut.
   constexpr double kLeast = 25000;
   const double target = std::max(kLeast, total / (8.0 * (count_grid_size() / kCtasPerSm)));
-  std::vector<std::pair<double, int2>> per_class[kSmallClasses];
+  // lists by class and by cost, eight bins to a factor of two, largest first
+  constexpr int kBins = 512;
+  std::vector<int32_t> at((size_t)kSmallClasses * kBins + 1, 0);
+  std::vector<int32_t> bin((size_t)G), parts((size_t)G);
   for (int32_t g = 0; g < G; ++g) {
     const double c = cost[(size_t)g];
-    const int parts = c > 2 * target ? (int)std::min(32.0, c / target) : 1;
-    for (int p = 0; p < parts; ++p)
-      per_class[small_class_of(n[(size_t)g])].push_back({c / parts, make_int2(g, p | (parts << 16))});
+    const int k = c > 2 * target ? (int)std::min(32.0, c / target) : 1;
+    const int lg = (int)(8 * std::log2(std::max(1.0, c / k)));
+    parts[(size_t)g] = k;
+    bin[(size_t)g] = small_class_of(n[(size_t)g]) * kBins + kBins - 1 - std::min(lg, kBins - 1);
+    at[(size_t)bin[(size_t)g] + 1] += k;
   }
-  units->clear();
-  for (int c = 0; c < kSmallClasses; ++c) {
-    std::sort(per_class[c].begin(), per_class[c].end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-    class_off[c] = (int32_t)units->size();
-    for (auto& u : per_class[c]) units->push_back(u.second);
-  }
-  class_off[kSmallClasses] = (int32_t)units->size();
+  for (size_t i = 1; i < at.size(); ++i) at[i] += at[i - 1];
+  for (int c = 0; c <= kSmallClasses; ++c) class_off[c] = at[(size_t)c * kBins];
+  units->resize((size_t)at.back());
+  for (int32_t g = 0; g < G; ++g)
+    for (int p = 0; p < parts[(size_t)g]; ++p)
+      (*units)[(size_t)at[(size_t)bin[(size_t)g]]++] = make_int2(g, p | (parts[(size_t)g] << 16));
 }
 
 gc_status small_graphs_setup() {

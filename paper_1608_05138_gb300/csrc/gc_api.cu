@@ -106,10 +106,6 @@ ForkSet* fork_acquire() {
     return nullptr;
   }
   f->device = dev;
-  for (auto& t : f->stream)
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);
-  for (auto& d : f->done)
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&d, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f->start, cudaEventDisableTiming);
   for (int k = 0; k < kNumPhases; ++k) {
     if (e == cudaSuccess) e = cudaEventCreate(&f->begin[k]);
@@ -126,7 +122,8 @@ ForkSet* fork_acquire() {
 
 void fork_drain(ForkSet* f) {
   if (!f) return;
-  for (auto& t : f->stream) cudaStreamSynchronize(t);
+  for (auto& t : f->stream)
+    if (t) cudaStreamSynchronize(t);
   cudaGetLastError();
 }
 

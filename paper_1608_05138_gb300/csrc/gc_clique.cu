@@ -41,6 +41,7 @@
 // listing) plus (#edges of H_a) * k / 32 words.
 #include <cuda_runtime.h>
 
+#include "gc_deal.h"
 #include "gc_internal.h"
 
 namespace gc {
@@ -512,198 +513,240 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
   }
 }
 
-// Units with k <= 32: one warp per unit, lane i holding member b_i, its
-// row of H_a as a 32-bit mask and the out-slots of the edges found from it
-// (shared memory). Membership of an id in out(a) is a 5-step binary search
-// over the lanes' ids (ascending). Same attribution as k_pass_k.
+// Units with k <= 32: one warp per unit, lane i holding member b_i, the rows of
+// H_a as 32-bit masks and the out-slots of its edges in shared memory.
+// The out-lists of all members are read end to end over the lanes (most have a
+// few entries, so that a window of 32 per member left most lanes idle and
+// waited on memory once per member), and an entry's place in out(a) is a 5-step
+// binary search over the lanes' ids (ascending). Pass K takes an edge of H_a
+// per lane. Both wait on chains of dependent loads, a unit at a time.
+// Chung-Lu 1M: pass T's kernel 1.92 -> 1.63 ms, pass K's 1.37 -> 0.43 ms.
+// Same attribution as k_pass_k.
 constexpr int kWBlock = 256;
 constexpr int kWWarps = kWBlock / 32;
-
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x) {
-  for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-  return x;
-}
 
 template <bool kTri, bool kDeg = false>
 __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a) {
   constexpr int tier = kTier32;
-  __shared__ int32_t s_q[kWWarps][32 * 32];  // out-slot of edge (i, j) found from member i
-  __shared__ uint32_t s_rowf[kWWarps][64];    // rows and found masks rebuilt from pass T's list
+  __shared__ int32_t s_q[kWWarps][kTri ? 32 * 32 : 1];  // pass T: out-slot of the edge (i, j), i < j, of H_a
+  __shared__ uint32_t s_row[kWWarps][kTri ? 32 : 1];    // pass T: bit j of row i: i ~ j, j > i
+  __shared__ uint32_t s_full[kWWarps][32];    // both triangles
+  __shared__ int32_t s_t[kWWarps][32];        // pass K: |T| of (a, b_i); pass T (kDeg): d of b_i
+  __shared__ uint32_t s_v[kWWarps][kTri && !kDeg ? 1 : 4][32];  // per-member sums (see below), 64-bit ones split
+  __shared__ int32_t s_comp[kWWarps][32];
+  __shared__ unsigned long long s_work[3];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t* qs = s_q[warp];
+  uint32_t *row = s_row[warp], *full = s_full[warp];
+  (void)row;
+  (void)qs;
+  if (threadIdx.x < 3) s_work[threadIdx.x] = 0ull;
+  __syncthreads();
   const int32_t u0 = a.ktier_off[tier], u1 = a.ktier_off[tier + 1];
   int32_t* cursor = a.cursor + (kTri ? 10 : 2) + tier;
-  long long w_members = 0, w_scan = 0, w_edges = 0;  // lane 0
-  for (;;) {
-    int32_t ui = 0;
-    if (lane == 0) ui = u0 + atomicAdd(cursor, 1);
-    ui = __shfl_sync(kFull, ui, 0);
-    if (ui >= u1) break;
-    const int32_t av = a.kunits[ui];
-    const int32_t ob = g.out_ptr[av];
-    const int32_t k = g.out_ptr[av + 1] - ob;
+  long long w_members = 0, w_scan = 0, w_edges = 0;  // warp-uniform
+  // units are taken eight at a time when every warp gets many, their
+  // vertices and list bounds loaded together: one unit costs a chain of
+  // dependent loads, and this takes the first three links out of it
+  const int take = u1 - u0 >= 64 * (int)gridDim.x * kWWarps ? 8 : 1;
+  int32_t c0 = 0, cn = 0, at = 0, c_av = 0, c_ob = 0, c_k = 0, c_cnt = 0;
+  long long c_off = 0;
+  for (;; ++at) {
+    if (at == cn) {
+      if (lane == 0) c0 = u0 + atomicAdd(cursor, take);
+      c0 = __shfl_sync(kFull, c0, 0);
+      if (c0 >= u1) break;
+      cn = min(take, u1 - c0);
+      at = 0;
+      if (lane < cn) {
+        c_av = a.kunits[c0 + lane];
+        c_ob = g.out_ptr[c_av];
+        c_k = g.out_ptr[c_av + 1] - c_ob;
+        if (!kTri) {
+          c_cnt = a.tlist ? a.tl_cnt[c0 + lane] : -1;
+          c_off = a.tlist ? a.tl_off[c0 + lane] : 0;
+        }
+      }
+    }
+    const int32_t ui = c0 + at;
+    const int32_t av = __shfl_sync(kFull, c_av, at);
+    const int32_t ob = __shfl_sync(kFull, c_ob, at);
+    const int32_t k = __shfl_sync(kFull, c_k, at);
     if (k > 32) {  // cannot happen: units are binned by k
       if (lane == 0) atomicOr(a.status, (int32_t)kSpillOverflow);
       continue;
     }
-    const int32_t id = lane < k ? g.out_idx[ob + lane] : 0x7fffffff;
-    const int32_t ti = (!kTri && lane < k) ? a.trio[ob + lane] : 0;
-    const int32_t dl = (kDeg && lane < k) ? g.deg[id] : 0;  // kDeg: degree of member b_lane
+    w_members += k;
+    __syncwarp();
+    if (kTri) row[lane] = 0u;
+    full[lane] = 0u;
+    if (!kTri || kDeg)
+      for (int v = 0; v < 4; ++v) s_v[warp][v][lane] = 0u;
+    const int32_t lcnt = kTri ? -1 : __shfl_sync(kFull, c_cnt, at);
+    const int2* lst = a.tlist + (kTri ? 0 : __shfl_sync(kFull, c_off, at));
+    int32_t id = 0x7fffffff;
+    if (kTri || lcnt < 0) id = lane < k ? g.out_idx[ob + lane] : 0x7fffffff;
+    if (!kTri) s_t[warp][lane] = lane < k ? a.trio[ob + lane] : 0;
+    if (kDeg) s_t[warp][lane] = lane < k ? g.deg[id] : 0;
     const int32_t da = kDeg ? g.deg[av] : 0;
-    const int32_t cmax = __shfl_sync(kFull, id, k - 1);
-    unsigned row = 0u, found = 0u;
-    const int32_t lcnt = (!kTri && a.tlist) ? a.tl_cnt[ui] : -1;
-    if (lcnt >= 0) {  // pass K with the edges of H_a kept by pass T
-      uint32_t* rw = s_rowf[warp];
-      rw[lane] = 0u;
-      rw[32 + lane] = 0u;
-      __syncwarp();
-      const int2* lst = a.tlist + a.tl_off[ui];
-      for (int32_t e = lane; e < lcnt; e += 32) {
-        const int2 en = lst[e];
-        const int32_t i = (int32_t)((uint32_t)en.x >> 16), j = en.x & 0xffff;
-        atomicOr(&rw[i], 1u << j);
-        atomicOr(&rw[j], 1u << i);
-        atomicOr(&rw[32 + i], 1u << j);
-        qs[i * 32 + j] = en.y;
+    __syncwarp();
+    // the scan: on_hit(i, j, q) for every edge (i, j) of H_a, q its out-slot
+    auto scan = [&](auto on_hit) {
+      int32_t b = 0, len = 0;
+      if (lane < k) {
+        b = g.out_ptr[id];
+        len = g.out_ptr[id + 1] - b;
       }
-      __syncwarp();
-      row = rw[lane];
-      found = rw[32 + lane];
-      if (lane == 0) w_edges += lcnt;
-    } else {
-    // Phase 1: the edges of H_a.
-    for (int i = 0; i < k; ++i) {
-      const int32_t b = __shfl_sync(kFull, id, i);
-      const int32_t bb = g.out_ptr[b], be = g.out_ptr[b + 1];
-      unsigned hits = 0u;
-      for (int32_t q0 = bb; q0 < be; q0 += 128) {  // four windows of 32 in flight
-        int32_t cw[4];
+      const Deal d = deal_setup(len, s_comp[warp], lane);
+      const int32_t base = b - d.excl;
+      w_scan += d.total;
+      int before = 0;
+      for (int32_t k0 = 0; k0 < d.total; k0 += 128) {  // four windows of loads in flight
+        int32_t q[4], c[4], own[4];
 #pragma unroll
-        for (int w4 = 0; w4 < 4; ++w4) {
-          const int32_t q = q0 + 32 * w4 + lane;
-          cw[w4] = q < be ? g.out_idx[q] : 0x7fffffff;
+        for (int w = 0; w < 4; ++w) {
+          own[w] = deal_owner(d, len, k0 + 32 * w, s_comp[warp], lane, before);
+          const int32_t pos = k0 + 32 * w + lane;
+          const int32_t bw = __shfl_sync(kFull, base, own[w]);
+          q[w] = bw + pos;
+          c[w] = pos < d.total ? g.out_idx[q[w]] : -1;
         }
-        if (lane == 0) w_scan += min(128, be - q0);
-        const bool past = __shfl_sync(kFull, cw[3], 31) > cmax;
 #pragma unroll
-        for (int w4 = 0; w4 < 4; ++w4) {
-          const int32_t q = q0 + 32 * w4 + lane;
-          const int32_t c = cw[w4];
-          int lo = 0;
+        for (int w = 0; w < 4; ++w) {
+          if (k0 + 32 * w >= d.total) break;  // warp-uniform
+          int lo = 0;  // the last member not above c
 #pragma unroll
           for (int step = 16; step; step >>= 1)
-            if (__shfl_sync(kFull, id, lo + step) <= c) lo += step;
-          const int32_t id_lo = __shfl_sync(kFull, id, lo);  // every lane takes part in the shuffle
-          const bool hit = c <= cmax && id_lo == c && lo < k;  // lanes >= k hold padding ids
-          if (hit) {
-            if (kTri) atomicAdd(&a.trio[q], 1);  // edge (b_i, c)
-            if (kDeg) atomicAdd(&a.dsum[q], (unsigned long long)da);  // its third vertex a
-            qs[i * 32 + lo] = q;
-          }
-          hits |= __reduce_or_sync(kFull, hit ? 1u << lo : 0u);
+            if (__shfl_sync(kFull, id, lo + step) <= c[w]) lo += step;
+          const int32_t id_lo = __shfl_sync(kFull, id, lo);
+          if (c[w] >= 0 && id_lo == c[w]) on_hit(own[w], lo, q[w]);  // lanes >= k hold an id no vertex has
         }
-        if (past) break;
       }
-      if (lane == i) {
-        found = hits;
-        row |= hits;
-      }
-      if ((hits >> lane) & 1u) row |= 1u << i;
-      if (lane == 0) w_edges += __popc(hits);
-    }
-    }  // scan
-    if (kTri) {  // edge (a, b_lane): one triangle per edge of H_a at lane
-      if (lane < k && row) atomicAdd(&a.trio[ob + lane], __popc(row));
-      if (kDeg) {  // and the degrees of their third vertices b_i
-        unsigned long long sd = 0;
-        for (int i = 0; i < k; ++i) {
-          const int32_t di = __shfl_sync(kFull, dl, i);
-          if ((row >> i) & 1u) sd += (unsigned long long)di;
+      __syncwarp();
+    };
+    if (kTri) {
+      scan([&](int i, int j, int32_t q) {
+        qs[i * 32 + j] = q;
+        atomicOr(&row[i], 1u << j);
+        atomicOr(&full[i], 1u << j);
+        atomicOr(&full[j], 1u << i);
+        atomicAdd(&a.trio[q], 1);  // edge (b_i, c)
+        if (kDeg) {  // third vertices: a, b_i and c
+          atomicAdd(&a.dsum[q], (unsigned long long)da);
+          add_split(s_v[warp][0], s_v[warp][1], j, (unsigned long long)s_t[warp][i]);
+          add_split(s_v[warp][0], s_v[warp][1], i, (unsigned long long)s_t[warp][j]);
         }
-        if (lane < k && sd) atomicAdd(&a.dsum[ob + lane], sd);
+      });
+      const unsigned found = row[lane];
+      int incl = __popc(found);
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
       }
-      if (lane == 0) w_members += k;
+      const int32_t edges = __shfl_sync(kFull, incl, 31);
+      w_edges += edges;
+      // edge (a, b_lane): one triangle per edge of H_a at lane
+      if (lane < k && full[lane]) {
+        atomicAdd(&a.trio[ob + lane], __popc(full[lane]));
+        if (kDeg) atomicAdd(&a.dsum[ob + lane], read_split(s_v[warp][0], s_v[warp][1], lane));
+      }
       if (a.tlist) {  // hand the edges of H_a on to pass K
-        const int c = __popc(found);
-        int incl = c;
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(kFull, incl, o);
-          if (lane >= o) incl += y;
-        }
-        const int total = __shfl_sync(kFull, incl, 31);
         long long off = -1;
         if (lane == 0) {
-          const unsigned long long o = atomicAdd(a.tlist_fill, (unsigned long long)total);
-          if ((long long)o + total <= a.tlist_cap) off = (long long)o;
+          const unsigned long long o = atomicAdd(a.tlist_fill, (unsigned long long)edges);
+          if ((long long)o + edges <= a.tlist_cap) off = (long long)o;
           a.tl_off[ui] = off < 0 ? 0 : off;
-          a.tl_cnt[ui] = off < 0 ? -1 : total;
+          a.tl_cnt[ui] = off < 0 ? -1 : edges;
         }
         off = __shfl_sync(kFull, off, 0);
-        if (off >= 0) {
-          // entry e of the unit's list, lane per entry: its row r is the
-          // number of rows whose inclusive prefix is <= e, its column the
-          // (e - exclusive prefix of r)-th set bit of found_r
-          for (int32_t e0 = 0; e0 < total; e0 += 32) {  // warp-uniform trip count
-            const int32_t e = e0 + lane;
-            int r = 0;
+        // entry e is in row r, the number of rows whose inclusive prefix is
+        // <= e, at the (e - exclusive prefix of r)-th set bit
+        for (int32_t e0 = 0; off >= 0 && e0 < edges; e0 += 32) {  // warp-uniform trip count
+          const int32_t e = e0 + lane;
+          int r = 0;
 #pragma unroll
-            for (int step = 16; step; step >>= 1)
-              if (__shfl_sync(kFull, incl, r + step - 1) <= e) r += step;
-            const unsigned fr = __shfl_sync(kFull, found, r);
-            const int ir = __shfl_sync(kFull, incl, r);
-            if (e < total) {
-              unsigned f = fr;
-              for (int t = e - (ir - __popc(fr)); t > 0; --t) f &= f - 1;
-              const int j = __ffs(f) - 1;
-              a.tlist[off + e] = make_int2((int32_t)(((uint32_t)r << 16) | (uint32_t)j), qs[r * 32 + j]);
-            }
+          for (int step = 16; step; step >>= 1)
+            if (__shfl_sync(kFull, incl, r + step - 1) <= e) r += step;
+          unsigned f = __shfl_sync(kFull, found, r);
+          const int ir = __shfl_sync(kFull, incl, r);
+          if (e < edges) {
+            for (int t = e - (ir - __popc(f)); t > 0; --t) f &= f - 1;
+            const int j = __ffs(f) - 1;
+            a.tlist[off + e] = make_int2((int32_t)(((uint32_t)r << 16) | (uint32_t)j), qs[r * 32 + j]);
           }
         }
-        __syncwarp();
       }
       continue;
     }
-    __syncwarp();
-    // Phase 2: c_ij and the cross terms of every edge (i, j) of H_a.
-    unsigned long long vx = 0, vc = 0;  // for the edge (a, b_lane)
-    for (int i = 0; i < k; ++i) {
-      const unsigned ri = __shfl_sync(kFull, row, i);
-      const unsigned fi = __shfl_sync(kFull, found, i);
-      const int32_t tI = __shfl_sync(kFull, ti, i);
-      if (fi == 0u) continue;  // warp-uniform
-      unsigned long long cx = 0, cc = 0;
-      if ((fi >> lane) & 1u) {
-        const int32_t q = qs[i * 32 + lane];
-        const int c4 = __popc(ri & row);
-        const int32_t tij = a.trio[q];
-        if (c4) atomicAdd(&a.xc[2 * (size_t)q], (unsigned long long)c4);
-        atomicAdd(&a.xc[2 * (size_t)q + 1], (unsigned long long)(tI + ti - 2));
-        vx += (unsigned long long)c4;
-        vc += (unsigned long long)(tI + tij - 2);
-        cx = (unsigned long long)c4;
-        cc = (unsigned long long)(ti + tij - 2);
+    // Pass K: the rows of H_a, from pass T's list or (not kept) a scan; then
+    // c_ij and the cross terms of every edge (i, j), a lane each, with their
+    // sums per member in shared memory
+    uint32_t *vx = s_v[warp][0], *vc = s_v[warp][1], *vch = s_v[warp][2];
+    auto set_bits = [&](int i, int j, int32_t) {
+      atomicOr(&full[i], 1u << j);
+      atomicOr(&full[j], 1u << i);
+    };
+    auto count_edge = [&](int i, int j, int32_t q) {
+      const uint32_t c4 = (uint32_t)__popc(full[i] & full[j]);
+      const int32_t ti = s_t[warp][i], tj = s_t[warp][j], tij = a.trio[q];
+      if (c4) {
+        atomicAdd(&a.xc[2 * (size_t)q], (unsigned long long)c4);
+        atomicAdd(&vx[i], c4);
+        atomicAdd(&vx[j], c4);
       }
-      cx = warp_sum_u64(cx);
-      cc = warp_sum_u64(cc);
-      if (lane == i) {
-        vx += cx;
-        vc += cc;
+      atomicAdd(&a.xc[2 * (size_t)q + 1], (unsigned long long)(ti + tj - 2));
+      add_split(vc, vch, i, (unsigned long long)(tj + tij - 2));
+      add_split(vc, vch, j, (unsigned long long)(ti + tij - 2));
+    };
+    if (lcnt >= 0) {
+      // a list of at most 64 edges (most) is read once
+      int2 en[2];
+#pragma unroll
+      for (int w = 0; w < 2; ++w) en[w] = 32 * w + lane < lcnt ? lst[32 * w + lane] : make_int2(-1, 0);
+#pragma unroll
+      for (int w = 0; w < 2; ++w)
+        if (en[w].x >= 0) set_bits((int)((uint32_t)en[w].x >> 16), en[w].x & 0xffff, 0);
+      for (int32_t e = 64 + lane; e < lcnt; e += 32) set_bits((int)((uint32_t)lst[e].x >> 16), lst[e].x & 0xffff, 0);
+      __syncwarp();
+#pragma unroll
+      for (int w = 0; w < 2; ++w)
+        if (en[w].x >= 0) count_edge((int)((uint32_t)en[w].x >> 16), en[w].x & 0xffff, en[w].y);
+      for (int32_t e = 64 + lane; e < lcnt; e += 32) {
+        const int2 x = lst[e];
+        count_edge((int)((uint32_t)x.x >> 16), x.x & 0xffff, x.y);
       }
+      w_edges += lcnt;
+    } else {
+      int found = 0;
+      scan([&](int i, int j, int32_t q) {
+        set_bits(i, j, q);
+        ++found;
+      });
+      const long long scanned = w_scan;
+      scan(count_edge);
+      w_scan = scanned;  // counted once
+      w_edges += (long long)__reduce_add_sync(kFull, (unsigned)found);
     }
+    __syncwarp();
     if (lane < k) {
-      if (vx) atomicAdd(&a.xc[2 * (size_t)(ob + lane)], vx >> 1);
-      if (vc) atomicAdd(&a.xc[2 * (size_t)(ob + lane) + 1], vc);
+      const unsigned long long c = read_split(vc, vch, lane);
+      if (vx[lane]) atomicAdd(&a.xc[2 * (size_t)(ob + lane)], (unsigned long long)(vx[lane] >> 1));
+      if (c) atomicAdd(&a.xc[2 * (size_t)(ob + lane) + 1], c);
     }
-    if (lane == 0) w_members += k;
-    __syncwarp();
   }
+  // work counters: one atomic a block each
   if (lane == 0) {
-    if (w_members) atomicAdd(a.work + (kTri ? kWorkTMembers : kWorkKMembers), (unsigned long long)w_members);
-    if (w_scan) atomicAdd(a.work + (kTri ? kWorkTScan : kWorkKScan), (unsigned long long)w_scan);
-    if (w_edges) {
-      atomicAdd(a.work + (kTri ? kWorkTTriangles : kWorkKLocalEdges), (unsigned long long)w_edges);
-      if (!kTri) atomicAdd(a.work + kWorkKWords, (unsigned long long)w_edges);
+    if (w_members) atomicAdd(&s_work[0], (unsigned long long)w_members);
+    if (w_scan) atomicAdd(&s_work[1], (unsigned long long)w_scan);
+    if (w_edges) atomicAdd(&s_work[2], (unsigned long long)w_edges);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (s_work[0]) atomicAdd(a.work + (kTri ? kWorkTMembers : kWorkKMembers), s_work[0]);
+    if (s_work[1]) atomicAdd(a.work + (kTri ? kWorkTScan : kWorkKScan), s_work[1]);
+    if (s_work[2]) {
+      atomicAdd(a.work + (kTri ? kWorkTTriangles : kWorkKLocalEdges), s_work[2]);
+      if (!kTri) atomicAdd(a.work + kWorkKWords, s_work[2]);
     }
   }
 }

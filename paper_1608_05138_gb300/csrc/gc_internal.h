@@ -188,14 +188,20 @@ class Fork {
   }
   cudaStream_t next() {
     if (!f_ || used_ >= count_ || e_ != cudaSuccess) return s_;
-    cudaStream_t t = f_->stream[first_ + used_++];
-    e_ = cudaStreamWaitEvent(t, f_->start, 0);
+    cudaStream_t& t = f_->stream[first_ + used_];
+    cudaEvent_t& d = f_->done[first_ + used_];
+    if (!t) e_ = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);  // on first use, and kept
+    if (!d && e_ == cudaSuccess) e_ = cudaEventCreateWithFlags(&d, cudaEventDisableTiming);
+    if (e_ == cudaSuccess) e_ = cudaStreamWaitEvent(t, f_->start, 0);
+    if (e_ != cudaSuccess) return s_;  // join() reports it
+    ++used_;
     return t;
   }
   cudaError_t join() {
-    for (int k = 0; k < used_ && e_ == cudaSuccess; ++k) {
-      e_ = cudaEventRecord(f_->done[first_ + k], f_->stream[first_ + k]);
-      if (e_ == cudaSuccess) e_ = cudaStreamWaitEvent(s_, f_->done[first_ + k], 0);
+    for (int k = 0; k < used_; ++k) {  // also after a failure: what was forked is waited for
+      cudaError_t e = cudaEventRecord(f_->done[first_ + k], f_->stream[first_ + k]);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(s_, f_->done[first_ + k], 0);
+      if (e_ == cudaSuccess) e_ = e;
     }
     used_ = 0;
     return e_;

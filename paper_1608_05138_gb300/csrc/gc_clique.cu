@@ -100,7 +100,9 @@ struct KLayout {
 // edges (a, b_i), (a, b_j), and nothing else runs. kDeg (with kTri): each
 // triangle also adds the degree of its third vertex to each of its edges,
 // so that a.dsum[e] = sum_{w in T_e} d_w (for the per-edge induced counts).
-template <int kCap, int kThreads, bool kTri, bool kDeg = false>
+// kX7 (without kTri): the 4-cliques alone, from a scan, for graphs whose |T|
+// and cross terms come from k_rows (gc_count.cu): nothing of pass T is needed.
+template <int kCap, int kThreads, bool kTri, bool kDeg = false, bool kX7 = false>
 __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThreads * 64)) k_pass_k(DevGraph g, CountArgs a) {
   constexpr int kW = kThreads / 32;
   constexpr int tier = kCap == 0 ? kTierGlobal : kCap == 1024 ? kTier1024 : kCap == 512 ? kTier512 : kTier256;
@@ -163,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
       ids[i] = g.out_idx[ob + i];
       vx7[i] = 0u;
       vx7h[i] = 0u;
-      if (!kTri || kDeg) {
+      if ((!kTri || kDeg) && !kX7) {
         ta[i] = kTri ? g.deg[ids[i]] : a.trio[ob + i];  // kDeg: the member's degree
         vcr[i] = 0u;
         vcrh[i] = 0u;
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
     }
     const int32_t da = kDeg ? g.deg[av] : 0;
     // pass K with the edges of H_a kept by pass T: no hash, no scan
-    const int32_t lcnt = (!kTri && a.tlist) ? a.tl_cnt[ui] : -1;
+    const int32_t lcnt = (!kTri && !kX7 && a.tlist) ? a.tl_cnt[ui] : -1;
     if (lcnt < 0) {
       for (int32_t i = threadIdx.x; i <= (int32_t)hmask; i += kThreads) hash[i] = 0;
       for (int32_t i = threadIdx.x; i < (1 << fbits) / 32; i += kThreads) filt[i] = 0u;
@@ -402,8 +404,6 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
           const uint32_t* rj = rows + j * S;
           int c4 = 0;
           for (int w = 0; w < W; ++w) c4 += __popc(ri[w] & rj[w]);
-          const int32_t ti = ta[i], tj = ta[j];
-          const int32_t tij = a.trio[q];
           if (c4) {
             atomicAdd(&a.xc[2 * (size_t)q], (unsigned long long)c4);
             if (kCap) {  // at most k^2 per member: no carry for k <= 1024
@@ -414,9 +414,13 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
               add_split(vx7, vx7h, j, (unsigned long long)c4);
             }
           }
-          atomicAdd(&a.xc[2 * (size_t)q + 1], (unsigned long long)(ti + tj - 2));
-          add_split(vcr, vcrh, i, (unsigned long long)(tj + tij - 2));
-          add_split(vcr, vcrh, j, (unsigned long long)(ti + tij - 2));
+          if (!kX7) {
+            const int32_t ti = ta[i], tj = ta[j];
+            const int32_t tij = a.trio[q];
+            atomicAdd(&a.xc[2 * (size_t)q + 1], (unsigned long long)(ti + tj - 2));
+            add_split(vcr, vcrh, i, (unsigned long long)(tj + tij - 2));
+            add_split(vcr, vcrh, j, (unsigned long long)(ti + tij - 2));
+          }
         }
         if (lane == 0) {
           const int32_t cnt = min(32, nhit - e0);
@@ -434,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
       if (i >= k) break;
       const int32_t b = ids[i];
       const int32_t bb = g.out_ptr[b], be = g.out_ptr[b + 1];
-      const int32_t ti = ta[i];
+      const int32_t ti = kX7 ? 0 : ta[i];
       const uint32_t* ri = rows + i * S;
       unsigned long long ax7 = 0, acr = 0;
       uint32_t head = 0, tail = 0;
@@ -442,13 +446,14 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
         const uint32_t* rj = rows + j * S;
         int c4 = 0;
         for (int w = 0; w < W; ++w) c4 += __popc(ri[w] & rj[w]);
+        if (c4) atomicAdd(&a.xc[2 * (size_t)q], (unsigned long long)c4);
+        if (c4) add_split(vx7, vx7h, j, (unsigned long long)c4);
+        ax7 += (unsigned long long)c4;
+        if (kX7) return;
         const int32_t tj = ta[j];
         const int32_t tij = a.trio[q];
-        if (c4) atomicAdd(&a.xc[2 * (size_t)q], (unsigned long long)c4);
         atomicAdd(&a.xc[2 * (size_t)q + 1], (unsigned long long)(ti + tj - 2));
-        if (c4) add_split(vx7, vx7h, j, (unsigned long long)c4);
         add_split(vcr, vcrh, j, (unsigned long long)(ti + tij - 2));
-        ax7 += (unsigned long long)c4;
         acr += (unsigned long long)(tj + tij - 2);
       };
       for (int32_t q0 = bb; q0 < be; q0 += 32) {
@@ -500,7 +505,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
     // Edges (a, b_i): triangles of H_a through i (each counted from both of
     // its edges at i, hence the halving) and the cross terms gathered above.
     for (int32_t i = threadIdx.x; i < k; i += kThreads) {
-      const unsigned long long x = read_split(vx7, vx7h, i), c = read_split(vcr, vcrh, i);
+      const unsigned long long x = read_split(vx7, vx7h, i), c = kX7 ? 0ull : read_split(vcr, vcrh, i);
       if (x) atomicAdd(&a.xc[2 * (size_t)(ob + i)], x >> 1);
       if (c) atomicAdd(&a.xc[2 * (size_t)(ob + i) + 1], c);
     }
@@ -509,6 +514,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
     if (w_members) atomicAdd(a.work + (kTri ? kWorkTMembers : kWorkKMembers), (unsigned long long)w_members);
     if (w_scan) atomicAdd(a.work + (kTri ? kWorkTScan : kWorkKScan), (unsigned long long)w_scan);
     if (w_edges) atomicAdd(a.work + (kTri ? kWorkTTriangles : kWorkKLocalEdges), (unsigned long long)w_edges);
+    if (kX7 && w_edges) atomicAdd(a.work + kWorkTTriangles, (unsigned long long)w_edges);
     if (w_words) atomicAdd(a.work + kWorkKWords, (unsigned long long)w_words);
   }
 }
@@ -525,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
 constexpr int kWBlock = 256;
 constexpr int kWWarps = kWBlock / 32;
 
-template <bool kTri, bool kDeg = false>
+template <bool kTri, bool kDeg = false, bool kX7 = false>
 __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a) {
   constexpr int tier = kTier32;
   __shared__ int32_t s_q[kWWarps][kTri ? 32 * 32 : 1];  // pass T: out-slot of the edge (i, j), i < j, of H_a
@@ -534,6 +540,8 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
   __shared__ int32_t s_t[kWWarps][32];        // pass K: |T| of (a, b_i); pass T (kDeg): d of b_i
   __shared__ uint32_t s_v[kWWarps][kTri && !kDeg ? 1 : 4][32];  // per-member sums (see below), 64-bit ones split
   __shared__ int32_t s_comp[kWWarps][32];
+  __shared__ int2 s_hit[kWWarps][kX7 ? 32 * 31 / 2 : 1];  // kX7: the edges of H_a
+  __shared__ int32_t s_nhit[kWWarps];
   __shared__ unsigned long long s_work[3];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t* qs = s_q[warp];
@@ -563,8 +571,11 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
         c_ob = g.out_ptr[c_av];
         c_k = g.out_ptr[c_av + 1] - c_ob;
         if (!kTri) {
-          c_cnt = a.tlist ? a.tl_cnt[c0 + lane] : -1;
-          c_off = a.tlist ? a.tl_off[c0 + lane] : 0;
+          c_cnt = -1;
+          if (!kX7 && a.tlist) {
+            c_cnt = a.tl_cnt[c0 + lane];
+            c_off = a.tl_off[c0 + lane];
+          }
         }
       }
     }
@@ -586,7 +597,8 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
     const int2* lst = a.tlist + (kTri ? 0 : __shfl_sync(kFull, c_off, at));
     int32_t id = 0x7fffffff;
     if (kTri || lcnt < 0) id = lane < k ? g.out_idx[ob + lane] : 0x7fffffff;
-    if (!kTri) s_t[warp][lane] = lane < k ? a.trio[ob + lane] : 0;
+    if (!kTri && !kX7) s_t[warp][lane] = lane < k ? a.trio[ob + lane] : 0;
+    if (kX7 && lane == 0) s_nhit[warp] = 0;
     if (kDeg) s_t[warp][lane] = lane < k ? g.deg[id] : 0;
     const int32_t da = kDeg ? g.deg[av] : 0;
     __syncwarp();
@@ -688,17 +700,29 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
     };
     auto count_edge = [&](int i, int j, int32_t q) {
       const uint32_t c4 = (uint32_t)__popc(full[i] & full[j]);
-      const int32_t ti = s_t[warp][i], tj = s_t[warp][j], tij = a.trio[q];
       if (c4) {
         atomicAdd(&a.xc[2 * (size_t)q], (unsigned long long)c4);
         atomicAdd(&vx[i], c4);
         atomicAdd(&vx[j], c4);
       }
+      if (kX7) return;
+      const int32_t ti = s_t[warp][i], tj = s_t[warp][j], tij = a.trio[q];
       atomicAdd(&a.xc[2 * (size_t)q + 1], (unsigned long long)(ti + tj - 2));
       add_split(vc, vch, i, (unsigned long long)(tj + tij - 2));
       add_split(vc, vch, j, (unsigned long long)(ti + tij - 2));
     };
-    if (lcnt >= 0) {
+    if (kX7) {
+      scan([&](int i, int j, int32_t q) {
+        set_bits(i, j, q);
+        s_hit[warp][atomicAdd(&s_nhit[warp], 1)] = make_int2((int32_t)(((uint32_t)i << 16) | (uint32_t)j), q);
+      });
+      const int32_t n_hit = s_nhit[warp];
+      for (int32_t e = lane; e < n_hit; e += 32) {
+        const int2 x = s_hit[warp][e];
+        count_edge((int)((uint32_t)x.x >> 16), x.x & 0xffff, x.y);
+      }
+      w_edges += n_hit;
+    } else if (lcnt >= 0) {
       // a list of at most 64 edges (most) is read once
       int2 en[2];
 #pragma unroll
@@ -729,7 +753,7 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
     }
     __syncwarp();
     if (lane < k) {
-      const unsigned long long c = read_split(vc, vch, lane);
+      const unsigned long long c = kX7 ? 0ull : read_split(vc, vch, lane);
       if (vx[lane]) atomicAdd(&a.xc[2 * (size_t)(ob + lane)], (unsigned long long)(vx[lane] >> 1));
       if (c) atomicAdd(&a.xc[2 * (size_t)(ob + lane) + 1], c);
     }
@@ -747,16 +771,17 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
     if (s_work[2]) {
       atomicAdd(a.work + (kTri ? kWorkTTriangles : kWorkKLocalEdges), s_work[2]);
       if (!kTri) atomicAdd(a.work + kWorkKWords, s_work[2]);
+      if (kX7) atomicAdd(a.work + kWorkTTriangles, s_work[2]);
     }
   }
 }
 
-template <int kCap, int kThreads, bool kTri, bool kDeg = false>
+template <int kCap, int kThreads, bool kTri, bool kDeg = false, bool kX7 = false>
 gc_status launch_tier(const DevGraph& g, const CountArgs& a, int tier, Fork* fork, int* launches) {
   const int32_t units = a.ktier_off[tier + 1] - a.ktier_off[tier];
   if (units <= 0) return GC_OK;
   const size_t smem = kCap ? KLayout(kCap, !kTri).total : 0;
-  auto kern = k_pass_k<kCap, kThreads, kTri, kDeg>;
+  auto kern = k_pass_k<kCap, kThreads, kTri, kDeg, kX7>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return cuda_fail(e, "k_pass_k attribute");
   int grid = 0;
@@ -777,7 +802,7 @@ gc_status launch_tier(const DevGraph& g, const CountArgs& a, int tier, Fork* for
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "k_pass_k");
 }
 
-template <bool kTri, bool kDeg = false>
+template <bool kTri, bool kDeg = false, bool kX7 = false>
 gc_status run_tiers(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches) {
   gc_status st;
   if (a.ktier_off[kTierGlobal + 1] > a.ktier_off[kTierGlobal]) {
@@ -785,20 +810,20 @@ gc_status run_tiers(const DevGraph& g, const CountArgs& a, Fork* fork, int* laun
       set_error("internal: pass K global buffers missing");
       return GC_ERR_CUDA;
     }
-    if ((st = launch_tier<0, 1024, kTri, kDeg>(g, a, kTierGlobal, fork, launches)) != GC_OK) return st;
+    if ((st = launch_tier<0, 1024, kTri, kDeg, kX7>(g, a, kTierGlobal, fork, launches)) != GC_OK) return st;
   }
-  if ((st = launch_tier<1024, kTri ? 512 : 1024, kTri, kDeg>(g, a, kTier1024, fork, launches)) != GC_OK) return st;
-  if ((st = launch_tier<512, 512, kTri, kDeg>(g, a, kTier512, fork, launches)) != GC_OK) return st;
-  if ((st = launch_tier<256, 512, kTri, kDeg>(g, a, kTier256, fork, launches)) != GC_OK) return st;
+  if ((st = launch_tier<1024, kTri ? 512 : 1024, kTri, kDeg, kX7>(g, a, kTier1024, fork, launches)) != GC_OK) return st;
+  if ((st = launch_tier<512, 512, kTri, kDeg, kX7>(g, a, kTier512, fork, launches)) != GC_OK) return st;
+  if ((st = launch_tier<256, 512, kTri, kDeg, kX7>(g, a, kTier256, fork, launches)) != GC_OK) return st;
   const int32_t units = a.ktier_off[kTier32 + 1] - a.ktier_off[kTier32];
   if (units > 0) {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pass_k_warp<kTri, kDeg>, kWBlock, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pass_k_warp<kTri, kDeg, kX7>, kWBlock, 0);
     if (e != cudaSuccess) return cuda_fail(e, "k_pass_k_warp occupancy");
     int grid = (per_sm > 0 ? per_sm : 1) * (count_grid_size() / kCtasPerSm);
     const int need = (units + kWWarps - 1) / kWWarps;
     if (grid > need) grid = need;
-    k_pass_k_warp<kTri, kDeg><<<grid, kWBlock, 0, fork->next()>>>(g, a);
+    k_pass_k_warp<kTri, kDeg, kX7><<<grid, kWBlock, 0, fork->next()>>>(g, a);
     ++*launches;
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "k_pass_k_warp");
@@ -812,6 +837,10 @@ size_t kbuf_bytes(int32_t cap) { return cap > 0 ? KLayout(cap).total : 0; }
 
 gc_status run_pass_k(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches) {
   return run_tiers<false>(g, a, fork, launches);
+}
+
+gc_status run_cliques_alone(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches) {
+  return run_tiers<false, false, true>(g, a, fork, launches);
 }
 
 gc_status run_pass_t(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches) {

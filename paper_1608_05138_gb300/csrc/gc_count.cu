@@ -322,6 +322,113 @@ __global__ void __launch_bounds__(kBlock) k_pass_c(DevGraph g, CountArgs a) {
   }
 }
 
+// ---------------- graphs of at most kSmemTableMax vertices: rows of common neighbours ----------------
+// For such a graph (of a union: every graph) a row of counters c(w) = |Gamma(u)
+// and Gamma(w)| over all vertices fits in shared memory, and gives for every
+// edge (u, v)
+//   |T|      = c(v)
+//   P(e)     = sum over w in Gamma(v), w != u, of c(w) - 1
+//   cross(e) = the sums over w in T of c(w) - 1 from u's row and from v's row
+// in two sweeps over the rows of u's neighbours: one adds the counters, one,
+// with a warp per neighbour v, reads them. So neither pass T nor pass C runs,
+// and the 4-cliques (the rest of pass K) need nothing from here: both run side
+// by side, where passes T and C, K, and the finish used to wait for each other
+// (G(1000, 0.3): 480 -> 356 us per count; G(2000, 0.01): 123 -> 103 us). Work is
+// sum d^2 counters, twice: it waits on loads in sparse graphs and on the
+// shared-memory pipe in dense ones. CTA per vertex, largest degree first.
+constexpr int kRowBlock = 256;
+constexpr uint32_t kMark = 0x80000000u;  // w is a neighbour of u
+__global__ void __launch_bounds__(kRowBlock) k_rows(DevGraph g, CountArgs a) {
+  extern __shared__ uint32_t cnt[];  // g.table_n
+  __shared__ unsigned long long s_work;
+  constexpr int kW = kRowBlock / 32;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int32_t u = g.n - 1 - (int32_t)blockIdx.x;
+  const int32_t ub = g.rp[u], d = g.rp[u + 1] - ub;
+  if (d == 0) return;
+  const int32_t gid = g.vgid ? g.vgid[u] : 0;
+  const int32_t base = g.gbase[gid], n = g.gn[gid];
+  for (int32_t i = threadIdx.x; i < n; i += kRowBlock) cnt[i] = 0u;
+  if (threadIdx.x == 0) s_work = 0ull;
+  __syncthreads();
+  // this warp's neighbours: warp, warp + kW, ..., 32 at a time, lane l the l-th
+  for (int32_t i0 = warp; i0 < d; i0 += 32 * kW) {
+    const int32_t i = i0 + kW * lane;
+    int32_t xb = 0, xe = 0;
+    if (i < d) {
+      const int32_t x = g.ci[ub + i];
+      xb = g.rp[x];
+      xe = g.rp[x + 1];
+      atomicOr(&cnt[x - base], kMark);
+    }
+    const int many = min(32, (d - i0 + kW - 1) / kW);
+    for (int j = 0; j < many; ++j) {
+      const int32_t b = __shfl_sync(0xffffffffu, xb, j), e = __shfl_sync(0xffffffffu, xe, j);
+      for (int32_t q0 = b; q0 < e; q0 += 128) {  // four windows of loads in flight
+        int32_t w[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) w[t] = q0 + 32 * t + lane < e ? g.ci[q0 + 32 * t + lane] : -1;
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+          if (w[t] >= 0) atomicAdd(&cnt[w[t] - base], 1u);
+      }
+    }
+  }
+  __syncthreads();
+  long long w_read = 0;
+  for (int32_t i0 = warp; i0 < d; i0 += 32 * kW) {
+    const int32_t i = i0 + kW * lane;
+    int32_t v = 0, vb = 0, ve = 0;
+    if (i < d) {
+      v = g.ci[ub + i];
+      vb = g.rp[v];
+      ve = g.rp[v + 1];
+    }
+    uint32_t my_p = 0, my_a = 0;
+    const int many = min(32, (d - i0 + kW - 1) / kW);
+    for (int j = 0; j < many; ++j) {
+      const int32_t b = __shfl_sync(0xffffffffu, vb, j), e = __shfl_sync(0xffffffffu, ve, j);
+      uint32_t p = 0, c = 0;  // below n^2 each
+      for (int32_t q0 = b; q0 < e; q0 += 128) {
+        int32_t w[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) w[t] = q0 + 32 * t + lane < e ? g.ci[q0 + 32 * t + lane] : u;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const uint32_t x = w[t] == u ? 1u : cnt[w[t] - base];
+          const uint32_t m = (x & ~kMark) - 1u;
+          p += m;
+          if (x & kMark) c += m;
+        }
+      }
+      w_read += e - b;
+      p = __reduce_add_sync(0xffffffffu, p);
+      c = __reduce_add_sync(0xffffffffu, c);
+      if (lane == j) {
+        my_p = p;
+        my_a = c;
+      }
+    }
+    if (i < d) {
+      // out-lists are the ends of the rows: the out-slot of the edge from the
+      // slot of its lower end, p in row x, is out_ptr[x + 1] - (rp[x + 1] - p)
+      const int32_t p = ub + i;
+      const int32_t o = v > u ? g.out_ptr[u + 1] - (ub + d - p)
+                              : g.out_ptr[v + 1] - (ve - min(max(g.rev[p], vb), ve - 1));
+      if ((uint32_t)o < (uint32_t)g.m) {  // out of range only for invalid input
+        if (v < u) {
+          a.trio[o] = (int32_t)(cnt[v - base] & ~kMark);
+          a.P[p] = my_p;
+        }
+        if (my_a) atomicAdd(&a.xc[2 * (size_t)o + 1], (unsigned long long)my_a);
+      }
+    }
+  }
+  if (lane == 0 && w_read) atomicAdd(&s_work, (unsigned long long)w_read);
+  __syncthreads();
+  if (threadIdx.x == 0) atomicAdd(a.work + kWorkCWedge, s_work);
+}
+
 // ---------------- pass C for hub units: the count table in shared memory ----------------
 // The same wedges and attribution as k_pass_c, for the units h whose wedges
 // (a few thousand hubs carry almost all of them on power-law graphs) would
@@ -970,6 +1077,13 @@ gc_status run_pass_c(const DevGraph& g, const CountArgs& a, cudaStream_t s) {
   const bool sm = a.tables == nullptr;
   if (sm) return launch(k_pass_c<true>, smem_bytes(true, g.table_n), g, a, s, "k_pass_c");
   return launch(k_pass_c<false>, smem_bytes(false, g.table_n), g, a, s, "k_pass_c");
+}
+
+gc_status run_rows(const DevGraph& g, const CountArgs& a, cudaStream_t s) {
+  if (g.n == 0) return GC_OK;
+  k_rows<<<g.n, kRowBlock, smem_bytes(true, g.table_n), s>>>(g, a);  // at most 16 KB
+  cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? GC_OK : cuda_fail(e, "k_rows");
 }
 
 gc_status run_pass_c_heavy(const DevGraph& g, const CountArgs& a, cudaStream_t s) {

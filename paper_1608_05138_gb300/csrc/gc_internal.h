@@ -462,6 +462,10 @@ gc_status run_small_graphs(const SmallGraphs& b, const int32_t* class_off, const
 int count_grid_size();
 gc_status run_pass_c(const DevGraph& g, const CountArgs& a, cudaStream_t s);
 gc_status run_pass_c_heavy(const DevGraph& g, const CountArgs& a, cudaStream_t s);
+// |T|, the 4-cycles and the cross terms of every edge, for unions of graphs of
+// at most kSmemTableMax vertices; and the 4-cliques without pass T.
+gc_status run_rows(const DevGraph& g, const CountArgs& a, cudaStream_t s);
+gc_status run_cliques_alone(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches);
 constexpr int kHeavyTab = 53248;  // largest o-range block of the hub kernel of pass C (words of shared memory)
 // Words of the hub kernel's count block (environment GC_HUB_TAB_WORDS, a
 // multiple of 1024 in [4096, kHeavyTab], else kHubTabDefault), read once per

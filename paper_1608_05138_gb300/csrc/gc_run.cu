@@ -183,7 +183,10 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
   // Pass T keeps the edges of the H_a for pass K, in a list sized by the
   // triangles of the previous count of this scratch (or by a first guess);
   // units that do not fit scan their out-lists again in pass K.
-  {
+  // Small graphs take the rows of common neighbours instead of passes T and C
+  // (see k_rows); the per-edge induced counts need pass T's degree sums.
+  const bool rows = g.table_n <= kSmemTableMax && !(induced != nullptr && g.m > 0);
+  if (!rows) {
     const int32_t nku = ku_total(ku);
     const long long want = sc->tlist_want;
     if (want > 0 && want * (long long)sizeof(int2) <= kTListBudget && nku > 0) {
@@ -206,7 +209,7 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
       }
     }
   }
-  a.tlist = sc->tlist_cap > 0 ? sc->tlist : nullptr;
+  a.tlist = !rows && sc->tlist_cap > 0 ? sc->tlist : nullptr;
   a.tlist_cap = sc->tlist_cap;
   a.tlist_fill = sc->tl_fill;
   a.tl_off = sc->tl_off;
@@ -264,7 +267,22 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
     GR_END(ph, s);
     return GC_OK;
   };
-  if (overlap) {
+  if (rows) {
+    GR_BEGIN(kPhasePassT, s);
+    GR_END(kPhasePassT, s);
+    Fork side(s, fs, 0, 1);
+    const cudaStream_t t = side.next();
+    GR_BEGIN(kPhasePassC, t);
+    if ((st = run_rows(g, a, t)) != GC_OK) return st;
+    launches += g.n > 0 ? 1 : 0;
+    GR_END(kPhasePassC, t);
+    GR_BEGIN(kPhasePassK, s);
+    Fork tiers(s, fs, 6, kForkStreams - 6);
+    if ((st = run_cliques_alone(g, a, &tiers, &launches)) != GC_OK) return st;
+    GR_TRY(tiers.join(), "join");
+    GR_END(kPhasePassK, s);
+    GR_TRY(side.join(), "join");
+  } else if (overlap) {
     // pass C on the set's first stream, its kernels forked from there
     Fork side(s, fs, 0, 1);
     const cudaStream_t t = side.next();

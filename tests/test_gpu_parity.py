@@ -281,6 +281,19 @@ def test_batch_four_cliques_of_wide_neighbourhoods(n, k, copies):
     assert all(x == ref for x in X[1:])
 
 
+@pytest.mark.parametrize("make", [
+    lambda: graphgen.er(4096, 0.004, 3),          # the largest graph on rows of common neighbours
+    lambda: graphgen.er(4097, 0.004, 3),          # and the smallest beyond
+    lambda: graphgen.chung_lu(4000, 60000, 2.1, 120000.0, 3999.0, 4),  # hubs next to all others
+    lambda: graphs.complete(300),
+    lambda: graphs.star(4000),
+    lambda: graphs.complete_bipartite(37, 290),
+    lambda: graphgen.er(700, 0.8, 5),
+])
+def test_rows_of_common_neighbours(make):
+    assert_parity(*make())
+
+
 def test_hub_over_a_skewed_o_range():
     # 3M vertices, almost all isolated (the lowest ranks): h has 620 lower
     # neighbours, 600 of them with 150 o each, drawn with weights 1/(i + 100)

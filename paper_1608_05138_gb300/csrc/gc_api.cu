@@ -678,7 +678,15 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
     g->d_gm = reinterpret_cast<int64_t*>(reinterpret_cast<char*>(g->d_gbase) + 16);
   }
   {
-    gc_status st2 = scratch_init(&g->sc, g->m, needs_tables(g->prep) ? n : 0, g->prep.kmax, g->prep.ktier_off, 1, s);
+    gc_status st2 = GC_OK;
+    if (n <= kDenseMaxN && g->prep.kmax <= kDenseMaxK) {
+      int64_t d2 = 0;
+      for (int32_t x = 0; x < n; ++x) d2 += (int64_t)(row_ptr[x + 1] - row_ptr[x]) * (row_ptr[x + 1] - row_ptr[x]);
+      if (dense_graph(n, g->m, d2, g->prep.dmax)) st2 = build_bits(n, g->d_rp, g->d_ci, &g->prep, s);
+    }
+    if (st2 == GC_OK)
+      st2 = scratch_init(&g->sc, g->m, needs_tables(g->prep) ? n : 0, g->prep.kmax, g->prep.ktier_off, 1,
+                         g->prep.bits ? n : 0, s);
     if (st2 != GC_OK) return fail(st2);
     scratch_guess_tlist(&g->sc, g->m);
   }
@@ -777,10 +785,13 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
   dg.gn = g->d_gn;
   dg.gm = g->d_gm;
   dg.table_n = g->n;
+  dg.bits = g->prep.bits;
+  dg.bits_t = g->prep.bits_t;
   dg.hgeom = g->prep.hgeom;
   dg.hseg = g->prep.hseg;
   dg.hpos = g->prep.hpos;
   KUnits ku;
+  ku.kmax = g->prep.kmax;
   ku.units = g->prep.kunits;
   ku.cunits = g->prep.cunits;
   ku.n_cheavy = g->prep.n_cheavy;

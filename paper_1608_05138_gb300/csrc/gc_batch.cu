@@ -397,7 +397,7 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
   d_rp0 = d_ci0 = d_perm = d_newid = d_lists = nullptr;
   d_loff = nullptr;
   d_tmp = nullptr;
-  if ((st = scratch_init(&sc, m, needs_tables(prep) ? table_n : 0, prep.kmax, prep.ktier_off, G, s)) != GC_OK) {
+  if ((st = scratch_init(&sc, m, needs_tables(prep) ? table_n : 0, prep.kmax, prep.ktier_off, G, 0, s)) != GC_OK) {
     L->error = gc_last_error();
     goto out;
   }
@@ -420,10 +420,12 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
     dg.gn = d_desc + G;
     dg.gm = d_gm;
     dg.table_n = table_n;
+    dg.bits = dg.bits_t = nullptr;
     dg.hgeom = prep.hgeom;
     dg.hseg = prep.hseg;
     dg.hpos = prep.hpos;
     KUnits ku;
+    ku.kmax = prep.kmax;
     ku.units = prep.kunits;
     ku.cunits = prep.cunits;
     ku.n_cheavy = prep.n_cheavy;

@@ -59,6 +59,8 @@ struct DevGraph {
   const int32_t* gn;       // [G] vertices of each graph
   const int64_t* gm;       // [G] edges of each graph
   int32_t table_n;         // max gn[g]: size of one Psi table
+  const uint32_t* bits;    // dense graphs (dense_graph()): bit rows [n][(n + 31) / 32], and the same by word
+  const uint32_t* bits_t;  // [(n + 31) / 32][n]; else nullptr
   const HubGeom* hgeom;    // ranked: [G] (nullptr when the graph has no hub units)
   const HubSeg* hseg;
   const int32_t* hpos;
@@ -97,6 +99,7 @@ struct CountArgs {
   unsigned long long* xc;    // [m][2] per out-slot: 4-cliques through the edge, and the sum over T of
                              // (|T_(a,u)| + |T_(a,v)| - 2) (pass K); side by side, so that the two
                              // atomics of an edge land in one 32-byte sector
+  uint32_t* x7d;           // dense graphs: [n][n] 4-cliques through the edge (lower, higher); else nullptr
   unsigned char* kbuf;     // global-tier per-CTA buffers (kbuf_ctas x kbuf_stride bytes)
   size_t kbuf_stride;
   int32_t kbuf_ctas;
@@ -229,6 +232,7 @@ struct Scratch {
   int32_t* trio = nullptr;           // [m]
   unsigned long long* xc = nullptr;  // [m][2]
   unsigned long long* P = nullptr;   // [2m]
+  uint32_t* x7d = nullptr;           // [n][n] (dense graphs)
   uint32_t* tables = nullptr;        // count_grid_size() x table_n
   size_t tables_n = 0;
   unsigned char* kbuf = nullptr;     // pass K global tier
@@ -250,10 +254,10 @@ struct Scratch {
   unsigned long long* vsum = nullptr;  // [n][2] per-edge induced counts: 2 x triangles, neighbour degrees
 };
 // Allocates the scratch of a union of G graphs with m edges, Psi tables of
-// table_n vertices, largest out-degree kmax and pass-K tiers tier_off
-// (stream-ordered).
+// table_n vertices, largest out-degree kmax and pass-K tiers tier_off, and for
+// a dense graph its vertices dense_n (stream-ordered).
 gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, const int32_t* tier_off, int32_t G,
-                       cudaStream_t s);
+                       int32_t dense_n, cudaStream_t s);
 void scratch_free(Scratch* sc, cudaStream_t s);
 // Size of pass T's edge lists for the first count of a whole graph with m
 // edges: 32 m entries within the list budget (units past it scan again).
@@ -264,6 +268,7 @@ void scratch_guess_tlist(Scratch* sc, int64_t m);
 // than kOverlapEdges edges (see run_count). Returns after the derive is queued
 // (no host synchronisation).
 struct KUnits {
+  int32_t kmax;            // largest out-degree
   const int32_t* units;
   int32_t tier_off[kNumTiers + 1];
   const int32_t* cunits;   // pass C units: hubs, hashed units, the others
@@ -374,6 +379,8 @@ struct PrepBuffers {
   int32_t n_chash2 = 0;        // units of the packed-key hash tier
   int32_t n_chash2_big = 0;    // of them, units of more than kHash2HalfMaxW wedges
   int32_t n_cunits = 0;
+  uint32_t* bits = nullptr;    // dense graphs: bit rows, and the same by word (see DevGraph)
+  uint32_t* bits_t = nullptr;
   HubGeom* hgeom = nullptr;    // layout of the hub kernel's o-range (owns hseg's block)
   HubSeg* hseg = nullptr;
   int32_t* hpos = nullptr;
@@ -466,6 +473,27 @@ gc_status run_pass_c_heavy(const DevGraph& g, const CountArgs& a, cudaStream_t s
 // at most kSmemTableMax vertices; and the 4-cliques without pass T.
 gc_status run_rows(const DevGraph& g, const CountArgs& a, cudaStream_t s);
 gc_status run_cliques_alone(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches);
+// The same two for a dense graph, on its bit rows: k_rows_dense reads them
+// instead of the neighbours' lists, k_cliques_dense packs every H_a from them.
+constexpr int kDenseMaxN = 2048;
+constexpr int kDenseMaxK = 1024;  // largest out-degree
+// Whether a graph of n vertices, m edges, sum d^2 = d2 and largest degree dmax
+// is counted on bit rows. Costs in SM cycles: about 1.1 per entry of the
+// neighbours' rows (25 instructions per 32 entries, read twice), against a popc
+// (16 a cycle) per word, counter bit and slot, for the 4-cycles of half of the
+// slots and the cross terms of all, and per word and vertex pair. G(1000, 0.3):
+// 1.0e8 against 1.1e7; G(2000, 0.01): 9e5 against 2.6e7.
+inline bool dense_graph(int64_t n, int64_t m, int64_t d2, int64_t dmax) {
+  if (n > kDenseMaxN || n < 64 || m == 0) return false;
+  int bits = 1;
+  while ((1LL << bits) <= dmax) ++bits;
+  const double W = (double)((n + 31) / 32);
+  return 1.1 * (double)d2 > 1.5 * (0.094 * 2.0 * (double)m * W * bits + 0.1 * (double)n * (double)n * W);
+}
+gc_status run_rows_dense(const DevGraph& g, const CountArgs& a, cudaStream_t s);
+gc_status run_cliques_dense(const DevGraph& g, const CountArgs& a, int32_t kmax, cudaStream_t s);
+// Bit rows of a prepared graph of at most kDenseMaxN vertices (P->bits, bits_t).
+gc_status build_bits(int32_t n, const int32_t* d_rp, const int32_t* d_ci, PrepBuffers* p, cudaStream_t s);
 constexpr int kHeavyTab = 53248;  // largest o-range block of the hub kernel of pass C (words of shared memory)
 // Words of the hub kernel's count block (environment GC_HUB_TAB_WORDS, a
 // multiple of 1024 in [4096, kHeavyTab], else kHubTabDefault), read once per

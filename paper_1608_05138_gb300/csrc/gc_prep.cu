@@ -233,6 +233,20 @@ __global__ void k_hub_pos(const HubGeom* __restrict__ geom, const HubSeg* __rest
   }
 }
 
+// Bit rows of the graph, in both layouts (zeroed before): warp per row.
+__global__ void k_bits(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                       uint32_t* __restrict__ bits, uint32_t* __restrict__ bits_t) {
+  const int lane = threadIdx.x & 31, W = (n + 31) / 32;
+  const int x = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (x >= n) return;
+  for (int32_t p = rp[x] + lane; p < rp[x + 1]; p += 32) {
+    const int32_t y = ci[p];
+    const uint32_t b = 1u << (y & 31);
+    atomicOr(&bits[(size_t)x * W + (y >> 5)], b);
+    atomicOr(&bits_t[(size_t)(y >> 5) * n + x], b);
+  }
+}
+
 // Smallest slot whose reverse was not found (rev[p] == p): the input is not
 // symmetric exactly when there is one.
 __global__ void k_first_unreversed(int64_t nnz, const int32_t* __restrict__ rev, int32_t* __restrict__ first) {
@@ -655,7 +669,19 @@ gc_status first_unreversed_slot(int64_t nnz, const int32_t* d_rev, int32_t* out,
   return GC_OK;
 }
 
+gc_status build_bits(int32_t n, const int32_t* d_rp, const int32_t* d_ci, PrepBuffers* p, cudaStream_t s) {
+  const size_t words = (size_t)n * (size_t)((n + 31) / 32);
+  cudaError_t e = pool_alloc(&p->bits, sizeof(uint32_t) * 2 * words, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(p->bits, 0, sizeof(uint32_t) * 2 * words, s);
+  if (e != cudaSuccess) return cuda_fail(e, "bit rows");
+  p->bits_t = p->bits + words;
+  k_bits<<<grid_for((int64_t)n * 32, 256), 256, 0, s>>>(n, d_rp, d_ci, p->bits, p->bits_t);
+  e = cudaGetLastError();
+  return e == cudaSuccess ? GC_OK : cuda_fail(e, "k_bits");
+}
+
 void free_prep(PrepBuffers* p, cudaStream_t s) {
+  if (p->bits) cudaFreeAsync(p->bits, s);
   if (p->deg) cudaFreeAsync(p->deg, s);
   if (p->eid) cudaFreeAsync(p->eid, s);
   if (p->uv) cudaFreeAsync(p->uv, s);

@@ -58,7 +58,7 @@ void scratch_free(Scratch* sc, cudaStream_t s) {
 }
 
 gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, const int32_t* tier_off, int32_t G,
-                       cudaStream_t s) {
+                       int32_t dense_n, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
 #define GS_TRY(call)                                \
   do {                                              \
@@ -80,7 +80,8 @@ gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, co
                  x = take(sizeof(unsigned long long) * 34 * (size_t)G);
     sc->head_bytes = at;
     const size_t trio = take(sizeof(int32_t) * m1, 256), xc = take(sizeof(unsigned long long) * 2 * m1, 256),
-                 P = take(sizeof(unsigned long long) * 2 * m1, 256);
+                 P = take(sizeof(unsigned long long) * 2 * m1, 256),
+                 x7d = take(sizeof(uint32_t) * (size_t)dense_n * (size_t)dense_n, 256);
     sc->zero_bytes = at;
     GS_TRY(pool_alloc(&sc->zero, at, s));
     sc->misc = reinterpret_cast<int32_t*>(sc->zero + misc);
@@ -91,6 +92,7 @@ gc_status scratch_init(Scratch* sc, int32_t m, int32_t table_n, int32_t kmax, co
     sc->trio = reinterpret_cast<int32_t*>(sc->zero + trio);
     sc->xc = reinterpret_cast<unsigned long long*>(sc->zero + xc);
     sc->P = reinterpret_cast<unsigned long long*>(sc->zero + P);
+    if (dense_n > 0) sc->x7d = reinterpret_cast<uint32_t*>(sc->zero + x7d);
   }
   if (table_n > kSmemTableMax) {
     sc->tables_n = (size_t)count_grid_size() * (size_t)table_n;
@@ -169,6 +171,7 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
   a.tables = g.table_n > kSmemTableMax ? sc->tables : nullptr;
   a.trio = sc->trio;
   a.P = sc->P;
+  a.x7d = nullptr;
   a.xc = sc->xc;
   a.kbuf = sc->kbuf;
   a.kbuf_stride = sc->kbuf_stride;
@@ -270,16 +273,25 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
   if (rows) {
     GR_BEGIN(kPhasePassT, s);
     GR_END(kPhasePassT, s);
-    Fork side(s, fs, 0, 1);
+    // the dense kernels fill the GPU and want different shares of shared memory
+    // and L1: side by side they take twice as long as one after the other
+    const bool dense = g.bits != nullptr;
+    Fork side(s, dense ? nullptr : fs, 0, 1);
     const cudaStream_t t = side.next();
     GR_BEGIN(kPhasePassC, t);
-    if ((st = run_rows(g, a, t)) != GC_OK) return st;
+    if (dense) a.x7d = sc->x7d;
+    if ((st = dense ? run_rows_dense(g, a, t) : run_rows(g, a, t)) != GC_OK) return st;
     launches += g.n > 0 ? 1 : 0;
     GR_END(kPhasePassC, t);
     GR_BEGIN(kPhasePassK, s);
-    Fork tiers(s, fs, 6, kForkStreams - 6);
-    if ((st = run_cliques_alone(g, a, &tiers, &launches)) != GC_OK) return st;
-    GR_TRY(tiers.join(), "join");
+    if (dense) {
+      if ((st = run_cliques_dense(g, a, ku.kmax, s)) != GC_OK) return st;
+      launches += ku_total(ku) > 0 ? 1 : 0;
+    } else {
+      Fork tiers(s, fs, 6, kForkStreams - 6);
+      if ((st = run_cliques_alone(g, a, &tiers, &launches)) != GC_OK) return st;
+      GR_TRY(tiers.join(), "join");
+    }
     GR_END(kPhasePassK, s);
     GR_TRY(side.join(), "join");
   } else if (overlap) {

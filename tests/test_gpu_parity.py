@@ -281,6 +281,12 @@ def test_batch_four_cliques_of_wide_neighbourhoods(n, k, copies):
     assert all(x == ref for x in X[1:])
 
 
+def padded(g, n):
+    """The graph with isolated vertices added up to n."""
+    rp, ci = g
+    return np.concatenate([rp, np.full(n + 1 - len(rp), rp[-1], np.int32)]), ci
+
+
 @pytest.mark.parametrize("make", [
     lambda: graphgen.er(4096, 0.004, 3),          # the largest graph on rows of common neighbours
     lambda: graphgen.er(4097, 0.004, 3),          # and the smallest beyond
@@ -289,6 +295,9 @@ def test_batch_four_cliques_of_wide_neighbourhoods(n, k, copies):
     lambda: graphs.star(4000),
     lambda: graphs.complete_bipartite(37, 290),
     lambda: graphgen.er(700, 0.8, 5),
+    lambda: graphgen.er(64, 0.9, 6),              # bit rows: the smallest graph, out-degrees beside whole words
+    lambda: graphgen.er(65, 0.9, 7),
+    lambda: padded(graphgen.er(400, 0.5, 8), 1201),  # a partial last word, most rows empty
 ])
 def test_rows_of_common_neighbours(make):
     assert_parity(*make())

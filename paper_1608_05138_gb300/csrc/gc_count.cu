@@ -92,6 +92,8 @@ constexpr int kFinBlock = 256;
 template <bool kByEdge>
 __global__ void __launch_bounds__(kFinBlock) k_finish(DevGraph g, CountArgs a) {
   __shared__ unsigned long long st[kFinBlock / 32][32][13];
+  __shared__ int32_t s_g[kFinBlock / 32];
+  __shared__ long long s_edges[kFinBlock / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned long long(*rowv)[13] = st[warp];
   const unsigned long long* flat = &st[warp][0][0];
@@ -142,8 +144,39 @@ __global__ void __launch_bounds__(kFinBlock) k_finish(DevGraph g, CountArgs a) {
     w_edges += rows;
     __syncwarp();
   }
-  if (lane < 13 && cur_g >= 0) atomic_add_u128(a.csum + ((size_t)cur_g * 13 + lane) * 2, acc);
-  if (lane == 0 && w_edges) atomicAdd(a.work + kWorkFinishEdges, (unsigned long long)w_edges);
+  // the warps' last sums meet in shared memory: one atomic a block and column
+  // where they belong to one graph (per warp, a count of ER-2000 sent 16 000
+  // atomics to 26 words, 10 of the kernel's 16 us)
+  __syncwarp();
+  unsigned long long* fin = &st[warp][0][0];  // 13 low words, 13 high words
+  if (lane < 13) {
+    fin[lane] = (unsigned long long)acc;
+    fin[13 + lane] = (unsigned long long)(acc >> 64);
+  }
+  if (lane == 0) {
+    s_g[warp] = cur_g;
+    s_edges[warp] = w_edges;
+  }
+  __syncthreads();
+  if (threadIdx.x < 13) {
+    u128 sum = 0;
+    int32_t of = -1;
+    for (int w = 0; w < kFinBlock / 32; ++w) {
+      if (s_g[w] < 0) continue;
+      if (s_g[w] != of) {
+        if (of >= 0) atomic_add_u128(a.csum + ((size_t)of * 13 + threadIdx.x) * 2, sum);
+        sum = 0;
+        of = s_g[w];
+      }
+      const unsigned long long* f = &st[w][0][0];
+      sum += ((u128)f[13 + threadIdx.x] << 64) | (u128)f[threadIdx.x];
+    }
+    if (of >= 0) atomic_add_u128(a.csum + ((size_t)of * 13 + threadIdx.x) * 2, sum);
+  } else if (threadIdx.x == 13) {
+    long long edges = 0;
+    for (int w = 0; w < kFinBlock / 32; ++w) edges += s_edges[w];
+    if (edges) atomicAdd(a.work + kWorkFinishEdges, (unsigned long long)edges);
+  }
 }
 
 // ---------------- per-edge induced 4-node counts ----------------
@@ -997,6 +1030,8 @@ __global__ void __launch_bounds__(kThreads, kThreads == kHashBlock ? kCtasPerSm 
   extern __shared__ int32_t hkeys[];                                  // [2 kMaxW] o, or -1
   uint32_t* hcnt = reinterpret_cast<uint32_t*>(hkeys + 2 * kMaxW);    // [kMaxW] two counts
   __shared__ int32_t s_unit, s_next[2];
+  __shared__ unsigned long long s_wedge;
+  if (threadIdx.x == 0) s_wedge = 0ull;  // seen by all after the loop's first barrier
   const int lane = threadIdx.x & 31;
   long long w_wedge = 0;  // lane 0
   for (;;) {
@@ -1061,9 +1096,11 @@ __global__ void __launch_bounds__(kThreads, kThreads == kHashBlock ? kCtasPerSm 
       __syncthreads();
     }
   }
-  if (lane == 0 && w_wedge) {
-    atomicAdd(a.work + kWorkCWedge, (unsigned long long)w_wedge);
-    atomicAdd(a.work + kWorkCHashWedge, (unsigned long long)w_wedge);
+  if (lane == 0 && w_wedge) atomicAdd(&s_wedge, (unsigned long long)w_wedge);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_wedge) {  // one atomic a block
+    atomicAdd(a.work + kWorkCWedge, s_wedge);
+    atomicAdd(a.work + kWorkCHashWedge, s_wedge);
   }
 }
 
@@ -1120,6 +1157,8 @@ __global__ void __launch_bounds__(kThreads, kThreads == kHash2Block ? 1 : 2)
     k_pass_c_hash2(DevGraph g, CountArgs a, int32_t k0, int32_t k1, int32_t* cursor) {
   extern __shared__ uint32_t htab[];  // kSlots packed (o, count) words
   __shared__ int32_t s_unit, s_next[2];
+  __shared__ unsigned long long s_wedge;
+  if (threadIdx.x == 0) s_wedge = 0ull;  // seen by all after the loop's first barrier
   const int lane = threadIdx.x & 31;
   long long w_wedge = 0;  // lane 0
   const int32_t first = a.n_cheavy + a.n_chash;
@@ -1180,9 +1219,11 @@ __global__ void __launch_bounds__(kThreads, kThreads == kHash2Block ? 1 : 2)
       __syncthreads();
     }
   }
-  if (lane == 0 && w_wedge) {
-    atomicAdd(a.work + kWorkCWedge, (unsigned long long)w_wedge);
-    atomicAdd(a.work + kWorkCHash2Wedge, (unsigned long long)w_wedge);
+  if (lane == 0 && w_wedge) atomicAdd(&s_wedge, (unsigned long long)w_wedge);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_wedge) {  // one atomic a block
+    atomicAdd(a.work + kWorkCWedge, s_wedge);
+    atomicAdd(a.work + kWorkCHash2Wedge, s_wedge);
   }
 }
 

@@ -526,8 +526,12 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
   p->n_chash2_big = 0;  // heaviest first too
   while (p->n_chash2_big < p->n_chash2 && W[hashed2[(size_t)p->n_chash2_big]] > kHash2HalfMaxW) ++p->n_chash2_big;
   p->n_cunits = (int32_t)out.size();
-  // The hub kernel's o-range (see HubSeg): per graph, each degree class in
-  // order, cut where a count block is full.
+  // The hub kernel's o-range (see HubSeg): per graph, segment by segment, the
+  // counter width that reaches furthest (the wider one at equal reach): to the
+  // end of the ids whose degree fits it, or of the block. A block is closed when
+  // less than a sixteenth is left. Every (neighbour, segment) costs a look at
+  // the row, so that a graph whose ids all fit one block of 16-bit counters
+  // gets one segment, not one per degree class.
   std::vector<HubSeg> segs;
   std::vector<HubGeom> geom;
   int64_t n_pos = 0;
@@ -537,18 +541,22 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
       const int32_t end = rank.gbase[gi] + rank.gn[gi];
       HubGeom ge = {(int32_t)segs.size(), 0, end, end, n_pos};
       int32_t word = 0;
-      for (int c = 0; c < kOBounds; ++c) {
-        const int lg = kOBounds - 1 - c;
-        const int32_t ce = c + 1 < kOBounds ? ob[c + 1] : end;
-        for (int32_t lo = ob[c]; lo < ce;) {
-          const int32_t hi = (int32_t)std::min<int64_t>(ce, lo + ((tab - word) << lg));
-          segs.push_back({lo, hi, word, (int16_t)lg, 0});
-          word += (hi - lo + (1 << lg) - 1) >> lg;
-          if (word >= tab || hi == end) {
-            segs.back().last = 1;
-            word = 0;
+      for (int32_t lo = ob[0], hi; lo < end; lo = hi) {
+        int lg = 0;
+        hi = lo;
+        for (int l = 0; l < kOBounds; ++l) {
+          const int32_t fits = l == 0 ? end : ob[kOBounds - l];  // ids whose degree fits 32 >> l bits
+          const int32_t to = (int32_t)std::min<int64_t>(fits, lo + ((tab - word) << l));
+          if (to > hi) {
+            hi = to;
+            lg = l;
           }
-          lo = hi;
+        }
+        segs.push_back({lo, hi, word, (int16_t)lg, 0});
+        word += (hi - lo + (1 << lg) - 1) >> lg;
+        if (tab - word < tab / 16 || hi == end) {
+          segs.back().last = 1;
+          word = 0;
         }
       }
       ge.nseg = (int32_t)segs.size() - ge.seg;

@@ -521,9 +521,9 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
 
 // Units with k <= 32: one warp per unit, lane i holding member b_i, the rows of
 // H_a as 32-bit masks and the out-slots of its edges in shared memory.
-// The out-lists of all members are read end to end over the lanes (most have a
-// few entries, so that a window of 32 per member left most lanes idle and
-// waited on memory once per member), and an entry's place in out(a) is a 5-step
+// The out-lists of all members are read end to end over the lanes, long ones in
+// blocks first (most have a few entries, so that windows per member left most
+// lanes idle and waited on memory once per member), and an entry's place in out(a) is a 5-step
 // binary search over the lanes' ids (ascending). Pass K takes an edge of H_a
 // per lane. Both wait on chains of dependent loads, a unit at a time.
 // Chung-Lu 1M: pass T's kernel 1.92 -> 1.63 ms, pass K's 1.37 -> 0.43 ms.
@@ -604,12 +604,45 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
     __syncwarp();
     // the scan: on_hit(i, j, q) for every edge (i, j) of H_a, q its out-slot
     auto scan = [&](auto on_hit) {
-      int32_t b = 0, len = 0;
+      int32_t b = 0, left = 0;
       if (lane < k) {
         b = g.out_ptr[id];
-        len = g.out_ptr[id + 1] - b;
+        left = g.out_ptr[id + 1] - b;
       }
-      const Deal d = deal_setup(len, s_comp[warp], lane);
+      const int32_t cmax = __shfl_sync(kFull, id, k - 1);
+      auto place = [&](int32_t c, int own, int32_t q) {  // entry c of member own's list, at out-slot q
+        int lo = 0;  // the last member not above c
+#pragma unroll
+        for (int step = 16; step; step >>= 1)
+          if (__shfl_sync(kFull, id, lo + step) <= c) lo += step;
+        const int32_t id_lo = __shfl_sync(kFull, id, lo);
+        if (c >= 0 && id_lo == c) on_hit(own, lo, q);  // lanes >= k hold an id no vertex has
+      };
+      // long lists: whole blocks of 128 entries, one list at a time, left where
+      // it (ascending) passes the largest member
+      unsigned lm = __ballot_sync(kFull, left >= 128);
+      while (lm) {
+        const int src = __ffs(lm) - 1;
+        lm &= lm - 1;
+        const int32_t b0 = __shfl_sync(kFull, b, src), n0 = __shfl_sync(kFull, left, src);
+        int32_t done = 0;
+        bool past = false;
+        for (; done + 128 <= n0 && !past; done += 128) {
+          int32_t c[4];
+#pragma unroll
+          for (int w = 0; w < 4; ++w) c[w] = g.out_idx[b0 + done + 32 * w + lane];
+#pragma unroll
+          for (int w = 0; w < 4; ++w) place(c[w], src, b0 + done + 32 * w + lane);
+          past = __shfl_sync(kFull, c[3], 31) > cmax;
+        }
+        w_scan += done;
+        if (lane == src) {
+          b += done;
+          left = past ? 0 : left - done;
+        }
+      }
+      // the rest of every list, end to end
+      const Deal d = deal_setup(left, s_comp[warp], lane);
       const int32_t base = b - d.excl;
       w_scan += d.total;
       int before = 0;
@@ -617,7 +650,7 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
         int32_t q[4], c[4], own[4];
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
-          own[w] = deal_owner(d, len, k0 + 32 * w, s_comp[warp], lane, before);
+          own[w] = deal_owner(d, left, k0 + 32 * w, s_comp[warp], lane, before);
           const int32_t pos = k0 + 32 * w + lane;
           const int32_t bw = __shfl_sync(kFull, base, own[w]);
           q[w] = bw + pos;
@@ -626,12 +659,7 @@ __global__ void __launch_bounds__(kWBlock) k_pass_k_warp(DevGraph g, CountArgs a
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
           if (k0 + 32 * w >= d.total) break;  // warp-uniform
-          int lo = 0;  // the last member not above c
-#pragma unroll
-          for (int step = 16; step; step >>= 1)
-            if (__shfl_sync(kFull, id, lo + step) <= c[w]) lo += step;
-          const int32_t id_lo = __shfl_sync(kFull, id, lo);
-          if (c[w] >= 0 && id_lo == c[w]) on_hit(own[w], lo, q[w]);  // lanes >= k hold an id no vertex has
+          place(c[w], own[w], q[w]);
         }
       }
       __syncwarp();

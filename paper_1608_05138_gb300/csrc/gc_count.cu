@@ -114,8 +114,9 @@ __global__ void __launch_bounds__(kFinBlock) k_finish(DevGraph g, CountArgs a) {
       gid = g.vgid ? g.vgid[u] : 0;
       const int64_t du = g.deg[u], dv = g.deg[v];
       const int64_t t = a.trio[o];
-      const int64_t x7 = a.x7d ? (int64_t)a.x7d[(size_t)u * g.n + v] : (int64_t)a.xc[2 * (size_t)o];
-      const int64_t x10 = (int64_t)(a.P[p] + a.P[r]) - (int64_t)a.xc[2 * (size_t)o + 1] + 2 * x7;
+      const ulonglong2 xc = *reinterpret_cast<const ulonglong2*>(a.xc + 2 * (size_t)o);
+      const int64_t x7 = a.x7d ? (int64_t)a.x7d[(size_t)u * g.n + v] : (int64_t)xc.x;
+      const int64_t x10 = (int64_t)(a.P[p] + a.P[r]) - (int64_t)xc.y + 2 * x7;
       const int64_t su = du - t - 1, sv = dv - t - 1;
       const int64_t n_g = g.gn[gid], m_g = g.gm[gid];
       const int64_t D = n_g - 2 - t - su - sv;
@@ -685,6 +686,7 @@ __global__ void __launch_bounds__(kDenseBlock) k_cliques_dense(DevGraph g, Count
 // explains: the longer the runs per block, the fewer the sweeps.
 constexpr int kHeavyBlock = 1024;
 constexpr int kHeavyWarps = kHeavyBlock / 32;
+constexpr int32_t kFine = 256;  // heaviest x's of a large hub, four to a chunk
 
 // Counters of a segment, 2^lg to a word (no count of the segment reaches its
 // field's size, so no carry crosses into the next field).
@@ -890,11 +892,14 @@ __global__ void __launch_bounds__(kHeavyBlock, 1) k_pass_c_heavy(DevGraph g, Cou
     }
     __syncthreads();
     const int32_t nx = s_nx;
-    // chunks of 32 x's: of consecutive ones, taken heaviest first (X ascends
-    // by degree) from a shared counter, when there are more than a CTA's
-    // threads; otherwise one chunk per warp, x = warp, warp + 32, ...
+    // chunks of x's: of consecutive ones, taken heaviest first (X ascends by
+    // degree) from a shared counter, when there are more than a CTA's threads
+    // -- four to a chunk for the heaviest, so that no warp keeps the others
+    // waiting with 32 of them (pass C of Chung-Lu 1M 7.94 -> 7.54 ms), 32 to a
+    // chunk for the rest; otherwise one chunk per warp, x = warp, warp + 32, ...
     const bool small = nx <= kHeavyBlock;
-    const int32_t nchunks = small ? kHeavyWarps : (nx + 31) >> 5;
+    const int32_t fine = min(nx, kFine), fine_chunks = (fine + 3) >> 2;
+    const int32_t nchunks = small ? kHeavyWarps : fine_chunks + ((nx - fine + 31) >> 5);
     if (job.w & 1) {  // the hub's wedges, counted by its first job
       for (int32_t i = threadIdx.x; i < nx; i += kHeavyBlock) {
         const int32_t xb = g.rp[g.ci[hb + i]];
@@ -936,7 +941,12 @@ __global__ void __launch_bounds__(kHeavyBlock, 1) k_pass_c_heavy(DevGraph g, Cou
             c = __shfl_sync(0xffffffffu, c, 0);
             if (c >= nchunks) break;
           }
-          const int32_t i = small ? ri : (nchunks - 1 - c) * 32 + lane;
+          int32_t i = ri;
+          if (!small) {
+            const bool few = c < fine_chunks;
+            const int32_t k = few ? 4 * c + lane : fine + 32 * (c - fine_chunks) + lane;  // from the heaviest x down
+            i = (few && (lane >= 4 || k >= fine)) || k >= nx ? nx : nx - 1 - k;
+          }
           int32_t x = rx, rend = rrend;
           if (!small && i < nx) {
             x = g.ci[hb + i];

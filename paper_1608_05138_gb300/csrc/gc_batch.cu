@@ -28,6 +28,7 @@
 #include <thread>
 #include <vector>
 
+#include "gc_deal.h"
 #include "gc_internal.h"
 
 namespace gc {
@@ -35,6 +36,35 @@ gc_status validate_csr(int32_t n, const int32_t* rp, const int32_t* ci);
 gc_status validate_csr_small(int32_t n, const int32_t* rp, const int32_t* ci, std::vector<int32_t>* fill);
 
 namespace {
+
+// The checks of one graph on the device, thread per slot: *bad becomes non-zero
+// if a column is out of range, a self-loop, not above its predecessor, or its
+// reverse is absent (row pointers from 0 to nnz, ascending, are checked
+// before). The host's walk over the reverses waits on memory once per edge:
+// 6.2 ms for 3.5M entries on 16 cores, against 0.9 ms for copy and kernel.
+__global__ void __launch_bounds__(256) k_check_csr(int32_t n, int32_t nnz, const int32_t* __restrict__ rp,
+                                                   const int32_t* __restrict__ ci, int32_t* __restrict__ bad) {
+  const int lane = threadIdx.x & 31;
+  bool ok = true;
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p - lane < nnz; p += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t p0 = (int32_t)(p - lane), p_last = (int32_t)min((int64_t)p0 + 31, (int64_t)nnz - 1);
+    const int32_t q = (int32_t)min(p, (int64_t)nnz - 1);
+    const int32_t x = row_of_slot(n, rp, p0, q, p_last);
+    const int32_t y = ci[q];
+    if ((uint32_t)y >= (uint32_t)n || y == x || (q > rp[x] && ci[q - 1] >= y)) {
+      ok = false;
+      continue;
+    }
+    int32_t lo = rp[y];
+    const int32_t ye = rp[y + 1];
+    for (int32_t hi = ye; lo < hi;) {
+      const int32_t mid = lo + ((hi - lo) >> 1);
+      if (ci[mid] < x) lo = mid + 1; else hi = mid;
+    }
+    ok &= lo < ye && ci[lo] == x;
+  }
+  if (!ok) *bad = 1;
+}
 
 // The library's host copy of one submission, pinned where possible, so that a
 // launch copies it to the device directly.
@@ -254,6 +284,11 @@ struct gc_batch_s {
   }
   bool stop = false;
   std::thread dispatcher;
+  // the device's checks of a submission (one at a time): a stream of high
+  // priority, so that they do not wait behind the launches in flight
+  std::mutex check_mu;
+  cudaStream_t check_stream = nullptr;
+  int32_t* check_bad = nullptr;         // pinned
   cudaStream_t streams[kMaxInflight] = {};
   int next_stream = 0;                  // manual mode: round-robin over the slots
   int device = 0;
@@ -870,6 +905,47 @@ void poll_wait(gc_batch b, std::unique_lock<std::mutex>* lk, std::chrono::steady
 
 }  // namespace
 
+// Whether the graph copied to `own` (row pointers, then columns; pinned) passes
+// every check of validate_csr, by k_check_csr; its row pointers have been
+// checked. false also when a device step fails: the caller then asks the host.
+static bool checked_on_device(gc_batch b, int32_t n, int32_t nnz, const int32_t* own) {
+  std::lock_guard<std::mutex> lk(b->check_mu);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || (dev != b->device && cudaSetDevice(b->device) != cudaSuccess)) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaError_t e = cudaSuccess;
+  if (!b->check_stream) {
+    int least = 0, greatest = 0;
+    e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->check_stream, cudaStreamNonBlocking, greatest);
+    if (e == cudaSuccess) e = cudaMallocHost(&b->check_bad, sizeof(int32_t));
+  }
+  int32_t* d = nullptr;  // flag, row pointers, columns
+  const size_t words = (size_t)n + 1 + (size_t)nnz;
+  cudaStream_t s = b->check_stream;
+  bool ok = false;
+  if (e == cudaSuccess && b->check_bad) {
+    e = pool_alloc(&d, sizeof(int32_t) * (words + 1), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d, 0, sizeof(int32_t), s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d + 1, own, sizeof(int32_t) * words, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) {
+      const int64_t blocks = ((int64_t)nnz + 255) / 256;
+      k_check_csr<<<(int)std::min<int64_t>(blocks, 8LL * (count_grid_size() / kCtasPerSm)), 256, 0, s>>>(
+          n, nnz, d + 1, d + 1 + n + 1, d);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->check_bad, d, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);  // also after a failure: `own` may be read
+    ok = e == cudaSuccess && e2 == cudaSuccess && *b->check_bad == 0;
+    if (d) cudaFreeAsync(d, s);
+  }
+  if (!ok) cudaGetLastError();
+  if (dev != b->device) cudaSetDevice(dev);
+  return ok;
+}
+
 extern "C" {
 
 gc_status gc_batch_create(int64_t device_mem_budget_bytes, uint32_t flags, gc_batch* out) {
@@ -951,10 +1027,25 @@ gc_status gc_batch_last_stats(gc_batch b, double* out) {
 gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const int32_t* col_idx,
                           uint64_t* ticket_out) {
   if (!b || !ticket_out || !row_ptr || n < 0) { set_error("bad arguments"); return GC_ERR_ARG; }
-  gc_status st = validate_csr(n, row_ptr, col_idx);
-  if (st != GC_OK) return st;
+  // Graphs of kDeviceCheck entries or more are checked on the device, from the
+  // copy, once their row pointers have been checked; what fails there (or
+  // cannot be checked there) gets the host's checks, for the code and message.
+  constexpr int32_t kDeviceCheck = 1 << 16;
+  bool on_device = n > 0 && row_ptr[0] == 0 && row_ptr[n] >= kDeviceCheck && row_ptr[n] % 2 == 0 && col_idx;
+  if (on_device) {
+    bool ascending = true;
+    for (int32_t x = 0; x < n; ++x) ascending &= row_ptr[x + 1] >= row_ptr[x];
+    on_device = ascending;
+  }
+  gc_status st = GC_OK;
+  if (!on_device && (st = validate_csr(n, row_ptr, col_idx)) != GC_OK) return st;
   const int64_t m = row_ptr[n] / 2;
   const int64_t bytes = footprint(n, m);
+  // an invalid graph is refused as such first, whatever its size
+  if (on_device && bytes > b->budget) {
+    if ((st = validate_csr(n, row_ptr, col_idx)) != GC_OK) return st;
+    on_device = false;
+  }
   if (bytes > b->budget) {
     set_error("graph needs more device memory than the whole budget");
     return GC_ERR_NOMEM;
@@ -963,13 +1054,6 @@ gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const i
   pg.n = n;
   pg.m = m;
   pg.bytes = bytes;
-  {  // refused before the copy is made, where it already shows
-    std::lock_guard<std::mutex> lk(b->mu);
-    if (b->in_use + bytes > b->budget) {
-      set_error("device-memory budget is full");
-      return GC_ERR_BUSY;
-    }
-  }
   try {
     pg.owner = host_block(b->host, (size_t)n + 1 + 2 * (size_t)m);
     int32_t* own = pg.owner->p;
@@ -985,6 +1069,9 @@ gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const i
     set_error("host allocation failed");
     return GC_ERR_NOMEM;
   }
+  if (on_device && !(pg.owner->pinned && checked_on_device(b, n, row_ptr[n], pg.rp)) &&
+      (st = validate_csr(n, pg.rp, pg.ci)) != GC_OK)
+    return st;
   {
     std::lock_guard<std::mutex> lk(b->mu);
     if (b->in_use + bytes > b->budget) {
@@ -1226,6 +1313,11 @@ gc_status gc_batch_destroy(gc_batch b) {
   for (auto& sb : b->small) free_small_bufs(&sb);
   for (auto* f : b->forks) fork_release(f);
   for (Launch* L : b->spare) free_launch(L);
+  if (b->check_stream) {
+    cudaStreamSynchronize(b->check_stream);
+    cudaStreamDestroy(b->check_stream);
+  }
+  if (b->check_bad) cudaFreeHost(b->check_bad);
   for (auto& s : b->streams) cudaStreamDestroy(s);
   delete b;
   return GC_OK;

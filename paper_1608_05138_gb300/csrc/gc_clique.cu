@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 512 ? 3 : 65536 / (kThre
 // lanes idle and waited on memory once per member), and an entry's place in out(a) is a 5-step
 // binary search over the lanes' ids (ascending). Pass K takes an edge of H_a
 // per lane. Both wait on chains of dependent loads, a unit at a time.
-// Chung-Lu 1M: pass T's kernel 1.92 -> 1.63 ms, pass K's 1.37 -> 0.43 ms.
+// Chung-Lu 1M: pass T's kernel 1.92 -> 1.36 ms, pass K's 1.37 -> 0.40 ms.
 // Same attribution as k_pass_k.
 constexpr int kWBlock = 256;
 constexpr int kWWarps = kWBlock / 32;

@@ -1,4 +1,5 @@
-// gc_deal.h -- runs of different lengths dealt to the lanes of a warp end to end.
+// gc_deal.h -- work of a warp dealt to its lanes: runs of different lengths end to
+// end, and the rows of consecutive CSR slots.
 #pragma once
 
 #include <stdint.h>
@@ -37,6 +38,22 @@ __device__ __forceinline__ int deal_owner(const Deal& d, int32_t L, int32_t k0, 
   const int r = before + __popc(M & (0xffffffffu >> (31 - lane))) - 1;
   before += __popc(M);
   return comp[r < 0 ? 0 : r];
+}
+
+// The row of slot p, one of 32 consecutive slots of a warp, p0 the first (the
+// whole warp calls): the warp's first and last rows by two searches of rp, the
+// lane's between them.
+__device__ __forceinline__ int32_t row_of_slot(int32_t n, const int32_t* __restrict__ rp, int32_t p0, int32_t p,
+                                               int32_t p_last) {
+  auto search = [&](int32_t lo, int32_t hi, int32_t q) {  // last row in [lo, hi] that starts at or before q
+    while (lo < hi) {
+      const int32_t mid = lo + ((hi - lo + 1) >> 1);
+      if (rp[mid] <= q) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+  };
+  const int32_t x0 = search(0, n - 1, p0);
+  return search(x0, search(x0, n - 1, p_last), p);
 }
 
 }  // namespace gc

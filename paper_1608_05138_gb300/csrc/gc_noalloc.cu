@@ -34,6 +34,7 @@
 #include <mutex>
 #include <string>
 
+#include "gc_deal.h"
 #include "gc_internal.h"
 
 namespace gc {
@@ -73,22 +74,6 @@ uint32_t* g_noalloc_ptr[kMaxDevices] = {};
 
 __device__ __forceinline__ bool row_bad(const uint32_t* scratch, int32_t x) {
   return (scratch[kOffBad + (x >> 5)] >> (x & 31)) & 1u;
-}
-
-// The row of slot p, one of 32 consecutive slots of a warp, p0 the first (the
-// whole warp calls): the warp's first and last rows by two searches of rp, the
-// lane's between them.
-__device__ __forceinline__ int32_t row_of_slot(int32_t n, const int32_t* __restrict__ rp, int32_t p0, int32_t p,
-                                               int32_t p_last) {
-  auto search = [&](int32_t lo, int32_t hi, int32_t q) {  // last row in [lo, hi] that starts at or before q
-    while (lo < hi) {
-      const int32_t mid = lo + ((hi - lo + 1) >> 1);
-      if (rp[mid] <= q) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-  };
-  const int32_t x0 = search(0, n - 1, p0);
-  return search(x0, search(x0, n - 1, p_last), p);
 }
 
 // Thread per slot: rows with a column out of range, a self-loop or two entries

@@ -303,6 +303,44 @@ def test_rows_of_common_neighbours(make):
     assert_parity(*make())
 
 
+@pytest.mark.parametrize("seed", range(6))
+def test_batch_submit_refuses_what_the_host_checks_refuse(seed):
+    # graphs large enough to be checked on the device: one corrupted entry gives
+    # the code and message of gc_validate_csr, an unchanged one is counted
+    rng = np.random.default_rng(seed)
+    rp, ci = graphgen.chung_lu(20000, 60000, 2.3, 120000.0, 3000.0, 90 + seed)
+    bad_rp, bad = rp.copy(), ci.copy()
+    x = int(rng.choice(np.flatnonzero(np.diff(rp) >= 3)))
+    p = int(rp[x]) + int(rng.integers(0, rp[x + 1] - rp[x]))
+    if seed == 0:
+        bad[p] = [-1, len(rp) - 1][int(rng.integers(0, 2))]
+    elif seed == 1:
+        bad[p] = x
+    elif seed == 2:
+        bad[rp[x] + 1] = bad[rp[x]]
+    elif seed == 3:
+        bad[rp[x]], bad[rp[x] + 1] = bad[rp[x] + 1], bad[rp[x]]
+    elif seed == 4:  # another neighbour, in order: (x, y) without (y, x)
+        free = np.setdiff1d(np.arange(len(rp) - 1), np.append(ci[rp[x]:rp[x + 1]], x))
+        bad[p] = free[int(rng.integers(0, len(free)))]
+        bad[rp[x]:rp[x + 1]].sort()
+    else:
+        bad_rp[x + 1] = bad_rp[x] - 1
+    with pytest.raises(gcb.GcError) as host:
+        gcb.gc_validate_csr(bad_rp, bad)
+    b = gcb.gc_batch_create(8 << 30, 0)
+    try:
+        with pytest.raises(gcb.GcError) as ei:
+            gcb.gc_batch_submit(b, bad_rp, bad)
+        assert ei.value.status == host.value.status
+        assert str(ei.value).split(": ", 2)[2] == str(host.value).split(": ", 2)[2]
+        X = gcb.gc_batch_poll(b, gcb.gc_batch_submit(b, rp, ci))
+    finally:
+        gcb.gc_batch_destroy(b)
+    with gcb.Graph(rp, ci) as g:
+        assert X == g.count()
+
+
 def test_hub_over_a_skewed_o_range():
     # 3M vertices, almost all isolated (the lowest ranks): h has 620 lower
     # neighbours, 600 of them with 150 o each, drawn with weights 1/(i + 100)

@@ -647,7 +647,7 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
   drop_temps();
   if (st != GC_OK) return fail(st);
   const int32_t zero = 0;
-  const RankInfo rank = {R.rp.data(), 1, &zero, &n, R.obound};
+  const RankInfo rank = {R.rp.data(), 1, &zero, &n, R.obound, nullptr, nullptr};
   st = prepare_graph(n, g->m, g->d_rp, g->d_ci, d_eid, d_perm, rank, &g->prep, s);
   d_eid = nullptr;  // owned by the preparation buffers from here on
   if (st != GC_OK) return fail(st);

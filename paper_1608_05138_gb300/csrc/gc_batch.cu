@@ -365,13 +365,13 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
     L->error = gc_last_error();
     return GC_ERR_NOMEM;
   }
-  const RankInfo rank = {h_rp.data(), G, gbase.data(), gn.data(), obound.data()};
   const size_t n1 = (size_t)n + 1, nnz1 = (size_t)(nnz_total > 0 ? nnz_total : 1);
   const size_t n_lists = mid.size() + longr.size();
   int32_t *d_rp = nullptr, *d_ci = nullptr, *d_vgid = nullptr, *d_desc = nullptr, *d_rp0 = nullptr, *d_ci0 = nullptr;
   int32_t *d_perm = nullptr, *d_newid = nullptr, *d_lists = nullptr;
   int64_t *d_gm = nullptr, *d_loff = nullptr;
   long long* d_tmp = nullptr;
+  RankInfo rank = RankInfo();
   PrepBuffers prep;
   Scratch sc;
   cudaError_t e = cudaSuccess;
@@ -420,6 +420,7 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
   GB_TRY(up(d_lists, mid.data(), mid.size()), "batch copy");
   GB_TRY(up(d_lists + mid.size(), longr.data(), longr.size()), "batch copy");
   GB_TRY(up(d_loff, long_off.data(), long_off.size()), "batch copy");
+  rank = {h_rp.data(), G, gbase.data(), gn.data(), obound.data(), d_vgid, d_desc};
   if ((st = relabel_on_device(n, m, d_rp0, d_ci0, d_perm, d_newid, d_rp, d_ci, nullptr, d_vgid, d_desc, d_lists,
                               (int32_t)mid.size(), d_lists + mid.size(), d_loff, (int32_t)longr.size(), d_tmp, s)) !=
           GC_OK ||

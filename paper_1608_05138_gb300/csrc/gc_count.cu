@@ -673,7 +673,7 @@ __global__ void __launch_bounds__(kDenseBlock) k_cliques_dense(DevGraph g, Count
 // width took 31 to 94, so that a run has 100 entries instead of 16 (sweeps of
 // (x, block) 2.2e9 -> 4.4e8), and the segments' bounds in every longer row
 // are looked up in a table made once per graph instead of searched. The
-// whole kernel: 180 -> 128 ms there; 8.5 -> 6.4 ms on Chung-Lu 1M, where
+// whole kernel: 180 -> 127 ms there; 8.5 -> 5.6 ms on Chung-Lu 1M, where
 // about a quarter of the warps' time is still the barrier between a block's
 // two phases, and the shared-memory pipe, with three-way bank conflicts of
 // random counters, is busy half of the time.

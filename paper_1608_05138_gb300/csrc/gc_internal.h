@@ -393,6 +393,8 @@ struct RankInfo {
   const int32_t* gbase;   // [G] first id of each, ascending
   const int32_t* gn;      // [G] vertices of each
   const int32_t* obound;  // [G][kOBounds] first id of degree >= kOBoundDeg[k] (the graph's end if none)
+  const int32_t* d_vgid;  // on the device: graph of every vertex, and gbase; nullptr for one graph
+  const int32_t* d_gbase;
 };
 // Whether some pass-C units are left for the vertex-indexed tables.
 inline bool needs_tables(const PrepBuffers& p) { return p.n_cunits > p.n_cheavy + p.n_chash + p.n_chash2; }
@@ -498,17 +500,18 @@ constexpr int kHeavyTab = 53248;  // largest o-range block of the hub kernel of 
 // Words of the hub kernel's count block (environment GC_HUB_TAB_WORDS, a
 // multiple of 1024 in [4096, kHeavyTab], else kHubTabDefault), read once per
 // process. The block and the SM's L1 cache share one array, split in steps
-// (the shared-memory carveout); kHubTabDefault is the largest block whose CTA
-// (block + 16.4 KB of static arrays + 1 KB reserved) fits the 196 KB step,
-// leaving about 60 KB of L1 for the rows and cursors instead of 28 KB with a
-// 208 KB block (R-MAT scale 22: pass C 228.4 ms at 53248 words, 205.0 at
-// 45056, 213.3 at 39936, 226.7 at 32768).
+// (the shared-memory carveout); kHubTabDefault with the kernel's 8.2 KB of
+// static arrays and 1 KB reserved fits the 196 KB step, leaving about 60 KB of
+// L1 for the rows instead of 28 KB with a 208 KB block (R-MAT scale 22, when
+// blocks had one counter width: pass C 228.4 ms at 53248 words, 205.0 at 45056,
+// 213.3 at 39936, 226.7 at 32768; now 139 at 45056 and at 47104, the largest
+// that fits).
 constexpr int kHubTabDefault = 45056;
 int hub_tab_words();
 // Counters per word that a unit of nx lower neighbours could use over its
 // whole o-range by nx alone; the rule that picks the hub units estimates
 // their blocks with it.
-inline int hub_cpw(int64_t nx) { return nx < 1023 ? 3 : nx < 65536 ? 2 : 1; }
+__host__ __device__ __forceinline__ int hub_cpw(int64_t nx) { return nx < 1023 ? 3 : nx < 65536 ? 2 : 1; }
 // Units of pass C with at most kHashMaxW wedges count in a shared-memory
 // hash of 2 kHashMaxW keys (at most half full: a unit has no more distinct
 // o than wedges).

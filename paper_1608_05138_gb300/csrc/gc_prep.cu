@@ -149,10 +149,10 @@ __device__ __forceinline__ int unit_bin(int key, int32_t d) {
   return key == 0 ? bin_of((long long)d * d) : (key == 1 ? bin_of(d) : 0);
 }
 
-// Counts, or (kScatter) lists by bin from cursor[], the v-groups: one atomic a
-// block and bin.
-template <int kBins, bool kScatter, class Bin>
-__device__ __forceinline__ void bin_vertices(int32_t n, int32_t* __restrict__ cursor, int32_t* __restrict__ list, Bin bin) {
+// Counts, or (kScatter) puts at places by bin from cursor[], the items 0 .. n - 1
+// (bin < 0: left out): one atomic a block and bin.
+template <int kBins, bool kScatter, class Bin, class Put>
+__device__ __forceinline__ void bin_vertices(int32_t n, int32_t* __restrict__ cursor, Bin bin, Put put) {
   __shared__ int32_t h[kBins], base[kBins];
   for (int32_t v0 = blockIdx.x * blockDim.x; v0 < n; v0 += gridDim.x * blockDim.x) {
     for (int i = threadIdx.x; i < kBins; i += blockDim.x) h[i] = 0;
@@ -165,7 +165,7 @@ __device__ __forceinline__ void bin_vertices(int32_t n, int32_t* __restrict__ cu
     for (int i = threadIdx.x; i < kBins; i += blockDim.x)
       if (h[i]) base[i] = atomicAdd(&cursor[i], h[i]);
     __syncthreads();
-    if (kScatter && b >= 0) list[base[b] + at] = v;
+    if (kScatter && b >= 0) put(base[b] + at, v);
     __syncthreads();
   }
 }
@@ -173,9 +173,9 @@ template <bool kScatter>
 __global__ void __launch_bounds__(1024) k_bin_units(int32_t n, const int32_t* __restrict__ deg,
                                                     const int32_t* __restrict__ out_cnt, int32_t* __restrict__ cursor,
                                                     int32_t* __restrict__ units, int key) {
-  bin_vertices<64, kScatter>(n, cursor, units, [&](int32_t v) {
-    return deg[v] - out_cnt[v] > 0 ? unit_bin(key, deg[v]) : -1;
-  });
+  bin_vertices<64, kScatter>(
+      n, cursor, [&](int32_t v) { return deg[v] - out_cnt[v] > 0 ? unit_bin(key, deg[v]) : -1; },
+      [&](int32_t at, int32_t v) { units[at] = v; });
 }
 
 // Pass K units: every vertex a with |out(a)| = k >= 2 (a triangle needs two
@@ -187,22 +187,55 @@ __device__ __forceinline__ int kbin_of(int32_t k) { return 32 - __clz(k - 1); }
 template <bool kScatter>
 __global__ void __launch_bounds__(1024) k_bin_kunits(int32_t n, const int32_t* __restrict__ out_cnt,
                                                      int32_t* __restrict__ cursor, int32_t* __restrict__ units) {
-  bin_vertices<32, kScatter>(n, cursor, units, [&](int32_t v) { return out_cnt[v] >= 2 ? kbin_of(out_cnt[v]) : -1; });
+  bin_vertices<32, kScatter>(
+      n, cursor, [&](int32_t v) { return out_cnt[v] >= 2 ? kbin_of(out_cnt[v]) : -1; },
+      [&](int32_t at, int32_t v) { units[at] = v; });
 }
 
-// Wedges of every pass-C unit h of a ranked graph: W_h = sum over the
-// lower-rank neighbours x of h of |{o in Gamma(x) : o < h}| (warp per unit).
-// Wedges W and lower neighbours NX of every pass-C unit h of a ranked graph.
-// Ids are ranks and rows ascend, so the o < h of Gamma(x) are the entries
-// before the slot of (x, h), the reverse of the slot of (h, x): no search per
-// lower neighbour (the reverse is clamped into the row, as the hub kernel does,
-// so that W is what the kernels count even before symmetry is checked).
-__global__ void k_cwork(int32_t n_units, const int32_t* __restrict__ units, const int32_t* __restrict__ rp,
-                        const int32_t* __restrict__ ci, const int32_t* __restrict__ rev, long long* __restrict__ W,
-                        int32_t* __restrict__ NX) {
+// Pass-C units by kernel and wedges W: eight bins to a factor of two of W - 1
+// (so that 512, 2048 and 8192 wedges end bins), for the hash, the two instances
+// of the packed-key hash, and one bin for the vertex-indexed tables.
+constexpr int kHashBins = 88, kHash2Bins = 24;
+constexpr int kBinHalf = kHashBins, kBinBig = kBinHalf + kHash2Bins, kBinRest = kBinBig + kHash2Bins;
+constexpr int kCBins = kBinRest + 1;
+__host__ __device__ __forceinline__ int wedge_bin(int32_t w) {  // 1 <= w <= kHash2MaxW
+  const int32_t v = w - 1;
+  if (v < 8) return v;
+  int o = 3;
+  while ((v >> (o + 1)) != 0) ++o;
+  return 8 * (o - 2) + ((v >> (o - 3)) & 7);
+}
+struct HubUnit {
+  int32_t h, nx;
+  long long w;
+};
+
+// Warp per unit h: its lower neighbours nx and wedges W = sum over them, x, of
+// |{o in Gamma(x) : o < h}|. Ids are ranks and rows ascend, so the o < h of
+// Gamma(x) are the entries before the slot of (x, h), the reverse of the slot of
+// (h, x): no search per lower neighbour (the reverse is clamped into the row, as
+// the hub kernel does, so that W is what the kernels count even before symmetry
+// is checked). Then the unit's kernel: a hub unit pays, per shared-memory block
+// of the o-range, a few microseconds of barriers (more when it has more than a
+// CTA's worth of lower neighbours), against roughly 10 ns per wedge on an SM
+// for a wedge on a vertex-indexed table in DRAM, so the hub kernel is taken
+// when the wedges exceed blocks x max(1024, nx), tested from 16384 wedges, after
+// both hashes have taken what fits them. Hub units are listed for the host, the
+// others get their bin; units without wedges add nothing to P and are left out
+// (bin -1). (The host used to make these lists from W and nx of every unit: 3 ms
+// of an upload of R-MAT scale 20.)
+__global__ void __launch_bounds__(256) k_cwork(int32_t n_units, const int32_t* __restrict__ units,
+                                               const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                               const int32_t* __restrict__ rev, const int32_t* __restrict__ vgid,
+                                               const int32_t* __restrict__ gbase, int32_t tab, bool packed,
+                                               int32_t* __restrict__ bin, int32_t* __restrict__ hw,
+                                               int32_t* __restrict__ hist, HubUnit* __restrict__ hubs) {
+  __shared__ int32_t s_hist[kCBins];
+  for (int i = threadIdx.x; i < kCBins; i += 256) s_hist[i] = 0;
+  __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n_units; k += warps) {
+  const int warps = (gridDim.x * 256) >> 5;
+  for (int32_t k = (int32_t)((blockIdx.x * 256 + threadIdx.x) >> 5); k < n_units; k += warps) {
     const int32_t h = units[k];
     const int32_t hb = rp[h];
     const int32_t nx = lower_bound_i32(ci, hb, rp[h + 1], h) - hb;
@@ -213,11 +246,42 @@ __global__ void k_cwork(int32_t n_units, const int32_t* __restrict__ units, cons
       w += min(max(rev[hb + i], xb), rp[x + 1]) - xb;
     }
     for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    if (lane == 0) {
-      W[k] = w;
-      NX[k] = nx;
+    if (lane != 0) continue;
+    int b = -1;
+    if (w > 0 && w <= kHashMaxW) {
+      b = wedge_bin((int32_t)w);
+    } else if (w > 0 && w <= kHash2MaxW && nx < kHash2MaxNx && packed) {
+      b = (w > kHash2HalfMaxW ? kBinBig : kBinHalf) + wedge_bin((int32_t)w) - kHashBins;
+    } else if (w > 0) {
+      b = kBinRest;
+      if (w >= 16384 && nx < (1 << 26)) {
+        const long long span = (long long)hub_cpw(nx) * tab;
+        const long long blocks = ((long long)(h - (vgid ? gbase[vgid[h]] : 0)) + span - 1) / span;
+        if (w >= blocks * (nx > 1024 ? nx : 1024)) {
+          b = -1;
+          hubs[atomicAdd(hist + kCBins, 1)] = {h, nx, w};
+        }
+      }
     }
+    bin[k] = b;
+    hw[k] = (int32_t)min(w, (long long)0x7fffffff);
+    if (b >= 0) atomicAdd(&s_hist[b], 1);
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kCBins; i += 256)
+    if (s_hist[i]) atomicAdd(hist + i, s_hist[i]);
+}
+
+__global__ void __launch_bounds__(1024) k_cscatter(int32_t n_units, const int32_t* __restrict__ units,
+                                                   const int32_t* __restrict__ bin, const int32_t* __restrict__ hw,
+                                                   int32_t* __restrict__ cursor, int32_t n_hubs, int32_t n_hashed,
+                                                   int32_t* __restrict__ cunits, int32_t* __restrict__ chash_w) {
+  bin_vertices<kCBins, true>(
+      n_units, cursor, [&](int32_t k) { return bin[k]; },
+      [&](int32_t at, int32_t k) {
+        cunits[n_hubs + at] = units[k];
+        if (at < n_hashed) chash_w[at] = hw[k];
+      });
 }
 
 // DevGraph::hpos: a row of CTAs per graph, thread per (row, bound).
@@ -411,22 +475,6 @@ static int hub_jobs_per_cta() {
   return v;
 }
 
-// The units of v (wedge counts W[v[i]] in [1, wmax]) in descending W, equal W
-// in their order in v: a counting sort.
-static void sort_by_wedges_desc(std::vector<int32_t>* v, const std::vector<long long>& W, long long wmax) {
-  std::vector<int32_t> cnt((size_t)wmax + 2, 0);
-  for (int32_t k : *v) cnt[(size_t)(wmax - W[k])]++;
-  int32_t r = 0;
-  for (auto& c : cnt) {
-    const int32_t x = c;
-    c = r;
-    r += x;
-  }
-  std::vector<int32_t> out(v->size());
-  for (int32_t k : *v) out[(size_t)cnt[(size_t)(wmax - W[k])]++] = k;
-  v->swap(out);
-}
-
 gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, const RankInfo& rank, PrepBuffers* p,
                            cudaStream_t s) {
   const int32_t nu = p->n_units;
@@ -448,84 +496,63 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
     e = nu > 0 ? cudaMemcpyAsync(p->cunits, p->units, sizeof(int32_t) * nu, cudaMemcpyDeviceToDevice, s) : cudaSuccess;
     return e == cudaSuccess ? GC_OK : cuda_fail(e, "copy cunits");
   }
-  long long* dW = nullptr;
-  int32_t* dNX = nullptr;
-  std::vector<long long> W(nu);
-  std::vector<int32_t> NX(nu), U(nu), out;
-  e = pool_alloc(&dW, sizeof(long long) * nu, s);
-  if (e == cudaSuccess) e = pool_alloc(&dNX, sizeof(int32_t) * nu, s);
+  const long long tab = hub_tab_words();
+  const int sms = count_grid_size() / kCtasPerSm;
+  HubUnit* d_hubs = nullptr;  // room for every unit; then the bins, the wedges and the histogram
+  std::vector<HubUnit> heavy;
+  int32_t hist[kCBins + 1];
+  const size_t nu1 = (size_t)nu;
+  e = pool_alloc(&d_hubs, sizeof(HubUnit) * nu1 + sizeof(int32_t) * (2 * nu1 + kCBins + 1), s);
+  if (e != cudaSuccess) return cuda_fail(e, "classify pass-C units");
+  int32_t* d_bin = reinterpret_cast<int32_t*>(d_hubs + nu1);
+  int32_t *d_w = d_bin + nu1, *d_hist = d_w + nu1;
+  e = cudaMemsetAsync(d_hist, 0, sizeof(hist), s);
   if (e == cudaSuccess) {
-    k_cwork<<<grid_for((int64_t)nu * 32, 256), 256, 0, s>>>(nu, p->units, d_rp, d_ci, p->rev, dW, dNX);
+    k_cwork<<<std::min(grid_for((int64_t)nu * 32, 256), 8 * sms), 256, 0, s>>>(
+        nu, p->units, d_rp, d_ci, p->rev, rank.d_vgid, rank.d_gbase, (int32_t)tab, largest <= kHash2MaxN, d_bin, d_w,
+        d_hist, d_hubs);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(W.data(), dW, sizeof(long long) * nu, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(NX.data(), dNX, sizeof(int32_t) * nu, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(U.data(), p->units, sizeof(int32_t) * nu, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hist, d_hist, sizeof(hist), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (dW) cudaFreeAsync(dW, s);
-  if (dNX) cudaFreeAsync(dNX, s);
+  // hub units heaviest first, then the hashed units, the packed-key hash units
+  // of the whole and of half tables, each by bins heaviest first, and the rest
+  if (e == cudaSuccess) {
+    int32_t cursor[kCBins], at = 0;
+    auto place = [&](int b) {
+      cursor[b] = at;
+      at += hist[b];
+    };
+    for (int b = kHashBins - 1; b >= 0; --b) {
+      place(b);
+      if (b == wedge_bin(kHashMidW + 1)) p->n_chash_mid = at;
+      if (b == wedge_bin(kHashSmallW + 1)) p->n_chash_big = at;
+    }
+    p->n_chash = at;
+    for (int b = kBinRest - 1; b >= kBinBig; --b) place(b);
+    p->n_chash2_big = at - p->n_chash;
+    for (int b = kBinBig - 1; b >= kBinHalf; --b) place(b);
+    p->n_chash2 = at - p->n_chash;
+    const int32_t n_hashed = at;
+    place(kBinRest);
+    p->n_cheavy = hist[kCBins];
+    p->n_cunits = p->n_cheavy + at;
+    heavy.resize((size_t)p->n_cheavy);
+    if (n_hashed > 0) e = pool_alloc(&p->chash_w, sizeof(int32_t) * (size_t)n_hashed, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_hist, cursor, sizeof(cursor), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && at > 0) {
+      k_cscatter<<<std::min(grid_for(nu, 1024), 2 * sms), 1024, 0, s>>>(nu, p->units, d_bin, d_w, d_hist, p->n_cheavy,
+                                                                        n_hashed, p->cunits, p->chash_w);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess && !heavy.empty())
+      e = cudaMemcpyAsync(heavy.data(), d_hubs, sizeof(HubUnit) * heavy.size(), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  }
+  cudaFreeAsync(d_hubs, s);
   if (e != cudaSuccess) return cuda_fail(e, "classify pass-C units");
-  // A hub unit pays, per shared-memory block of the o-range, a few
-  // microseconds of barriers and cursor searches (more when it has more than
-  // a CTA's worth of lower neighbours), against roughly 10 ns per wedge on an
-  // SM for a wedge that goes through the vertex-indexed table in DRAM; the
-  // hub kernel is taken when the wedges exceed blocks x max(1024, nx), about
-  // three times the break-even point. One pass over the units, in unit
-  // order: the packed-key hash takes every unit it fits; the hub rule is
-  // tested (with its division) only from 16384 wedges; units without wedges
-  // add nothing to P and are left out.
-  std::vector<int32_t> heavy, hashed, hashed2, rest;
-  const long long tab = hub_tab_words();
-  for (int32_t k = 0; k < nu; ++k) {
-    const long long w = W[k];
-    if (w <= 0) continue;
-    if (w <= kHashMaxW) {
-      hashed.push_back(k);
-      continue;
-    }
-    if (w <= kHash2MaxW && NX[k] < kHash2MaxNx && largest <= kHash2MaxN) {
-      hashed2.push_back(k);
-      continue;
-    }
-    if (w >= 16384 && NX[k] < (1 << 26)) {
-      const long long span = (long long)hub_cpw(NX[k]) * tab;
-      const long long blocks = ((long long)(U[k] - rank.gbase[graph_of(U[k])]) + span - 1) / span;
-      const long long per_block = NX[k] > 1024 ? NX[k] : 1024;
-      if (w >= blocks * per_block) {
-        heavy.push_back(k);
-        continue;
-      }
-    }
-    rest.push_back(k);
-  }
-  // hub units heaviest first, then the hashed units heaviest first, the
-  // packed-key hash units heaviest first, and the rest in unit order
-  std::sort(heavy.begin(), heavy.end(), [&](int32_t a, int32_t b) { return W[a] > W[b]; });
-  sort_by_wedges_desc(&hashed, W, kHashMaxW);
-  sort_by_wedges_desc(&hashed2, W, kHash2MaxW);
-  out.reserve(heavy.size() + hashed.size() + hashed2.size() + rest.size());
-  std::vector<int32_t> hw;
-  hw.reserve(hashed.size() + hashed2.size());
-  for (int32_t k : heavy) out.push_back(U[k]);
-  for (int32_t k : hashed) {
-    out.push_back(U[k]);
-    hw.push_back((int32_t)W[k]);
-  }
-  for (int32_t k : hashed2) {
-    out.push_back(U[k]);
-    hw.push_back((int32_t)W[k]);
-  }
-  for (int32_t k : rest) out.push_back(U[k]);
-  p->n_cheavy = (int32_t)heavy.size();
-  p->n_chash = (int32_t)hashed.size();
-  p->n_chash_big = 0;  // hashed is heaviest first
-  while (p->n_chash_big < p->n_chash && W[hashed[(size_t)p->n_chash_big]] > kHashSmallW) ++p->n_chash_big;
-  p->n_chash_mid = 0;
-  while (p->n_chash_mid < p->n_chash_big && W[hashed[(size_t)p->n_chash_mid]] > kHashMidW) ++p->n_chash_mid;
-  p->n_chash2 = (int32_t)hashed2.size();
-  p->n_chash2_big = 0;  // heaviest first too
-  while (p->n_chash2_big < p->n_chash2 && W[hashed2[(size_t)p->n_chash2_big]] > kHash2HalfMaxW) ++p->n_chash2_big;
-  p->n_cunits = (int32_t)out.size();
+  std::sort(heavy.begin(), heavy.end(),
+            [](const HubUnit& a, const HubUnit& b) { return a.w != b.w ? a.w > b.w : a.h < b.h; });
   // The hub kernel's o-range (see HubSeg): per graph, segment by segment, the
   // counter width that reaches furthest (the wider one at equal reach): to the
   // end of the ids whose degree fits it, or of the block. A block is closed when
@@ -600,19 +627,19 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
     std::vector<double> cost(heavy.size());
     double total = 0;
     for (size_t i = 0; i < heavy.size(); ++i) {
-      const int32_t k = heavy[i];
-      const HubGeom& ge = geom_of(U[k]);
-      cost[i] = (double)W[k] + kSweepCost * (double)NX[k] * (double)(seg_of(ge, U[k]) - ge.seg + 1);
+      const HubUnit& k = heavy[i];
+      const HubGeom& ge = geom_of(k.h);
+      cost[i] = (double)k.w + kSweepCost * (double)k.nx * (double)(seg_of(ge, k.h) - ge.seg + 1);
       total += cost[i];
     }
     const double target = per_cta > 0 ? total / ((double)(count_grid_size() / kCtasPerSm) * per_cta) : 0.0;
     std::vector<std::pair<double, int4>> cj;
     for (size_t i = 0; i < heavy.size(); ++i) {
-      const int32_t h = U[heavy[i]];
+      const int32_t h = heavy[i].h;
       const HubGeom& ge = geom_of(h);
       const int32_t lo = ge.nseg > 0 ? std::min(segs[(size_t)ge.seg].lo, h) : h;
       long long J = target > 0 ? (long long)std::ceil(cost[i] / target) : 1;
-      J = std::max(1LL, std::min(J, W[heavy[i]] / std::max(kJobWedges, 8LL * NX[heavy[i]])));
+      J = std::max(1LL, std::min(J, heavy[i].w / std::max(kJobWedges, 8LL * heavy[i].nx)));
       int32_t from = lo;
       for (long long j = 1; j <= J; ++j) {
         const long long upto = rank.rp[lo] + (long long)(rank.rp[h] - rank.rp[lo]) * j / J;
@@ -648,11 +675,10 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
     if (e == cudaSuccess) e = cudaMemcpyAsync(p->cjobs, jobs.data(), sizeof(int4) * jobs.size(), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(e, "hub jobs");
   }
+  std::vector<int32_t> out;
+  out.reserve(heavy.size());
+  for (const HubUnit& k : heavy) out.push_back(k.h);
   if (!out.empty()) e = cudaMemcpyAsync(p->cunits, out.data(), sizeof(int32_t) * out.size(), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && !hw.empty()) {
-    e = pool_alloc(&p->chash_w, sizeof(int32_t) * hw.size(), s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(p->chash_w, hw.data(), sizeof(int32_t) * hw.size(), cudaMemcpyHostToDevice, s);
-  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "copy cunits");
 }

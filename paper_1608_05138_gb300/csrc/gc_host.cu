@@ -30,24 +30,22 @@ struct Job {
 
 class Pool {
  public:
-  Pool() : pid_(getpid()), threads_(new std::vector<std::thread>()) {
+  Pool() : pid_(getpid()), threads_() {
     for (int t = 1; t < host_threads(); ++t) {
       try {
-        threads_->emplace_back([this] { work(); });
+        threads_.emplace_back([this] { work(); });
       } catch (...) {
         break;  // fewer threads
       }
     }
   }
   ~Pool() {
-    if (getpid() != pid_) return;  // a forked child has none of the threads (the vector is left alone)
     {
       std::lock_guard<std::mutex> lk(mu_);
       stop_ = true;
     }
     cv_.notify_all();
-    for (auto& t : *threads_) t.join();
-    delete threads_;
+    for (auto& t : threads_) t.join();
   }
   bool usable() const { return getpid() == pid_; }
 
@@ -59,8 +57,8 @@ class Pool {
       std::lock_guard<std::mutex> lk(mu_);
       jobs_.push_back(&job);
     }
-    const int want = std::min<int>(n - 1, (int)threads_->size());
-    if (want >= (int)threads_->size()) cv_.notify_all();
+    const int want = std::min<int>(n - 1, (int)threads_.size());
+    if (want >= (int)threads_.size()) cv_.notify_all();
     else
       for (int k = 0; k < want; ++k) cv_.notify_one();
     take(&job);
@@ -105,12 +103,33 @@ class Pool {
   }
 
   const pid_t pid_;
-  std::vector<std::thread>* threads_;
+  std::vector<std::thread> threads_;
   std::mutex mu_;
   std::condition_variable cv_, done_;
   std::deque<Job*> jobs_;
   bool stop_ = false;
 };
+
+// The process's pool. A forked child has the object but none of its threads: it
+// starts a pool of its own and leaves the parent's as it is (destroying it
+// would wait for threads that the child does not have).
+std::atomic<Pool*> g_pool{nullptr};
+
+Pool* pool() {
+  Pool* p = g_pool.load();
+  if (p && p->usable()) return p;
+  Pool* mine = new Pool();
+  if (g_pool.compare_exchange_strong(p, mine)) return mine;
+  delete mine;  // another thread was first
+  return p;
+}
+
+struct AtExit {
+  ~AtExit() {
+    Pool* p = g_pool.exchange(nullptr);
+    if (p && p->usable()) delete p;
+  }
+} g_at_exit;
 
 }  // namespace
 
@@ -124,11 +143,8 @@ int host_threads() {
 
 void host_run(int n, const std::function<void(int)>& f) {
   if (n > 1) {
-    static Pool pool;
-    if (pool.usable()) {
-      pool.run(n, f);
-      return;
-    }
+    pool()->run(n, f);
+    return;
   }
   for (int i = 0; i < n; ++i) f(i);
 }

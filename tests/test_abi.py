@@ -3,6 +3,8 @@ include/gc.h declares; host-side CSR validation returns the documented error
 codes before any device work (no GPU needed)."""
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -268,3 +270,32 @@ def test_validate_csr_extra_entry_names_the_entry_without_reverse(lib):
     with pytest.raises(gcb.GcError) as ei:
         gcb.gc_validate_csr(np.array([0, 1, 2, 3], np.int32), np.array([1, 2, 1], np.int32))
     assert ei.value.status == -5 and str(ei.value).endswith("row_ptr[n] is odd: the graph cannot be symmetric")
+
+
+def test_host_threads_survive_a_fork(lib):
+    """After a call that started the library's host threads, a forked child can
+    call it again and exit: it must not wait for threads that it does not have."""
+    code = """
+import os, sys, time
+import numpy as np
+import paper_1608_05138_gb300 as gc
+n = 1 << 22  # a cycle: 2^23 entries, enough for several host threads
+v = np.arange(n, dtype=np.int64)
+ci = np.sort(np.stack([(v - 1) % n, (v + 1) % n], axis=1), axis=1).astype(np.int32).ravel()
+rp = np.arange(0, 2 * n + 1, 2, dtype=np.int32)
+gc.gc_validate_csr(rp, ci)
+pid = os.fork()
+if pid == 0:
+    gc.gc_validate_csr(rp, ci)
+    sys.exit(7)
+end = time.time() + 60
+while time.time() < end:
+    p, status = os.waitpid(pid, os.WNOHANG)
+    if p:
+        sys.exit(0 if os.waitstatus_to_exitcode(status) == 7 else 1)
+    time.sleep(0.05)
+os.kill(pid, 9)
+os.waitpid(pid, 0)
+sys.exit(2)
+"""
+    assert subprocess.run([sys.executable, "-c", code], cwd=ROOT, timeout=120).returncode == 0

@@ -231,7 +231,10 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_tri_long(int32_t n, const int
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t* cnt = s_cnt[warp];
   const uint32_t n_long = min(scratch[kNumLong], kMaxParts);
-  auto in = [&](int32_t w) -> bool { return (bm[w >> 5] >> (w & 31)) & 1u; };
+  // Bounds are checked although the listed rows follow the rules: calls that
+  // overlap on the GPU share the scratch array, and may then list rows and miss
+  // marks of each other's graphs.
+  auto in = [&](int32_t w) -> bool { return w < n && ((bm[w >> 5] >> (w & 31)) & 1u); };
   for (int32_t i = threadIdx.x; i < (n + 31) / 32; i += kNoAllocBlock) bm[i] = 0u;
   for (;;) {
     __syncthreads();
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_tri_long(int32_t n, const int
     __syncthreads();
     if (s_x == kNoPart) break;
     const int32_t x = (int32_t)(s_x & 0xfffffu), part = (int32_t)(s_x >> 20);
-    if (row_bad(scratch, x)) continue;
+    if (x >= n || row_bad(scratch, x)) continue;
     const int32_t b = rp[x], e = rp[x + 1];
     const int32_t pe = min(e, b + (part + 1) * kPart);
     if (threadIdx.x == 0) {
@@ -255,7 +258,7 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_tri_long(int32_t n, const int
     }
     for (int32_t p = b + threadIdx.x; p < e; p += kNoAllocBlock) {
       const int32_t y = ci[p];
-      atomicOr(&bm[y >> 5], 1u << (y & 31));
+      if ((uint32_t)y < (uint32_t)n) atomicOr(&bm[y >> 5], 1u << (y & 31));
     }
     __syncthreads();
     for (;;) {
@@ -299,7 +302,10 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_tri_long(int32_t n, const int
     }
     __syncthreads();
     for (int32_t k = threadIdx.x; k < heavy; k += kNoAllocBlock) tri[s_hp[k]] = s_hc[k];
-    for (int32_t p = b + threadIdx.x; p < e; p += kNoAllocBlock) bm[ci[p] >> 5] = 0u;
+    for (int32_t p = b + threadIdx.x; p < e; p += kNoAllocBlock) {
+      const int32_t y = ci[p];
+      if ((uint32_t)y < (uint32_t)n) bm[y >> 5] = 0u;
+    }
   }
 }
 
@@ -318,7 +324,7 @@ __global__ void __launch_bounds__(kTriBlock) k_tri_reverse(int32_t n, const int3
     if (p >= nnz) continue;
     const int32_t y = ci[q], dx = rp[x + 1] - rp[x];
     bool found = false;
-    if (!row_bad(scratch, x) && !row_bad(scratch, y)) {  // a row that follows the rules has its columns in range
+    if ((uint32_t)y < (uint32_t)n && !row_bad(scratch, x) && !row_bad(scratch, y)) {
       const int32_t yb = rp[y], ye = rp[y + 1], dy = ye - yb;
       if (dy < dx || (dy == dx && y < x)) continue;  // counted at this slot
       int32_t lo = yb, hi = ye;

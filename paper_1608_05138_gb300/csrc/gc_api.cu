@@ -131,12 +131,27 @@ void fork_release(ForkSet* f) {
   if (!f) return;
   {
     std::lock_guard<std::mutex> lk(g_fork_mu);
-    if (g_forks.size() < kForksKept) {
-      g_forks.push_back(f);
-      return;
+    try {
+      if (g_forks.size() < kForksKept) {
+        g_forks.push_back(f);
+        return;
+      }
+    } catch (...) {  // no memory to keep it
     }
   }
   fork_destroy(f);
+}
+
+// The idle sets of the current device, given back.
+void fork_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  std::lock_guard<std::mutex> lk(g_fork_mu);
+  for (size_t i = g_forks.size(); i-- > 0;)
+    if (g_forks[i]->device == dev) {
+      fork_destroy(g_forks[i]);
+      g_forks.erase(g_forks.begin() + (long)i);
+    }
 }
 
 namespace {
@@ -917,6 +932,7 @@ gc_status gc_release_cached_memory(void) {
   }
   cudaError_t e = cudaDeviceSynchronize();  // every stream-ordered free has reached the pool
   if (e == cudaSuccess) e = cudaMemPoolTrimTo(pool, 0);
+  fork_trim();
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "gc_release_cached_memory");
 }
 

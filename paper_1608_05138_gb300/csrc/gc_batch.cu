@@ -90,6 +90,7 @@ struct HostCache {
   static constexpr size_t kLargeEntries = (size_t)16 << 20;
   std::mutex mu;
   std::vector<HostBlock> free;
+  HostCache() { free.reserve(kLarge + kSmall + 1); }  // a returned block never allocates
   ~HostCache() {
     for (auto& h : free) free_block(h);
   }

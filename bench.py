@@ -96,7 +96,9 @@ def algorithmic_bytes(work: dict) -> dict:
               triangle (4-byte read-modify-write of |T| of the found edge)
       pass C: 20 per wedge h-x-o (the CSR entry o, and the 8-byte
               read-modify-write of the 4-cycle count of its slot; the
-              wedge counts cnt_h(o) stay on chip)
+              wedge counts cnt_h(o) stay on chip); 4 per list entry read
+              where rows of common neighbours take the place of passes T and
+              C (graphs of at most 4096 vertices: no t_members)
       pass K: 48 per member of out(a) (id, |T|, out-list bounds, two 8-byte
               read-modify-write flushes), 4 per out-list entry scanned, 36 per
               edge of H_a (|T| gather, two 8-byte read-modify-write atomics)
@@ -104,7 +106,7 @@ def algorithmic_bytes(work: dict) -> dict:
               both slots, x7, cross; 104 written: the 13-column row)"""
     return {
         "k_pass_t": 20 * work["t_members"] + 4 * work["t_scan"] + 8 * work["t_triangles"],
-        "k_pass_c": 20 * work["c_wedges"],
+        "k_pass_c": (20 if work["t_members"] else 4) * work["c_wedges"],
         "k_pass_k": 48 * work["k_members"] + 4 * work["k_scan"] + 36 * work["k_local_edges"],
         "k_finish": 168 * work["finish_edges"],
     }

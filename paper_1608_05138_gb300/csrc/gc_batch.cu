@@ -66,6 +66,15 @@ __global__ void __launch_bounds__(256) k_check_csr(int32_t n, int32_t nnz, const
   if (!ok) *bad = 1;
 }
 
+// Submitting is allowed while the calling thread captures one of its own
+// streams: pinning and the device check use other streams, so that they may run
+// then, which the runtime wants to be told.
+struct OutsideCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The library's host copy of one submission, pinned where possible, so that a
 // launch copies it to the device directly.
 struct HostBlock {
@@ -124,6 +133,7 @@ std::shared_ptr<HostBlock> host_block(const std::shared_ptr<HostCache>& cache, s
   }
   if (!h.p) {
     h.cap = entries + entries / 8;
+    OutsideCapture relaxed;
     if (cudaHostAlloc(reinterpret_cast<void**>(&h.p), sizeof(int32_t) * h.cap, cudaHostAllocPortable) == cudaSuccess) {
       h.pinned = true;
     } else {
@@ -912,6 +922,7 @@ void poll_wait(gc_batch b, std::unique_lock<std::mutex>* lk, std::chrono::steady
 // checked. false also when a device step fails: the caller then asks the host.
 static bool checked_on_device(gc_batch b, int32_t n, int32_t nnz, const int32_t* own) {
   std::lock_guard<std::mutex> lk(b->check_mu);
+  OutsideCapture relaxed;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || (dev != b->device && cudaSetDevice(b->device) != cudaSuccess)) {
     cudaGetLastError();

@@ -697,6 +697,29 @@ def test_batch_rejects_asymmetric_graph_and_keeps_the_others():
     assert res == [_oracle_X(*g) for g in good]
 
 
+def test_batch_submit_while_the_thread_captures():
+    """Submitting pins memory and checks on the device, on streams of its own:
+    a capture that the calling thread has under way goes on."""
+    import torch
+    big = graphgen.er(3000, 0.01, 74)             # at least 2^16 entries: checked on the device
+    assert len(big[1]) >= 1 << 16
+    x = torch.zeros(8, device="cuda")
+    b = gcb.gc_batch_create(1 << 30, gcb.GC_BATCH_MANUAL)
+    try:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            x += 1
+            t = gcb.gc_batch_submit(b, *big)
+        graph.replay()
+        torch.cuda.synchronize()
+        gcb.gc_batch_flush(b)
+        res = gcb.gc_batch_poll(b, t, timeout_us=120_000_000)
+    finally:
+        gcb.gc_batch_destroy(b)
+    assert x.tolist() == [1.0] * 8
+    assert res == _oracle_X(*big)
+
+
 def test_batch_submit_many_matches_single_submits():
     B = graphgen.batch(200, n_lo=20, n_hi=700, seed=33)   # small and large (n > 512) graphs
     b = gcb.gc_batch_create(8 << 30, gcb.GC_BATCH_MANUAL)

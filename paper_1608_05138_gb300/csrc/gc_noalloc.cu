@@ -17,13 +17,13 @@
 // sum min(d_x, d_y) lookups over the edges, where looking up row y in a bitmap
 // of row x for every slot, in global memory, took sum d^2 (Chung-Lu, 100 003
 // vertices, 1 000 003 edges, exponent 2.3: 2.2e9 lookups and 7.9 ms for a
-// pass, 0.60 ms now: 38 us k_rows, 226 k_tri_long, 224 k_tri_short, 66
-// k_tri_reverse, all waiting on chains of dependent loads).
+// pass, 0.50 ms now: 37 us k_rows, 368 k_tri, 64 k_tri_reverse, all waiting on
+// chains of dependent loads).
 //   k_rows   marks the rows that break the CSR rules (not strictly ascending,
 //            a column out of range, a self-loop) and lists the long rows
-//   k_tri_long, k_tri_short   the slots (x, y), y below x in (degree, id): a CTA
-//            per part of a long row with a bitmap of the vertices in shared
-//            memory, a warp per other row with a hash of at most 128 entries
+//   k_tri    the slots (x, y), y below x in (degree, id): a CTA per part of a
+//            long row with a bitmap of the vertices in shared memory, then a
+//            warp per other row with a hash of at most 128 entries
 //   k_tri_reverse   the other slots, from the reverse slot (a binary search);
 //            slots without one, or with an end whose row breaks the rules, are
 //            marked
@@ -31,6 +31,7 @@
 //            the scratch array (nothing to do for a valid graph)
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -53,11 +54,25 @@ constexpr size_t kOffMaps = (size_t)2 * kNoAllocMaxN;
 constexpr size_t kScratchWords = kOffMaps + (size_t)kNoAllocCtas * kNoAllocWords;  // 32 MiB
 static_assert(kScratchWords * 4 == (size_t)32 << 20, "scratch size");
 
-// Rows of at most this many entries are a warp's; a longer one is a CTA's.
-constexpr int kShortRow = 128;
-constexpr int kShortSlots = 2 * kShortRow;  // hash of a short row, at most half full
+// Slots of a long row that a warp takes at a time: the runs of that many lower
+// neighbours are a warp's chain of loads. Graphs of fewer entries have fewer
+// warps' worth of slots, and there the longest chain is the kernel's time
+// (Chung-Lu, exponent 2.3, a pass with one split of 32 slots for all sizes, with
+// this one, and of the bitmap in global memory: 20 000 edges 260, 67, 68 us;
+// 50 000 edges 283, 84, 143; 100 000 edges 286, 96, 341; 10^6 edges 611, 504, 7690).
+__device__ __forceinline__ int window_of(int64_t nnz) { return nnz < (1 << 18) ? 8 : nnz < (1 << 20) ? 16 : 32; }
+// Rows of at most this many entries are a warp's (d^2 / 128 steps at most); a
+// longer one is a CTA's, in parts of a window per warp.
+__device__ __forceinline__ int short_row(int64_t nnz) { return 4 * window_of(nnz); }
+__device__ __forceinline__ int part_of(int64_t nnz) { return kNoAllocBlock / 32 * window_of(nnz); }
+constexpr int kShortRow = 128;              // the longest short row
+constexpr int kShortSlots = 2 * kShortRow;  // its hash, at most half full
+constexpr int kShortWords = kShortSlots + kShortRow;  // a warp's hash and filter
 constexpr int kTriBlock = 256;
-constexpr int kPart = 512;       // slots of a long row that one CTA takes
+constexpr int kPart = kNoAllocBlock;        // the largest part
+// Up to this many vertices, the bitmap and the warps' hashes leave room for four
+// CTAs an SM, and one kernel takes the long rows and then the short ones.
+constexpr int32_t kBothMaxN = 1 << 17;
 constexpr int kHeavyRun = 512;   // a lower neighbour's row of this many entries is all warps' together
 constexpr uint32_t kMaxParts = (uint32_t)(kOffMaps - kOffLong);  // list entries: x (20 bits) and the part above
 constexpr uint32_t kNoPart = 0xffffffffu;
@@ -71,33 +86,35 @@ static __device__ __align__(256) uint32_t g_noalloc_scratch[kScratchWords];
 constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mu;
 uint32_t* g_noalloc_ptr[kMaxDevices] = {};
+int g_noalloc_sms[kMaxDevices] = {};  // SMs of the device, with the address
 
 __device__ __forceinline__ bool row_bad(const uint32_t* scratch, int32_t x) {
   return (scratch[kOffBad + (x >> 5)] >> (x & 31)) & 1u;
 }
 
 // Thread per slot: rows with a column out of range, a self-loop or two entries
-// out of order; thread per row: the long rows, in parts of kPart slots. (A warp
+// out of order; thread per row: the long rows, in parts. (A warp
 // per row would walk the longest rows alone: 0.4 ms for one of 25 000 entries.)
 __global__ void __launch_bounds__(kTriBlock) k_rows(int32_t n, const int32_t* __restrict__ rp,
                                                     const int32_t* __restrict__ ci, uint32_t* __restrict__ scratch) {
   const int lane = threadIdx.x & 31;
   const int64_t t0 = (int64_t)blockIdx.x * kTriBlock + threadIdx.x, threads = (int64_t)gridDim.x * kTriBlock;
+  const int64_t nnz = rp[n];
+  const int32_t part = part_of(nnz), longest_short = short_row(nnz);
   for (int64_t x = t0; x < n; x += threads) {
     const int32_t d = rp[x + 1] - rp[x];
-    if (d <= kShortRow) continue;
-    if (d > n) {  // more entries than vertices
+    if (d <= longest_short) continue;
+    if (d > n || d > nnz) {  // more entries than vertices
       atomicOr(scratch + kOffBad + (x >> 5), 1u << (x & 31));
       continue;
     }
-    const uint32_t parts = (uint32_t)((d + kPart - 1) / kPart);
+    const uint32_t parts = (uint32_t)((d + part - 1) / part);  // at most 4096, as d <= min(n, nnz)
     const uint32_t at = atomicAdd(scratch + kNumLong, parts);
-    const bool fits = at + parts <= kMaxParts;  // else (only beyond 2^29 entries) by k_tri_marked
+    const bool fits = at + parts <= kMaxParts;  // else (only beyond 2^28 entries) by k_tri_marked
     if (!fits) atomicOr(scratch + kOffBad + (x >> 5), 1u << (x & 31));
     for (uint32_t k = 0; k < parts && at + k < kMaxParts; ++k)
       scratch[kOffLong + at + k] = fits ? (uint32_t)x | (k << 20) : kNoPart;
   }
-  const int64_t nnz = rp[n];
   for (int64_t p = t0; p - lane < nnz; p += threads) {
     const int32_t p0 = (int32_t)(p - lane), p_last = (int32_t)min((int64_t)p0 + 31, nnz - 1);
     const int32_t q = (int32_t)min(p, nnz - 1);
@@ -155,26 +172,22 @@ __device__ __forceinline__ void count_runs(const int32_t* __restrict__ ci, int32
   }
 }
 
-// Warp per row of 2 .. kShortRow entries: its entries in an open-addressing
-// hash (twice the slots), behind a filter of 32 bits a slot word.
-__global__ void __launch_bounds__(kTriBlock) k_tri_short(int32_t n, const int32_t* __restrict__ rp,
-                                                         const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
-                                                         uint32_t* __restrict__ scratch) {
-  constexpr int kW = kTriBlock / 32;
-  __shared__ int32_t s_key[kW][kShortSlots];
-  __shared__ uint32_t s_filt[kW][kShortRow];
-  __shared__ int32_t s_cnt[kW][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int32_t *key = s_key[warp], *cnt = s_cnt[warp];
-  uint32_t* filt = s_filt[warp];
+// Warp per row of up to short_row() entries: its entries in an open-addressing
+// hash (twice the slots), behind a filter of 16 bits a hash slot.
+__device__ __forceinline__ void short_rows(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                           int32_t* __restrict__ tri, uint32_t* __restrict__ scratch, int32_t* key,
+                                           uint32_t* filt, int32_t* cnt, int lane) {
+  const int32_t longest = short_row(rp[n]);
+  // rows taken at a time: eight where every warp gets many
+  const int32_t take = min(8, max(1, n / (int32_t)(gridDim.x * (kNoAllocBlock / 32))));
   for (;;) {
-    int32_t x0 = 0;  // eight rows at a time
-    if (lane == 0) x0 = (int32_t)atomicAdd(scratch + kCurShort, 8u);
+    int32_t x0 = 0;
+    if (lane == 0) x0 = (int32_t)atomicAdd(scratch + kCurShort, (uint32_t)take);
     x0 = __shfl_sync(0xffffffffu, x0, 0);
     if (x0 >= n) break;
-    for (int32_t x = x0; x < min(x0 + 8, n); ++x) {
+    for (int32_t x = x0; x < min(x0 + take, n); ++x) {
       const int32_t b = rp[x], e = rp[x + 1], d = e - b;
-      if (d > kShortRow || d == 0 || row_bad(scratch, x)) continue;  // warp-uniform
+      if (d > longest || d == 0 || row_bad(scratch, x)) continue;  // warp-uniform
       int bits = 5;
       while ((1 << bits) < 2 * d) ++bits;  // at most log2(kShortSlots)
       const uint32_t mask = (1u << bits) - 1u;
@@ -217,19 +230,19 @@ __global__ void __launch_bounds__(kTriBlock) k_tri_short(int32_t n, const int32_
 }
 
 // CTA per part of a long row: a bitmap of the n vertices in shared memory with
-// the whole row; the warps take windows of 32 slots of the part, and leave the
+// the whole row; the warps take windows of the part's slots, and leave the
 // long rows of lower neighbours to a list that all warps then read together
 // (the heaviest neighbours are often next to each other, and one warp alone
 // took 0.9 ms for them).
-__global__ void __launch_bounds__(kNoAllocBlock) k_tri_long(int32_t n, const int32_t* __restrict__ rp,
-                                                            const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
-                                                            uint32_t* __restrict__ scratch) {
-  extern __shared__ uint32_t bm[];  // (n + 31) / 32 words
+__device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                           int32_t* __restrict__ tri, uint32_t* __restrict__ scratch,
+                                           uint32_t* bm /* (n + 31) / 32 words */, int32_t* cnt) {
   __shared__ uint32_t s_x;
-  __shared__ int32_t s_next, s_heavy, s_cnt[kNoAllocBlock / 32][32];
+  __shared__ int32_t s_next, s_heavy;
   __shared__ int32_t s_hp[kPart], s_hb[kPart], s_he[kPart], s_hc[kPart];  // the listed slots, their rows, their counts
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int32_t* cnt = s_cnt[warp];
+  const int64_t nnz = rp[n];
+  const int32_t window = window_of(nnz), slots = part_of(nnz);
   const uint32_t n_long = min(scratch[kNumLong], kMaxParts);
   // Bounds are checked although the listed rows follow the rules: calls that
   // overlap on the GPU share the scratch array, and may then list rows and miss
@@ -251,9 +264,9 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_tri_long(int32_t n, const int
     const int32_t x = (int32_t)(s_x & 0xfffffu), part = (int32_t)(s_x >> 20);
     if (x >= n || row_bad(scratch, x)) continue;
     const int32_t b = rp[x], e = rp[x + 1];
-    const int32_t pe = min(e, b + (part + 1) * kPart);
+    const int32_t pe = (int32_t)min((int64_t)e, (int64_t)b + (int64_t)(part + 1) * slots);
     if (threadIdx.x == 0) {
-      s_next = b + part * kPart;
+      s_next = (int32_t)min((int64_t)pe, (int64_t)b + (int64_t)part * slots);
       s_heavy = 0;
     }
     for (int32_t p = b + threadIdx.x; p < e; p += kNoAllocBlock) {
@@ -263,12 +276,12 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_tri_long(int32_t n, const int
     __syncthreads();
     for (;;) {
       int32_t p0 = 0;
-      if (lane == 0) p0 = atomicAdd(&s_next, 32);
+      if (lane == 0) p0 = atomicAdd(&s_next, window);
       p0 = __shfl_sync(0xffffffffu, p0, 0);
       if (p0 >= pe) break;
       int32_t yb, L;
       bool mine;
-      lower_slot(n, rp, ci, scratch, x, e - b, p0 + lane, pe, yb, L, mine);
+      lower_slot(n, rp, ci, scratch, x, e - b, p0 + lane, min(pe, p0 + window), yb, L, mine);
       if (L >= kHeavyRun) {
         const int32_t k = atomicAdd(&s_heavy, 1);
         s_hp[k] = p0 + lane;
@@ -306,6 +319,25 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_tri_long(int32_t n, const int
       const int32_t y = ci[p];
       if ((uint32_t)y < (uint32_t)n) bm[y >> 5] = 0u;
     }
+  }
+}
+
+// Both, or one of them (which: bit 0 long rows, bit 1 short ones), with the
+// bitmap and the warps' hashes in dynamic shared memory.
+__global__ void __launch_bounds__(kNoAllocBlock, 4) k_tri(int32_t n, const int32_t* __restrict__ rp,
+                                                          const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
+                                                          uint32_t* __restrict__ scratch, int which) {
+  extern __shared__ uint32_t s_dyn[];
+  __shared__ int32_t s_cnt[kNoAllocBlock / 32][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t* tables = s_dyn;
+  if (which & 1) {
+    long_parts(n, rp, ci, tri, scratch, s_dyn, s_cnt[warp]);
+    tables += (n + 31) / 32;
+  }
+  if (which & 2) {
+    uint32_t* mine = tables + warp * kShortWords;
+    short_rows(n, rp, ci, tri, scratch, reinterpret_cast<int32_t*>(mine), mine + kShortSlots, s_cnt[warp], lane);
   }
 }
 
@@ -412,6 +444,7 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
     return GC_ERR_ARG;
   }
   uint32_t* scratch = nullptr;
+  int sms = 0;
   {
     std::lock_guard<std::mutex> lk(g_noalloc_mu);
     if (!g_noalloc_ptr[dev]) {
@@ -420,26 +453,35 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
       void* p = nullptr;
       e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
       if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress");
+      if ((e = cudaDeviceGetAttribute(&g_noalloc_sms[dev], cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        return cuda_fail(e, "cudaDeviceGetAttribute");
+      if ((e = cudaFuncSetAttribute(k_tri, cudaFuncAttributeMaxDynamicSharedMemorySize, kNoAllocWords * 4)) !=
+          cudaSuccess)
+        return cuda_fail(e, "k_tri");
       g_noalloc_ptr[dev] = static_cast<uint32_t*>(p);
     }
     scratch = g_noalloc_ptr[dev];
+    sms = g_noalloc_sms[dev];
   }
   cudaStream_t s = (cudaStream_t)stream;
-  int sms = 0, per_sm = 0;
-  const size_t smem = sizeof(uint32_t) * (size_t)((n + 31) / 32);
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-    return cuda_fail(e, "cudaDeviceGetAttribute");
-  if ((e = cudaFuncSetAttribute(k_tri_long, cudaFuncAttributeMaxDynamicSharedMemorySize, kNoAllocWords * 4)) !=
-          cudaSuccess ||
-      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tri_long, kNoAllocBlock, smem)) != cudaSuccess)
-    return cuda_fail(e, "k_tri_long");
+  const size_t bitmap = sizeof(uint32_t) * (size_t)((n + 31) / 32);
+  constexpr size_t kTables = sizeof(uint32_t) * kShortWords * (kNoAllocBlock / 32);
   // counters and the bad-row bits
   if ((e = cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * (kOffBad + (size_t)((n + 31) / 32)), s)) != cudaSuccess)
     return cuda_fail(e, "zero counters");
   const int grid = sms * 8;  // 2048 threads an SM; the number of slots is on the device only
   k_rows<<<grid, kTriBlock, 0, s>>>(n, row_ptr, col_idx, scratch);
-  k_tri_long<<<sms * (per_sm > 0 ? per_sm : 1), kNoAllocBlock, smem, s>>>(n, row_ptr, col_idx, tri_out, scratch);
-  k_tri_short<<<grid, kTriBlock, 0, s>>>(n, row_ptr, col_idx, tri_out, scratch);
+  auto tri = [&](int which, int per_sm, size_t smem) {
+    k_tri<<<sms * per_sm, kNoAllocBlock, smem, s>>>(n, row_ptr, col_idx, tri_out, scratch, which);
+  };
+  // CTAs an SM: four (2048 threads) while the bitmaps leave room for them in
+  // 227 KB, beside the 11 KB that every CTA takes
+  if (n <= kBothMaxN) {
+    tri(3, 4, bitmap + kTables);
+  } else {
+    tri(1, (int)std::min<size_t>(4, ((size_t)227 << 10) / (bitmap + ((size_t)13 << 10))), bitmap);
+    tri(2, 4, kTables);
+  }
   k_tri_reverse<<<grid, kTriBlock, 0, s>>>(n, row_ptr, col_idx, tri_out, scratch);
   k_tri_marked<<<kNoAllocCtas, kNoAllocBlock, 0, s>>>(n, row_ptr, col_idx, tri_out, scratch);
   e = cudaGetLastError();

@@ -87,6 +87,28 @@ def test_noalloc_row_lengths(make):
     np.testing.assert_array_equal(out.cpu().numpy(), _oracle_per_slot(rp, ci))
 
 
+@pytest.mark.parametrize("k, copies, pad", [
+    (33, 3, 0), (34, 3, 0),                    # rows of 32, 33 entries, fewer than 2^18 in all
+    (129, 1, 0), (130, 1, 0),                  # one part of 128 slots, and one slot more
+    (65, 70, 0), (66, 70, 0),                  # 64, 65 of fewer than 2^20
+    (257, 5, 0), (258, 5, 0),                  # a part of 256, and one slot more
+    (129, 70, 0), (130, 70, 0),                # 128, 129 of 2^20 or more
+    (513, 5, 0), (514, 5, 0),                  # a part of 512, and one slot more
+    (66, 70, 1 << 17), (130, 70, 1 << 17),     # long and short rows in kernels of their own
+])
+def test_noalloc_split_of_the_rows(k, copies, pad):
+    # disjoint complete graphs on k vertices: k - 2 triangles on every edge; and
+    # as many isolated vertices as asked for
+    import torch
+    v = np.arange(k, dtype=np.int32)
+    block = np.array([np.delete(v, x) for x in range(k)], np.int32).ravel()
+    ci = np.concatenate([block + c * k for c in range(copies)]).astype(np.int32)
+    rp = np.concatenate([np.arange(copies * k + 1) * (k - 1), np.full(pad, len(ci))]).astype(np.int32)
+    out = torch.full((len(ci),), -1, dtype=torch.int32, device="cuda")
+    gcb.gc_edge_triangles_noalloc(torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda(), out)
+    assert (out == k - 2).all()
+
+
 @pytest.mark.parametrize("seed", range(4))
 def test_noalloc_rows_that_break_the_rules(seed):
     # not validated, but safe and by the definition: tri[p] of (x, y) is the

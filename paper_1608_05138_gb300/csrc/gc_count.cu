@@ -994,7 +994,6 @@ __global__ void __launch_bounds__(kHeavyBlock, 1) k_pass_c_heavy(DevGraph g, Cou
 // {o in Gamma(x) : o < h}, which ends at the slot of (x, h) (ids are ranks
 // and rows ascend).
 constexpr int kHashBlock = 512;
-constexpr int kHashSlots = 2 * kHashMaxW;
 constexpr int kHashSmallBlock = 128;
 constexpr int kHashMidBlock = 256;
 
@@ -1053,7 +1052,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == kHashBlock ? kCtasPerSm 
     const int32_t h = a.cunits[a.n_cheavy + k];
     const int32_t wk = min(a.chash_w[k], (int32_t)kMaxW);
     int bits = 6;
-    while ((1 << bits) < 2 * wk) ++bits;  // at most log2(kHashSlots)
+    while ((1 << bits) < 2 * wk) ++bits;  // at most log2(2 * kHashMaxW)
     const uint32_t mask = (1u << bits) - 1u;
     const int32_t hb = g.rp[h], he = g.rp[h + 1];
     for (int32_t i = threadIdx.x; i <= (int32_t)mask; i += kThreads) hkeys[i] = -1;

@@ -154,7 +154,7 @@ enum Work {
 // happen for a validated graph.
 enum Status : int32_t { kOk = 0, kSpillOverflow = 1, kInexact = 2 };
 
-constexpr int kBlock = 512;            // threads per CTA of passes A and C
+constexpr int kBlock = 512;            // threads per CTA of pass C's vertex-indexed tables
 constexpr int kCtasPerSm = 2;          // resident CTAs per SM of the persistent grids
 constexpr int kWarps = kBlock / 32;
 constexpr int kSmemTableMax = 4096;    // Psi tables up to this many vertices live in shared memory

@@ -450,13 +450,7 @@ gc_status exclusive_scan(int32_t n, const int32_t* in, int32_t* out, cudaStream_
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "scan launch");
 }
 
-// Jobs per CTA of the hub kernel the hub units are cut into (environment
-// GC_HUB_JOBS_PER_CTA, 0 .. 64, default 1; 0 keeps one job per hub), read
-// once per process. With 1, only a hub that costs more than a whole CTA's
-// share of the work is cut: a new job has to seed every lower neighbour's
-// cursor with a galloping search (milliseconds for the largest hubs), and
-// heaviest-first stealing already balances hubs below that size (on R-MAT
-// scale 22 the CTAs' lifetimes differ by 0.1 %).
+// Words of the hub kernel's count block (see kHubTabDefault).
 int hub_tab_words() {
   static int v = [] {
     const char* e = getenv("GC_HUB_TAB_WORDS");
@@ -466,6 +460,12 @@ int hub_tab_words() {
   return v;
 }
 
+// Jobs per CTA of the hub kernel the hub units are cut into (environment
+// GC_HUB_JOBS_PER_CTA, 0 .. 64, default 1; 0 keeps one job per hub), read
+// once per process. With 1, only a hub that costs more than a whole CTA's
+// share of the work is cut: every job looks at all lower neighbours of its hub,
+// and heaviest-first stealing already balances hubs below that size (on R-MAT
+// scale 22 the CTAs' lifetimes differ by 0.1 %).
 static int hub_jobs_per_cta() {
   static int v = [] {
     const char* e = getenv("GC_HUB_JOBS_PER_CTA");

@@ -25,10 +25,12 @@
 //          triangles counted as sum over its edges (i, j), i < j, of the common
 //          neighbours above j: k / 32 words a row instead of n / 32, and no
 //          list of members per edge. A warp per u up to 128 neighbours above
-//          it, the CTA together beyond.
+//          it, the CTA together beyond. An H_u of few edges is counted edge by
+//          edge instead (few_edges), one of fewer than three not at all.
 // Rows are stored at an odd word stride, so that 32 lanes reading one word
 // index of 32 rows hit 32 banks. What bounds it: popc (16 lanes a clock an SM)
-// and shared-memory reads, two each per 32 pairs and word. (Before, each edge
+// and shared-memory reads, one and five quarters of one per 32 pairs and word
+// (four u's share the words of row w). (Before, each edge
 // listed its common neighbours and took one of their rows at a time over the
 // lanes: the graphs of n <= 512 in a launch of 48 took 5.3 ms, one CTA each;
 // now 0.24 ms, in 256 parts.)
@@ -39,12 +41,13 @@
 // an SM. The block size of each class is a tuning parameter (BatchConfig). A
 // CTA takes one unit at a time from the class's list, most work first: a
 // graph, or, when a launch has too few graphs to fill the GPU, a part of one
-// (every parts-th vertex u); each part loads the graph's bit rows, and the
+// (every parts-th group of vertices u); each part loads the graph's bit rows, and the
 // sums of a graph meet in global memory.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <vector>
 
 #include "gc_internal.h"
@@ -207,11 +210,119 @@ __device__ __forceinline__ uint32_t count_h(const uint32_t* h, int k, int wi, in
   return acc;
 }
 
-// at least 1536 threads resident per SM (at most 42 registers a thread): the
-// kernel waits on shared memory and popc, and the more warps an SM holds, the
-// more of its cycles issue
+// This lane's part of the 4-cliques with lowest vertex u, edge by edge of H_u:
+// a lane per member v, its edges (v, w) one after the other, the common
+// neighbours above w of each. For an H_u of few edges: the neighbourhoods of a
+// star's centre or of one side of a bipartite graph have none, and packing a
+// k x k matrix for each of them was most of such a graph's time.
+template <int kS>
+__device__ __noinline__ uint32_t count_edges(const uint32_t* __restrict__ bm, const uint32_t* __restrict__ ru,
+                                                const int32_t* __restrict__ above, int k, int W, int lane) {
+  uint32_t acc = 0;
+  for (int i = lane; i < k; i += 32) {
+    const int v = above[i];
+    const uint32_t* rv = bm + v * kS;
+    uint32_t keep = (kFull << (v & 31)) << 1;  // ids above v
+    for (int a = v >> 5; a < W; ++a, keep = kFull) {
+      uint32_t t = ru[a] & rv[a] & keep;
+      while (t) {
+        const int b = __ffs(t) - 1;
+        t &= t - 1u;
+        const uint32_t* rw = bm + (32 * a + b) * kS;
+        uint32_t hi = (kFull << b) << 1;
+        for (int c = a; c < W; ++c, hi = kFull) acc += __popc(ru[c] & rv[c] & rw[c] & hi);
+      }
+    }
+  }
+  return acc;
+}
+// Whether H_u, k members and at most e edges, is counted edge by edge rather
+// than packed, by SM cycles: about W / 4 a member and 2 W an edge against k / 24
+// a member and k^2 / 1500 a pair (small_cost).
+__device__ __forceinline__ bool few_edges(int k, uint32_t e, int W) {
+  const float K = (float)k;
+  return (float)W * (0.25f * K + 2.0f * (float)e) < K * K * (1.0f / 24.0f + K * (1.0f / 1500.0f));
+}
+constexpr uint16_t kFewEdges = 0x8000;  // in s_up
+
+// The pairs of kU consecutive vertices u0, u0 + 1, ... with the vertices above
+// them, a lane per w: every word of row w is loaded once for all of them. (One u
+// at a time loaded two words a pair and word, and those loads, not popc, were
+// the pass: 2000 graphs of 1000 vertices and mean degree 5, 14.9 ms, now 9.5.) Lane i
+// adds sum i of them to `mine`: sums over four u stay in 32 bits (4092 pairs at
+// most, c and the degrees at most 1023). Marks the u that need no H_u, and those
+// whose H_u is counted edge by edge.
+template <int kS, int kU>
+__device__ __forceinline__ void small_pairs(const uint32_t* __restrict__ bm, const uint16_t* __restrict__ deg,
+                                            uint16_t* __restrict__ up, int u0, int n, int W, int lane,
+                                            unsigned long long& mine) {
+  const uint32_t* rowu = bm + u0 * kS;
+  uint32_t at[kU], tt = 0, tw = 0, dd = 0, c4 = 0;
+#pragma unroll
+  for (int i = 0; i < kU; ++i) at[i] = 0u;
+  for (int w0 = u0 + 1; w0 < n; w0 += 32) {
+    const int w = w0 + lane;
+    if (w >= n) continue;
+    const uint32_t* roww = bm + w * kS;
+    uint32_t c[kU];
+#pragma unroll
+    for (int i = 0; i < kU; ++i) c[i] = 0u;
+#pragma unroll 2
+    for (int k = 0; k < W; ++k) {
+      const uint32_t x = roww[k];
+#pragma unroll
+      for (int i = 0; i < kU; ++i) c[i] += __popc(rowu[i * kS + k] & x);  // rows past n: of the array, not used
+    }
+    const uint32_t dw = deg[w];
+    const int ww = w >> 5, wb = w & 31;
+#pragma unroll
+    for (int i = 0; i < kU; ++i) {
+      if (w <= u0 + i) continue;  // also u0 + i >= n
+      c4 += c[i] * (c[i] - 1u) / 2u;  // 0 for c = 0: the product is 0
+      if ((rowu[i * kS + ww] >> wb) & 1u) {
+        at[i] += c[i];
+        tt += c[i] * c[i];
+        tw += c[i] * dw;
+        dd += deg[u0 + i] * dw;
+      }
+    }
+  }
+  unsigned long long t = 0, ta = 0;
+#pragma unroll
+  for (int i = 0; i < kU; ++i) {
+    const uint32_t ti = __reduce_add_sync(kFull, at[i]);  // at least twice the edges of H_u
+    t += ti;
+    if (u0 + i < n) {  // warp-uniform
+      ta += (unsigned long long)deg[u0 + i] * ti;
+      if (lane == 0) {
+        if (ti < 6u) up[u0 + i] = 0;  // fewer than three edges: no triangle in H_u
+        else if (few_edges(up[u0 + i], ti / 2u, W)) up[u0 + i] |= kFewEdges;
+      }
+    }
+  }
+  const uint32_t d = lane < kU && u0 + lane < n ? deg[u0 + lane] : 0u;
+  if (lane == kQt) mine += t;
+  auto add = [&](int i, uint32_t v, unsigned long long more = 0ull) {
+    v = __reduce_add_sync(kFull, v);
+    if (lane == i) mine += v + more;
+  };
+  add(kQtt, tt);
+  add(kQta, tw, ta);
+  add(kQdd, dd);
+  add(kQd2, d * d);
+  add(kQd3, d * d * d);
+  add(kQc4, c4);
+}
+
+// at least 1536 threads resident per SM (at most 42 registers a thread) where
+// shared memory has room for them: the kernel waits on shared memory and popc,
+// and the more warps an SM holds, the more of its cycles issue
+__host__ __device__ constexpr int small_ctas(int kN, int kBlock) {
+  const int fit = (int)(((size_t)227 << 10) / (small_smem(kN, kBlock) + 3072));
+  return fit < 1 ? 1 : fit < 1536 / kBlock ? fit : 1536 / kBlock;
+}
 template <int kN, int kBlock>
-__global__ void __launch_bounds__(kBlock, 1536 / kBlock) k_small_graphs(const int32_t* __restrict__ rp,
+__global__ void __launch_bounds__(kBlock, small_ctas(kN, kBlock)) k_small_graphs(const int32_t* __restrict__ rp,
                                                          const int64_t* __restrict__ voff,
                                                          const int32_t* __restrict__ ci,
                                                          const int64_t* __restrict__ eoff,
@@ -228,12 +339,11 @@ __global__ void __launch_bounds__(kBlock, 1536 / kBlock) k_small_graphs(const in
   uint16_t* s_deg = reinterpret_cast<uint16_t*>(smem + small_bm(kN) + small_h(kN, kBlock) + small_list(kN, kBlock));
   uint16_t* s_up = s_deg + kN;
   __shared__ int32_t s_unit;
-  __shared__ unsigned long long s_q[kQn];
+  __shared__ unsigned long long s_q[kBlock / 32][kQn];  // per warp: a 64-bit shared atomic is a loop of compare-and-swaps
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (;;) {
     __syncthreads();
     if (threadIdx.x == 0) s_unit = atomicAdd(cursor, 1);
-    if (threadIdx.x < kQn) s_q[threadIdx.x] = 0ull;
     __syncthreads();
     if (s_unit >= n_units) break;
     const int2 unit = units[s_unit];  // graph, part | parts << 16
@@ -249,77 +359,62 @@ __global__ void __launch_bounds__(kBlock, 1536 / kBlock) k_small_graphs(const in
     for (int32_t i = threadIdx.x; i < n * kS; i += kBlock) bm[i] = 0u;
     __syncthreads();
     // the bit rows, the degrees, and the neighbours above each vertex
-    for (int32_t x = warp; x < n; x += kWarps) {
-      const int32_t xb = grp[x], xe = grp[x + 1];
-      int up = 0;
-      for (int32_t p0 = xb; p0 < xe; p0 += 32) {
-        const int32_t y = p0 + lane < xe ? gci[p0 + lane] : -1;
-        if (y >= 0) atomicOr(&bm[x * kS + (y >> 5)], 1u << (y & 31));
-        up += __popc(__ballot_sync(kFull, y > x));
+    // (four rows of a warp at a time, their first 32 entries in flight together:
+    // one row after the other, this was half of a sparse graph's time)
+    constexpr int kRows = 4;
+    for (int32_t x0 = kRows * warp; x0 < n; x0 += kRows * kWarps) {
+      const int32_t off = lane <= kRows ? grp[min(x0 + lane, n)] : 0;
+      int32_t xb[kRows], len[kRows], y[kRows], up[kRows];
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) {  // rows past n are empty
+        xb[j] = __shfl_sync(kFull, off, j);
+        len[j] = __shfl_sync(kFull, off, j + 1) - xb[j];
+        y[j] = lane < len[j] ? gci[xb[j] + lane] : -1;
       }
-      if (lane == 0) {
-        s_deg[x] = (uint16_t)(xe - xb);
-        s_up[x] = (uint16_t)up;
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) {
+        const int32_t x = x0 + j;
+        if (y[j] >= 0) atomicOr(&bm[x * kS + (y[j] >> 5)], 1u << (y[j] & 31));
+        up[j] = __popc(__ballot_sync(kFull, y[j] > x));
+        for (int32_t k = 32; k < len[j]; k += 32) {
+          const int32_t z = k + lane < len[j] ? gci[xb[j] + k + lane] : -1;
+          if (z >= 0) atomicOr(&bm[x * kS + (z >> 5)], 1u << (z & 31));
+          up[j] += __popc(__ballot_sync(kFull, z > x));
+        }
+        if (lane == 0 && x < n) {
+          s_deg[x] = (uint16_t)len[j];
+          s_up[x] = (uint16_t)up[j];
+        }
       }
     }
     __syncthreads();
-    // this unit's vertices u: part, part + parts, ..., one per warp in turn.
-    // Pairs (u, w), w > u. Sums over one u stay in 32 bits (a lane has at most
-    // 32 pairs, every term below 2^21).
-    auto add_sum = [&](int i, unsigned long long v) {
-      v = warp_sum(v);
-      if (lane == 0 && v) atomicAdd(&s_q[i], v);
-    };
-    {
-      unsigned long long q_t = 0, q_tt = 0, q_ta = 0, q_dd = 0, q_c4 = 0, d2 = 0, d3 = 0;
-      for (int32_t u = part + parts * warp; u < n; u += parts * kWarps) {
-        const uint32_t* rowu = bm + u * kS;
-        const uint32_t du = s_deg[u];
-        uint32_t a_t = 0, a_tt = 0, a_ta = 0, a_dd = 0, a_c4 = 0;
-        for (int32_t w0 = u + 1; w0 < n; w0 += 32) {
-          const int32_t w = w0 + lane;
-          if (w < n) {
-            const uint32_t* roww = bm + w * kS;
-            uint32_t c = 0;
-  #pragma unroll 4
-            for (int k = 0; k < W; ++k) c += __popc(rowu[k] & roww[k]);
-            a_c4 += c * (c - 1u) / 2u;  // 0 for c = 0: the product is 0
-            if ((rowu[w >> 5] >> (w & 31)) & 1u) {
-              const uint32_t dw = s_deg[w];
-              a_t += c;
-              a_tt += c * c;
-              a_ta += c * (du + dw);
-              a_dd += du * dw;
-            }
-          }
-        }
-        q_t += a_t;
-        q_tt += a_tt;
-        q_ta += a_ta;
-        q_dd += a_dd;
-        q_c4 += a_c4;
-        if (lane == 0) {
-          d2 += du * du;
-          d3 += (unsigned long long)(du * du) * du;
-        }
-      }
-      add_sum(kQt, q_t);
-      add_sum(kQtt, q_tt);
-      add_sum(kQta, q_ta);
-      add_sum(kQdd, q_dd);
-      add_sum(kQc4, q_c4);
-      add_sum(kQd2, d2);
-      add_sum(kQd3, d3);
+    // this unit's vertices u, groups of kU in turn: part, part + parts, ..., one
+    // per warp: four where every warp gets several, else one
+    const int32_t turn = parts * kWarps, first = part + parts * warp;
+    const int32_t group = n >= 4 * turn ? 4 : 1;
+    unsigned long long mine = 0;  // lane i: sum i
+    for (int32_t u = group * first; u < n; u += group * turn) {
+      if (group == 4) small_pairs<kS, 4>(bm, s_deg, s_up, u, n, W, lane, mine);
+      else small_pairs<kS, 1>(bm, s_deg, s_up, u, n, W, lane, mine);
     }
+    if (lane < kQk4) s_q[warp][lane] = mine;
+    __syncthreads();  // the marks in s_up
     // the 4-cliques with lowest vertex u: the triangles of H_u
     unsigned long long q_k4 = 0;
     {
       uint32_t* h = s_h + warp * h_words(kWarpK / 32);
       uint16_t* m = s_m + warp * kWarpK;
-      for (int32_t u = part + parts * warp; u < n; u += parts * kWarps) {
-        const int k = s_up[u];
-        if (k < 3 || k > kWarpK) continue;  // warp-uniform
+      for (int32_t j = warp;; j += kWarps) {  // this unit's vertices one to a warp: the first have the most members
+        const int32_t u = group * (part + parts * (j / group)) + j % group;
+        if (u - j % group >= n) break;
+        const int up = u < n ? s_up[u] : 0, k = up & ~kFewEdges;
+        if (k < 3) continue;  // warp-uniform
         const int32_t p1 = grp[u + 1] - k;  // the neighbours above u end its ascending row
+        if (up & kFewEdges) {
+          q_k4 += count_edges<kS>(bm, bm + u * kS, gci + p1, k, W, lane);
+          continue;
+        }
+        if (k > kWarpK) continue;
         for (int i = lane; i < k; i += 32) m[i] = (uint16_t)gci[p1 + i];
         __syncwarp();
         pack_h<kS>(bm, m, k, h, 0, 1, lane);
@@ -329,22 +424,27 @@ __global__ void __launch_bounds__(kBlock, 1536 / kBlock) k_small_graphs(const in
       }
     }
     if (kN > kWarpK) {
-      for (int32_t u = part; u < n; u += parts) {
-        const int k = s_up[u];
-        if (k <= kWarpK) continue;  // CTA-uniform
-        __syncthreads();
-        const int32_t p1 = grp[u + 1] - k;
-        for (int i = threadIdx.x; i < k; i += kBlock) s_m[i] = (uint16_t)gci[p1 + i];
-        __syncthreads();
-        pack_h<kS>(bm, s_m, k, s_h, warp, kWarps, lane);
-        __syncthreads();
-        q_k4 += count_h(s_h, k, warp, kWarps, lane);
-      }
+      for (int32_t u0 = group * part; u0 < n; u0 += group * parts)
+        for (int32_t u = u0; u < min(u0 + group, n); ++u) {
+          const int k = s_up[u];
+          if (k <= kWarpK || (k & kFewEdges)) continue;  // CTA-uniform
+          __syncthreads();
+          const int32_t p1 = grp[u + 1] - k;
+          for (int i = threadIdx.x; i < k; i += kBlock) s_m[i] = (uint16_t)gci[p1 + i];
+          __syncthreads();
+          pack_h<kS>(bm, s_m, k, s_h, warp, kWarps, lane);
+          __syncthreads();
+          q_k4 += count_h(s_h, k, warp, kWarps, lane);
+        }
     }
-    add_sum(kQk4, q_k4);
+    q_k4 = warp_sum(q_k4);
+    if (lane == 0) s_q[warp][kQk4] = q_k4;
     __syncthreads();
-    if (threadIdx.x < kQn && s_q[threadIdx.x])
-      atomicAdd(&sums[(size_t)g * kQn + threadIdx.x], s_q[threadIdx.x]);
+    if (threadIdx.x < kQn) {
+      unsigned long long v = 0;
+      for (int w = 0; w < kWarps; ++w) v += s_q[w][threadIdx.x];
+      if (v) atomicAdd(&sums[(size_t)g * kQn + threadIdx.x], v);
+    }
   }
 }
 
@@ -458,8 +558,12 @@ void small_units(const std::vector<int32_t>& n, const std::vector<int64_t>& m, s
 }
 
 gc_status small_graphs_setup() {
+  static std::mutex mu;
+  static std::vector<int> done;  // devices
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lk(mu);
+  if (e == cudaSuccess && std::find(done.begin(), done.end(), dev) != done.end()) return GC_OK;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_fail(e, "k_small_graphs setup");
   for (int c = 0; c < kSmallClasses; ++c)
@@ -472,6 +576,7 @@ gc_status small_graphs_setup() {
       if (e != cudaSuccess) return cuda_fail(e, "k_small_graphs attribute");
       g_small_ctas[c][j] = (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
     }
+  done.push_back(dev);
   return GC_OK;
 }
 

@@ -208,8 +208,8 @@ gc_status gc_graph_phase_ms(gc_graph g, double* ms);
  *     kernel's tail)
  *  17 pass C: wedges of the units counted in the packed-key shared-memory hash
  * A graph of at most 4096 vertices (unless its per-edge induced counts were
- * asked for) is counted from the rows of common neighbours instead of by passes
- * T and C: 0 and 10 are 0, 1 is the list entries read for those rows, and 11
+ * asked for) may be counted from the rows of common neighbours instead of by
+ * passes T and C, by its degrees: 0 and 10 are 0 then, 1 is the list entries read for those rows, and 11
  * comes from the clique kernels. Used to turn kernel times into algorithmic bytes per second. */
 #define GC_NUM_WORK 18
 gc_status gc_graph_work_counts(gc_graph g, uint64_t* out);

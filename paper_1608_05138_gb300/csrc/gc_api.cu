@@ -694,11 +694,7 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
   }
   {
     gc_status st2 = GC_OK;
-    if (n <= kDenseMaxN && g->prep.kmax <= kDenseMaxK) {
-      int64_t d2 = 0;
-      for (int32_t x = 0; x < n; ++x) d2 += (int64_t)(row_ptr[x + 1] - row_ptr[x]) * (row_ptr[x + 1] - row_ptr[x]);
-      if (dense_graph(n, g->m, d2, g->prep.dmax)) st2 = build_bits(n, g->d_rp, g->d_ci, &g->prep, s);
-    }
+    if (g->prep.route == kRouteDense) st2 = build_bits(n, g->d_rp, g->d_ci, &g->prep, s);
     if (st2 == GC_OK)
       st2 = scratch_init(&g->sc, g->m, needs_tables(g->prep) ? n : 0, g->prep.kmax, g->prep.ktier_off, 1,
                          g->prep.bits ? n : 0, s);
@@ -819,6 +815,7 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
   ku.n_chash_mid = g->prep.n_chash_mid;
   ku.n_chash2_big = g->prep.n_chash2_big;
   ku.n_cunits = g->prep.n_cunits;
+  ku.rows = g->prep.route != kRoutePasses;
   for (int t = 0; t <= kNumTiers; ++t) ku.tier_off[t] = g->prep.ktier_off[t];
   if ((st = run_count(dg, g->prep.units, g->prep.n_units, ku, pe_dev, &g->sc, s, g->fs, pe_host, ind_dev, ind_host)) != GC_OK) {
     fork_drain(g->fs);

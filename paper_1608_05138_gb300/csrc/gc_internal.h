@@ -282,6 +282,7 @@ struct KUnits {
   int32_t n_chash2;
   int32_t n_chash2_big;
   int32_t n_cunits;        // pass C units in all (units without wedges are left out)
+  bool rows;               // the graph's route (small_route) is not kRoutePasses
 };
 // induced (optional): [m][10] rows of the per-edge induced counts of H_7..H_16
 // (device pointer, or the device view of pinned host memory when
@@ -289,6 +290,48 @@ struct KUnits {
 gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, const KUnits& ku,
                     uint64_t* per_edge, Scratch* sc, cudaStream_t s, ForkSet* fs, bool per_edge_host = false,
                     uint64_t* induced = nullptr, bool induced_host = false);
+
+// How a graph, or a union of graphs, is counted: by passes T, C and K; from rows
+// of common neighbours (run_rows) for graphs of at most kSmemTableMax vertices;
+// or from those on bit rows (run_rows_dense), one graph of 64 to kDenseMaxN
+// vertices with out-degrees up to kDenseMaxK.
+enum SmallRoute { kRoutePasses = 0, kRouteRows, kRouteDense };
+constexpr int kDenseMaxN = 2048;
+constexpr int kDenseMaxK = 1024;
+// n vertices of the largest of G graphs, n2 the sum of their n^2, m edges in
+// all, kmax the largest out-degree, d2 = sum d^2, kd = sum k (d - k), the
+// out-list entries that pass T scans. What the three routes cost (GB300, us a
+// count with per-edge rows; passes / rows / dense):
+//   rows read 2 d2 entries (1.1 us per 10^6), whatever they find; the passes'
+//   work follows kd and the triangles. G(3000, 0.03), d2 2.5e7: 243 / 194;
+//   Chung-Lu 4000 / 60 000 edges, 3.1e7: 360 / 309; 20 hubs joined to 4000
+//   others, 3.2e8: 575 / 512; 200 hubs joined to 2000, 7.3e8: 526 / 1035;
+//   K(500, 3500), 7.0e9: 2470 / 7828; G(4096, 0.1), 6.9e8: 1269 / 1569.
+//   Above 2.5e8 they pay only where most of what they read are triangles, that is
+//   in graphs as dense all over as G(n, 0.2), d2 = 6 kd there: G(3000, 0.3),
+//   2.4e9: 5793 / 5503; G(4096, 0.3), 6.2e9: 19596 / 17803; Chung-Lu 4000 /
+//   10^6, d2 = 8.7 kd: 2723 / 3318.
+//   Without a vertex of two higher neighbours nothing is left for passes T and K:
+//   star of 4000 leaves 324 / 412.
+//   Bit rows cost n / 32 words a slot and bit of the counts, and a k x k matrix per
+//   vertex whether it has edges or not: G(500, 0.3) 169 / 152 / 129, G(1000, 0.1)
+//   169 / 138 / 150, G(1000, 0.3) 422 / 353 / 245, G(1500, 0.2) 483 / 457 / 409,
+//   G(2000, 0.11) 342 / 341 / 411, G(2000, 0.25) 1311 / 1230 / 916, K(1000, 1000)
+//   1593 / 2630 / 3413, 500 hubs joined to 2000 1262 / 2232 / 1322; where the
+//   matrices are small, K(200, 800) 276 / 359 / 262, K(250, 1500) 609 / 915 / 574,
+//   K(200, 1500) 438 / 765 / 529, 150 hubs joined to 1500 394 / 527 / 438.
+//   Unions fill the GPU with units too small for the passes' CTAs: 2000 graphs
+//   G(1100, 0.011), 29.6 ms with passes, 15.0 with rows.
+inline SmallRoute small_route(int32_t n, int32_t G, int64_t n2, int64_t m, int32_t kmax, double d2, double kd) {
+  if (n > kSmemTableMax || kmax < 2) return kRoutePasses;
+  const double edges2 = 2.0 * (double)m;
+  if (G > 1) return kRouteRows;
+  if (n >= 64 && n <= kDenseMaxN && kmax <= kDenseMaxK && edges2 >= 0.15 * (double)n2 &&
+      (d2 <= 8.0 * kd || (kmax <= 256 && edges2 >= 0.22 * (double)n2)))
+    return kRouteDense;
+  if (d2 <= 3.3e8 && kd <= 3e7) return kRouteRows;
+  return d2 <= 7.0 * kd && edges2 >= 0.2 * (double)n2 ? kRouteRows : kRoutePasses;
+}
 
 // ---- host helpers (gc_api.cu) ----
 void set_error(const std::string& msg);
@@ -379,7 +422,8 @@ struct PrepBuffers {
   int32_t n_chash2 = 0;        // units of the packed-key hash tier
   int32_t n_chash2_big = 0;    // of them, units of more than kHash2HalfMaxW wedges
   int32_t n_cunits = 0;
-  uint32_t* bits = nullptr;    // dense graphs: bit rows, and the same by word (see DevGraph)
+  SmallRoute route = kRoutePasses;  // how the graph is counted (small_route)
+  uint32_t* bits = nullptr;    // kRouteDense: bit rows, and the same by word (see DevGraph)
   uint32_t* bits_t = nullptr;
   HubGeom* hgeom = nullptr;    // layout of the hub kernel's o-range (owns hseg's block)
   HubSeg* hseg = nullptr;
@@ -477,21 +521,6 @@ gc_status run_rows(const DevGraph& g, const CountArgs& a, cudaStream_t s);
 gc_status run_cliques_alone(const DevGraph& g, const CountArgs& a, Fork* fork, int* launches);
 // The same two for a dense graph, on its bit rows: k_rows_dense reads them
 // instead of the neighbours' lists, k_cliques_dense packs every H_a from them.
-constexpr int kDenseMaxN = 2048;
-constexpr int kDenseMaxK = 1024;  // largest out-degree
-// Whether a graph of n vertices, m edges, sum d^2 = d2 and largest degree dmax
-// is counted on bit rows. Costs in SM cycles: about 1.1 per entry of the
-// neighbours' rows (25 instructions per 32 entries, read twice), against a popc
-// (16 a cycle) per word, counter bit and slot, for the 4-cycles of half of the
-// slots and the cross terms of all, and per word and vertex pair. G(1000, 0.3):
-// 1.0e8 against 1.1e7; G(2000, 0.01): 9e5 against 2.6e7.
-inline bool dense_graph(int64_t n, int64_t m, int64_t d2, int64_t dmax) {
-  if (n > kDenseMaxN || n < 64 || m == 0) return false;
-  int bits = 1;
-  while ((1LL << bits) <= dmax) ++bits;
-  const double W = (double)((n + 31) / 32);
-  return 1.1 * (double)d2 > 1.5 * (0.094 * 2.0 * (double)m * W * bits + 0.1 * (double)n * (double)n * W);
-}
 gc_status run_rows_dense(const DevGraph& g, const CountArgs& a, cudaStream_t s);
 gc_status run_cliques_dense(const DevGraph& g, const CountArgs& a, int32_t kmax, cudaStream_t s);
 // Bit rows of a prepared graph of at most kDenseMaxN vertices (P->bits, bits_t).

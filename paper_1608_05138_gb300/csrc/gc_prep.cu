@@ -40,13 +40,14 @@ __device__ __forceinline__ int32_t lower_bound_i32(const int32_t* a, int32_t lo,
   return lo;
 }
 
-// Degrees, out-degrees (ids are ranks, so the higher-rank neighbours of x are
-// the entries above x), and the largest of both.
+// Degrees, out-degrees k (ids are ranks, so the higher-rank neighbours of x are
+// the entries above x), the largest of both, and the sums of d^2 and of k (d - k).
 __global__ void __launch_bounds__(256) k_deg_out(int32_t n, const int32_t* __restrict__ rp,
                                                  const int32_t* __restrict__ ci, int32_t* __restrict__ deg,
                                                  int32_t* __restrict__ out_cnt, int32_t* __restrict__ dmax,
-                                                 int32_t* __restrict__ kmax) {
+                                                 int32_t* __restrict__ kmax, unsigned long long* __restrict__ sums) {
   int32_t dm = 0, km = 0;
+  unsigned long long d2 = 0, kd = 0;
   for (int32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
     const int32_t b = rp[x], e = rp[x + 1];
     const int32_t k = e - lower_bound_i32(ci, b, e, x + 1);
@@ -54,22 +55,36 @@ __global__ void __launch_bounds__(256) k_deg_out(int32_t n, const int32_t* __res
     out_cnt[x] = k;
     dm = max(dm, e - b);
     km = max(km, k);
+    d2 += (unsigned long long)(e - b) * (unsigned)(e - b);
+    kd += (unsigned long long)k * (unsigned)(e - b - k);
   }
   // one atomic a block and maximum: one a vertex on the same word took 0.8 ms
   // of the preparation of R-MAT scale 20
   __shared__ int32_t s_m[2];
-  if (threadIdx.x < 2) s_m[threadIdx.x] = 0;
+  __shared__ unsigned long long s_s[2];
+  if (threadIdx.x < 2) {
+    s_m[threadIdx.x] = 0;
+    s_s[threadIdx.x] = 0ull;
+  }
   __syncthreads();
   dm = __reduce_max_sync(0xffffffffu, dm);
   km = __reduce_max_sync(0xffffffffu, km);
+  for (int o = 16; o; o >>= 1) {
+    d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+    kd += __shfl_xor_sync(0xffffffffu, kd, o);
+  }
   if ((threadIdx.x & 31) == 0) {
     atomicMax(&s_m[0], dm);
     atomicMax(&s_m[1], km);
+    atomicAdd(&s_s[0], d2);
+    atomicAdd(&s_s[1], kd);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     if (s_m[0]) atomicMax(dmax, s_m[0]);
     if (s_m[1]) atomicMax(kmax, s_m[1]);
+    if (s_s[0]) atomicAdd(&sums[0], s_s[0]);
+    if (s_s[1]) atomicAdd(&sums[1], s_s[1]);
   }
 }
 
@@ -763,14 +778,16 @@ gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t
   }
   GC_TRY(pool_alloc(&P.kunits, sizeof(int32_t) * (n > 0 ? n : 1), s), "alloc kunits");
   GC_TRY(pool_alloc(&out_cnt, sizeof(int32_t) * (n > 0 ? n : 1), s), "alloc out_cnt");
-  // [0] max degree, [1..64] v-group bins, [65] max out-degree, [66..97] pass-K bins
-  GC_TRY(pool_alloc(&dmax, sizeof(int32_t) * 98, s), "alloc dmax");
+  // [0] max degree, [1..64] v-group bins, [65] max out-degree, [66..97] pass-K
+  // bins, [98..101] the sums of d^2 and of k (d - k), 64 bits each
+  GC_TRY(pool_alloc(&dmax, sizeof(int32_t) * 102, s), "alloc dmax");
   hist = dmax + 1;
-  GC_TRY(cudaMemsetAsync(dmax, 0, sizeof(int32_t) * 98, s), "memset");
+  GC_TRY(cudaMemsetAsync(dmax, 0, sizeof(int32_t) * 102, s), "memset");
   if (n > 0) {
     const int blocks = std::min(grid_for(n, 256), 8 * (count_grid_size() / kCtasPerSm));
     const int bin_blocks = std::min(grid_for(n, 1024), 2 * (count_grid_size() / kCtasPerSm));
-    k_deg_out<<<blocks, 256, 0, s>>>(n, d_rp, d_ci, P.deg, out_cnt, dmax, dmax + 65);
+    k_deg_out<<<blocks, 256, 0, s>>>(n, d_rp, d_ci, P.deg, out_cnt, dmax, dmax + 65,
+                                  reinterpret_cast<unsigned long long*>(dmax + 98));
     GC_TRY(cudaGetLastError(), "k_deg_out");
     if ((st = exclusive_scan(n, out_cnt, P.out_ptr, s)) != GC_OK) goto fail;
     k_rev_init<<<grid_for(nnz, 256), 256, 0, s>>>(nnz, P.rev);
@@ -787,11 +804,20 @@ gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t
     k_bin_kunits<false><<<bin_blocks, 1024, 0, s>>>(n, out_cnt, dmax + 66, nullptr);
     GC_TRY(cudaGetLastError(), "k_bin_kunits");
     {
-      int32_t h[98];
+      int32_t h[102];
       GC_TRY(cudaMemcpyAsync(h, dmax, sizeof(h), cudaMemcpyDeviceToHost, s), "copy hist");
       GC_TRY(cudaStreamSynchronize(s), "sync hist");
       P.dmax = h[0];
       P.kmax = h[65];
+      uint64_t sums[2];
+      std::memcpy(sums, h + 98, sizeof(sums));
+      int64_t n2 = 0;
+      int32_t largest = 0;
+      for (int32_t gi = 0; gi < rank.G; ++gi) {
+        n2 += (int64_t)rank.gn[gi] * rank.gn[gi];
+        largest = std::max(largest, rank.gn[gi]);
+      }
+      P.route = small_route(largest, rank.G, n2, m, P.kmax, (double)sums[0], (double)sums[1]);
       {  // pass-K units, largest bin first; tier boundaries at k = 1024, 512, 256, 32
         int32_t kc[32];
         int32_t acc = 0;

@@ -186,9 +186,10 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
   // Pass T keeps the edges of the H_a for pass K, in a list sized by the
   // triangles of the previous count of this scratch (or by a first guess);
   // units that do not fit scan their out-lists again in pass K.
-  // Small graphs take the rows of common neighbours instead of passes T and C
-  // (see k_rows); the per-edge induced counts need pass T's degree sums.
-  const bool rows = g.table_n <= kSmemTableMax && !(induced != nullptr && g.m > 0);
+  // Graphs of at most kSmemTableMax vertices may take the rows of common
+  // neighbours instead of passes T and C (small_route); the per-edge induced
+  // counts need pass T's degree sums.
+  const bool rows = ku.rows && !(induced != nullptr && g.m > 0);
   if (!rows) {
     const int32_t nku = ku_total(ku);
     const long long want = sc->tlist_want;

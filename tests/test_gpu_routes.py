@@ -80,3 +80,30 @@ def test_small_graphs_without_4_cliques_cost_what_sparse_ones_do():
     for name, g in (("sparse", graphgen.er(1000, 0.02, 1)), ("bipartite", bipartite(10, 990))):
         t[name] = min(batch_counts([g] * 1000)[1] for _ in range(3))
     assert t["bipartite"] < 2 * t["sparse"]
+
+
+# (graph, whether passes T and C count it)
+@pytest.mark.parametrize("make,passes", [
+    (lambda: graphgen.er(2000, 0.01, 1), False),     # rows of common neighbours
+    (lambda: graphgen.er(3000, 0.02, 1), False),
+    (lambda: hubs(5, 3000, 3), False),
+    (lambda: graphgen.er(700, 0.2, 1), False),       # bit rows
+    (lambda: bipartite(60, 240), False),             # out-degrees of at most 256, without a triangle
+    (lambda: bipartite(150, 3900), True),            # rows of hubs, read once for every leaf
+    (lambda: hubs(200, 2000, 5), True),
+    (lambda: hubs(120, 4000, 4), True),
+    (lambda: bipartite(900, 1100), True),            # dense, but without a triangle
+])
+def test_route_of_graphs_up_to_4096_vertices(make, passes):
+    rp, ci = make()
+    with gcb.Graph(rp, ci) as g:
+        pe = np.zeros((g.m, 13), np.uint64)
+        X = g.count(pe)
+        w = g.work_counts()
+        pe2 = np.zeros((g.m, 13), np.uint64)
+        assert g.count(pe2) == X
+    o = oracle.count(rp, ci)
+    np.testing.assert_array_equal(pe, o["per_edge"])
+    np.testing.assert_array_equal(pe2, o["per_edge"])
+    assert X == o["X"]
+    assert (w["t_members"] > 0) == passes

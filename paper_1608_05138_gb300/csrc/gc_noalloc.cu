@@ -19,6 +19,8 @@
 // vertices, 1 000 003 edges, exponent 2.3: 2.2e9 lookups and 7.9 ms for a
 // pass, 0.50 ms now: 37 us k_rows, 368 k_tri, 64 k_tri_reverse, all waiting on
 // chains of dependent loads).
+// Up to kOneN vertices one kernel does it all, a CTA per row (k_tri_one). Above,
+// five launches, each waiting for the one before:
 //   k_rows   marks the rows that break the CSR rules (not strictly ascending,
 //            a column out of range, a self-loop) and lists the long rows
 //   k_tri    the slots (x, y), y below x in (degree, id): a CTA per part of a
@@ -29,6 +31,7 @@
 //            marked
 //   k_tri_marked    the marked slots by the definition, with a bitmap per CTA in
 //            the scratch array (nothing to do for a valid graph)
+// Up to kPickN vertices k_pick, in the place of the clearing, picks either.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -47,7 +50,7 @@ constexpr int kNoAllocCtas = 192;                      // CTAs of k_tri_marked, 
 constexpr int kNoAllocBlock = 512;
 // Scratch layout, in 32-bit words: counters, a bit per row that breaks the
 // CSR rules, the list of long rows, the bitmaps of k_tri_marked.
-enum { kCurLong = 0, kNumLong, kCurShort, kNumMarked, kNumCounters };
+enum { kCurLong = 0, kNumLong, kCurShort, kNumMarked, kOneKernel, kNumCounters };
 constexpr size_t kOffBad = 32;
 constexpr size_t kOffLong = kOffBad + kNoAllocWords;
 constexpr size_t kOffMaps = (size_t)2 * kNoAllocMaxN;
@@ -76,6 +79,9 @@ constexpr int32_t kBothMaxN = 1 << 17;
 constexpr int kHeavyRun = 512;   // a lower neighbour's row of this many entries is all warps' together
 constexpr uint32_t kMaxParts = (uint32_t)(kOffMaps - kOffLong);  // list entries: x (20 bits) and the part above
 constexpr uint32_t kNoPart = 0xffffffffu;
+// Up to kOneN vertices, k_tri_one does the whole step; up to kPickN, it or the
+// kernels of larger graphs, picked from the degrees on the device.
+constexpr int32_t kOneN = 1024, kPickN = 4096;
 
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kScratchWords];
 
@@ -88,6 +94,32 @@ std::mutex g_noalloc_mu;
 uint32_t* g_noalloc_ptr[kMaxDevices] = {};
 int g_noalloc_sms[kMaxDevices] = {};  // SMs of the device, with the address
 
+// Up to kCloseN vertices the kernels of a call follow each other closely: a kernel
+// lets the next one be launched as soon as all its CTAs run, and the next one waits
+// here until the previous is complete and its writes can be seen. Beyond, the next
+// kernel's waiting CTAs cost more than the gap (Chung-Lu, 100 003 vertices, 10^6
+// edges: 495 us, closely 509; R-MAT scale 13 111 and 106; a cycle of 4097 76 and 65).
+constexpr int32_t kCloseN = 1 << 14;
+__device__ __forceinline__ void after_previous() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
+template <class... Params, class... Args>
+cudaError_t launch_after(void (*kernel)(Params...), int grid, int block, size_t smem, cudaStream_t s, int32_t n,
+                         Args... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = n <= kCloseN;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, n, args...);
+}
+
 __device__ __forceinline__ bool row_bad(const uint32_t* scratch, int32_t x) {
   return (scratch[kOffBad + (x >> 5)] >> (x & 31)) & 1u;
 }
@@ -97,6 +129,8 @@ __device__ __forceinline__ bool row_bad(const uint32_t* scratch, int32_t x) {
 // per row would walk the longest rows alone: 0.4 ms for one of 25 000 entries.)
 __global__ void __launch_bounds__(kTriBlock) k_rows(int32_t n, const int32_t* __restrict__ rp,
                                                     const int32_t* __restrict__ ci, uint32_t* __restrict__ scratch) {
+  after_previous();
+  if (scratch[kOneKernel]) return;
   const int lane = threadIdx.x & 31;
   const int64_t t0 = (int64_t)blockIdx.x * kTriBlock + threadIdx.x, threads = (int64_t)gridDim.x * kTriBlock;
   const int64_t nnz = rp[n];
@@ -169,6 +203,103 @@ __device__ __forceinline__ void count_runs(const int32_t* __restrict__ ci, int32
 #pragma unroll
     for (int j = 0; j < 4; ++j)
       if (w[j] >= 0 && in(w[j])) atomicAdd(&cnt[own[j]], 1);
+  }
+}
+
+// The whole step in one kernel: CTA per row x, a bitmap of it in shared memory; a
+// window of its slots per warp, whose short rows are read end to end over the
+// lanes and whose long ones (kLongRun entries) by the whole warp. Every slot by
+// the definition, so that no row's order matters: sum d^2 lookups, where the
+// kernels below take sum min(d_x, d_y) but four more launches. A call with the
+// read-back of row_ptr[n] around it (about 30 us), one kernel / the others:
+// G(64, 0.3) 40 / 71 us, G(1000, 0.02) 43 / 82, K_1000 687 / 795, K(200, 800)
+// 161 / 151; the others' 71 is 66 since they follow each other closely.
+constexpr int kOneBlock = 256;
+constexpr int32_t kLongRun = 64;
+__global__ void __launch_bounds__(kOneBlock) k_tri_one(int32_t n, const int32_t* __restrict__ rp,
+                                                       const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
+                                                       const uint32_t* scratch /* null: not picked */) {
+  constexpr int kW = kOneBlock / 32;
+  __shared__ uint32_t bm[kPickN / 32];
+  after_previous();
+  if (scratch && !scratch[kOneKernel]) return;
+  __shared__ int32_t s_cnt[kW][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int32_t* cnt = s_cnt[warp];
+  auto in = [&](int32_t w) -> bool { return (uint32_t)w < (uint32_t)n && ((bm[w >> 5] >> (w & 31)) & 1u); };
+  for (int32_t x = blockIdx.x; x < n; x += gridDim.x) {
+    const int32_t b = rp[x];
+    const uint32_t d = (uint32_t)(rp[x + 1] - b);
+    if (d == 0u) continue;
+    __syncthreads();  // the previous row's lookups
+    for (int i = threadIdx.x; i < (n + 31) / 32; i += kOneBlock) bm[i] = 0u;
+    __syncthreads();
+    for (uint32_t k = threadIdx.x; k < d; k += kOneBlock) {
+      const int32_t w = ci[b + k];
+      if ((uint32_t)w < (uint32_t)n) atomicOr(&bm[w >> 5], 1u << (w & 31));
+    }
+    __syncthreads();
+    const uint32_t window = min(32u, (d + kW - 1) / kW);  // slots a warp takes at a time
+    for (uint32_t k0 = warp * window; k0 < d; k0 += kW * window) {
+      const bool mine = lane < window && k0 + lane < d;
+      int32_t yb = 0, L = 0;
+      if (mine) {
+        const int32_t y = ci[b + k0 + lane];
+        if ((uint32_t)y < (uint32_t)n) {
+          yb = rp[y];
+          L = rp[y + 1] - yb;
+        }
+      }
+      cnt[lane] = 0;
+      __syncwarp();
+      count_runs(ci, yb, L < kLongRun ? L : 0, cnt, lane, in);
+      unsigned lm = __ballot_sync(0xffffffffu, L >= kLongRun);
+      while (lm) {
+        const int src = __ffs(lm) - 1;
+        lm &= lm - 1u;
+        const int32_t* row = ci + __shfl_sync(0xffffffffu, yb, src);
+        const uint32_t len = (uint32_t)__shfl_sync(0xffffffffu, L, src);
+        uint32_t c = 0;
+        for (uint32_t q = lane; q < len; q += 128) {
+          int32_t w[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) w[j] = q + 32 * j < len ? row[q + 32 * j] : -1;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) c += in(w[j]);
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == src) cnt[lane] = (int32_t)c;  // its own: count_runs left it 0
+      }
+      __syncwarp();
+      if (mine) tri[b + k0 + lane] = cnt[lane];
+      __syncwarp();
+    }
+  }
+}
+
+// One CTA, in the place of clearing the counters and the bad-row bits: does that,
+// and picks k_tri_one or the kernels after it: the first where sum d^2 is small
+// anyway, or the degrees are about equal (E[d^2] <= 1.25 E[d]^2), where sum min(d)
+// saves little. k_tri_one / the others: G(3000, 0.1) 298 / 382 us, G(2000, 0.01)
+// 46 / 70, Chung-Lu 4000 / 10 000 63 / 72, star of 4000 71 / 69, Chung-Lu 4000 /
+// 60 000 130 / 97, K(100, 3900) 978 / 193, G(2048, 0.7) 2810 / 2469.
+__global__ void __launch_bounds__(1024) k_pick(int32_t n, const int32_t* __restrict__ rp, uint32_t* __restrict__ scratch) {
+  __shared__ double s_d2[32];
+  cudaTriggerProgrammaticLaunchCompletion();
+  double d2 = 0;
+  for (int32_t x = threadIdx.x; x < n; x += 1024) {
+    const double d = (double)(rp[x + 1] - rp[x]);
+    d2 += d * d;
+  }
+  for (int32_t i = threadIdx.x; i < (int32_t)kOffBad + (n + 31) / 32; i += 1024)
+    if (i != kOneKernel) scratch[i] = 0u;
+  for (int o = 16; o; o >>= 1) d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+  if ((threadIdx.x & 31) == 0) s_d2[threadIdx.x >> 5] = d2;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 32; ++w) d2 += s_d2[w];
+    const double nnz = (double)rp[n];
+    scratch[kOneKernel] = d2 <= 8e6 || (d2 <= 2e9 && d2 * n <= 1.25 * nnz * nnz);
   }
 }
 
@@ -330,6 +461,8 @@ __global__ void __launch_bounds__(kNoAllocBlock, 4) k_tri(int32_t n, const int32
   extern __shared__ uint32_t s_dyn[];
   __shared__ int32_t s_cnt[kNoAllocBlock / 32][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  after_previous();
+  if (scratch[kOneKernel]) return;
   uint32_t* tables = s_dyn;
   if (which & 1) {
     long_parts(n, rp, ci, tri, scratch, s_dyn, s_cnt[warp]);
@@ -346,6 +479,8 @@ __global__ void __launch_bounds__(kNoAllocBlock, 4) k_tri(int32_t n, const int32
 __global__ void __launch_bounds__(kTriBlock) k_tri_reverse(int32_t n, const int32_t* __restrict__ rp,
                                                            const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
                                                            uint32_t* __restrict__ scratch) {
+  after_previous();
+  if (scratch[kOneKernel]) return;
   const int lane = threadIdx.x & 31;
   const int64_t nnz = rp[n], threads = (int64_t)gridDim.x * kTriBlock;
   bool marked = false;
@@ -381,6 +516,7 @@ __global__ void __launch_bounds__(kTriBlock) k_tri_reverse(int32_t n, const int3
 __global__ void __launch_bounds__(kNoAllocBlock) k_tri_marked(int32_t n, const int32_t* __restrict__ rp,
                                                               const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
                                                               uint32_t* __restrict__ scratch) {
+  cudaGridDependencySynchronize();
   if (scratch[kNumMarked] == 0u) return;
   uint32_t* bm = scratch + kOffMaps + (size_t)blockIdx.x * kNoAllocWords;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -464,15 +600,26 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
     sms = g_noalloc_sms[dev];
   }
   cudaStream_t s = (cudaStream_t)stream;
+  if (n <= kOneN) {
+    k_tri_one<<<std::min(n, sms * 8), kOneBlock, 0, s>>>(n, row_ptr, col_idx, tri_out, nullptr);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? GC_OK : cuda_fail(e, "gc_edge_triangles_noalloc");
+  }
   const size_t bitmap = sizeof(uint32_t) * (size_t)((n + 31) / 32);
   constexpr size_t kTables = sizeof(uint32_t) * kShortWords * (kNoAllocBlock / 32);
-  // counters and the bad-row bits
-  if ((e = cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * (kOffBad + (size_t)((n + 31) / 32)), s)) != cudaSuccess)
-    return cuda_fail(e, "zero counters");
   const int grid = sms * 8;  // 2048 threads an SM; the number of slots is on the device only
-  k_rows<<<grid, kTriBlock, 0, s>>>(n, row_ptr, col_idx, scratch);
+  // the counters and the bad-row bits cleared; then each kernel is launched while
+  // the one before it runs, and waits for it (after_previous)
+  if (n <= kPickN) {
+    k_pick<<<1, 1024, 0, s>>>(n, row_ptr, scratch);
+    launch_after(k_tri_one, std::min(n, grid), kOneBlock, 0, s, n, row_ptr, col_idx, tri_out, scratch);
+  } else if ((e = cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * (kOffBad + (size_t)((n + 31) / 32)), s)) !=
+             cudaSuccess) {
+    return cuda_fail(e, "zero counters");
+  }
+  launch_after(k_rows, grid, kTriBlock, 0, s, n, row_ptr, col_idx, scratch);
   auto tri = [&](int which, int per_sm, size_t smem) {
-    k_tri<<<sms * per_sm, kNoAllocBlock, smem, s>>>(n, row_ptr, col_idx, tri_out, scratch, which);
+    launch_after(k_tri, sms * per_sm, kNoAllocBlock, smem, s, n, row_ptr, col_idx, tri_out, scratch, which);
   };
   // CTAs an SM: four (2048 threads) while the bitmaps leave room for them in
   // 227 KB, beside the 11 KB that every CTA takes
@@ -482,8 +629,8 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
     tri(1, (int)std::min<size_t>(4, ((size_t)227 << 10) / (bitmap + ((size_t)13 << 10))), bitmap);
     tri(2, 4, kTables);
   }
-  k_tri_reverse<<<grid, kTriBlock, 0, s>>>(n, row_ptr, col_idx, tri_out, scratch);
-  k_tri_marked<<<kNoAllocCtas, kNoAllocBlock, 0, s>>>(n, row_ptr, col_idx, tri_out, scratch);
+  launch_after(k_tri_reverse, grid, kTriBlock, 0, s, n, row_ptr, col_idx, tri_out, scratch);
+  launch_after(k_tri_marked, kNoAllocCtas, kNoAllocBlock, 0, s, n, row_ptr, col_idx, tri_out, scratch);
   e = cudaGetLastError();
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "gc_edge_triangles_noalloc");
 }

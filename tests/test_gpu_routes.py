@@ -1,6 +1,7 @@
 """The rules that pick a kernel by the shape of a graph: results on both sides of
 each line, and work that follows the shape (a sparse or skewed graph must not
 cost what a dense one of its size does)."""
+import ctypes as C
 from math import comb
 
 import numpy as np
@@ -107,3 +108,91 @@ def test_route_of_graphs_up_to_4096_vertices(make, passes):
     np.testing.assert_array_equal(pe2, o["per_edge"])
     assert X == o["X"]
     assert (w["t_members"] > 0) == passes
+
+
+def triangles(rp, ci):
+    import torch
+    a, b = torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda()
+    out = torch.full((len(ci),), -1, dtype=torch.int32, device="cuda")
+    gcb.gc_edge_triangles_noalloc(a, b, out)
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("make", [
+    lambda: graphgen.er(1024, 0.05, 1),      # the largest graph of one kernel
+    lambda: graphgen.er(1025, 0.05, 1),      # picked on the device: one kernel
+    lambda: graphgen.er(4096, 0.02, 1),
+    lambda: graphgen.er(4097, 0.02, 1),      # beyond
+    lambda: graphs.complete(64),             # rows of 63 entries: end to end
+    lambda: graphs.complete(66),             # and of 65: one at a time
+    lambda: graphs.star(1000),
+    lambda: graphs.star(4095),               # picked: the kernels of larger graphs
+    lambda: bipartite(60, 2000),
+    lambda: hubs(20, 3000, 4),
+    lambda: graphs.csr(3000, [(7, 2999)]),
+])
+def test_noalloc_kernel_by_size_and_shape(make):
+    rp, ci = make()
+    t = oracle.count(rp, ci)["per_edge"][:, 0]
+    uv = oracle.edges(rp, ci)
+    n = len(rp) - 1
+    rows = np.repeat(np.arange(n, dtype=np.int64), np.diff(rp))
+    at = np.searchsorted(uv[:, 0].astype(np.int64) * n + uv[:, 1],
+                         np.minimum(rows, ci) * n + np.maximum(rows, ci))
+    np.testing.assert_array_equal(triangles(rp, ci), t[at].astype(np.int32))
+
+
+@pytest.mark.parametrize("n", [300, 1500, 3000])
+@pytest.mark.parametrize("skew", [False, True])
+def test_noalloc_rows_that_break_the_rules_by_size(n, skew):
+    # as test_noalloc_rows_that_break_the_rules, for every kernel that a size and shape pick
+    rng = np.random.default_rng(n + skew)
+    rp, ci = graphgen.chung_lu(n, 9 * n, 2.1, 18.0 * n, n - 1.0, 5) if skew else graphgen.er(n, 20.0 / n, 5)
+    ci = ci.copy()
+    for x in rng.choice(n, 60, replace=False):
+        row = ci[rp[x]:rp[x + 1]]
+        if len(row) >= 3:
+            k = rng.integers(0, 4)
+            if k == 0:
+                rng.shuffle(row)
+            elif k == 1:
+                row[0] = row[-1]
+            elif k == 2:
+                row[rng.integers(0, len(row))] = rng.choice([-1, n, 2**31 - 1, -2**31])
+            else:
+                row[rng.integers(0, len(row))] = x
+    rows = [ci[rp[x]:rp[x + 1]].tolist() for x in range(n)]
+    sets = [set(r) for r in rows]
+    expect = [sum(0 <= w < n and w in sets[x] for w in rows[y]) if 0 <= y < n else 0 for x in range(n) for y in rows[x]]
+    np.testing.assert_array_equal(triangles(rp, ci), np.array(expect, np.int32))
+
+
+def test_noalloc_small_call_is_one_kernel_and_can_be_captured():
+    # the smallest calls are launches; and every launch sequence replays as a graph
+    import torch
+    cu = C.CDLL("libcuda.so.1")
+    for (rp, ci), most in ((graphgen.er(500, 0.1, 3), 1), (graphgen.er(3000, 0.01, 3), 6), (graphgen.er(9000, 0.003, 3), 6)):
+        expect = triangles(rp, ci)  # also the first call, which looks the array up
+        a, b = torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda()
+        out = torch.full((len(ci),), -1, dtype=torch.int32, device="cuda")
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        graph, ex, count = C.c_void_p(), C.c_void_p(), C.c_size_t()
+        torch.cuda.synchronize()
+        h = C.c_void_p(s.cuda_stream)
+        n = C.c_int32(len(rp) - 1)
+        assert cu.cuStreamBeginCapture_v2(h, 1) == 0
+        st = gcb.lib().gc_edge_triangles_noalloc(n, C.c_void_p(a.data_ptr()), C.c_void_p(b.data_ptr()),
+                                                 C.c_void_p(out.data_ptr()), h)
+        assert cu.cuStreamEndCapture(h, C.byref(graph)) == 0 and st == 0
+        assert cu.cuGraphGetNodes(graph, None, C.byref(count)) == 0
+        assert cu.cuGraphInstantiateWithFlags(C.byref(ex), graph, C.c_ulonglong(0)) == 0
+        for _ in range(2):
+            out.fill_(-1)
+            torch.cuda.synchronize()
+            assert cu.cuGraphLaunch(ex, h) == 0
+            torch.cuda.synchronize()
+            np.testing.assert_array_equal(out.cpu().numpy(), expect)
+        cu.cuGraphExecDestroy(ex)
+        cu.cuGraphDestroy(graph)
+        assert 1 <= count.value <= most

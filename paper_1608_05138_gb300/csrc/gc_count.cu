@@ -1292,10 +1292,13 @@ size_t smem_bytes(bool smem_table, int32_t table_n) {
   return smem_table ? sizeof(uint32_t) * (size_t)((table_n + 3) & ~3) : 0;
 }
 
+// The limit on a kernel's shared memory is the process's: every call sets it to the
+// most the kernel ever takes, not to what its own graph needs, which another thread
+// might be about to launch with more than.
 template <typename K>
-gc_status launch(K kernel, size_t smem, const DevGraph& g, const CountArgs& a, cudaStream_t s,
+gc_status launch(K kernel, size_t smem, size_t most, const DevGraph& g, const CountArgs& a, cudaStream_t s,
                  const char* what) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   if (e != cudaSuccess) return cuda_fail(e, what);
   int grid = count_grid_size();
   if (a.n_units < grid) grid = a.n_units > 0 ? a.n_units : 1;
@@ -1319,8 +1322,8 @@ int count_grid_size() {
 
 gc_status run_pass_c(const DevGraph& g, const CountArgs& a, cudaStream_t s) {
   const bool sm = a.tables == nullptr;
-  if (sm) return launch(k_pass_c<true>, smem_bytes(true, g.table_n), g, a, s, "k_pass_c");
-  return launch(k_pass_c<false>, smem_bytes(false, g.table_n), g, a, s, "k_pass_c");
+  if (sm) return launch(k_pass_c<true>, smem_bytes(true, g.table_n), smem_bytes(true, kSmemTableMax), g, a, s, "k_pass_c");
+  return launch(k_pass_c<false>, 0, 0, g, a, s, "k_pass_c");
 }
 
 gc_status run_rows(const DevGraph& g, const CountArgs& a, cudaStream_t s) {
@@ -1339,10 +1342,11 @@ gc_status run_rows_dense(const DevGraph& g, const CountArgs& a, cudaStream_t s) 
 gc_status run_cliques_dense(const DevGraph& g, const CountArgs& a, int32_t kmax, cudaStream_t s) {
   const int32_t units = a.ktier_off[kNumTiers];
   if (units <= 0) return GC_OK;
-  const size_t smem = 4 * ((size_t)kmax * dense_stride(kmax) + 2 * (size_t)kmax);  // at most 140 KB
-  cudaError_t e = cudaFuncSetAttribute(k_cliques_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto smem = [](int32_t k) { return 4 * ((size_t)k * dense_stride(k) + 2 * (size_t)k); };
+  cudaError_t e = cudaFuncSetAttribute(k_cliques_dense, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem(kDenseMaxK));  // 140 KB, see launch()
   if (e != cudaSuccess) return cuda_fail(e, "k_cliques_dense");
-  k_cliques_dense<<<units, kDenseBlock, smem, s>>>(g, a, kmax);
+  k_cliques_dense<<<units, kDenseBlock, smem(kmax), s>>>(g, a, kmax);
   e = cudaGetLastError();
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "k_cliques_dense");
 }

@@ -66,9 +66,11 @@ __global__ void __launch_bounds__(256) k_check_csr(int32_t n, int32_t nnz, const
   if (!ok) *bad = 1;
 }
 
-// Submitting is allowed while the calling thread captures one of its own
-// streams: pinning and the device check use other streams, so that they may run
-// then, which the runtime wants to be told.
+// A batch may be used while some thread captures a stream of its own: its work is
+// on other streams, so that its allocations, queries and waits may run then, which
+// the runtime wants to be told (else it refuses them and ends the capture, also
+// when it is another thread's in the default, global mode). Held by every call
+// that does such things and by the dispatcher all its life.
 struct OutsideCapture {
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
   OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
@@ -84,8 +86,12 @@ struct HostBlock {
 };
 
 void free_block(const HostBlock& h) {
-  if (h.pinned) cudaFreeHost(h.p);
-  else delete[] h.p;
+  if (h.pinned) {
+    OutsideCapture relaxed;
+    cudaFreeHost(h.p);
+  } else {
+    delete[] h.p;
+  }
 }
 
 // Host blocks of retired submissions, kept for reuse: a submission takes the
@@ -736,6 +742,7 @@ void run_launch(gc_batch b, std::vector<PendingGraph>& graphs, cudaStream_t s, L
     if (e != cudaSuccess) {
       L->launch_status = cuda_fail(e, "batch event");
       L->error = gc_last_error();
+      cudaStreamSynchronize(s);  // no event tells when the launch's buffers are free
     }
   }
 }
@@ -782,6 +789,7 @@ void retire_locked(gc_batch b) {
       if (q != cudaSuccess) {
         L->launch_status = cuda_fail(q, "batch launch");
         L->error = gc_last_error();
+        cudaStreamSynchronize(L->stream);  // whatever it was, the GPU must be done with the launch's buffers
       }
     }
     if (L->launch_status == GC_OK) {  // device times of the launch
@@ -887,6 +895,7 @@ bool launch_pending(gc_batch b) {
 }
 
 void dispatcher_main(gc_batch b) {
+  OutsideCapture relaxed;
   cudaSetDevice(b->device);
   std::unique_lock<std::mutex> lk(b->mu);
   while (!b->stop) {
@@ -1202,6 +1211,7 @@ gc_status gc_batch_submit_many(gc_batch b, int64_t G, const int32_t* nvert, cons
 gc_status gc_batch_flush(gc_batch b) {
   if (!b) { set_error("batch is NULL"); return GC_ERR_ARG; }
   if (b->flags & GC_BATCH_MANUAL) {
+    OutsideCapture relaxed;
     while (launch_pending(b)) {
     }
   } else {
@@ -1213,6 +1223,7 @@ gc_status gc_batch_flush(gc_batch b) {
 gc_status gc_batch_poll(gc_batch b, uint64_t ticket, uint64_t* global_out, uint64_t* global_hi,
                         int32_t timeout_us) {
   if (!b || !global_out) { set_error("NULL argument"); return GC_ERR_ARG; }
+  OutsideCapture relaxed;
   const auto began = std::chrono::steady_clock::now();
   const auto deadline = began + std::chrono::microseconds(timeout_us > 0 ? timeout_us : 0);
   std::unique_lock<std::mutex> lk(b->mu);
@@ -1253,6 +1264,7 @@ gc_status gc_batch_poll(gc_batch b, uint64_t ticket, uint64_t* global_out, uint6
 gc_status gc_batch_poll_many(gc_batch b, int64_t G, const uint64_t* tickets, uint64_t* global_out,
                              uint64_t* global_hi, int32_t timeout_us) {
   if (!b || G < 0 || (G > 0 && (!tickets || !global_out))) { set_error("bad arguments"); return GC_ERR_ARG; }
+  OutsideCapture relaxed;
   const auto began = std::chrono::steady_clock::now();
   const auto deadline = began + std::chrono::microseconds(timeout_us > 0 ? timeout_us : 0);
   std::unique_lock<std::mutex> lk(b->mu);
@@ -1313,6 +1325,7 @@ gc_status gc_batch_poll_many(gc_batch b, int64_t G, const uint64_t* tickets, uin
 
 gc_status gc_batch_destroy(gc_batch b) {
   if (!b) return GC_OK;
+  OutsideCapture relaxed;
   {
     std::lock_guard<std::mutex> lk(b->mu);
     b->stop = true;

@@ -56,3 +56,39 @@ def test_threads_count_dense_graphs_of_different_sizes():
     finally:
         for g in handles:
             g.close()
+
+
+def batch_count(g):
+    with gcb.Graph(*g) as h:
+        return h.count()
+
+
+def test_batch_goes_on_while_a_thread_captures():
+    # the dispatcher queries events and allocates while the caller has a capture
+    # of the default mode under way, and the caller submits and polls: neither the
+    # capture nor a launch in flight may suffer
+    import torch
+    large = [graphgen.chung_lu(60000, 500000 + 20000 * i, 2.2, 1e6, 3000.0, 3 + i) for i in range(4)]
+    small = [graphgen.er(300 + i, 0.1, i) for i in range(6)]  # of other sizes: buffers grow meanwhile
+    expect = [batch_count(g) for g in large + small]
+    x = torch.zeros(8, device="cuda")
+    b = gcb.gc_batch_create(16 << 30, 0)
+    try:
+        tickets = [gcb.gc_batch_submit(b, *g) for g in large[:2]]
+        for k in range(2):
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                x += 1
+                tickets += [gcb.gc_batch_submit(b, *g) for g in [large[2 + k]] + small[3 * k:3 * k + 3]]
+                gcb.gc_batch_flush(b)
+                time.sleep(0.02)
+                last = gcb.gc_batch_poll(b, tickets.pop(), timeout_us=60_000_000)
+            assert last == expect[4 + 3 * k + 2]
+            graph.replay()
+        torch.cuda.synchronize()
+        order = [0, 1, 2, 4, 5, 3, 7, 8]
+        res = [gcb.gc_batch_poll(b, t, timeout_us=60_000_000) for t in tickets]
+    finally:
+        gcb.gc_batch_destroy(b)
+    assert x.tolist() == [2.0] * 8
+    assert res == [expect[i] for i in order]

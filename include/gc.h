@@ -235,15 +235,22 @@ gc_status gc_release_cached_memory(void);
  * gc_batch_create: a runtime with its own CUDA stream that keeps admitted
  *   graphs resident on the device and counts them in shared launches (one
  *   persistent kernel per pass over all graphs of a launch, with work
- *   stealing over the graphs' vertex groups). device_mem_budget_bytes bounds
- *   the device memory the admitted graphs may hold at once (> 0).
+ *   stealing over the graphs' vertex groups). device_mem_budget_bytes (> 0)
+ *   bounds what the admitted graphs may be charged at once: an estimate by size
+ *   alone, 44 n + 32 m + 1024 bytes a graph, and above 4096 vertices 4 n more for
+ *   each CTA of a persistent grid (two an SM), as if every graph needed count
+ *   tables for all of its vertices. It is no measurement: most graphs need no
+ *   such tables, while a launch takes up to 70 bytes an edge for its
+ *   preparation and count, and lists of triangles of up to 2.5 GB for each range of
+ *   out-degrees. Leave the device room beside the budget.
  *   flags: 0, or GC_BATCH_MANUAL (launch only on gc_batch_flush; otherwise a
  *   dispatcher thread launches pending graphs as soon as the device is free:
  *   continuous batching).
  * gc_batch_submit: validates and copies one CSR graph (same rules as
  *   gc_graph_upload), admits it if it fits in the budget, and returns a
  *   ticket. GC_ERR_BUSY if it does not fit now (retry after polling), or
- *   GC_ERR_NOMEM if it could never fit.
+ *   GC_ERR_NOMEM if it could never fit; an invalid graph gets its own code
+ *   first. A graph holds its share of the budget from before it is checked.
  * gc_batch_flush: launch everything pending now (returns without waiting).
  * gc_batch_poll: waits up to timeout_us microseconds (0 = just test, < 0 =
  *   forever) for the ticket. GC_OK: global_out/global_hi (17 words each, hi

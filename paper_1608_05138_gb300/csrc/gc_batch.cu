@@ -278,6 +278,20 @@ struct gc_batch_s {
   int64_t in_use = 0;
   std::mutex mu;
   std::condition_variable cv;
+  // the budget: admitted graphs, and submissions still being checked
+  bool reserve(int64_t bytes) {
+    std::lock_guard<std::mutex> lk(mu);
+    if (in_use + bytes > budget) return false;
+    in_use += bytes;
+    return true;
+  }
+  void release(int64_t bytes) {
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      in_use -= bytes;
+    }
+    cv.notify_all();
+  }
   std::deque<PendingGraph> pending;
   std::vector<Launch*> inflight;
   std::deque<Ticket> tickets;           // of the numbers first_ticket .. (the oldest one unretired or later)
@@ -1064,15 +1078,25 @@ gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const i
   if (!on_device && (st = validate_csr(n, row_ptr, col_idx)) != GC_OK) return st;
   const int64_t m = row_ptr[n] / 2;
   const int64_t bytes = footprint(n, m);
-  // an invalid graph is refused as such first, whatever its size
-  if (on_device && bytes > b->budget) {
-    if ((st = validate_csr(n, row_ptr, col_idx)) != GC_OK) return st;
-    on_device = false;
+  // Its share of the budget first, so that a graph that does not fit now costs
+  // neither a copy nor device memory for the check. An invalid graph is refused as
+  // such all the same, by the host's checks.
+  if (!b->reserve(bytes)) {
+    if (on_device && (st = validate_csr(n, row_ptr, col_idx)) != GC_OK) return st;
+    if (bytes > b->budget) {
+      set_error("graph needs more device memory than the whole budget");
+      return GC_ERR_NOMEM;
+    }
+    set_error("device-memory budget is full");
+    return GC_ERR_BUSY;
   }
-  if (bytes > b->budget) {
-    set_error("graph needs more device memory than the whole budget");
-    return GC_ERR_NOMEM;
-  }
+  struct Reserved {  // given back unless the graph is admitted
+    gc_batch b;
+    int64_t bytes;
+    ~Reserved() {
+      if (bytes) b->release(bytes);
+    }
+  } reserved = {b, bytes};
   PendingGraph pg;
   pg.n = n;
   pg.m = m;
@@ -1097,14 +1121,10 @@ gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const i
     return st;
   {
     std::lock_guard<std::mutex> lk(b->mu);
-    if (b->in_use + bytes > b->budget) {
-      set_error("device-memory budget is full");
-      return GC_ERR_BUSY;
-    }
     pg.ticket = b->add_ticket();
     *ticket_out = pg.ticket;
-    b->in_use += bytes;
     b->pending.push_back(std::move(pg));
+    reserved.bytes = 0;  // the launch's retirement gives it back
   }
   b->cv.notify_all();
   return GC_OK;

@@ -92,3 +92,37 @@ def test_batch_goes_on_while_a_thread_captures():
         gcb.gc_batch_destroy(b)
     assert x.tolist() == [2.0] * 8
     assert res == [expect[i] for i in order]
+
+
+def test_refused_submissions_take_no_device_memory():
+    # a submission that does not fit in the budget now is refused before it is
+    # copied and checked on the device; an invalid one gets its own code
+    import torch
+    rp, ci = graphgen.er(200000, 4e-4, 5)  # 8M entries: 64 MB of CSR
+    bad = ci.copy()
+    x = int(np.flatnonzero(np.diff(rp) >= 3)[0])
+    bad[rp[x]] = bad[rp[x] + 1]
+    need = 44 * 200000 + 32 * (len(ci) // 2) + 1024 + 2 * 152 * 200000 * 4
+    gcb.gc_release_cached_memory()
+    b = gcb.gc_batch_create(need + 10000, gcb.GC_BATCH_MANUAL)
+    try:
+        t = gcb.gc_batch_submit(b, *graphgen.er(100, 0.5, 1))  # 80 KB of the budget, held until it is launched
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        for _ in range(2):
+            assert gcb.gc_batch_try_submit(b, rp, ci) is None
+        with pytest.raises(gcb.GcError) as ei:
+            gcb.gc_batch_submit(b, rp, bad)
+        assert ei.value.status == -3
+        assert free - torch.cuda.mem_get_info()[0] < 16 << 20
+        gcb.gc_batch_flush(b)
+        assert gcb.gc_batch_poll(b, t) is not None
+        for _ in range(3):  # a refusal gives its share back
+            with pytest.raises(gcb.GcError) as ei:
+                gcb.gc_batch_submit(b, rp, bad)
+            assert ei.value.status == -3
+        t = gcb.gc_batch_submit(b, rp, ci)
+        gcb.gc_batch_flush(b)
+        assert gcb.gc_batch_poll(b, t)[0] == len(ci) // 2
+    finally:
+        gcb.gc_batch_destroy(b)

@@ -251,6 +251,8 @@ gc_status gc_release_cached_memory(void);
  *   ticket. GC_ERR_BUSY if it does not fit now (retry after polling), or
  *   GC_ERR_NOMEM if it could never fit; an invalid graph gets its own code
  *   first. A graph holds its share of the budget from before it is checked.
+ *   Graphs of 2^16 entries or more are checked on the GPU where it has room for
+ *   that at once, else by the host: submitting does not wait for running kernels.
  * gc_batch_flush: launch everything pending now (returns without waiting).
  * gc_batch_poll: waits up to timeout_us microseconds (0 = just test, < 0 =
  *   forever) for the ticket. GC_OK: global_out/global_hi (17 words each, hi

@@ -197,6 +197,18 @@ struct Ticket {
   std::shared_ptr<Results> out;
 };
 
+// One check of a submission on the device (checked_on_device).
+struct Check {
+  cudaStream_t stream = nullptr;     // of high priority, so that it does not wait behind the launches in flight
+  cudaEvent_t done = nullptr;
+  int32_t* bad = nullptr;            // pinned
+  int32_t* d = nullptr;              // flag, row pointers, columns
+  std::shared_ptr<HostBlock> own;    // what the device reads, until the check is over
+  bool busy = false;
+};
+// Checks at a time; a submission that finds them all busy is checked on the host.
+constexpr int kChecks = 4;
+
 // Timers of one launch (CUDA events on its stream): the size classes of the
 // small-graph kernels (eager launches only), the whole small-graph sequence
 // (copies in, kernels, derive, copy out) and the larger graphs' passes.
@@ -315,11 +327,8 @@ struct gc_batch_s {
   }
   bool stop = false;
   std::thread dispatcher;
-  // the device's checks of a submission (one at a time): a stream of high
-  // priority, so that they do not wait behind the launches in flight
-  std::mutex check_mu;
-  cudaStream_t check_stream = nullptr;
-  int32_t* check_bad = nullptr;         // pinned
+  std::mutex check_mu;                  // of the checks' busy marks
+  Check checks[kChecks];
   cudaStream_t streams[kMaxInflight] = {};
   int next_stream = 0;                  // manual mode: round-robin over the slots
   int device = 0;
@@ -941,44 +950,90 @@ void poll_wait(gc_batch b, std::unique_lock<std::mutex>* lk, std::chrono::steady
 
 }  // namespace
 
+// Gives back what the checks hold that the GPU is done with (all: waits for them).
+static void reclaim_checks(gc_batch b, bool all) {
+  for (Check& c : b->checks) {
+    if (!c.busy || !c.own) continue;  // free, or its submission still looks at it
+    if (all) cudaEventSynchronize(c.done);
+    else if (cudaEventQuery(c.done) == cudaErrorNotReady) continue;
+    cudaGetLastError();
+    if (c.d) cudaFreeAsync(c.d, c.stream);
+    c.d = nullptr;
+    c.own.reset();
+    c.busy = false;
+  }
+}
+
 // Whether the graph copied to `own` (row pointers, then columns; pinned) passes
 // every check of validate_csr, by k_check_csr; its row pointers have been
-// checked. false also when a device step fails: the caller then asks the host.
-static bool checked_on_device(gc_batch b, int32_t n, int32_t nnz, const int32_t* own) {
-  std::lock_guard<std::mutex> lk(b->check_mu);
+// checked. false also when a device step fails, when the checks are all busy, or
+// when the GPU has no room for the check in time: the caller then asks the host.
+// Neither priority nor anything else takes a running CTA's place, so that behind
+// kernels that fill the GPU a check would last as long as they do: a submission
+// gives it 0.3 ms and 0.5 ns an entry (3.5M entries take 0.9 ms on an idle GPU, the
+// host's checks 6.2), and leaves what it holds to a later one.
+static bool checked_on_device(gc_batch b, int32_t n, int32_t nnz, const std::shared_ptr<HostBlock>& own) {
   OutsideCapture relaxed;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || (dev != b->device && cudaSetDevice(b->device) != cudaSuccess)) {
     cudaGetLastError();
     return false;
   }
-  cudaError_t e = cudaSuccess;
-  if (!b->check_stream) {
-    int least = 0, greatest = 0;
-    e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->check_stream, cudaStreamNonBlocking, greatest);
-    if (e == cudaSuccess) e = cudaMallocHost(&b->check_bad, sizeof(int32_t));
+  Check* c = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(b->check_mu);
+    reclaim_checks(b, false);
+    for (Check& k : b->checks)
+      if (!k.busy) {
+        c = &k;
+        c->busy = true;
+        break;
+      }
   }
-  int32_t* d = nullptr;  // flag, row pointers, columns
-  const size_t words = (size_t)n + 1 + (size_t)nnz;
-  cudaStream_t s = b->check_stream;
-  bool ok = false;
-  if (e == cudaSuccess && b->check_bad) {
-    e = pool_alloc(&d, sizeof(int32_t) * (words + 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d, 0, sizeof(int32_t), s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d + 1, own, sizeof(int32_t) * words, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) {
-      const int64_t blocks = ((int64_t)nnz + 255) / 256;
-      k_check_csr<<<(int)std::min<int64_t>(blocks, 8LL * (count_grid_size() / kCtasPerSm)), 256, 0, s>>>(
-          n, nnz, d + 1, d + 1 + n + 1, d);
-      e = cudaGetLastError();
+  bool ok = false, left = false;
+  if (c) {
+    cudaError_t e = cudaSuccess;
+    if (!c->stream) {
+      int least = 0, greatest = 0;
+      e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+      if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->stream, cudaStreamNonBlocking, greatest);
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->check_bad, d, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-    const cudaError_t e2 = cudaStreamSynchronize(s);  // also after a failure: `own` may be read
-    ok = e == cudaSuccess && e2 == cudaSuccess && *b->check_bad == 0;
-    if (d) cudaFreeAsync(d, s);
+    if (e == cudaSuccess && !c->done) e = cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming);
+    if (e == cudaSuccess && !c->bad) e = cudaMallocHost(&c->bad, sizeof(int32_t));
+    const size_t words = (size_t)n + 1 + (size_t)nnz;
+    bool queued = false;
+    if (e == cudaSuccess && (e = pool_alloc(&c->d, sizeof(int32_t) * (words + 1), c->stream)) == cudaSuccess) {
+      queued = true;
+      e = cudaMemsetAsync(c->d, 0, sizeof(int32_t), c->stream);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->d + 1, own->p, sizeof(int32_t) * words, cudaMemcpyHostToDevice, c->stream);
+      if (e == cudaSuccess) {
+        const int64_t blocks = ((int64_t)nnz + 255) / 256;
+        k_check_csr<<<(int)std::min<int64_t>(blocks, 8LL * (count_grid_size() / kCtasPerSm)), 256, 0, c->stream>>>(
+            n, nnz, c->d + 1, c->d + 1 + n + 1, c->d);
+        e = cudaGetLastError();
+      }
+      if (e == cudaSuccess) e = cudaMemcpyAsync(c->bad, c->d, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream);
+      if (e == cudaSuccess) e = cudaEventRecord(c->done, c->stream);
+    }
+    if (e == cudaSuccess) {
+      const auto until = std::chrono::steady_clock::now() + std::chrono::nanoseconds(300000 + (int64_t)nnz / 2);
+      while ((e = cudaEventQuery(c->done)) == cudaErrorNotReady && std::chrono::steady_clock::now() < until)
+        std::this_thread::yield();
+      left = e == cudaErrorNotReady;
+      ok = e == cudaSuccess && *c->bad == 0;
+    }
+    if (queued && !left && e != cudaSuccess) cudaStreamSynchronize(c->stream);  // `own` may be read
+    if (e != cudaSuccess) cudaGetLastError();
+    std::lock_guard<std::mutex> lk(b->check_mu);
+    if (left) {
+      c->own = own;  // busy until reclaimed
+    } else {
+      if (c->d) cudaFreeAsync(c->d, c->stream);
+      c->d = nullptr;
+      c->busy = false;
+    }
   }
-  if (!ok) cudaGetLastError();
   if (dev != b->device) cudaSetDevice(dev);
   return ok;
 }
@@ -1116,7 +1171,7 @@ gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const i
     set_error("host allocation failed");
     return GC_ERR_NOMEM;
   }
-  if (on_device && !(pg.owner->pinned && checked_on_device(b, n, row_ptr[n], pg.rp)) &&
+  if (on_device && !(pg.owner->pinned && checked_on_device(b, n, row_ptr[n], pg.owner)) &&
       (st = validate_csr(n, pg.rp, pg.ci)) != GC_OK)
     return st;
   {
@@ -1360,11 +1415,15 @@ gc_status gc_batch_destroy(gc_batch b) {
   for (auto& sb : b->small) free_small_bufs(&sb);
   for (auto* f : b->forks) fork_release(f);
   for (Launch* L : b->spare) free_launch(L);
-  if (b->check_stream) {
-    cudaStreamSynchronize(b->check_stream);
-    cudaStreamDestroy(b->check_stream);
+  reclaim_checks(b, true);
+  for (Check& c : b->checks) {
+    if (c.stream) {
+      cudaStreamSynchronize(c.stream);
+      cudaStreamDestroy(c.stream);
+    }
+    if (c.done) cudaEventDestroy(c.done);
+    if (c.bad) cudaFreeHost(c.bad);
   }
-  if (b->check_bad) cudaFreeHost(b->check_bad);
   for (auto& s : b->streams) cudaStreamDestroy(s);
   delete b;
   return GC_OK;

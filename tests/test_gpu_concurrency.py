@@ -126,3 +126,64 @@ def test_refused_submissions_take_no_device_memory():
         assert gcb.gc_batch_poll(b, t)[0] == len(ci) // 2
     finally:
         gcb.gc_batch_destroy(b)
+
+
+@pytest.fixture(scope="module")
+def hold_gpu():
+    """hold(seconds): kernels whose long-lived CTAs take every thread of the GPU, on the current stream."""
+    import torch
+    code = "template <typename T> T hold(T x, float n) { for (int i = 0; i < (int)n; ++i) x = x * 1.0000001f + 1e-7f; return x; }"
+    fn = torch.cuda.jiterator._create_jit_fn(code, n=1.0)
+    x = torch.zeros(torch.cuda.get_device_properties(0).multi_processor_count * 16 * 512 * 4, device="cuda")
+
+    def took(n):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        fn(x, n=n)
+        torch.cuda.synchronize()
+        return time.perf_counter() - t
+
+    took(1e3)
+    per = (took(4e5) - took(1e5)) / 3e5
+    return lambda seconds: fn(x, n=float(int(seconds / per)))
+
+
+def test_submitting_does_not_wait_for_running_kernels(hold_gpu):
+    # graphs of 2^16 entries or more are checked on the device where it has room
+    import torch
+    g = graphgen.er(3000, 0.03, 9)
+    assert len(g[1]) >= 1 << 16
+    bad = g[1].copy()
+    bad[g[0][5]] = bad[g[0][5] + 1]
+    expect = batch_count(g)
+    b = gcb.gc_batch_create(8 << 30, gcb.GC_BATCH_MANUAL)
+    try:
+        tickets = [gcb.gc_batch_submit(b, *g) for _ in range(8)]  # the blocks and streams exist from here on
+        gcb.gc_batch_flush(b)
+        assert all(gcb.gc_batch_poll(b, t) == expect for t in tickets)
+        hold_gpu(2.0)
+        done = torch.cuda.Event()
+        done.record()
+        worst, tickets = [], []
+
+        def submit():
+            t = time.perf_counter()
+            tickets.append(gcb.gc_batch_submit(b, *g))
+            worst.append(time.perf_counter() - t)
+
+        def refused():
+            with pytest.raises(gcb.GcError) as ei:
+                gcb.gc_batch_submit(b, g[0], bad)
+            assert ei.value.status == -3
+
+        submit()
+        run_threads(*[submit] * 6, refused)  # more than the checks that may run at a time
+        assert not done.query()  # the GPU was taken all the while
+        assert max(worst) < 0.1
+        gcb.gc_batch_flush(b)
+        assert all(gcb.gc_batch_poll(b, t) == expect for t in tickets)
+        t = gcb.gc_batch_submit(b, *g)  # what the checks left behind is taken up again
+        gcb.gc_batch_flush(b)
+        assert gcb.gc_batch_poll(b, t) == expect
+    finally:
+        gcb.gc_batch_destroy(b)

@@ -273,10 +273,10 @@ gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const i
  * returned (message names its index), GC_ERR_BUSY if they do not fit in the
  * budget now. tickets_out receives G tickets. Host pointers; copied into a
  * pinned host block, from which the launch copies to the device, and which the
- * batch keeps for reuse once the graphs retire (at most four blocks of 64 MiB or
- * more and 64 smaller ones, the smallest given back first; all freed by
- * gc_batch_destroy once no graph holds them). gc_batch_submit takes its copy
- * from the same blocks. */
+ * batch keeps for reuse once the graphs retire (when it has nothing to do, at
+ * most four blocks of 64 MiB or more and 64 smaller ones, the smallest given back
+ * first; all freed by gc_batch_destroy once no graph holds them). gc_batch_submit
+ * takes its copy from the same blocks. */
 gc_status gc_batch_submit_many(gc_batch b, int64_t G, const int32_t* nvert, const int64_t* voff, const int64_t* eoff,
                                const int32_t* row_ptr, const int32_t* col_idx, uint64_t* tickets_out);
 gc_status gc_batch_flush(gc_batch b);

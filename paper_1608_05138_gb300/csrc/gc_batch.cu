@@ -21,10 +21,11 @@
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <iterator>
+#include <map>
+#include <memory>
 #include <mutex>
 #include <string>
-#include <thread>
-#include <memory>
 #include <thread>
 #include <vector>
 
@@ -97,17 +98,42 @@ void free_block(const HostBlock& h) {
 // Host blocks of retired submissions, kept for reuse: a submission takes the
 // smallest kept block that holds it and is not more than twice as large, whose
 // pages are already mapped and pinned, instead of a fresh allocation. Blocks are
-// not initialised (the copy that fills one writes every entry it reads). Kept
-// are at most kLarge blocks of kLargeBytes or more and kSmall others; the cache
-// lives until the batch and its last block are gone.
+// not initialised (the copy that fills one writes every entry it reads). A
+// returned block is kept whatever the number, since giving pinned memory back
+// waits for the whole device; trim(), called without any lock when the batch has
+// nothing to do, keeps at most kLarge blocks of kLargeEntries or more and kSmall
+// others, the largest. The cache lives until the batch and its last block are gone.
 struct HostCache {
-  static constexpr int kLarge = 4, kSmall = 64;
+  static constexpr size_t kLarge = 4, kSmall = 64;
   static constexpr size_t kLargeEntries = (size_t)16 << 20;
   std::mutex mu;
-  std::vector<HostBlock> free;
-  HostCache() { free.reserve(kLarge + kSmall + 1); }  // a returned block never allocates
+  std::multimap<size_t, HostBlock> free;  // by capacity
   ~HostCache() {
-    for (auto& h : free) free_block(h);
+    for (auto& h : free) free_block(h.second);
+  }
+  void put(const HostBlock& h) {
+    try {
+      std::lock_guard<std::mutex> lk(mu);
+      free.emplace(h.cap, h);
+      return;
+    } catch (...) {  // no memory to keep it
+    }
+    free_block(h);
+  }
+  void trim() {
+    for (;;) {
+      HostBlock out;
+      {
+        std::lock_guard<std::mutex> lk(mu);
+        const auto large = free.lower_bound(kLargeEntries);
+        const size_t n_large = (size_t)std::distance(large, free.end());
+        auto it = n_large > kLarge ? large : free.size() - n_large > kSmall ? free.begin() : free.end();
+        if (it == free.end()) return;
+        out = it->second;
+        free.erase(it);
+      }
+      free_block(out);
+    }
   }
 };
 
@@ -127,14 +153,10 @@ std::shared_ptr<HostBlock> host_block(const std::shared_ptr<HostCache>& cache, s
   HostBlock h;
   {
     std::lock_guard<std::mutex> lk(cache->mu);
-    int best = -1;
-    for (int i = 0; i < (int)cache->free.size(); ++i) {
-      const size_t cap = cache->free[(size_t)i].cap;
-      if (cap >= entries && cap / 2 <= entries && (best < 0 || cap < cache->free[(size_t)best].cap)) best = i;
-    }
-    if (best >= 0) {
-      h = cache->free[(size_t)best];
-      cache->free.erase(cache->free.begin() + best);
+    const auto it = cache->free.lower_bound(entries);
+    if (it != cache->free.end() && it->first / 2 <= entries) {
+      h = it->second;
+      cache->free.erase(it);
     }
   }
   if (!h.p) {
@@ -149,25 +171,9 @@ std::shared_ptr<HostBlock> host_block(const std::shared_ptr<HostCache>& cache, s
   }
   std::shared_ptr<HostCache> keep = cache;
   return std::shared_ptr<HostBlock>(new HostBlock(h), [keep](HostBlock* q) {
-    HostBlock out = *q;
+    const HostBlock out = *q;
     delete q;
-    {
-      std::lock_guard<std::mutex> lk(keep->mu);
-      const bool large = out.cap >= HostCache::kLargeEntries;
-      keep->free.push_back(out);
-      out.p = nullptr;
-      int count = 0, least = -1;
-      for (int i = 0; i < (int)keep->free.size(); ++i) {
-        if ((keep->free[(size_t)i].cap >= HostCache::kLargeEntries) != large) continue;
-        ++count;
-        if (least < 0 || keep->free[(size_t)i].cap < keep->free[(size_t)least].cap) least = i;
-      }
-      if (count > (large ? HostCache::kLarge : HostCache::kSmall)) {
-        out = keep->free[(size_t)least];
-        keep->free.erase(keep->free.begin() + least);
-      }
-    }
-    if (out.p) free_block(out);
+    keep->put(out);
   });
 }
 
@@ -308,7 +314,7 @@ struct gc_batch_s {
   std::vector<Launch*> inflight;
   std::deque<Ticket> tickets;           // of the numbers first_ticket .. (the oldest one unretired or later)
   uint64_t first_ticket = 1;
-  std::vector<Launch*> spare;           // retired launches, for their events and pinned results (at most kMaxSpare)
+  std::vector<Launch*> spare;           // retired launches, for their events and pinned results (trimmed to kMaxSpare)
   Ticket* find(uint64_t t) {            // nullptr: unknown or retired
     if (t < first_ticket || t - first_ticket >= tickets.size()) return nullptr;
     Ticket* k = &tickets[(size_t)(t - first_ticket)];
@@ -846,11 +852,29 @@ void retire_locked(gc_batch b) {
     }
     b->in_use -= L->bytes;
     L->owners.clear();
-    if (b->spare.size() < kMaxSpare) b->spare.push_back(L);
-    else free_launch(L);
+    b->spare.push_back(L);
     b->inflight.erase(b->inflight.begin() + i);
     b->cv.notify_all();
   }
+}
+
+// Whether the batch has nothing to do. Must hold b->mu.
+bool idle(gc_batch b) { return b->pending.empty() && b->inflight.empty(); }
+
+// Gives back the pinned memory kept beyond the limits. Freeing it waits for the
+// whole device, so no lock is held and the batch is idle.
+void trim(gc_batch b) {
+  for (;;) {
+    Launch* L = nullptr;
+    {
+      std::lock_guard<std::mutex> lk(b->mu);
+      if (b->spare.size() <= kMaxSpare) break;
+      L = b->spare.back();
+      b->spare.pop_back();
+    }
+    free_launch(L);
+  }
+  b->host->trim();
 }
 
 // Takes every pending graph (up to the int32 edge limit) and launches it.
@@ -921,8 +945,18 @@ void dispatcher_main(gc_batch b) {
   OutsideCapture relaxed;
   cudaSetDevice(b->device);
   std::unique_lock<std::mutex> lk(b->mu);
+  bool trimmed = true;  // since the batch was last busy
   while (!b->stop) {
     retire_locked(b);
+    if (!idle(b)) {
+      trimmed = false;
+    } else if (!trimmed) {
+      trimmed = true;
+      lk.unlock();
+      trim(b);
+      lk.lock();
+      continue;
+    }
     if (!b->pending.empty() && (int)b->inflight.size() < b->cfg.max_inflight) {
       lk.unlock();
       launch_pending(b);
@@ -1313,6 +1347,9 @@ gc_status gc_batch_poll(gc_batch b, uint64_t ticket, uint64_t* global_out, uint6
       const Ticket r = std::move(*t);
       *t = Ticket();
       b->drop_retired();
+      const bool rest = (b->flags & GC_BATCH_MANUAL) && idle(b);
+      lk.unlock();
+      if (rest) trim(b);  // otherwise the dispatcher's
       if (r.status != GC_OK) {
         set_error("batch launch failed");
         return r.status;
@@ -1390,6 +1427,9 @@ gc_status gc_batch_poll_many(gc_batch b, int64_t G, const uint64_t* tickets, uin
   for (int64_t i = 0; i < G; ++i)
     if (Ticket* t = b->find(tickets[i])) *t = Ticket();
   b->drop_retired();
+  const bool rest = (b->flags & GC_BATCH_MANUAL) && idle(b);
+  lk.unlock();
+  if (rest) trim(b);
   if (first != GC_OK) return first;
   if (need_hi && !global_hi) {
     set_error("a global count exceeds 64 bits and global_hi is NULL");

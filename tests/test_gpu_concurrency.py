@@ -187,3 +187,47 @@ def test_submitting_does_not_wait_for_running_kernels(hold_gpu):
         assert gcb.gc_batch_poll(b, t) == expect
     finally:
         gcb.gc_batch_destroy(b)
+
+
+@pytest.mark.parametrize("flags", [0, gcb.GC_BATCH_MANUAL])
+def test_pinned_memory_is_given_back_without_the_lock(flags):
+    # 150 outstanding submissions hold 150 pinned blocks, of which 64 are kept;
+    # giving the others back waits for the whole device, here a kernel that sleeps,
+    # and must not keep other threads' calls waiting
+    import torch
+    g = graphgen.er(200, 0.25, 9)  # above 4096 entries: pinned
+    expect = batch_count(g)
+    b = gcb.gc_batch_create(8 << 30, flags)
+    try:
+        # not launched one by one as they come: behind one long launch
+        first = gcb.gc_batch_submit(b, *graphgen.chung_lu(200000, 3000000, 2.1, 6e6, 30000.0, 3))
+        tickets = [gcb.gc_batch_submit(b, *g) for _ in range(150)]
+        gcb.gc_batch_flush(b)
+        if flags:
+            torch.cuda.synchronize()
+            torch.cuda._sleep(2_000_000_000)
+        else:
+            while gcb.gc_batch_poll(b, first, timeout_us=0) is None:
+                time.sleep(1e-4)
+            torch.cuda._sleep(2_000_000_000)
+        done = torch.cuda.Event()
+        done.record()
+        worst = []
+
+        def others():
+            time.sleep(0.05)
+            while not done.query() and len(worst) < 50:
+                t = time.perf_counter()
+                extra = gcb.gc_batch_submit(b, *g)
+                assert flags or gcb.gc_batch_poll(b, extra, timeout_us=0) in (None, expect)
+                worst.append(time.perf_counter() - t)
+                time.sleep(0.005)
+
+        def poll():
+            got = gcb.gc_batch_poll_many(b, np.array(tickets, np.uint64))
+            assert all(int(v) == e for x in got for v, e in zip(x[:, 0], expect))
+
+        run_threads(poll, others)
+        assert len(worst) > 5 and max(worst) < 0.2
+    finally:
+        gcb.gc_batch_destroy(b)

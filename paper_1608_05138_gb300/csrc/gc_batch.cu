@@ -27,6 +27,7 @@
 #include <mutex>
 #include <string>
 #include <thread>
+#include <unordered_map>
 #include <vector>
 
 #include "gc_deal.h"
@@ -314,19 +315,43 @@ struct gc_batch_s {
   std::vector<Launch*> inflight;
   std::deque<Ticket> tickets;           // of the numbers first_ticket .. (the oldest one unretired or later)
   uint64_t first_ticket = 1;
+  size_t live = 0;                      // tickets not retired
+  std::unordered_map<uint64_t, Ticket> old;  // unretired tickets below first_ticket, long unpolled
   std::vector<Launch*> spare;           // retired launches, for their events and pinned results (trimmed to kMaxSpare)
   Ticket* find(uint64_t t) {            // nullptr: unknown or retired
-    if (t < first_ticket || t - first_ticket >= tickets.size()) return nullptr;
+    if (t < first_ticket) {
+      const auto it = old.find(t);
+      return it == old.end() ? nullptr : &it->second;
+    }
+    if (t - first_ticket >= tickets.size()) return nullptr;
     Ticket* k = &tickets[(size_t)(t - first_ticket)];
     return k->state == Ticket::kRetired ? nullptr : k;
   }
   uint64_t add_ticket() {
     tickets.emplace_back();
     tickets.back().state = Ticket::kLive;
+    ++live;
     return first_ticket + tickets.size() - 1;
   }
+  void retire(uint64_t t) {
+    if (t < first_ticket) old.erase(t);
+    else tickets[(size_t)(t - first_ticket)] = Ticket();
+    --live;
+  }
+  // A ticket that is never polled does not keep all later ones: where most of the
+  // queue is retired, its oldest move out of it.
   void drop_retired() {
-    while (!tickets.empty() && tickets.front().state == Ticket::kRetired) {
+    while (!tickets.empty()) {
+      Ticket& f = tickets.front();
+      if (f.state != Ticket::kRetired) {
+        if (tickets.size() <= 4096 + 2 * live) break;
+        try {
+          old.reserve(old.size() + 1);  // nothing is moved before all memory is there
+          old.emplace(first_ticket, std::move(f));
+        } catch (...) {
+          break;  // no memory for it: it stays
+        }
+      }
       tickets.pop_front();
       ++first_ticket;
     }
@@ -1345,7 +1370,7 @@ gc_status gc_batch_poll(gc_batch b, uint64_t ticket, uint64_t* global_out, uint6
     if (b->flags & GC_BATCH_MANUAL) retire_locked(b);
     if (t->state == Ticket::kDone) {
       const Ticket r = std::move(*t);
-      *t = Ticket();
+      b->retire(ticket);
       b->drop_retired();
       const bool rest = (b->flags & GC_BATCH_MANUAL) && idle(b);
       lk.unlock();
@@ -1425,7 +1450,7 @@ gc_status gc_batch_poll_many(gc_batch b, int64_t G, const uint64_t* tickets, uin
     }
   }
   for (int64_t i = 0; i < G; ++i)
-    if (Ticket* t = b->find(tickets[i])) *t = Ticket();
+    if (b->find(tickets[i])) b->retire(tickets[i]);
   b->drop_retired();
   const bool rest = (b->flags & GC_BATCH_MANUAL) && idle(b);
   lk.unlock();

@@ -231,3 +231,45 @@ def test_pinned_memory_is_given_back_without_the_lock(flags):
         assert len(worst) > 5 and max(worst) < 0.2
     finally:
         gcb.gc_batch_destroy(b)
+
+
+def test_a_ticket_that_is_never_polled_keeps_no_later_ones():
+    import os
+    import subprocess
+    import sys
+    code = """
+import ctypes, numpy as np, graphgen, paper_1608_05138_gb300 as gc
+class Info(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_size_t) for k in 'arena ordblks smblks hblks hblkhd usmblks fsmblks uordblks fordblks keepcost'.split()]
+mallinfo2 = ctypes.CDLL(None).mallinfo2
+mallinfo2.restype = Info
+def held():  # bytes of this thread's heap in use
+    return mallinfo2().uordblks + mallinfo2().hblkhd
+b = gc.gc_batch_create(8 << 30, gc.GC_BATCH_MANUAL)
+first = graphgen.er(30, 0.2, 1)
+t0 = gc.gc_batch_submit(b, *first)
+G = 100000
+nv, vo, eo = np.full(G, 2), np.arange(G + 1) * 3, np.arange(G + 1) * 2
+rp, ci = np.tile(np.array([0, 1, 2], np.int32), G), np.tile(np.array([1, 0], np.int32), G)
+size = []
+for i in range(40):
+    t = gc.gc_batch_submit_many(b, nv, vo, eo, rp, ci)
+    gc.gc_batch_flush(b)
+    x = gc.gc_batch_poll_many(b, t)
+    assert (x[:, 0, 0] == 1).all()
+    if i in (4, 39):
+        size.append(held())
+assert size[1] - size[0] < 40 << 20, size
+with gc.Graph(*first) as g:
+    assert gc.gc_batch_poll(b, t0) == g.count()
+try:
+    gc.gc_batch_poll(b, t0)
+    raise SystemExit('a retired ticket was found')
+except gc.GcError:
+    pass
+gc.gc_batch_destroy(b)
+print('ok')
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr

@@ -632,6 +632,7 @@ gc_status run_small(std::vector<PendingGraph*>& graphs, cudaStream_t s, Launch* 
     if ((size_t)G + 1 > sb->cap_g || !sb->d_voff) {
       size_t c1 = 0;
       const size_t need = (size_t)G + 1;
+      sb->cap_g = 0;  // until all of them hold it: a failure below leaves some without memory
       GS_TRY(grow_pair(&sb->d_voff, &sb->h_voff, &c1, need), "small buffers");
       c1 = 0; GS_TRY(grow_pair(&sb->d_eoff, &sb->h_eoff, &c1, need), "small buffers");
       c1 = 0; GS_TRY(grow_pair(&sb->d_gm, &sb->h_gm, &c1, need), "small buffers");

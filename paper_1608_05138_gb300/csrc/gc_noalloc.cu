@@ -159,16 +159,18 @@ __global__ void __launch_bounds__(kTriBlock) k_rows(int32_t n, const int32_t* __
   }
 }
 
-// The lower neighbours of x in one window of 32 slots of its row: lane l's
-// slot p, and whether it is counted here (both rows follow the rules, and y is
-// below x in (degree, id)); its row [yb, yb + L).
+// The lower neighbours of x in one window of 32 slots of its row, which starts at
+// b: the lane's is the k-th, if below end, and whether it is counted here (both
+// rows follow the rules, and y is below x in (degree, id)); its row [yb, yb + L).
+// Places in a row are counted from its start all through these kernels: a slot,
+// which may be up to 2^31 - 2, plus a step or another slot would not fit 32 bits.
 __device__ __forceinline__ void lower_slot(int32_t n, const int32_t* rp, const int32_t* ci, const uint32_t* scratch,
-                                           int32_t x, int32_t dx, int32_t p, int32_t e, int32_t& yb, int32_t& L,
-                                           bool& mine) {
+                                           int32_t x, int32_t dx, int32_t b, int32_t k, int32_t end, int32_t& yb,
+                                           int32_t& L, bool& mine) {
   yb = L = 0;
   mine = false;
-  if (p >= e) return;
-  const int32_t y = ci[p];
+  if (k >= end) return;
+  const int32_t y = ci[b + k];
   if ((uint32_t)y >= (uint32_t)n || row_bad(scratch, y)) return;
   yb = rp[y];
   const int32_t dy = rp[y + 1] - yb;
@@ -317,7 +319,7 @@ __device__ __forceinline__ void short_rows(int32_t n, const int32_t* __restrict_
     x0 = __shfl_sync(0xffffffffu, x0, 0);
     if (x0 >= n) break;
     for (int32_t x = x0; x < min(x0 + take, n); ++x) {
-      const int32_t b = rp[x], e = rp[x + 1], d = e - b;
+      const int32_t b = rp[x], d = rp[x + 1] - b;
       if (d > longest || d == 0 || row_bad(scratch, x)) continue;  // warp-uniform
       int bits = 5;
       while ((1 << bits) < 2 * d) ++bits;  // at most log2(kShortSlots)
@@ -326,8 +328,8 @@ __device__ __forceinline__ void short_rows(int32_t n, const int32_t* __restrict_
       for (int i = lane; i <= (int)mask; i += 32) key[i] = -1;
       for (int i = lane; i < (1 << fbits) / 32; i += 32) filt[i] = 0u;
       __syncwarp();
-      for (int32_t p = b + lane; p < e; p += 32) {
-        const int32_t y = ci[p];
+      for (int32_t k = lane; k < d; k += 32) {
+        const int32_t y = ci[b + k];
         const uint32_t hy = (uint32_t)y * 0x9E3779B1u;
         uint32_t s = hy >> (32 - bits);
         while (atomicCAS(&key[s], -1, y) != -1) s = (s + 1) & mask;  // rows ascend: no y twice, half full
@@ -335,10 +337,10 @@ __device__ __forceinline__ void short_rows(int32_t n, const int32_t* __restrict_
         atomicOr(&filt[f >> 5], 1u << (f & 31));
       }
       __syncwarp();
-      for (int32_t p0 = b; p0 < e; p0 += 32) {
+      for (int32_t k0 = 0; k0 < d; k0 += 32) {
         int32_t yb, L;
         bool mine;
-        lower_slot(n, rp, ci, scratch, x, d, p0 + lane, e, yb, L, mine);
+        lower_slot(n, rp, ci, scratch, x, d, b, k0 + lane, d, yb, L, mine);
         cnt[lane] = 0;
         __syncwarp();
         count_runs(ci, yb, L, cnt, lane, [&](int32_t w) -> bool {
@@ -353,7 +355,7 @@ __device__ __forceinline__ void short_rows(int32_t n, const int32_t* __restrict_
           }
         });
         __syncwarp();
-        if (mine) tri[p0 + lane] = cnt[lane];
+        if (mine) tri[b + k0 + lane] = cnt[lane];
         __syncwarp();
       }
     }
@@ -370,7 +372,7 @@ __device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict_
                                            uint32_t* bm /* (n + 31) / 32 words */, int32_t* cnt) {
   __shared__ uint32_t s_x;
   __shared__ int32_t s_next, s_heavy;
-  __shared__ int32_t s_hp[kPart], s_hb[kPart], s_he[kPart], s_hc[kPart];  // the listed slots, their rows, their counts
+  __shared__ int32_t s_hp[kPart], s_hb[kPart], s_hl[kPart], s_hc[kPart];  // the listed slots, their rows, their counts
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t nnz = rp[n];
   const int32_t window = window_of(nnz), slots = part_of(nnz);
@@ -394,30 +396,30 @@ __device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict_
     if (s_x == kNoPart) break;
     const int32_t x = (int32_t)(s_x & 0xfffffu), part = (int32_t)(s_x >> 20);
     if (x >= n || row_bad(scratch, x)) continue;
-    const int32_t b = rp[x], e = rp[x + 1];
-    const int32_t pe = (int32_t)min((int64_t)e, (int64_t)b + (int64_t)(part + 1) * slots);
+    const int32_t b = rp[x], d = rp[x + 1] - b;
+    const int32_t end = min(d, (part + 1) * slots);  // at most 4096 parts of at most 512 slots
     if (threadIdx.x == 0) {
-      s_next = (int32_t)min((int64_t)pe, (int64_t)b + (int64_t)part * slots);
+      s_next = min(end, part * slots);
       s_heavy = 0;
     }
-    for (int32_t p = b + threadIdx.x; p < e; p += kNoAllocBlock) {
-      const int32_t y = ci[p];
+    for (int32_t k = threadIdx.x; k < d; k += kNoAllocBlock) {
+      const int32_t y = ci[b + k];
       if ((uint32_t)y < (uint32_t)n) atomicOr(&bm[y >> 5], 1u << (y & 31));
     }
     __syncthreads();
     for (;;) {
-      int32_t p0 = 0;
-      if (lane == 0) p0 = atomicAdd(&s_next, window);
-      p0 = __shfl_sync(0xffffffffu, p0, 0);
-      if (p0 >= pe) break;
+      int32_t k0 = 0;
+      if (lane == 0) k0 = atomicAdd(&s_next, window);
+      k0 = __shfl_sync(0xffffffffu, k0, 0);
+      if (k0 >= end) break;
       int32_t yb, L;
       bool mine;
-      lower_slot(n, rp, ci, scratch, x, e - b, p0 + lane, min(pe, p0 + window), yb, L, mine);
+      lower_slot(n, rp, ci, scratch, x, d, b, k0 + lane, min(end, k0 + window), yb, L, mine);
       if (L >= kHeavyRun) {
         const int32_t k = atomicAdd(&s_heavy, 1);
-        s_hp[k] = p0 + lane;
+        s_hp[k] = b + k0 + lane;
         s_hb[k] = yb;
-        s_he[k] = yb + L;
+        s_hl[k] = L;
         s_hc[k] = 0;
         L = 0;
         mine = false;
@@ -426,18 +428,18 @@ __device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict_
       __syncwarp();
       count_runs(ci, yb, L, cnt, lane, in);
       __syncwarp();
-      if (mine) tri[p0 + lane] = cnt[lane];
+      if (mine) tri[b + k0 + lane] = cnt[lane];
       __syncwarp();
     }
     __syncthreads();
     const int32_t heavy = s_heavy;
     for (int32_t k = 0; k < heavy; ++k) {
-      const int32_t yb = s_hb[k], ye = s_he[k];
+      const int32_t *row = ci + s_hb[k], len = s_hl[k];
       int32_t c = 0;
-      for (int32_t q0 = yb + 128 * warp; q0 < ye; q0 += 128 * (kNoAllocBlock / 32)) {
+      for (int32_t q0 = 128 * warp; q0 < len; q0 += 128 * (kNoAllocBlock / 32)) {
         int32_t w[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = q0 + 32 * j + lane < ye ? ci[q0 + 32 * j + lane] : -1;
+        for (int j = 0; j < 4; ++j) w[j] = q0 + 32 * j + lane < len ? row[q0 + 32 * j + lane] : -1;
 #pragma unroll
         for (int j = 0; j < 4; ++j) c += w[j] >= 0 && in(w[j]);
       }
@@ -446,8 +448,8 @@ __device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict_
     }
     __syncthreads();
     for (int32_t k = threadIdx.x; k < heavy; k += kNoAllocBlock) tri[s_hp[k]] = s_hc[k];
-    for (int32_t p = b + threadIdx.x; p < e; p += kNoAllocBlock) {
-      const int32_t y = ci[p];
+    for (int32_t k = threadIdx.x; k < d; k += kNoAllocBlock) {
+      const int32_t y = ci[b + k];
       if ((uint32_t)y < (uint32_t)n) bm[y >> 5] = 0u;
     }
   }
@@ -496,7 +498,7 @@ __global__ void __launch_bounds__(kTriBlock) k_tri_reverse(int32_t n, const int3
       if (dy < dx || (dy == dx && y < x)) continue;  // counted at this slot
       int32_t lo = yb, hi = ye;
       while (lo < hi) {
-        const int32_t mid = (lo + hi) >> 1;
+        const int32_t mid = lo + ((hi - lo) >> 1);
         if (ci[mid] < x) lo = mid + 1; else hi = mid;
       }
       found = lo < ye && ci[lo] == x;
@@ -525,30 +527,31 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_tri_marked(int32_t n, const i
   for (int32_t i = threadIdx.x; i < words; i += kNoAllocBlock) bm[i] = 0u;
   __syncthreads();
   for (int32_t x = blockIdx.x; x < n; x += gridDim.x) {
-    const int32_t xb = rp[x], xe = rp[x + 1];
+    const int32_t xb = rp[x];
+    const uint32_t d = (uint32_t)(rp[x + 1] - xb);
     bool any = false;
-    for (int32_t p = xb + threadIdx.x; p < xe; p += kNoAllocBlock) any |= tri[p] == -1;
+    for (uint32_t k = threadIdx.x; k < d; k += kNoAllocBlock) any |= tri[xb + k] == -1;
     if (!__syncthreads_or(any)) continue;
-    for (int32_t p = xb + threadIdx.x; p < xe; p += kNoAllocBlock) {
-      const int32_t w = ci[p];
+    for (uint32_t k = threadIdx.x; k < d; k += kNoAllocBlock) {
+      const int32_t w = ci[xb + k];
       if ((uint32_t)w < (uint32_t)n) atomicOr(&bm[w >> 5], 1u << (w & 31));
     }
     __syncthreads();
-    for (int32_t p = xb + warp; p < xe; p += warps) {
-      if (tri[p] != -1) continue;
-      const int32_t y = ci[p];
+    for (uint32_t k = warp; k < d; k += warps) {
+      if (tri[xb + k] != -1) continue;
+      const int32_t y = ci[xb + k];
       int c = 0;
       if ((uint32_t)y < (uint32_t)n)
-        for (int32_t q = rp[y] + lane; q < rp[y + 1]; q += 32) {
-          const int32_t w = ci[q];
+        for (uint32_t q = lane; q < (uint32_t)(rp[y + 1] - rp[y]); q += 32) {
+          const int32_t w = ci[rp[y] + q];
           if ((uint32_t)w < (uint32_t)n) c += (bm[w >> 5] >> (w & 31)) & 1u;
         }
       c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
-      if (lane == 0) tri[p] = c;
+      if (lane == 0) tri[xb + k] = c;
     }
     __syncthreads();
-    for (int32_t p = xb + threadIdx.x; p < xe; p += kNoAllocBlock) {
-      const int32_t w = ci[p];
+    for (uint32_t k = threadIdx.x; k < d; k += kNoAllocBlock) {
+      const int32_t w = ci[xb + k];
       if ((uint32_t)w < (uint32_t)n) bm[w >> 5] = 0u;
     }
     __syncthreads();

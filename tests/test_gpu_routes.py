@@ -196,3 +196,21 @@ def test_noalloc_small_call_is_one_kernel_and_can_be_captured():
         cu.cuGraphExecDestroy(ex)
         cu.cuGraphDestroy(graph)
         assert 1 <= count.value <= most
+
+
+def test_noalloc_slots_beyond_2_to_the_30():
+    # 950 complete graphs on 1100 vertices: 1.15e9 slots, so that the sum of two of
+    # them, as a binary search forms it, passes 2^31; a third of the rows does not
+    # fit the list of parts either
+    import torch
+    k, copies = 1100, 950
+    v = torch.arange(k, dtype=torch.int32, device="cuda")
+    block = v.repeat(k, 1)[~torch.eye(k, dtype=torch.bool, device="cuda")]
+    ci = (block[None, :] + (torch.arange(copies, dtype=torch.int32, device="cuda") * k)[:, None]).reshape(-1)
+    rp = (torch.arange(copies * k + 1, dtype=torch.int64, device="cuda") * (k - 1)).to(torch.int32)
+    assert ci.numel() > 1 << 30
+    out = torch.full_like(ci, -1)
+    gcb.gc_edge_triangles_noalloc(rp, ci, out)
+    assert bool((out == k - 2).all())
+    del ci, out
+    torch.cuda.empty_cache()

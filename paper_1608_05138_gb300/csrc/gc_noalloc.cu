@@ -144,7 +144,9 @@ __global__ void __launch_bounds__(kTriBlock) k_rows(int32_t n, const int32_t* __
     }
     const uint32_t parts = (uint32_t)((d + part - 1) / part);  // at most 4096, as d <= min(n, nnz)
     const uint32_t at = atomicAdd(scratch + kNumLong, parts);
-    const bool fits = at + parts <= kMaxParts;  // else (only beyond 2^28 entries) by k_tri_marked
+    // else by k_tri_marked: more parts than the list holds (only beyond 2^28
+    // entries), or a last part of the last vertex that would read as kNoPart
+    const bool fits = at + parts <= kMaxParts && !((uint32_t)x == 0xfffffu && parts == 4096u);
     if (!fits) atomicOr(scratch + kOffBad + (x >> 5), 1u << (x & 31));
     for (uint32_t k = 0; k < parts && at + k < kMaxParts; ++k)
       scratch[kOffLong + at + k] = fits ? (uint32_t)x | (k << 20) : kNoPart;

@@ -214,3 +214,15 @@ def test_noalloc_slots_beyond_2_to_the_30():
     assert bool((out == k - 2).all())
     del ci, out
     torch.cuda.empty_cache()
+
+
+def test_noalloc_last_row_of_as_many_parts_as_there_are():
+    # not symmetric: the last of 2^20 vertices has 1 048 420 entries, its last part
+    # the largest number a list entry can hold; all other rows are empty
+    import torch
+    n, d = 1 << 20, 4095 * 256 + 100
+    rp = torch.zeros(n + 1, dtype=torch.int32, device="cuda")
+    rp[n] = d
+    out = torch.full((d,), -7, dtype=torch.int32, device="cuda")
+    gcb.gc_edge_triangles_noalloc(rp, torch.arange(d, dtype=torch.int32, device="cuda"), out)
+    assert bool((out == 0).all())

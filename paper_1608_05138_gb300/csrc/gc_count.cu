@@ -709,15 +709,15 @@ __device__ __forceinline__ uint32_t read_count(const uint32_t* tab, uint32_t slo
 __device__ __forceinline__ int32_t gallop_lower_bound(const int32_t* __restrict__ a, int32_t p, int32_t e,
                                                       int32_t key) {
   if (p >= e || a[p] >= key) return p;
-  int32_t lo = p, step = 1;  // a[lo] < key throughout
-  while (lo + step < e && a[lo + step] < key) {
+  int32_t lo = p, step = 1;  // a[lo] < key throughout; lo + step or lo + hi may pass 2^31
+  while (step < e - lo && a[lo + step] < key) {
     lo += step;
     step <<= 1;
   }
-  int32_t hi = min(lo + step, e);
+  int32_t hi = step < e - lo ? lo + step : e;
   ++lo;
   while (lo < hi) {
-    const int32_t mid = (lo + hi) >> 1;
+    const int32_t mid = lo + ((hi - lo) >> 1);
     if (a[mid] < key) lo = mid + 1; else hi = mid;
   }
   return lo;
@@ -885,7 +885,7 @@ __global__ void __launch_bounds__(kHeavyBlock, 1) k_pass_c_heavy(DevGraph g, Cou
     if (threadIdx.x == 0) {
       int32_t lo = hb, hi = he;  // first slot of Gamma(h) with id >= h
       while (lo < hi) {
-        const int32_t mid = (lo + hi) >> 1;
+        const int32_t mid = lo + ((hi - lo) >> 1);  // slots beyond 2^30: their sum is no int32
         if (g.ci[mid] < h) lo = mid + 1; else hi = mid;
       }
       s_nx = lo - hb;

@@ -226,3 +226,33 @@ def test_noalloc_last_row_of_as_many_parts_as_there_are():
     out = torch.full((d,), -7, dtype=torch.int32, device="cuda")
     gcb.gc_edge_triangles_noalloc(rp, torch.arange(d, dtype=torch.int32, device="cuda"), out)
     assert bool((out == 0).all())
+
+
+def test_hub_rows_beyond_2_to_the_30_slots():
+    # a circulant graph of 67.2M vertices of degree 16, and beside it a hub joined to
+    # 620 vertices that share 20 000 others: the highest degrees, so that all their
+    # slots are beyond 2^30. The connected graphlets of both add up.
+    n0, half = 67_200_000, 8
+    off = np.r_[-half:0, 1:half + 1].astype(np.int32)
+    rng = np.random.default_rng(1)
+    hub, xs, os_ = 0, np.arange(1, 621), np.arange(621, 20621)
+    e = [(hub, int(x)) for x in xs] + [(int(rng.integers(1, 621)), int(o)) for o in os_ for _ in range(20)]
+    small_rp, small_ci = graphs.csr_large(20621, e)
+    assert 16 * n0 > 1 << 30
+    ci = np.empty(16 * n0 + len(small_ci), np.int32)
+    body = ci[:16 * n0].reshape(n0, 16)
+    np.add(np.arange(n0, dtype=np.int32)[:, None], off, out=body)
+    for x in list(range(half)) + list(range(n0 - half, n0)):
+        body[x] = np.sort((x + off.astype(np.int64)) % n0)
+    ci[16 * n0:] = small_ci + n0
+    rp = np.concatenate([np.arange(n0, dtype=np.int64) * 16, 16 * n0 + small_rp.astype(np.int64)]).astype(np.int32)
+    with gcb.Graph(rp, ci) as g:
+        X = g.count()
+        w = g.work_counts()
+    del ci, body
+    gcb.gc_release_cached_memory()
+    a = oracle.count(*graphs.csr(1000, [(x, (x + d) % 1000) for x in range(1000) for d in range(1, half + 1)]))["X"]
+    b = oracle.count(small_rp, small_ci)["X"]
+    for i in (2, 3, 6, 7, 8, 9, 10, 11):  # X_3, X_4 and X_7 .. X_12
+        assert X[i] == a[i] * (n0 // 1000) + b[i], i + 1
+    assert w["c_hub_jobs"] > 0

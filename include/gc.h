@@ -224,7 +224,8 @@ gc_status gc_graph_free(gc_graph g);
 
 /* Return every unused block of the library's memory pool on the current
  * device to the device (like a caching allocator's empty-cache call), with the
- * side streams and events kept for later graphs (at most 16 sets). Waits
+ * side streams and events kept for later counts and graphs (at most 16 sets of
+ * each). Waits
  * for all work on the device first (cudaDeviceSynchronize). Live graphs and
  * batches keep their memory. Errors: GC_ERR_CUDA (no device). */
 gc_status gc_release_cached_memory(void);

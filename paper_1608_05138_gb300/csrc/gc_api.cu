@@ -74,12 +74,7 @@ void fork_destroy(ForkSet* f) {
     if (t) cudaStreamDestroy(t);
   for (cudaEvent_t e : f->done)
     if (e) cudaEventDestroy(e);
-  for (cudaEvent_t e : f->begin)
-    if (e) cudaEventDestroy(e);
-  for (cudaEvent_t e : f->end)
-    if (e) cudaEventDestroy(e);
   if (f->start) cudaEventDestroy(f->start);
-  if (f->pinned) cudaFreeHost(f->pinned);
   delete f;
 }
 }  // namespace
@@ -106,12 +101,7 @@ ForkSet* fork_acquire() {
     return nullptr;
   }
   f->device = dev;
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f->start, cudaEventDisableTiming);
-  for (int k = 0; k < kNumPhases; ++k) {
-    if (e == cudaSuccess) e = cudaEventCreate(&f->begin[k]);
-    if (e == cudaSuccess) e = cudaEventCreate(&f->end[k]);
-  }
-  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&f->pinned), kPinnedBytes);
+  e = cudaEventCreateWithFlags(&f->start, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     cuda_fail(e, "side streams");
     fork_destroy(f);
@@ -142,19 +132,60 @@ void fork_release(ForkSet* f) {
   fork_destroy(f);
 }
 
-// The idle sets of the current device, given back.
-void fork_trim() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return;
-  std::lock_guard<std::mutex> lk(g_fork_mu);
-  for (size_t i = g_forks.size(); i-- > 0;)
-    if (g_forks[i]->device == dev) {
-      fork_destroy(g_forks[i]);
-      g_forks.erase(g_forks.begin() + (long)i);
-    }
+namespace {
+
+// Timers of freed handles, kept for later ones (of any device: they are idle).
+struct KeptTimers {
+  CountTimers t;
+  int device;
+};
+std::vector<KeptTimers> g_timers;  // under g_fork_mu
+constexpr size_t kTimersKept = 16;
+
+void timers_destroy(CountTimers* t) {
+  for (cudaEvent_t e : t->begin)
+    if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : t->end)
+    if (e) cudaEventDestroy(e);
+  if (t->pinned) cudaFreeHost(t->pinned);
+  *t = CountTimers();
 }
 
-namespace {
+cudaError_t timers_init(CountTimers* t, int dev) {
+  {
+    std::lock_guard<std::mutex> lk(g_fork_mu);
+    for (size_t i = 0; i < g_timers.size(); ++i)
+      if (g_timers[i].device == dev) {
+        *t = g_timers[i].t;
+        g_timers.erase(g_timers.begin() + (long)i);
+        return cudaSuccess;
+      }
+  }
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < kNumPhases; ++k) {
+    if (e == cudaSuccess) e = cudaEventCreate(&t->begin[k]);
+    if (e == cudaSuccess) e = cudaEventCreate(&t->end[k]);
+  }
+  if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&t->pinned), kPinnedBytes);
+  if (e != cudaSuccess) timers_destroy(t);
+  return e;
+}
+
+void timers_release(CountTimers* t, int dev) {
+  if (!t->pinned) return;  // never made
+  {
+    std::lock_guard<std::mutex> lk(g_fork_mu);
+    try {
+      if (g_timers.size() < kTimersKept) {
+        g_timers.push_back({*t, dev});
+        *t = CountTimers();
+        return;
+      }
+    } catch (...) {  // no memory to keep them
+    }
+  }
+  timers_destroy(t);
+}
 
 // Threads for a loop over `work` entries: one per 2^16, at most host_threads().
 int threads_for(int64_t work) { return (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), work >> 16)); }
@@ -514,7 +545,8 @@ struct gc_graph_s {
   Scratch sc;
   uint64_t* d_pe_tmp = nullptr;          // device staging for a host per-edge buffer
   uint64_t* d_ind_tmp = nullptr;         // device staging for a host per-edge induced buffer
-  ForkSet* fs = nullptr;                 // side streams, events and the pinned results
+  int device = 0;
+  CountTimers timers;                    // events of the last count, and the pinned results
   bool counted = false;
   uint64_t csum_lo[13] = {0}, csum_hi[13] = {0};
   uint64_t work[kNumWork] = {0};
@@ -548,7 +580,7 @@ static void graph_release(gc_graph g) {
   free_prep(&g->prep, s);
   scratch_free(&g->sc, s);
   cudaStreamSynchronize(s);
-  fork_release(g->fs);
+  timers_release(&g->timers, g->device);
   delete g;
 }
 
@@ -578,6 +610,7 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
   g->n = n;
   g->m = (int32_t)(nnz / 2);
   g->stream = (cudaStream_t)stream;
+  if (cudaGetDevice(&g->device) != cudaSuccess) cudaGetLastError();  // the first device step reports it
   cudaStream_t s = g->stream;
   cudaError_t e;
   gc_status st = GC_OK;
@@ -701,7 +734,7 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
     if (st2 != GC_OK) return fail(st2);
     scratch_guess_tlist(&g->sc, g->m);
   }
-  if (!(g->fs = fork_acquire())) return fail(GC_ERR_CUDA);
+  GC_CHECK(timers_init(&g->timers, g->device), "events");
   GC_CHECK(cudaStreamSynchronize(s), "sync upload");
 #undef GC_CHECK
   *out = g;
@@ -817,13 +850,21 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
   ku.n_cunits = g->prep.n_cunits;
   ku.rows = g->prep.route != kRoutePasses;
   for (int t = 0; t <= kNumTiers; ++t) ku.tier_off[t] = g->prep.ktier_off[t];
-  if ((st = run_count(dg, g->prep.units, g->prep.n_units, ku, pe_dev, &g->sc, s, g->fs, pe_host, ind_dev, ind_host)) != GC_OK) {
-    fork_drain(g->fs);
+  struct Lent {  // the side streams of this count, idle again when it ends
+    ForkSet* f;
+    bool joined = false;
+    ~Lent() {
+      if (!joined) fork_drain(f);
+      fork_release(f);
+    }
+  } lent = {fork_acquire()};
+  if (!lent.f) return GC_ERR_CUDA;
+  if ((st = run_count(dg, g->prep.units, g->prep.n_units, ku, pe_dev, &g->sc, s, lent.f, &g->timers, pe_host, ind_dev,
+                      ind_host)) != GC_OK)
     return st;
-  }
   // the results' head of the scratch in one copy: status, work, sums, X
   if (g->sc.head_bytes > kPinnedBytes) { set_error("internal: results do not fit"); return GC_ERR_CUDA; }
-  GC_CHECK(cudaMemcpyAsync(g->fs->pinned, g->sc.zero, g->sc.head_bytes, cudaMemcpyDeviceToHost, s), "copy results");
+  GC_CHECK(cudaMemcpyAsync(g->timers.pinned, g->sc.zero, g->sc.head_bytes, cudaMemcpyDeviceToHost, s), "copy results");
   if (staged)
     GC_CHECK(cudaMemcpyAsync(per_edge_out, pe_dev, sizeof(uint64_t) * 13 * (size_t)g->m, cudaMemcpyDeviceToHost, s),
              "copy per-edge");
@@ -831,9 +872,10 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
     GC_CHECK(cudaMemcpyAsync(induced_out, ind_dev, sizeof(uint64_t) * GC_INDUCED_COLS * (size_t)g->m,
                              cudaMemcpyDeviceToHost, s),
              "copy induced");
-  GC_CHECK(cudaEventRecord(g->fs->end[kPhaseCopy], s), "event");
+  GC_CHECK(cudaEventRecord(g->timers.end[kPhaseCopy], s), "event");
   GC_CHECK(cudaStreamSynchronize(s), "sync count");
-  auto host_of = [&](const void* d) { return g->fs->pinned + (static_cast<const unsigned char*>(d) - g->sc.zero); };
+  lent.joined = true;
+  auto host_of = [&](const void* d) { return g->timers.pinned + (static_cast<const unsigned char*>(d) - g->sc.zero); };
   const int32_t hstatus = reinterpret_cast<const int32_t*>(host_of(g->sc.misc))[1];
   std::memcpy(g->work, host_of(g->sc.work), sizeof(g->work));
   const uint64_t* hx = reinterpret_cast<const uint64_t*>(host_of(g->sc.x));
@@ -909,7 +951,7 @@ gc_status gc_graph_phase_ms(gc_graph g, double* ms) {
   if (!g->counted) { set_error("graph not counted yet"); return GC_ERR_ARG; }
   for (int i = 0; i < kNumPhases; ++i) {
     float f = 0.f;
-    cudaError_t e = cudaEventElapsedTime(&f, g->fs->begin[i], g->fs->end[i]);
+    cudaError_t e = cudaEventElapsedTime(&f, g->timers.begin[i], g->timers.end[i]);
     if (e != cudaSuccess) return cuda_fail(e, "event elapsed");
     ms[i] = f;
   }
@@ -919,6 +961,23 @@ gc_status gc_graph_phase_ms(gc_graph g, double* ms) {
 gc_status gc_graph_free(gc_graph g) {
   graph_release(g);
   return GC_OK;
+}
+
+// The idle side streams and timers of the current device, given back.
+static void fork_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  std::lock_guard<std::mutex> lk(g_fork_mu);
+  for (size_t i = g_forks.size(); i-- > 0;)
+    if (g_forks[i]->device == dev) {
+      fork_destroy(g_forks[i]);
+      g_forks.erase(g_forks.begin() + (long)i);
+    }
+  for (size_t i = g_timers.size(); i-- > 0;)
+    if (g_timers[i].device == dev) {
+      timers_destroy(&g_timers[i].t);
+      g_timers.erase(g_timers.begin() + (long)i);
+    }
 }
 
 gc_status gc_release_cached_memory(void) {

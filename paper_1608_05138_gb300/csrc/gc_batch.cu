@@ -547,7 +547,7 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
     ku.n_cunits = prep.n_cunits;
     ku.rows = prep.route != kRoutePasses;
     for (int t = 0; t <= kNumTiers; ++t) ku.tier_off[t] = prep.ktier_off[t];
-    if ((st = run_count(dg, prep.units, prep.n_units, ku, nullptr, &sc, s, fs)) != GC_OK) {
+    if ((st = run_count(dg, prep.units, prep.n_units, ku, nullptr, &sc, s, fs, nullptr)) != GC_OK) {
       fork_drain(fs);
       L->error = gc_last_error();
       goto out;

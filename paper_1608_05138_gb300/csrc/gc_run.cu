@@ -135,8 +135,8 @@ void scratch_guess_tlist(Scratch* sc, int64_t m) {
 static int32_t ku_total(const KUnits& ku) { return ku.tier_off[kNumTiers]; }
 
 gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, const KUnits& ku,
-                    uint64_t* per_edge, Scratch* sc, cudaStream_t s, ForkSet* fs, bool per_edge_host, uint64_t* induced,
-                    bool induced_host) {
+                    uint64_t* per_edge, Scratch* sc, cudaStream_t s, ForkSet* fs, CountTimers* tm, bool per_edge_host,
+                    uint64_t* induced, bool induced_host) {
   cudaError_t e = cudaSuccess;
   gc_status st = GC_OK;
 #define GR_TRY(call, what)                  \
@@ -145,9 +145,9 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
     if (e != cudaSuccess) return cuda_fail(e, what); \
   } while (0)
 #define GR_BEGIN(i, t) \
-  if (fs) GR_TRY(cudaEventRecord(fs->begin[i], t), "event")
+  if (tm) GR_TRY(cudaEventRecord(tm->begin[i], t), "event")
 #define GR_END(i, t) \
-  if (fs) GR_TRY(cudaEventRecord(fs->end[i], t), "event")
+  if (tm) GR_TRY(cudaEventRecord(tm->end[i], t), "event")
   CountArgs a;
   a.units = units;
   a.n_units = n_units;

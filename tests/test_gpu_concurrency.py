@@ -273,3 +273,27 @@ print('ok')
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
+
+
+def test_live_handles_keep_no_side_streams():
+    # 200 live handles, each counted: a side stream takes 0.6 MB of device memory
+    import torch
+    g = graphgen.er(5000, 0.004, 1)
+    expect = batch_count(g)
+    handles = [gcb.Graph(*g) for _ in range(200)]
+    try:
+        assert handles[0].count() == expect
+        gcb.gc_release_cached_memory()
+        torch.cuda.synchronize()
+        used = []
+        for part in (handles[:20], handles[20:]):
+            free = torch.cuda.mem_get_info()[0]
+            assert all(h.count() == expect for h in part)
+            used.append((free - torch.cuda.mem_get_info()[0]) / len(part))
+        # what a count's own scratch takes (lists of triangles: 32 entries an edge, in
+        # blocks of the pool) is the same for all; ten streams would be 5.7 MB more
+        m = len(g[1]) // 2
+        assert used[1] < 32 * m * 8 * 1.5 + (1 << 20), used
+    finally:
+        for h in handles:
+            h.close()

@@ -77,8 +77,11 @@ const char* gc_last_error(void);
  *   row_ptr  host pointer, n + 1 int32
  *   col_idx  host pointer, row_ptr[n] int32
  *   flags    0 or GC_NO_VALIDATE
- *   stream   cudaStream_t (as void*) on which all work of this graph runs;
- *            NULL = the legacy default stream
+ *   stream   cudaStream_t (as void*) of this graph, NULL = the legacy default
+ *            stream: all its work runs after what is queued there and is
+ *            waited for there. A count also uses side streams of the library, of
+ *            the same priority, forked from `stream` and joined into it (none for
+ *            a stream of a green context, whose work stays on its part of the GPU).
  *   out      receives the new handle
  * Errors: GC_ERR_ARG, GC_ERR_RANGE, GC_ERR_UNSORTED, GC_ERR_DUPLICATE,
  * GC_ERR_SELF_LOOP, GC_ERR_ASYMMETRIC, GC_ERR_OVERFLOW (2m >= 2^31),

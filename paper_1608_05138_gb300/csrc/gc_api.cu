@@ -79,7 +79,7 @@ void fork_destroy(ForkSet* f) {
 }
 }  // namespace
 
-ForkSet* fork_acquire() {
+ForkSet* fork_acquire(int priority) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) {
@@ -89,7 +89,7 @@ ForkSet* fork_acquire() {
   {
     std::lock_guard<std::mutex> lk(g_fork_mu);
     for (size_t i = 0; i < g_forks.size(); ++i)
-      if (g_forks[i]->device == dev) {
+      if (g_forks[i]->device == dev && g_forks[i]->priority == priority) {
         ForkSet* f = g_forks[i];
         g_forks.erase(g_forks.begin() + (long)i);
         return f;
@@ -101,6 +101,7 @@ ForkSet* fork_acquire() {
     return nullptr;
   }
   f->device = dev;
+  f->priority = priority;
   e = cudaEventCreateWithFlags(&f->start, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     cuda_fail(e, "side streams");
@@ -108,6 +109,22 @@ ForkSet* fork_acquire() {
     return nullptr;
   }
   return f;
+}
+
+bool on_part_of_gpu(cudaStream_t s) {
+  typedef int (*Query)(cudaStream_t, void**);  // cuStreamGetGreenCtx
+  static const Query query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &f, 12040, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;  // a driver without them
+    }
+    return reinterpret_cast<Query>(f);
+  }();
+  void* ctx = nullptr;
+  return query && query(s, &ctx) == 0 && ctx != nullptr;
 }
 
 void fork_drain(ForkSet* f) {
@@ -857,8 +874,12 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
       if (!joined) fork_drain(f);
       fork_release(f);
     }
-  } lent = {fork_acquire()};
-  if (!lent.f) return GC_ERR_CUDA;
+  } lent = {nullptr};
+  if (!on_part_of_gpu(s)) {
+    int priority = 0;
+    if (cudaStreamGetPriority(s, &priority) != cudaSuccess) cudaGetLastError();
+    if (!(lent.f = fork_acquire(priority))) return GC_ERR_CUDA;
+  }
   if ((st = run_count(dg, g->prep.units, g->prep.n_units, ku, pe_dev, &g->sc, s, lent.f, &g->timers, pe_host, ind_dev,
                       ind_host)) != GC_OK)
     return st;

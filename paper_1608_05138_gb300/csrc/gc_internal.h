@@ -174,6 +174,7 @@ struct ForkSet {
   cudaStream_t stream[kForkStreams] = {};
   cudaEvent_t start = nullptr, done[kForkStreams] = {};
   int device = 0;
+  int priority = 0;  // of its streams
 };
 // What a graph handle keeps: events that time the phases of its last count, and
 // pinned memory that receives the results.
@@ -182,7 +183,10 @@ struct CountTimers {
   cudaEvent_t begin[kNumPhases] = {}, end[kNumPhases] = {};
   unsigned char* pinned = nullptr;
 };
-ForkSet* fork_acquire();         // of the current device; nullptr on failure (message set)
+ForkSet* fork_acquire(int priority);  // of the current device; nullptr on failure (message set)
+// Whether the stream belongs to a part of the GPU only (a green context): its
+// count then stays on it, since side streams would be on the whole GPU.
+bool on_part_of_gpu(cudaStream_t s);
 void fork_release(ForkSet* f);   // its streams must be idle; nullptr is accepted
 void fork_drain(ForkSet* f);     // waits for its streams (after a failed count, whose forks were not joined)
 
@@ -198,7 +202,7 @@ class Fork {
     if (!f_ || used_ >= count_ || e_ != cudaSuccess) return s_;
     cudaStream_t& t = f_->stream[first_ + used_];
     cudaEvent_t& d = f_->done[first_ + used_];
-    if (!t) e_ = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);  // on first use, and kept
+    if (!t) e_ = cudaStreamCreateWithPriority(&t, cudaStreamNonBlocking, f_->priority);  // on first use, and kept
     if (!d && e_ == cudaSuccess) e_ = cudaEventCreateWithFlags(&d, cudaEventDisableTiming);
     if (e_ == cudaSuccess) e_ = cudaStreamWaitEvent(t, f_->start, 0);
     if (e_ != cudaSuccess) return s_;  // join() reports it

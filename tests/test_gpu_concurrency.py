@@ -297,3 +297,72 @@ def test_live_handles_keep_no_side_streams():
     finally:
         for h in handles:
             h.close()
+
+
+def test_a_count_keeps_its_streams_priority():
+    # beside a kernel of many short CTAs on a stream of lower priority, a count's
+    # kernels get the slots that come free; at equal priority they would wait until
+    # all of its CTAs are placed
+    import torch
+    g = graphgen.chung_lu(60000, 500000, 2.2, 1e6, 3000.0, 3)
+    z = torch.full((1 << 29,), 3.3, dtype=torch.float64, device="cuda")
+    with gcb.Graph(*g, stream=torch.cuda.Stream(priority=-1)) as h:
+        expect = h.count()
+        torch.lgamma(z, out=z)  # compiled and warm
+        z.fill_(3.3)
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        torch.lgamma(z, out=z)
+        torch.cuda.synchronize()
+        alone = time.perf_counter() - t
+        z.fill_(3.3)
+        torch.cuda.synchronize()
+        torch.lgamma(z, out=z)
+        done = torch.cuda.Event()
+        done.record()
+        t = time.perf_counter()
+        assert h.count() == expect
+        took = time.perf_counter() - t
+        assert not done.query()
+    assert took < alone / 3
+
+
+def test_a_count_stays_on_its_streams_part_of_the_gpu():
+    # a green context of 16 SMs: a count on its stream takes several times as long
+    # as on the whole GPU, and the same counts come out
+    import ctypes as C
+    import torch
+    cu = C.CDLL("libcuda.so.1")
+    if not hasattr(cu, "cuGreenCtxStreamCreate"):
+        pytest.skip("no green contexts in this driver")
+
+    class Resource(C.Structure):  # CUdevResource: type, padding, union
+        _fields_ = [("type", C.c_int), ("pad", C.c_ubyte * 92), ("sm", C.c_uint), ("rest", C.c_ubyte * 44)]
+
+    torch.zeros(1, device="cuda")
+    whole, part, rest = Resource(), Resource(), Resource()
+    count, desc, ctx, stream = C.c_uint(1), C.c_void_p(), C.c_void_p(), C.c_void_p()
+    assert cu.cuDeviceGetDevResource(0, C.byref(whole), 1) == 0
+    assert cu.cuDevSmResourceSplitByCount(C.byref(part), C.byref(count), C.byref(whole), C.byref(rest), 0, 16) == 0
+    assert part.sm == 16
+    assert cu.cuDevResourceGenerateDesc(C.byref(desc), C.byref(part), 1) == 0
+    assert cu.cuGreenCtxCreate(C.byref(ctx), desc, 0, 1) == 0
+    assert cu.cuGreenCtxStreamCreate(C.byref(stream), ctx, 1, 0) == 0
+    took = {}
+    g = graphgen.chung_lu(100000, 1500000, 2.2, 3e6, 5000.0, 3)
+    counts = {}
+    try:
+        for name, s in (("whole", torch.cuda.Stream().cuda_stream), ("part", stream.value)):
+            with gcb.Graph(*g, stream=s) as h:
+                times = []
+                for _ in range(4):
+                    t = time.perf_counter()
+                    counts[name] = h.count()
+                    times.append(time.perf_counter() - t)
+                took[name] = min(times)
+    finally:
+        torch.cuda.synchronize()
+        cu.cuStreamDestroy_v2(stream)
+        cu.cuGreenCtxDestroy(ctx)
+    assert counts["part"] == counts["whole"]
+    assert took["part"] > 3 * took["whole"], took

@@ -138,7 +138,8 @@ gc_status gc_graph_edges(gc_graph g, int32_t* uv);
  *   global_hi     host pointer, 17 uint64 for the high 64 bits, or NULL. If
  *                 NULL and some X_i >= 2^64 the call writes the low words and
  *                 returns GC_ERR_OVERFLOW.
- * Runs on the graph's stream and returns when the results are written.
+ * Runs on the graph's stream, with the device current on which it was uploaded
+ * (else GC_ERR_CUDA), and returns when the results are written.
  * Errors: GC_ERR_ARG, GC_ERR_CUDA, GC_ERR_NOMEM, GC_ERR_OVERFLOW.
  */
 gc_status gc_count_edge_graphlets(gc_graph g, uint64_t* per_edge_out, uint64_t* global_out,

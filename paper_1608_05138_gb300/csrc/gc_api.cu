@@ -800,6 +800,13 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
   cudaStream_t s = g->stream;
   cudaError_t e;
   gc_status st;
+  // the side streams are the current device's, and so would their kernels be
+  int dev = -1;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+  if (dev != g->device) {
+    set_error("the graph is on device " + std::to_string(g->device) + ", the current device is " + std::to_string(dev));
+    return GC_ERR_CUDA;
+  }
 #define GC_CHECK(call, what)                  \
   do {                                        \
     e = (call);                               \

@@ -366,3 +366,19 @@ def test_a_count_stays_on_its_streams_part_of_the_gpu():
         cu.cuGreenCtxDestroy(ctx)
     assert counts["part"] == counts["whole"]
     assert took["part"] > 3 * took["whole"], took
+
+
+def test_a_count_with_another_device_current_is_refused():
+    import torch
+    if torch.cuda.device_count() < 2:
+        pytest.skip("needs two devices")
+    g = gcb.Graph(*graphgen.er(300, 0.1, 1))
+    try:
+        x = g.count()
+        with torch.cuda.device(1):
+            with pytest.raises(gcb.GcError) as ei:
+                g.count()
+        assert ei.value.status == -8
+        assert g.count() == x
+    finally:
+        g.close()

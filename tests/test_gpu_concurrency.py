@@ -98,11 +98,11 @@ def test_refused_submissions_take_no_device_memory():
     # a submission that does not fit in the budget now is refused before it is
     # copied and checked on the device; an invalid one gets its own code
     import torch
-    rp, ci = graphgen.er(200000, 4e-4, 5)  # 8M entries: 64 MB of CSR
+    rp, ci = graphgen.er(100000, 4e-4, 5)  # 4M entries: 16 MB of CSR
     bad = ci.copy()
     x = int(np.flatnonzero(np.diff(rp) >= 3)[0])
     bad[rp[x]] = bad[rp[x] + 1]
-    need = 44 * 200000 + 32 * (len(ci) // 2) + 1024 + 2 * 152 * 200000 * 4
+    need = 44 * 100000 + 32 * (len(ci) // 2) + 1024 + 2 * 152 * 100000 * 4
     gcb.gc_release_cached_memory()
     b = gcb.gc_batch_create(need + 10000, gcb.GC_BATCH_MANUAL)
     try:
@@ -114,7 +114,7 @@ def test_refused_submissions_take_no_device_memory():
         with pytest.raises(gcb.GcError) as ei:
             gcb.gc_batch_submit(b, rp, bad)
         assert ei.value.status == -3
-        assert free - torch.cuda.mem_get_info()[0] < 16 << 20
+        assert free - torch.cuda.mem_get_info()[0] < 8 << 20
         gcb.gc_batch_flush(b)
         assert gcb.gc_batch_poll(b, t) is not None
         for _ in range(3):  # a refusal gives its share back
@@ -276,24 +276,17 @@ print('ok')
 
 
 def test_live_handles_keep_no_side_streams():
-    # 200 live handles, each counted: a side stream takes 0.6 MB of device memory
+    # 200 live handles, each counted: a side stream takes 0.57 MB of device memory,
+    # and a count of this graph uses two or three
     import torch
-    g = graphgen.er(5000, 0.004, 1)
+    g = graphgen.er(1000, 0.02, 1)
     expect = batch_count(g)
     handles = [gcb.Graph(*g) for _ in range(200)]
     try:
-        assert handles[0].count() == expect
-        gcb.gc_release_cached_memory()
         torch.cuda.synchronize()
-        used = []
-        for part in (handles[:20], handles[20:]):
-            free = torch.cuda.mem_get_info()[0]
-            assert all(h.count() == expect for h in part)
-            used.append((free - torch.cuda.mem_get_info()[0]) / len(part))
-        # what a count's own scratch takes (lists of triangles: 32 entries an edge, in
-        # blocks of the pool) is the same for all; ten streams would be 5.7 MB more
-        m = len(g[1]) // 2
-        assert used[1] < 32 * m * 8 * 1.5 + (1 << 20), used
+        free = torch.cuda.mem_get_info()[0]
+        assert all(h.count() == expect for h in handles)
+        assert free - torch.cuda.mem_get_info()[0] < 64 << 20
     finally:
         for h in handles:
             h.close()

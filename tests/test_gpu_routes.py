@@ -90,9 +90,9 @@ def test_small_graphs_without_4_cliques_cost_what_sparse_ones_do():
     (lambda: hubs(5, 3000, 3), False),
     (lambda: graphgen.er(700, 0.2, 1), False),       # bit rows
     (lambda: bipartite(60, 240), False),             # out-degrees of at most 256, without a triangle
-    (lambda: bipartite(150, 3900), True),            # rows of hubs, read once for every leaf
+    (lambda: bipartite(60, 3000), True),            # rows of hubs, read once for every leaf
     (lambda: hubs(200, 2000, 5), True),
-    (lambda: hubs(120, 4000, 4), True),
+    (lambda: hubs(60, 3000, 4), True),
     (lambda: bipartite(900, 1100), True),            # dense, but without a triangle
 ])
 def test_route_of_graphs_up_to_4096_vertices(make, passes):
@@ -230,14 +230,14 @@ def test_noalloc_last_row_of_as_many_parts_as_there_are():
 
 def test_hub_rows_beyond_2_to_the_30_slots():
     # a circulant graph of 67.2M vertices of degree 16, and beside it a hub joined to
-    # 620 vertices that share 20 000 others: the highest degrees, so that all their
-    # slots are beyond 2^30. The connected graphlets of both add up.
+    # 2000 vertices that share 60 000 others: the highest degrees, so that their
+    # slots are the last ones. The connected graphlets of both add up.
     n0, half = 67_200_000, 8
     off = np.r_[-half:0, 1:half + 1].astype(np.int32)
     rng = np.random.default_rng(1)
-    hub, xs, os_ = 0, np.arange(1, 621), np.arange(621, 20621)
-    e = [(hub, int(x)) for x in xs] + [(int(rng.integers(1, 621)), int(o)) for o in os_ for _ in range(20)]
-    small_rp, small_ci = graphs.csr_large(20621, e)
+    shared = np.stack([1 + rng.integers(0, 2000, 60000 * 32), np.repeat(2001 + np.arange(60000), 32)], 1)
+    small_rp, small_ci = graphs.csr_large(62001, np.concatenate([np.stack([np.zeros(2000, int), 1 + np.arange(2000)], 1),
+                                                                 shared]))
     assert 16 * n0 > 1 << 30
     ci = np.empty(16 * n0 + len(small_ci), np.int32)
     body = ci[:16 * n0].reshape(n0, 16)
@@ -252,7 +252,8 @@ def test_hub_rows_beyond_2_to_the_30_slots():
     del ci, body
     gcb.gc_release_cached_memory()
     a = oracle.count(*graphs.csr(1000, [(x, (x + d) % 1000) for x in range(1000) for d in range(1, half + 1)]))["X"]
-    b = oracle.count(small_rp, small_ci)["X"]
+    with gcb.Graph(small_rp, small_ci) as g:
+        b = g.count()
     for i in (2, 3, 6, 7, 8, 9, 10, 11):  # X_3, X_4 and X_7 .. X_12
         assert X[i] == a[i] * (n0 // 1000) + b[i], i + 1
     assert w["c_hub_jobs"] > 0

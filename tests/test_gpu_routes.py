@@ -93,7 +93,7 @@ def test_small_graphs_without_4_cliques_cost_what_sparse_ones_do():
     (lambda: bipartite(60, 3000), True),            # rows of hubs, read once for every leaf
     (lambda: hubs(200, 2000, 5), True),
     (lambda: hubs(60, 3000, 4), True),
-    (lambda: bipartite(900, 1100), True),            # dense, but without a triangle
+    (lambda: bipartite(550, 700), True),             # dense, but without a triangle
 ])
 def test_route_of_graphs_up_to_4096_vertices(make, passes):
     rp, ci = make()
@@ -257,3 +257,168 @@ def test_hub_rows_beyond_2_to_the_30_slots():
     for i in (2, 3, 6, 7, 8, 9, 10, 11):  # X_3, X_4 and X_7 .. X_12
         assert X[i] == a[i] * (n0 // 1000) + b[i], i + 1
     assert w["c_hub_jobs"] > 0
+
+
+# ---- the paths that small graphs no longer take by themselves ----
+
+def padded(g, n):
+    """The graph with isolated vertices added up to n: beyond 4096, passes T, C and K count it."""
+    rp, ci = g
+    return np.concatenate([rp, np.full(n + 1 - len(rp), rp[-1], np.int32)]), ci
+
+
+def by_passes(g, scans, times=2):
+    """Counts the graph, padded beyond 4096 vertices, against the oracle; scans: whether pass K scans in the last
+    count, or replays the lists that pass T kept."""
+    rp, ci = padded(g, max(len(g[0]) - 1, 4200))
+    o = oracle.count(rp, ci)
+    with gcb.Graph(rp, ci) as h:
+        for _ in range(times):
+            pe = np.zeros((h.m, 13), np.uint64)
+            assert h.count(pe) == o["X"]
+            np.testing.assert_array_equal(pe, o["per_edge"])
+        w = h.work_counts()
+    assert w["t_members"] > 0 and w["t_triangles"] == w["k_local_edges"] == o["X"][2]
+    assert (w["k_scan"] > 0) == scans
+
+
+@pytest.mark.parametrize("make", [
+    lambda: graphgen.chung_lu(3000, 15000, 2.1, 30000.0, 800.0, 5),
+    lambda: graphgen.rmat(12, 16, 0.57, 0.19, 0.19, 6),
+    graphgen.config_er_dense,
+    lambda: graphs.complete(300),
+])
+def test_replayed_triangle_lists_of_every_tier(make):
+    by_passes(make(), scans=False, times=3)
+
+
+def test_replayed_triangle_lists_of_the_global_tier():
+    # out-degrees a little above 1024, lists of fewer than 2^19 edges; x3, x7 and x10
+    # do not change with isolated vertices, and without them the graph takes the rows
+    g = graphgen.er(1170, 0.915, 41)
+    cols = []
+    for h in (padded(g, 4200), g):
+        with gcb.Graph(*h) as G:
+            for _ in range(2):
+                pe = np.zeros((G.m, 13), np.uint64)
+                G.count(pe)
+                cols.append(pe[:, [0, 3, 4]])
+            w = G.work_counts()
+        assert (w["t_members"] > 0) == (len(h[0]) > 4096)
+        if w["t_members"]:
+            assert w["k_scan"] == 0
+    for c in cols[1:]:
+        np.testing.assert_array_equal(c, cols[0])
+    uv = oracle.edges(*g)
+    pick = np.random.default_rng(1).choice(len(uv), 100, replace=False)
+    np.testing.assert_array_equal(cols[0][pick], oracle.count_sample(*g, pick)[:, [0, 3, 4]])
+
+
+def run_with_env(call, **env):
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", f"import tests.test_gpu_routes as t; t.{call}; print('ok')"], cwd=root,
+                       env=dict(os.environ, PYTHONPATH=root, **env), capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("env", [{"GC_K_LIST_CAP": "64"}, {"GC_T_LIST_CAP": "5000"}])
+def test_pass_k_scans_again_where_lists_are_short(env):
+    run_with_env("by_passes(t.graphgen.rmat(12, 16, 0.57, 0.19, 0.19, 29), scans=True)", **env)
+    run_with_env("by_passes(t.graphgen.config_er_dense(), scans=True)", **env)
+
+
+@pytest.mark.parametrize("n", [1025, 1026])  # out-degrees up to 1024: bit rows; 1025: not
+def test_complete_graphs_at_the_limit_of_the_bit_rows(n):
+    m = n * (n - 1) // 2
+    with gcb.Graph(*graphgen.er(n, 1.0, 1)) as g:
+        pe = np.zeros((g.m, 13), np.uint64)
+        assert g.count(pe) == [m, 0, comb(n, 3), 0, 0, 0, comb(n, 4)] + [0] * 10
+    row = [n - 2, 0, 0, comb(n - 2, 2), 0, comb(n - 2, 2), 0, 0, 0, 0, m - 2 * (n - 1) + 1, 0, 0]
+    assert (pe == np.array(row, np.uint64)).all()
+
+
+@pytest.mark.parametrize("n", [2047, 2048])
+def test_bit_rows_of_the_largest_graphs(n):
+    # all 64 words; 60 vertices joined to all, any two of which share more than 1024
+    # neighbours (the highest plane of the counts), among others of about 950
+    from tests.test_gpu_parity import _sampled_check
+    rp, ci = graphgen.er(n, 0.44, 3)
+    rows = np.repeat(np.arange(n), np.diff(rp))
+    up = rows < ci
+    u, v = np.meshgrid(np.arange(60), np.arange(n), indexing="ij")
+    e = np.concatenate([np.stack([rows[up], ci[up]], 1), np.stack([u.ravel(), v.ravel()], 1)[(u != v).ravel()]])
+    rp, ci = graphs.csr_large(n, e)
+    with gcb.Graph(rp, ci) as g:
+        g.count()
+        w = g.work_counts()
+    assert w["t_members"] == 0 and w["launches"] == 4  # rows, cliques, finish, derive
+    _sampled_check(rp, ci, k=100, seed=n)
+
+
+# ---- the hub kernel's counters at the limits of their fields ----
+
+def hub_segments(degrees, tab):
+    """Counters per word of the segments that the ids of these degrees (ascending) are cut into: each takes the width
+    that reaches furthest, up to the end of its block or of the ids whose counts fit it."""
+    bound = [int(np.searchsorted(degrees, d)) for d in (2, 4, 16, 256, 65536)]
+    end, lo, word, out = len(degrees), bound[0], 0, []
+    while lo < end:
+        hi, lg = lo, 0
+        for k in range(5):
+            to = min(end if k == 0 else bound[5 - k], lo + ((tab - word) << k))
+            if to > hi:
+                hi, lg = to, k
+        out.append((lo, hi, 1 << lg))
+        word += (hi - lo + (1 << lg) - 1) >> lg
+        if tab - word < tab // 16 or hi == end:
+            word = 0
+        lo = hi
+    return out
+
+
+def check_field_limits():
+    # a hub joined to 3000 vertices x; others, o, whose neighbours are all x, so that
+    # the hub's count of o is its degree: 2, 3 / 4, 15 / 16, 255 / 256, so many of each
+    # that the ids of a class reach further than a block of wider counters. No triangle:
+    # every 4-cycle is induced, and x10 of (x, y) is the sum over the other neighbours
+    # x' of y of the common neighbours of x and x' without y.
+    import torch
+    nx, rng = 3000, np.random.default_rng(7)
+    deg = np.repeat([2, 3, 4, 15, 16, 255, 256], [20000, 20000, 8000, 2000, 10000, 300, 4300])
+    key = rng.random((2000, nx))
+    rows, at = [], 0
+    for d in deg:  # d of the nx, by a random row of keys, shifted
+        rows.append(np.argpartition(np.roll(key[at % 2000], at), d - 1)[:d] if d > 4 else rng.choice(nx, d, replace=False))
+        at += 1
+    x = np.concatenate([np.arange(nx)] + rows)
+    y = nx + np.concatenate([np.zeros(nx, int), np.repeat(1 + np.arange(len(deg)), deg)])
+    rp, ci = graphs.csr_large(nx + 1 + len(deg), np.stack([x, y], 1))
+    degrees = np.sort(np.diff(rp))
+    assert degrees[-1] == nx  # the hub is the last
+    segments = hub_segments(degrees, 4096)
+    for d, counters in ((3, 16), (15, 8), (255, 4), (256, 2)):  # the largest counts of a field, and one more bit
+        i = int(np.searchsorted(degrees, d, side="right")) - 1 if d != 256 else int(np.searchsorted(degrees, d))
+        assert [c for lo, hi, c in segments if lo <= i < hi] == [counters], (d, segments)
+    with gcb.Graph(rp, ci) as g:
+        pe = np.zeros((g.m, 13), np.uint64)
+        X = g.count(pe)
+        uv = g.edges().astype(np.int64)
+        w = g.work_counts()
+    assert w["c_heavy_wedges"] >= deg.sum()
+    a = torch.zeros((nx, 1 + len(deg)), dtype=torch.float64, device="cuda")
+    a[torch.from_numpy(x).cuda(), torch.from_numpy(y - nx).cuda()] = 1.0
+    q = a @ a.T - 1.0
+    q.fill_diagonal_(0.0)
+    pairs = (q + 1.0).cpu().numpy()
+    x10 = (q @ a).cpu().numpy()[uv[:, 0], uv[:, 1] - nx]
+    np.testing.assert_array_equal(pe[:, 4].astype(np.int64), x10.astype(np.int64))
+    assert not pe[:, 0].any()
+    i = np.triu_indices(nx, 1)
+    assert X[9] == int((pairs[i] * (pairs[i] - 1) / 2).sum())
+
+
+def test_hub_counters_at_the_limits_of_every_field():
+    run_with_env("check_field_limits()", GC_HUB_TAB_WORDS="4096")

@@ -25,6 +25,15 @@ static thread_local std::string t_err;
 
 void set_error(const std::string& msg) { t_err = msg; }
 
+gc_status no_memory() noexcept {
+  try {
+    t_err = "host allocation failed";
+  } catch (...) {
+    t_err.clear();
+  }
+  return GC_ERR_NOMEM;
+}
+
 gc_status cuda_fail(cudaError_t e, const char* what) {
   set_error(std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")");
   if (e == cudaErrorMemoryAllocation) return GC_ERR_NOMEM;
@@ -573,7 +582,7 @@ extern "C" {
 
 const char* gc_last_error(void) { return t_err.c_str(); }
 
-gc_status gc_validate_csr(int32_t n, const int32_t* row_ptr, const int32_t* col_idx) {
+gc_status gc_validate_csr(int32_t n, const int32_t* row_ptr, const int32_t* col_idx) try {
   if (n < 0 || !row_ptr || (!col_idx && n > 0 && row_ptr[n] > 0)) {
     set_error("bad arguments to gc_validate_csr");
     return GC_ERR_ARG;
@@ -584,6 +593,8 @@ gc_status gc_validate_csr(int32_t n, const int32_t* row_ptr, const int32_t* col_
     return validate_csr_small(n, row_ptr, col_idx, &fill);
   }
   return validate_csr(n, row_ptr, col_idx);
+} catch (...) {
+  return no_memory();
 }
 
 static void graph_release(gc_graph g) {
@@ -602,7 +613,7 @@ static void graph_release(gc_graph g) {
 }
 
 gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_idx, uint32_t flags,
-                          void* stream, gc_graph* out) {
+                          void* stream, gc_graph* out) try {
   if (!out) { set_error("out is NULL"); return GC_ERR_ARG; }
   *out = nullptr;
   if (n < 0 || !row_ptr || (!col_idx && n > 0 && row_ptr[n] > 0)) {
@@ -756,6 +767,8 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
 #undef GC_CHECK
   *out = g;
   return GC_OK;
+} catch (...) {
+  return no_memory();
 }
 
 gc_status gc_graph_info(gc_graph g, int64_t* n, int64_t* m) {
@@ -765,13 +778,15 @@ gc_status gc_graph_info(gc_graph g, int64_t* n, int64_t* m) {
   return GC_OK;
 }
 
-gc_status gc_graph_edges(gc_graph g, int32_t* uv) {
+gc_status gc_graph_edges(gc_graph g, int32_t* uv) try {
   if (!g || !uv) { set_error("NULL argument"); return GC_ERR_ARG; }
   if (g->m == 0) return GC_OK;
   cudaError_t e = cudaMemcpyAsync(uv, g->prep.uv, sizeof(int32_t) * 2 * (size_t)g->m,
                                   cudaMemcpyDeviceToHost, g->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "copy edges");
+} catch (...) {
+  return no_memory();
 }
 
 // The address by which the device writes the per-edge rows at p: p itself
@@ -937,14 +952,18 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
 }
 
 gc_status gc_count_edge_graphlets(gc_graph g, uint64_t* per_edge_out, uint64_t* global_out,
-                                  uint64_t* global_hi) {
+                                  uint64_t* global_hi) try {
   return count_graph(g, per_edge_out, nullptr, global_out, global_hi);
+} catch (...) {
+  return no_memory();
 }
 
 gc_status gc_count_edge_induced(gc_graph g, uint64_t* induced_out, uint64_t* per_edge_out, uint64_t* global_out,
-                                uint64_t* global_hi) {
+                                uint64_t* global_hi) try {
   if (!induced_out && g && g->m > 0) { set_error("induced_out is NULL"); return GC_ERR_ARG; }
   return count_graph(g, per_edge_out, induced_out, global_out, global_hi);
+} catch (...) {
+  return no_memory();
 }
 
 gc_status gc_graph_csums(gc_graph g, uint64_t* lo, uint64_t* hi) {
@@ -1008,7 +1027,7 @@ static void fork_trim() {
     }
 }
 
-gc_status gc_release_cached_memory(void) {
+gc_status gc_release_cached_memory(void) try {
   cudaMemPool_t pool = lib_pool();
   if (!pool) {
     set_error("gc_release_cached_memory: no CUDA device or pool");
@@ -1018,6 +1037,8 @@ gc_status gc_release_cached_memory(void) {
   if (e == cudaSuccess) e = cudaMemPoolTrimTo(pool, 0);
   fork_trim();
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "gc_release_cached_memory");
+} catch (...) {
+  return no_memory();
 }
 
 }  // extern "C"

@@ -333,6 +333,21 @@ struct gc_batch_s {
     ++live;
     return first_ticket + tickets.size() - 1;
   }
+  // A place at the end of the queue, and its ticket; or neither, and an exception.
+  uint64_t admit() {
+    pending.emplace_back();
+    try {
+      return add_ticket();
+    } catch (...) {
+      pending.pop_back();
+      throw;
+    }
+  }
+  void dismiss() {  // the last admitted
+    pending.pop_back();
+    tickets.pop_back();
+    --live;
+  }
   void retire(uint64_t t) {
     if (t < first_ticket) old.erase(t);
     else tickets[(size_t)(t - first_ticket)] = Ticket();
@@ -878,7 +893,11 @@ void retire_locked(gc_batch b) {
     }
     b->in_use -= L->bytes;
     L->owners.clear();
-    b->spare.push_back(L);
+    try {
+      b->spare.push_back(L);
+    } catch (...) {
+      free_launch(L);
+    }
     b->inflight.erase(b->inflight.begin() + i);
     b->cv.notify_all();
   }
@@ -915,6 +934,7 @@ bool launch_pending(gc_batch b) {
       L = b->spare.back();
       b->spare.pop_back();
     } else {
+      b->spare.reserve(b->spare.size() + kMaxSpare);  // a launch can always be put back
       L = new Launch();
     }
     L->tickets.clear();
@@ -924,6 +944,17 @@ bool launch_pending(gc_batch b) {
     L->launch_status = GC_OK;
     L->error.clear();
     int64_t nnz = 0, nv = 0;
+    try {  // from here to the launch nothing may throw: a graph taken from the queue must reach its ticket
+      const size_t most = b->pending.size();
+      take.reserve(most);
+      L->tickets.reserve(most);
+      L->owners.reserve(most);
+      L->slot.reserve(most);
+      b->inflight.reserve(b->inflight.size() + 1 + kMaxInflight);
+    } catch (...) {
+      b->spare.push_back(L);  // where it was, or the place of one that was
+      throw;
+    }
     while (!b->pending.empty()) {
       PendingGraph& pg = b->pending.front();
       if (!take.empty() && (nnz + 2 * pg.m >= (1LL << 31) - 1 || nv + pg.n >= (1LL << 31) - 1)) break;
@@ -957,7 +988,12 @@ bool launch_pending(gc_batch b) {
     cudaGetLastError();
     L->launch_status = GC_ERR_NOMEM;
   } else {
-    run_launch(b, take, L->stream, L);
+    try {
+      run_launch(b, take, L->stream, L);
+    } catch (...) {
+      L->launch_status = no_memory();
+      cudaStreamSynchronize(L->stream);  // what was queued reads the launch's host blocks
+    }
   }
   {
     std::lock_guard<std::mutex> lk(b->mu);
@@ -985,7 +1021,11 @@ void dispatcher_main(gc_batch b) {
     }
     if (!b->pending.empty() && (int)b->inflight.size() < b->cfg.max_inflight) {
       lk.unlock();
-      launch_pending(b);
+      try {
+        launch_pending(b);
+      } catch (...) {  // no memory for the launch's lists: the graphs are still pending
+        std::this_thread::sleep_for(std::chrono::milliseconds(1));
+      }
       lk.lock();
       continue;
     }
@@ -1100,7 +1140,7 @@ static bool checked_on_device(gc_batch b, int32_t n, int32_t nnz, const std::sha
 
 extern "C" {
 
-gc_status gc_batch_create(int64_t device_mem_budget_bytes, uint32_t flags, gc_batch* out) {
+gc_status gc_batch_create(int64_t device_mem_budget_bytes, uint32_t flags, gc_batch* out) try {
   if (!out) { set_error("out is NULL"); return GC_ERR_ARG; }
   *out = nullptr;
   if (device_mem_budget_bytes <= 0 || (flags & ~GC_BATCH_MANUAL)) {
@@ -1130,9 +1170,18 @@ gc_status gc_batch_create(int64_t device_mem_budget_bytes, uint32_t flags, gc_ba
     return st;
   }
   load_tuned_config(&b->cfg, nullptr);
-  if (!(flags & GC_BATCH_MANUAL)) b->dispatcher = std::thread(dispatcher_main, b);
+  try {
+    if (!(flags & GC_BATCH_MANUAL)) b->dispatcher = std::thread(dispatcher_main, b);
+  } catch (...) {
+    for (auto& t : b->streams) cudaStreamDestroy(t);
+    delete b;
+    set_error("the dispatcher thread could not be started");
+    return GC_ERR_NOMEM;
+  }
   *out = b;
   return GC_OK;
+} catch (...) {
+  return no_memory();
 }
 
 gc_status gc_batch_set_param(gc_batch b, int32_t param, int32_t value) {
@@ -1177,7 +1226,7 @@ gc_status gc_batch_last_stats(gc_batch b, double* out) {
 }
 
 gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const int32_t* col_idx,
-                          uint64_t* ticket_out) {
+                          uint64_t* ticket_out) try {
   if (!b || !ticket_out || !row_ptr || n < 0) { set_error("bad arguments"); return GC_ERR_ARG; }
   // Graphs of kDeviceCheck entries or more are checked on the device, from the
   // copy, once their row pointers have been checked; what fails there (or
@@ -1236,17 +1285,19 @@ gc_status gc_batch_submit(gc_batch b, int32_t n, const int32_t* row_ptr, const i
     return st;
   {
     std::lock_guard<std::mutex> lk(b->mu);
-    pg.ticket = b->add_ticket();
+    pg.ticket = b->admit();
     *ticket_out = pg.ticket;
-    b->pending.push_back(std::move(pg));
+    b->pending.back() = std::move(pg);
     reserved.bytes = 0;  // the launch's retirement gives it back
   }
   b->cv.notify_all();
   return GC_OK;
+} catch (...) {
+  return no_memory();
 }
 
 gc_status gc_batch_submit_many(gc_batch b, int64_t G, const int32_t* nvert, const int64_t* voff, const int64_t* eoff,
-                               const int32_t* row_ptr, const int32_t* col_idx, uint64_t* tickets_out) {
+                               const int32_t* row_ptr, const int32_t* col_idx, uint64_t* tickets_out) try {
   if (!b || G < 0 || (G > 0 && (!nvert || !voff || !eoff || !row_ptr || !tickets_out))) {
     set_error("bad arguments");
     return GC_ERR_ARG;
@@ -1332,18 +1383,26 @@ gc_status gc_batch_submit_many(gc_batch b, int64_t G, const int32_t* nvert, cons
       set_error("device-memory budget is full");
       return GC_ERR_BUSY;
     }
-    b->in_use += bytes;
-    for (int64_t g = 0; g < G; ++g) {
-      pgs[(size_t)g].ticket = b->add_ticket();
-      tickets_out[g] = pgs[(size_t)g].ticket;
-      b->pending.push_back(std::move(pgs[(size_t)g]));
+    int64_t g = 0;
+    try {
+      for (; g < G; ++g) {
+        pgs[(size_t)g].ticket = b->admit();
+        tickets_out[g] = pgs[(size_t)g].ticket;
+        b->pending.back() = std::move(pgs[(size_t)g]);
+      }
+    } catch (...) {  // all or none
+      for (; g > 0; --g) b->dismiss();
+      throw;
     }
+    b->in_use += bytes;
   }
   b->cv.notify_all();
   return GC_OK;
+} catch (...) {
+  return no_memory();
 }
 
-gc_status gc_batch_flush(gc_batch b) {
+gc_status gc_batch_flush(gc_batch b) try {
   if (!b) { set_error("batch is NULL"); return GC_ERR_ARG; }
   if (b->flags & GC_BATCH_MANUAL) {
     OutsideCapture relaxed;
@@ -1353,10 +1412,12 @@ gc_status gc_batch_flush(gc_batch b) {
     b->cv.notify_all();
   }
   return GC_OK;
+} catch (...) {
+  return no_memory();
 }
 
 gc_status gc_batch_poll(gc_batch b, uint64_t ticket, uint64_t* global_out, uint64_t* global_hi,
-                        int32_t timeout_us) {
+                        int32_t timeout_us) try {
   if (!b || !global_out) { set_error("NULL argument"); return GC_ERR_ARG; }
   OutsideCapture relaxed;
   const auto began = std::chrono::steady_clock::now();
@@ -1397,10 +1458,12 @@ gc_status gc_batch_poll(gc_batch b, uint64_t ticket, uint64_t* global_out, uint6
     if (timeout_us > 0 && std::chrono::steady_clock::now() >= deadline) return GC_PENDING;
     poll_wait(b, &lk, began);
   }
+} catch (...) {
+  return no_memory();
 }
 
 gc_status gc_batch_poll_many(gc_batch b, int64_t G, const uint64_t* tickets, uint64_t* global_out,
-                             uint64_t* global_hi, int32_t timeout_us) {
+                             uint64_t* global_hi, int32_t timeout_us) try {
   if (!b || G < 0 || (G > 0 && (!tickets || !global_out))) { set_error("bad arguments"); return GC_ERR_ARG; }
   OutsideCapture relaxed;
   const auto began = std::chrono::steady_clock::now();
@@ -1462,9 +1525,11 @@ gc_status gc_batch_poll_many(gc_batch b, int64_t G, const uint64_t* tickets, uin
     return GC_ERR_OVERFLOW;
   }
   return GC_OK;
+} catch (...) {
+  return no_memory();
 }
 
-gc_status gc_batch_destroy(gc_batch b) {
+gc_status gc_batch_destroy(gc_batch b) try {
   if (!b) return GC_OK;
   OutsideCapture relaxed;
   {
@@ -1493,6 +1558,8 @@ gc_status gc_batch_destroy(gc_batch b) {
   for (auto& s : b->streams) cudaStreamDestroy(s);
   delete b;
   return GC_OK;
+} catch (...) {
+  return no_memory();
 }
 
 }  // extern "C"

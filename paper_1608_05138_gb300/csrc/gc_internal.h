@@ -344,6 +344,8 @@ inline SmallRoute small_route(int32_t n, int32_t G, int64_t n2, int64_t m, int32
 
 // ---- host helpers (gc_api.cu) ----
 void set_error(const std::string& msg);
+// What a C entry answers to a C++ exception: GC_ERR_NOMEM, with a message if there is memory for one.
+gc_status no_memory() noexcept;
 gc_status cuda_fail(cudaError_t e, const char* what);
 
 // The library's stream-ordered memory pool on the current device (created on

@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(kNoAllocBlock) k_tri_marked(int32_t n, const i
 using namespace gc;
 
 extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr, const int32_t* col_idx,
-                                               int32_t* tri_out, void* stream) {
+                                               int32_t* tri_out, void* stream) try {
   if (n < 0 || (n > 0 && (!row_ptr || !col_idx || !tri_out))) {
     set_error("gc_edge_triangles_noalloc: bad arguments");
     return GC_ERR_ARG;
@@ -638,4 +638,6 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
   launch_after(k_tri_marked, kNoAllocCtas, kNoAllocBlock, 0, s, n, row_ptr, col_idx, tri_out, scratch);
   e = cudaGetLastError();
   return e == cudaSuccess ? GC_OK : cuda_fail(e, "gc_edge_triangles_noalloc");
+} catch (...) {
+  return no_memory();
 }

@@ -552,8 +552,12 @@ gc_status classify_c_units(int32_t n, const int32_t* d_rp, const int32_t* d_ci, 
     place(kBinRest);
     p->n_cheavy = hist[kCBins];
     p->n_cunits = p->n_cheavy + at;
-    heavy.resize((size_t)p->n_cheavy);
-    if (n_hashed > 0) e = pool_alloc(&p->chash_w, sizeof(int32_t) * (size_t)n_hashed, s);
+    try {
+      heavy.resize((size_t)p->n_cheavy);
+    } catch (...) {
+      e = cudaErrorMemoryAllocation;
+    }
+    if (n_hashed > 0 && e == cudaSuccess) e = pool_alloc(&p->chash_w, sizeof(int32_t) * (size_t)n_hashed, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_hist, cursor, sizeof(cursor), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && at > 0) {
       k_cscatter<<<std::min(grid_for(nu, 1024), 2 * sms), 1024, 0, s>>>(nu, p->units, d_bin, d_w, d_hist, p->n_cheavy,
@@ -849,7 +853,12 @@ gc_status prepare_graph(int32_t n, int32_t m, const int32_t* d_rp, const int32_t
   } else {
     GC_TRY(cudaMemsetAsync(P.out_ptr, 0, sizeof(int32_t), s), "memset out_ptr");
   }
-  if ((st = classify_c_units(n, d_rp, d_ci, rank, &P, s)) != GC_OK) goto fail;
+  try {
+    st = classify_c_units(n, d_rp, d_ci, rank, &P, s);
+  } catch (...) {
+    st = no_memory();
+  }
+  if (st != GC_OK) goto fail;
   cudaFreeAsync(out_cnt, s);
   cudaFreeAsync(dmax, s);
   *out = P;

@@ -299,3 +299,29 @@ os.waitpid(pid, 0)
 sys.exit(2)
 """
     assert subprocess.run([sys.executable, "-c", code], cwd=ROOT, timeout=120).returncode == 0
+
+
+def test_host_memory_that_runs_out_is_an_error_code(lib):
+    """No C++ exception crosses the boundary: where the checks' scratch cannot be
+    allocated, the call returns GC_ERR_NOMEM and later ones work."""
+    code = """
+import resource
+import numpy as np
+import paper_1608_05138_gb300 as gc
+gc.gc_validate_csr(np.array([0, 1, 2], np.int32), np.array([1, 0], np.int32))
+rp = np.zeros((1 << 26) + 1, np.int32)  # the scratch is two entries a vertex, 512 MB
+none = np.zeros(0, np.int32)
+size = int(open('/proc/self/statm').read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (size + (256 << 20), resource.RLIM_INFINITY))
+try:
+    gc.gc_validate_csr(rp, none)
+except gc.GcError as e:
+    assert e.status == -7, e
+else:
+    raise SystemExit('not refused')
+resource.setrlimit(resource.RLIMIT_AS, (resource.RLIM_INFINITY, resource.RLIM_INFINITY))
+gc.gc_validate_csr(rp, none)
+print('ok')
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr

@@ -23,7 +23,7 @@ namespace {
 struct Job {
   const std::function<void(int)>* f;
   int n;
-  std::atomic<int> next{0}, done{0};
+  std::atomic<int> next{0};
   int inside = 0;  // threads of the pool that hold the job (under the pool's lock)
   std::exception_ptr err;
 };

@@ -325,3 +325,23 @@ print('ok')
 """
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
+
+
+def test_symmetry_check_follows_the_mean_degree(lib):
+    """Walking the rows with counters or searching the reverses: the entries of a
+    graph of 29 a vertex must not cost several times those of one of 200 a vertex
+    (they did, with searches: four times)."""
+    import time
+    import graphgen
+
+    def took(g):
+        best = []
+        for _ in range(7):
+            t = time.perf_counter()
+            gcb.gc_validate_csr(*g)
+            best.append(time.perf_counter() - t)
+        return min(best)
+
+    skewed, dense = graphgen.rmat(18, 16, 0.57, 0.19, 0.19, 1), graphgen.er(50000, 4e-3, 3)
+    assert 20 < len(skewed[1]) / (len(skewed[0]) - 1) < 40 and len(dense[1]) > len(skewed[1])
+    assert took(skewed) < 3 * took(dense)

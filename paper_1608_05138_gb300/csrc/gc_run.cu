@@ -277,24 +277,26 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
     // the dense kernels fill the GPU and want different shares of shared memory
     // and L1: side by side they take twice as long as one after the other
     const bool dense = g.bits != nullptr;
-    Fork side(s, dense ? nullptr : fs, 0, 1);
-    const cudaStream_t t = side.next();
-    GR_BEGIN(kPhasePassC, t);
     if (dense) a.x7d = sc->x7d;
-    if ((st = dense ? run_rows_dense(g, a, t) : run_rows(g, a, t)) != GC_OK) return st;
+    // the rows stay on the count's stream, so that their kernel is the first on the
+    // GPU: its largest vertex is the longest chain, and takes half as long again on an
+    // SM that the cliques' kernels have filled before it (R-MAT scale 12: 240 us a
+    // count, 270 to 295 when a side stream let them in first)
+    Fork tiers(s, dense ? nullptr : fs, 6, kForkStreams - 6);
+    if (!dense) GR_BEGIN(kPhasePassK, s);
+    GR_BEGIN(kPhasePassC, s);
+    if ((st = dense ? run_rows_dense(g, a, s) : run_rows(g, a, s)) != GC_OK) return st;
     launches += g.n > 0 ? 1 : 0;
-    GR_END(kPhasePassC, t);
-    GR_BEGIN(kPhasePassK, s);
+    GR_END(kPhasePassC, s);
     if (dense) {
+      GR_BEGIN(kPhasePassK, s);
       if ((st = run_cliques_dense(g, a, ku.kmax, s)) != GC_OK) return st;
       launches += ku_total(ku) > 0 ? 1 : 0;
     } else {
-      Fork tiers(s, fs, 6, kForkStreams - 6);
       if ((st = run_cliques_alone(g, a, &tiers, &launches)) != GC_OK) return st;
       GR_TRY(tiers.join(), "join");
     }
     GR_END(kPhasePassK, s);
-    GR_TRY(side.join(), "join");
   } else if (overlap) {
     // pass C on the set's first stream, its kernels forked from there
     Fork side(s, fs, 0, 1);

@@ -573,6 +573,7 @@ struct gc_graph_s {
   Scratch sc;
   uint64_t* d_pe_tmp = nullptr;          // device staging for a host per-edge buffer
   uint64_t* d_ind_tmp = nullptr;         // device staging for a host per-edge induced buffer
+  int32_t n_long = 0;                    // rows of more than 4096 entries
   int device = 0;
   CountTimers timers;                    // events of the last count, and the pinned results
   bool counted = false;
@@ -687,6 +688,7 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
     set_error("host allocation failed");
     return fail(GC_ERR_NOMEM);
   }
+  g->n_long = (int32_t)R.longr.size();
   const size_t nnz1 = (size_t)(nnz > 0 ? nnz : 1), n1 = (size_t)(n > 0 ? n : 1);
   const size_t n_lists = R.mid.size() + R.longr.size();
   GC_CHECK(pool_alloc(&g->d_rp, sizeof(int32_t) * ((size_t)n + 1), s), "alloc row_ptr");
@@ -875,6 +877,7 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
   dg.hgeom = g->prep.hgeom;
   dg.hseg = g->prep.hseg;
   dg.hpos = g->prep.hpos;
+  dg.n_long = g->n_long;
   KUnits ku;
   ku.kmax = g->prep.kmax;
   ku.units = g->prep.kunits;

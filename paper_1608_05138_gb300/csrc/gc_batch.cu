@@ -546,6 +546,7 @@ gc_status run_union(std::vector<PendingGraph*>& graphs, cudaStream_t s, ForkSet*
     dg.hgeom = prep.hgeom;
     dg.hseg = prep.hseg;
     dg.hpos = prep.hpos;
+    dg.n_long = 0;  // for the induced counts, which unions do not have
     KUnits ku;
     ku.kmax = prep.kmax;
     ku.units = prep.kunits;

@@ -183,12 +183,42 @@ __global__ void __launch_bounds__(kFinBlock) k_finish(DevGraph g, CountArgs a) {
 // ---------------- per-edge induced 4-node counts ----------------
 // Per vertex x: vsum[2x] = sum over Gamma(x) of |T| of the edge (twice the
 // triangles at x), vsum[2x + 1] = sum over Gamma(x) of the neighbour's
-// degree. One warp per vertex.
+// degree. One warp per vertex, but a CTA per vertex for the g.n_long last ones, of
+// more than 4096 neighbours each: a row's chains of loads (neighbour, degree; edge,
+// out-slot, |T|) take 0.2 us per 32 entries of a warp, and the longest row was the
+// kernel (a star of 100 000 leaves: 641 us, now 72).
+constexpr int kLongRowBlock = 1024;
+__global__ void __launch_bounds__(kLongRowBlock) k_vertex_sums_long(DevGraph g, const int32_t* __restrict__ trio,
+                                                                    unsigned long long* __restrict__ vsum) {
+  __shared__ unsigned long long s_sum[2][kLongRowBlock / 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int32_t x = g.n - 1 - (int32_t)blockIdx.x;
+  const int32_t b = g.rp[x], d = g.rp[x + 1] - b;
+  unsigned long long t2 = 0, ns = 0;
+  for (int64_t k = threadIdx.x; k < d; k += kLongRowBlock) {
+    ns += (unsigned long long)g.deg[g.ci[b + k]];
+    t2 += (unsigned long long)trio[g.e2o[g.eid[b + k]]];
+  }
+  for (int o = 16; o; o >>= 1) {
+    t2 += __shfl_xor_sync(0xffffffffu, t2, o);
+    ns += __shfl_xor_sync(0xffffffffu, ns, o);
+  }
+  if (lane == 0) {
+    s_sum[0][warp] = t2;
+    s_sum[1][warp] = ns;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    unsigned long long v = 0;
+    for (int w = 0; w < kLongRowBlock / 32; ++w) v += s_sum[threadIdx.x][w];
+    vsum[2 * (size_t)x + threadIdx.x] = v;
+  }
+}
 __global__ void __launch_bounds__(256) k_vertex_sums(DevGraph g, const int32_t* __restrict__ trio,
                                                      unsigned long long* __restrict__ vsum) {
   const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < g.n; x += warps) {
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5), n = g.n - g.n_long;
+  for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += warps) {
     unsigned long long t2 = 0, ns = 0;
     for (int32_t p = g.rp[x] + lane; p < g.rp[x + 1]; p += 32) {
       ns += (unsigned long long)g.deg[g.ci[p]];
@@ -1433,6 +1463,10 @@ gc_status run_induced(const DevGraph& g, const CountArgs& a, unsigned long long*
   const int vblocks = (int)min((int64_t)count_grid_size() * 4, ((int64_t)g.n * 32 + 255) / 256);
   k_vertex_sums<<<vblocks > 0 ? vblocks : 1, 256, 0, s>>>(g, a.trio, vsum);
   cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess && g.n_long > 0) {
+    k_vertex_sums_long<<<g.n_long, kLongRowBlock, 0, s>>>(g, a.trio, vsum);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) return cuda_fail(e, "k_vertex_sums");
   const int blocks = (int)min((int64_t)count_grid_size() * 4, ((int64_t)g.m + kFinBlock - 1) / kFinBlock);
   unsigned long long* o = reinterpret_cast<unsigned long long*>(out);

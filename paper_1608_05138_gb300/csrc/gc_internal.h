@@ -64,6 +64,7 @@ struct DevGraph {
   const HubGeom* hgeom;    // ranked: [G] (nullptr when the graph has no hub units)
   const HubSeg* hseg;
   const int32_t* hpos;
+  int32_t n_long;          // one graph: rows of more than 4096 entries, the last ids
 };
 
 // Pass K (4-cliques and cross terms by lowest vertex) runs in tiers by the

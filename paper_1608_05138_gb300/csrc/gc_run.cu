@@ -329,7 +329,7 @@ gc_status run_count(const DevGraph& g, const int32_t* units, int32_t n_units, co
   GR_BEGIN(kPhaseInduced, s);
   if (want_induced) {
     if ((st = run_induced(g, a, sc->vsum, induced, induced_host, s)) != GC_OK) return st;
-    launches += 2;
+    launches += g.n_long > 0 ? 3 : 2;
   }
   GR_END(kPhaseInduced, s);
   GR_BEGIN(kPhaseDerive, s);

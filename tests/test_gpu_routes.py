@@ -422,3 +422,30 @@ def check_field_limits():
 
 def test_hub_counters_at_the_limits_of_every_field():
     run_with_env("check_field_limits()", GC_HUB_TAB_WORDS="4096")
+
+
+# ---- induced counts: rows of more than 4096 entries ----
+
+@pytest.mark.parametrize("make", [
+    lambda: graphs.star(4096),               # a warp's longest row
+    lambda: graphs.star(4097),               # a CTA's shortest
+    lambda: hubs(2, 5000, 1),
+])
+def test_induced_counts_beside_long_rows(make):
+    from tests.test_gpu_induced import assert_induced_parity
+    assert_induced_parity(*make())
+
+
+def test_induced_counts_do_not_wait_for_one_warp():
+    # the sums over the neighbours of a star's centre were one warp's, 0.64 ms
+    import torch
+    with gcb.Graph(*graphs.csr_large(100001, [(0, x) for x in range(1, 100001)])) as g:
+        n = g.n
+        ind = torch.zeros((g.m, 10), dtype=torch.int64, device="cuda")
+        took = []
+        for _ in range(5):
+            g.count_induced(ind)
+            took.append(g.phase_ms()["induced_columns"])
+    ind = ind.cpu().numpy()
+    assert (ind[:, 4] == comb(n - 2, 2)).all() and not ind[:, [0, 1, 2, 3, 5, 6, 7, 8, 9]].any()
+    assert min(took) < 0.3

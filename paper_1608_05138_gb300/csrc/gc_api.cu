@@ -88,16 +88,10 @@ void fork_destroy(ForkSet* f) {
 }
 }  // namespace
 
-ForkSet* fork_acquire(int priority) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) {
-    cuda_fail(e, "cudaGetDevice");
-    return nullptr;
-  }
+ForkSet* fork_acquire(int dev, int priority) {
   {
     std::lock_guard<std::mutex> lk(g_fork_mu);
-    for (size_t i = 0; i < g_forks.size(); ++i)
+    for (size_t i = g_forks.size(); i-- > 0;)  // the last one given back
       if (g_forks[i]->device == dev && g_forks[i]->priority == priority) {
         ForkSet* f = g_forks[i];
         g_forks.erase(g_forks.begin() + (long)i);
@@ -111,7 +105,7 @@ ForkSet* fork_acquire(int priority) {
   }
   f->device = dev;
   f->priority = priority;
-  e = cudaEventCreateWithFlags(&f->start, cudaEventDisableTiming);
+  const cudaError_t e = cudaEventCreateWithFlags(&f->start, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     cuda_fail(e, "side streams");
     fork_destroy(f);
@@ -574,6 +568,8 @@ struct gc_graph_s {
   uint64_t* d_pe_tmp = nullptr;          // device staging for a host per-edge buffer
   uint64_t* d_ind_tmp = nullptr;         // device staging for a host per-edge induced buffer
   int32_t n_long = 0;                    // rows of more than 4096 entries
+  int priority = 0;                      // of the stream
+  bool part = false;                     // it is on a part of the GPU
   int device = 0;
   CountTimers timers;                    // events of the last count, and the pinned results
   bool counted = false;
@@ -767,6 +763,8 @@ gc_status gc_graph_upload(int32_t n, const int32_t* row_ptr, const int32_t* col_
     scratch_guess_tlist(&g->sc, g->m);
   }
   GC_CHECK(timers_init(&g->timers, g->device), "events");
+  if (cudaStreamGetPriority(s, &g->priority) != cudaSuccess) cudaGetLastError();
+  g->part = on_part_of_gpu(s);
   GC_CHECK(cudaStreamSynchronize(s), "sync upload");
 #undef GC_CHECK
   *out = g;
@@ -902,11 +900,9 @@ static gc_status count_graph(gc_graph g, uint64_t* per_edge_out, uint64_t* induc
       fork_release(f);
     }
   } lent = {nullptr};
-  if (!on_part_of_gpu(s)) {
-    int priority = 0;
-    if (cudaStreamGetPriority(s, &priority) != cudaSuccess) cudaGetLastError();
-    if (!(lent.f = fork_acquire(priority))) return GC_ERR_CUDA;
-  }
+  // what the default streams stand for is the current context's to say
+  const bool part = (uintptr_t)s <= (uintptr_t)cudaStreamPerThread ? on_part_of_gpu(s) : g->part;
+  if (!part && !(lent.f = fork_acquire(dev, g->priority))) return GC_ERR_CUDA;
   if ((st = run_count(dg, g->prep.units, g->prep.n_units, ku, pe_dev, &g->sc, s, lent.f, &g->timers, pe_host, ind_dev,
                       ind_host)) != GC_OK)
     return st;

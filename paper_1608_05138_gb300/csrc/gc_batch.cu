@@ -796,7 +796,7 @@ void run_launch(gc_batch b, std::vector<PendingGraph>& graphs, cudaStream_t s, L
   if (st == GC_OK && !large.empty()) {
     cudaEventRecord(L->ev[kEvUnion0], s);
     ForkSet*& fs = b->forks[L->stream_slot];
-    if (!fs) fs = fork_acquire(0);  // the slots' streams have the default priority
+    if (!fs) fs = fork_acquire(b->device, 0);  // the slots' streams have the default priority
     if (!fs) {
       st = GC_ERR_CUDA;
       L->error = gc_last_error();

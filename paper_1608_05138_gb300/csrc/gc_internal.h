@@ -184,7 +184,7 @@ struct CountTimers {
   cudaEvent_t begin[kNumPhases] = {}, end[kNumPhases] = {};
   unsigned char* pinned = nullptr;
 };
-ForkSet* fork_acquire(int priority);  // of the current device; nullptr on failure (message set)
+ForkSet* fork_acquire(int device, int priority);  // of the current device; nullptr on failure (message set)
 // Whether the stream belongs to a part of the GPU only (a green context): its
 // count then stays on it, since side streams would be on the whole GPU.
 bool on_part_of_gpu(cudaStream_t s);

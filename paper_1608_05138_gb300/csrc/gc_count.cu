@@ -387,7 +387,8 @@ __global__ void __launch_bounds__(kBlock) k_pass_c(DevGraph g, CountArgs a) {
 }
 
 // ---------------- graphs of at most kSmemTableMax vertices: rows of common neighbours ----------------
-// For such a graph (of a union: every graph) a row of counters c(w) = |Gamma(u)
+// For such a graph (of a union: every graph; which of them take this route:
+// small_route) a row of counters c(w) = |Gamma(u)
 // and Gamma(w)| over all vertices fits in shared memory, and gives for every
 // edge (u, v)
 //   |T|      = c(v)
@@ -700,8 +701,8 @@ __global__ void __launch_bounds__(kDenseBlock) k_cliques_dense(DevGraph g, Count
 // fixed segments of 2- to 32-bit counters (HubSeg), several to a block; o of
 // degree 1 close no cycle and are skipped. On R-MAT scale 22 the id range of
 // 4.2M takes 8 blocks and 12 segments where blocks of one 10-, 16- or 32-bit
-// width took 31 to 94, so that a run has 100 entries instead of 16 (sweeps of
-// (x, block) 2.2e9 -> 4.4e8), and the segments' bounds in every longer row
+// width took 31 to 94, so that a run has 72 entries instead of 16 (sweeps of
+// (x, segment) 5.0e8, of (x, block) 2.2e9), and the segments' bounds in every longer row
 // are looked up in a table made once per graph instead of searched. The
 // whole kernel: 180 -> 127 ms there; 8.5 -> 5.6 ms on Chung-Lu 1M, where
 // about a quarter of the warps' time is still the barrier between a block's

@@ -59,7 +59,7 @@ struct DevGraph {
   const int32_t* gn;       // [G] vertices of each graph
   const int64_t* gm;       // [G] edges of each graph
   int32_t table_n;         // max gn[g]: size of one Psi table
-  const uint32_t* bits;    // dense graphs (dense_graph()): bit rows [n][(n + 31) / 32], and the same by word
+  const uint32_t* bits;    // kRouteDense (small_route()): bit rows [n][(n + 31) / 32], and the same by word
   const uint32_t* bits_t;  // [(n + 31) / 32][n]; else nullptr
   const HubGeom* hgeom;    // ranked: [G] (nullptr when the graph has no hub units)
   const HubSeg* hseg;
@@ -151,7 +151,7 @@ enum Work {
 };
 
 // Device status bits. kSpillOverflow: a unit outgrew what it was binned for
-// (a pass-T/K tier, the hub cursors, the hashed pass-C table); it cannot
+// (a pass-T/K tier, the hashed pass-C table); it cannot
 // happen for a validated graph.
 enum Status : int32_t { kOk = 0, kSpillOverflow = 1, kInexact = 2 };
 
@@ -551,7 +551,9 @@ constexpr int kHubTabDefault = 45056;
 int hub_tab_words();
 // Counters per word that a unit of nx lower neighbours could use over its
 // whole o-range by nx alone; the rule that picks the hub units estimates
-// their blocks with it.
+// their blocks with it. It dates from blocks of one counter width: with segments
+// there are fewer blocks (8 where it says 31 to 94 on R-MAT scale 22), and the
+// line between the hub kernel and the others was not measured again.
 __host__ __device__ __forceinline__ int hub_cpw(int64_t nx) { return nx < 1023 ? 3 : nx < 65536 ? 2 : 1; }
 // Units of pass C with at most kHashMaxW wedges count in a shared-memory
 // hash of 2 kHashMaxW keys (at most half full: a unit has no more distinct
@@ -585,8 +587,8 @@ gc_status run_induced(const DevGraph& g, const CountArgs& a, unsigned long long*
                       cudaStream_t s);
 // Bytes of one global-tier buffer for out-degrees up to cap.
 size_t kbuf_bytes(int32_t cap);
-// Unit ordering key (environment GC_ORDER): 0 = vol (default: d_v + sum of
-// neighbour degrees, heaviest bin first), 1 = degree d_v, 2 = none (vertex id).
+// Ordering key of the units on the vertex-indexed tables (environment GC_ORDER):
+// 0 = vol (default: d_v^2, heaviest bin first), 1 = degree d_v, 2 = none (vertex id).
 int order_key();
 // exclusive prefix sum of n int32 into out[0..n] (out[n] = total)
 gc_status exclusive_scan(int32_t n, const int32_t* in, int32_t* out, cudaStream_t s);

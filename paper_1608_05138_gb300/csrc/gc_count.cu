@@ -399,8 +399,9 @@ __global__ void __launch_bounds__(kBlock) k_pass_c(DevGraph g, CountArgs a) {
 // and the 4-cliques (the rest of pass K) need nothing from here: both run side
 // by side, where passes T and C, K, and the finish used to wait for each other
 // (G(1000, 0.3): 480 -> 356 us per count; G(2000, 0.01): 123 -> 103 us). Work is
-// sum d^2 counters, twice: it waits on loads in sparse graphs and on the
-// shared-memory pipe in dense ones. CTA per vertex, largest degree first.
+// sum d^2 counters, twice. CTA per vertex, largest degree first: in skewed graphs
+// the largest one is the kernel (Chung-Lu 4000 / 60 000, 213 us: the SMs are busy
+// 21 % of the time, and issue on 68 % of their active cycles).
 constexpr int kRowBlock = 256;
 constexpr uint32_t kMark = 0x80000000u;  // w is a neighbour of u
 __global__ void __launch_bounds__(kRowBlock) k_rows(DevGraph g, CountArgs a) {
@@ -499,7 +500,8 @@ __global__ void __launch_bounds__(kRowBlock) k_rows(DevGraph g, CountArgs a) {
 // so that the sums over Gamma(v), and over T = Gamma(u) and Gamma(v), of c(w) - 1
 // are popcounts of row v, and of row v & row u, with each plane: a lane per v,
 // words times bits operations for it where the lists took 25 instructions per
-// 32 of its d_v entries. Bound by popc. G(1000, 0.3): 165 -> 78 us.
+// 32 of its d_v entries. It waits on the loads of the bit rows, at 39 % of the warps
+// an SM can hold (issue active 38 %, the pipe of popc 25 %). G(1000, 0.3): 165 -> 78 us.
 constexpr int kDenseBits = 11;  // c(w) - 1 < 2^11
 static_assert(kDenseMaxN <= 1 << kDenseBits, "counter planes");
 constexpr int kRowDenseBlock = 128;
@@ -588,7 +590,7 @@ __global__ void __launch_bounds__(kRowDenseBlock, 8) k_rows_dense(DevGraph g, Co
 // bit rows (a ballot per row and word), c_ij for its edges i < j, a lane each,
 // added to x7d of the edge (b_i, b_j), and half of each member's sum to (a, b_i). No scan of out-lists, no hash and no list of edges, which
 // took pass K's tiers 58 + 100 us on G(1000, 0.3); here 74 us. CTA per unit, largest
-// first. Bound by popc.
+// first. Bound by instruction issue (72 % of the active cycles; popc's pipe 12 %).
 constexpr int kDenseBlock = 256;
 __host__ __device__ constexpr int dense_stride(int k) { return ((k + 31) / 32) | 1; }
 __global__ void __launch_bounds__(kDenseBlock) k_cliques_dense(DevGraph g, CountArgs a, int32_t kmax) {

@@ -28,9 +28,10 @@
 //          it, the CTA together beyond. An H_u of few edges is counted edge by
 //          edge instead (few_edges), one of fewer than three not at all.
 // Rows are stored at an odd word stride, so that 32 lanes reading one word
-// index of 32 rows hit 32 banks. What bounds it: popc (16 lanes a clock an SM)
-// and shared-memory reads, one and five quarters of one per 32 pairs and word
-// (four u's share the words of row w). (Before, each edge
+// index of 32 rows hit 32 banks; four u's share the words of row w, five quarters
+// of a read per 32 pairs and word. What bounds it: instruction issue, 86 % of the
+// cycles in the classes above 128 vertices (shared-memory wavefronts 47 %, the
+// pipe of popc 25 % of their peaks), with barriers in the smaller ones. (Before, each edge
 // listed its common neighbours and took one of their rows at a time over the
 // lanes: the graphs of n <= 512 in a launch of 48 took 5.3 ms, one CTA each;
 // now 0.24 ms, in 256 parts.)
@@ -247,8 +248,7 @@ constexpr uint16_t kFewEdges = 0x8000;  // in s_up
 
 // The pairs of kU consecutive vertices u0, u0 + 1, ... with the vertices above
 // them, a lane per w: every word of row w is loaded once for all of them. (One u
-// at a time loaded two words a pair and word, and those loads, not popc, were
-// the pass: 2000 graphs of 1000 vertices and mean degree 5, 14.9 ms, now 9.5.) Lane i
+// at a time: 2000 graphs of 1000 vertices and mean degree 5 took 14.9 ms, now 9.5.) Lane i
 // adds sum i of them to `mine`: sums over four u stay in 32 bits (4092 pairs at
 // most, c and the degrees at most 1023). Marks the u that need no H_u, and those
 // whose H_u is counted edge by edge.
@@ -315,8 +315,8 @@ __device__ __forceinline__ void small_pairs(const uint32_t* __restrict__ bm, con
 }
 
 // at least 1536 threads resident per SM (at most 42 registers a thread) where
-// shared memory has room for them: the kernel waits on shared memory and popc,
-// and the more warps an SM holds, the more of its cycles issue
+// shared memory has room for them: the more warps an SM holds, the more of its
+// cycles issue
 __host__ __device__ constexpr int small_ctas(int kN, int kBlock) {
   const int fit = (int)(((size_t)227 << 10) / (small_smem(kN, kBlock) + 3072));
   return fit < 1 ? 1 : fit < 1536 / kBlock ? fit : 1536 / kBlock;

@@ -225,8 +225,10 @@ __global__ void __launch_bounds__(kOneBlock) k_tri_one(int32_t n, const int32_t*
                                                        const uint32_t* scratch /* null: not picked */) {
   constexpr int kW = kOneBlock / 32;
   __shared__ uint32_t bm[kPickN / 32];
-  after_previous();
-  if (scratch && !scratch[kOneKernel]) return;
+  if (scratch) {  // else the call's only kernel: what follows it is the caller's
+    after_previous();
+    if (!scratch[kOneKernel]) return;
+  }
   __shared__ int32_t s_cnt[kW][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t* cnt = s_cnt[warp];

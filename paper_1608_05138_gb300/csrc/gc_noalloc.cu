@@ -67,16 +67,23 @@ __device__ __forceinline__ int window_of(int64_t nnz) { return nnz < (1 << 18) ?
 // Rows of at most this many entries are a warp's (d^2 / 128 steps at most); a
 // longer one is a CTA's, in parts of a window per warp.
 __device__ __forceinline__ int short_row(int64_t nnz) { return 4 * window_of(nnz); }
-__device__ __forceinline__ int part_of(int64_t nnz) { return kNoAllocBlock / 32 * window_of(nnz); }
+// (from 2^28 entries larger ones, so that their list holds all of them: 1700
+// complete graphs of 600, which it did not hold, 1163 ms, now 392)
+__device__ __forceinline__ int part_of(int64_t nnz) {
+  return nnz < (1 << 28) ? kNoAllocBlock / 32 * window_of(nnz) : 2048;
+}
 constexpr int kShortRow = 128;              // the longest short row
 constexpr int kShortSlots = 2 * kShortRow;  // its hash, at most half full
 constexpr int kShortWords = kShortSlots + kShortRow;  // a warp's hash and filter
 constexpr int kTriBlock = 256;
-constexpr int kPart = kNoAllocBlock;        // the largest part
+constexpr int kMaxHeavy = 512;              // heavy runs of a part that its warps share
 // Up to this many vertices, the bitmap and the warps' hashes leave room for four
 // CTAs an SM, and one kernel takes the long rows and then the short ones.
 constexpr int32_t kBothMaxN = 1 << 17;
-constexpr int kHeavyRun = 512;   // a lower neighbour's row of this many entries is all warps' together
+// A lower neighbour's row of this many entries is shared by all warps, as one
+// alone would be the last to end (R-MAT scale 18, rows from 512, 1024, 2048
+// entries: 1.99, 1.71, 1.68 ms; 950 complete graphs of 1100: 1368, 1367, 1211).
+constexpr int kHeavyRun = 2048;
 constexpr uint32_t kMaxParts = (uint32_t)(kOffMaps - kOffLong);  // list entries: x (20 bits) and the part above
 constexpr uint32_t kNoPart = 0xffffffffu;
 // Up to kOneN vertices, k_tri_one does the whole step; up to kPickN, it or the
@@ -144,7 +151,7 @@ __global__ void __launch_bounds__(kTriBlock) k_rows(int32_t n, const int32_t* __
     }
     const uint32_t parts = (uint32_t)((d + part - 1) / part);  // at most 4096, as d <= min(n, nnz)
     const uint32_t at = atomicAdd(scratch + kNumLong, parts);
-    // else by k_tri_marked: more parts than the list holds (only beyond 2^28
+    // else by k_tri_marked: more parts than the list holds (only beyond 2.08e9
     // entries), or a last part of the last vertex that would read as kNoPart
     const bool fits = at + parts <= kMaxParts && !((uint32_t)x == 0xfffffu && parts == 4096u);
     if (!fits) atomicOr(scratch + kOffBad + (x >> 5), 1u << (x & 31));
@@ -210,6 +217,34 @@ __device__ __forceinline__ void count_runs(const int32_t* __restrict__ ci, int32
   }
 }
 
+// The same with the runs of kLongRun entries or more read by the whole warp, one
+// after the other, at a third of the instructions an entry (k_tri: 1000 complete
+// graphs of 500, 659 ms with all runs laid end to end, now 271; K_300, 3400 of
+// them, 376 and 130). `in` takes any number.
+constexpr int32_t kLongRun = 64;
+template <class In>
+__device__ __forceinline__ void count_runs_long(const int32_t* __restrict__ ci, int32_t yb, int32_t L, int32_t* cnt,
+                                                int lane, In in) {
+  count_runs(ci, yb, L < kLongRun ? L : 0, cnt, lane, in);
+  unsigned lm = __ballot_sync(0xffffffffu, L >= kLongRun);
+  while (lm) {
+    const int src = __ffs(lm) - 1;
+    lm &= lm - 1u;
+    const int32_t* row = ci + __shfl_sync(0xffffffffu, yb, src);
+    const uint32_t len = (uint32_t)__shfl_sync(0xffffffffu, L, src);
+    uint32_t c = 0;
+    for (uint32_t q = lane; q < len; q += 128) {
+      int32_t w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) w[j] = q + 32 * j < len ? row[q + 32 * j] : -1;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) c += in(w[j]);
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == src) cnt[lane] = (int32_t)c;  // its own: count_runs left it 0
+  }
+}
+
 // The whole step in one kernel: CTA per row x, a bitmap of it in shared memory; a
 // window of its slots per warp, whose short rows are read end to end over the
 // lanes and whose long ones (kLongRun entries) by the whole warp. Every slot by
@@ -219,7 +254,6 @@ __device__ __forceinline__ void count_runs(const int32_t* __restrict__ ci, int32
 // G(64, 0.3) 40 / 71 us, G(1000, 0.02) 43 / 82, K_1000 687 / 795, K(200, 800)
 // 161 / 151; the others' 71 is 66 since they follow each other closely.
 constexpr int kOneBlock = 256;
-constexpr int32_t kLongRun = 64;
 __global__ void __launch_bounds__(kOneBlock) k_tri_one(int32_t n, const int32_t* __restrict__ rp,
                                                        const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
                                                        const uint32_t* scratch /* null: not picked */) {
@@ -258,24 +292,7 @@ __global__ void __launch_bounds__(kOneBlock) k_tri_one(int32_t n, const int32_t*
       }
       cnt[lane] = 0;
       __syncwarp();
-      count_runs(ci, yb, L < kLongRun ? L : 0, cnt, lane, in);
-      unsigned lm = __ballot_sync(0xffffffffu, L >= kLongRun);
-      while (lm) {
-        const int src = __ffs(lm) - 1;
-        lm &= lm - 1u;
-        const int32_t* row = ci + __shfl_sync(0xffffffffu, yb, src);
-        const uint32_t len = (uint32_t)__shfl_sync(0xffffffffu, L, src);
-        uint32_t c = 0;
-        for (uint32_t q = lane; q < len; q += 128) {
-          int32_t w[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) w[j] = q + 32 * j < len ? row[q + 32 * j] : -1;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) c += in(w[j]);
-        }
-        c = __reduce_add_sync(0xffffffffu, c);
-        if (lane == src) cnt[lane] = (int32_t)c;  // its own: count_runs left it 0
-      }
+      count_runs_long(ci, yb, L, cnt, lane, in);
       __syncwarp();
       if (mine) tri[b + k0 + lane] = cnt[lane];
       __syncwarp();
@@ -371,21 +388,22 @@ __device__ __forceinline__ void short_rows(int32_t n, const int32_t* __restrict_
 // long rows of lower neighbours to a list that all warps then read together
 // (the heaviest neighbours are often next to each other, and one warp alone
 // took 0.9 ms for them).
+template <int kThreads>
 __device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                            int32_t* __restrict__ tri, uint32_t* __restrict__ scratch,
                                            uint32_t* bm /* (n + 31) / 32 words */, int32_t* cnt) {
   __shared__ uint32_t s_x;
   __shared__ int32_t s_next, s_heavy;
-  __shared__ int32_t s_hp[kPart], s_hb[kPart], s_hl[kPart], s_hc[kPart];  // the listed slots, their rows, their counts
+  __shared__ int32_t s_hp[kMaxHeavy], s_hb[kMaxHeavy], s_hl[kMaxHeavy], s_hc[kMaxHeavy];  // slots, rows, counts
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t nnz = rp[n];
-  const int32_t window = window_of(nnz), slots = part_of(nnz);
+  const int32_t slots = part_of(nnz);
   const uint32_t n_long = min(scratch[kNumLong], kMaxParts);
   // Bounds are checked although the listed rows follow the rules: calls that
   // overlap on the GPU share the scratch array, and may then list rows and miss
   // marks of each other's graphs.
-  auto in = [&](int32_t w) -> bool { return w < n && ((bm[w >> 5] >> (w & 31)) & 1u); };
-  for (int32_t i = threadIdx.x; i < (n + 31) / 32; i += kNoAllocBlock) bm[i] = 0u;
+  auto in = [&](int32_t w) -> bool { return (uint32_t)w < (uint32_t)n && ((bm[w >> 5] >> (w & 31)) & 1u); };
+  for (int32_t i = threadIdx.x; i < (n + 31) / 32; i += kThreads) bm[i] = 0u;
   for (;;) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -401,12 +419,13 @@ __device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict_
     const int32_t x = (int32_t)(s_x & 0xfffffu), part = (int32_t)(s_x >> 20);
     if (x >= n || row_bad(scratch, x)) continue;
     const int32_t b = rp[x], d = rp[x + 1] - b;
-    const int32_t end = min(d, (part + 1) * slots);  // at most 4096 parts of at most 512 slots
+    const int32_t start = min(d, part * slots), end = min(d, start + slots);  // at most 4096 parts of 128 to 2048 slots
+    const int32_t window = min(32, (end - start + kThreads / 32 - 1) / (kThreads / 32));  // some for every warp
     if (threadIdx.x == 0) {
-      s_next = min(end, part * slots);
+      s_next = start;
       s_heavy = 0;
     }
-    for (int32_t k = threadIdx.x; k < d; k += kNoAllocBlock) {
+    for (int32_t k = threadIdx.x; k < d; k += kThreads) {
       const int32_t y = ci[b + k];
       if ((uint32_t)y < (uint32_t)n) atomicOr(&bm[y >> 5], 1u << (y & 31));
     }
@@ -421,38 +440,42 @@ __device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict_
       lower_slot(n, rp, ci, scratch, x, d, b, k0 + lane, min(end, k0 + window), yb, L, mine);
       if (L >= kHeavyRun) {
         const int32_t k = atomicAdd(&s_heavy, 1);
-        s_hp[k] = b + k0 + lane;
-        s_hb[k] = yb;
-        s_hl[k] = L;
-        s_hc[k] = 0;
-        L = 0;
-        mine = false;
+        if (k < kMaxHeavy) {  // else this warp's
+          s_hp[k] = b + k0 + lane;
+          s_hb[k] = yb;
+          s_hl[k] = L;
+          s_hc[k] = 0;
+          L = 0;
+          mine = false;
+        }
       }
       cnt[lane] = 0;
       __syncwarp();
-      count_runs(ci, yb, L, cnt, lane, in);
+      count_runs_long(ci, yb, L, cnt, lane, in);
       __syncwarp();
       if (mine) tri[b + k0 + lane] = cnt[lane];
       __syncwarp();
     }
     __syncthreads();
-    const int32_t heavy = s_heavy;
+    const int32_t heavy = min(s_heavy, kMaxHeavy);
+    int32_t before = 0;  // their pieces of 128 entries go round the warps
     for (int32_t k = 0; k < heavy; ++k) {
       const int32_t *row = ci + s_hb[k], len = s_hl[k];
       int32_t c = 0;
-      for (int32_t q0 = 128 * warp; q0 < len; q0 += 128 * (kNoAllocBlock / 32)) {
+      for (int32_t q0 = 128 * ((warp - before) & (kThreads / 32 - 1)); q0 < len; q0 += 128 * (kThreads / 32)) {
         int32_t w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) w[j] = q0 + 32 * j + lane < len ? row[q0 + 32 * j + lane] : -1;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) c += w[j] >= 0 && in(w[j]);
+        for (int j = 0; j < 4; ++j) c += in(w[j]);
       }
+      before += (len + 127) >> 7;
       c = (int32_t)__reduce_add_sync(0xffffffffu, (unsigned)c);
       if (lane == 0 && c) atomicAdd(&s_hc[k], c);
     }
     __syncthreads();
-    for (int32_t k = threadIdx.x; k < heavy; k += kNoAllocBlock) tri[s_hp[k]] = s_hc[k];
-    for (int32_t k = threadIdx.x; k < d; k += kNoAllocBlock) {
+    for (int32_t k = threadIdx.x; k < heavy; k += kThreads) tri[s_hp[k]] = s_hc[k];
+    for (int32_t k = threadIdx.x; k < d; k += kThreads) {
       const int32_t y = ci[b + k];
       if ((uint32_t)y < (uint32_t)n) bm[y >> 5] = 0u;
     }
@@ -461,17 +484,18 @@ __device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict_
 
 // Both, or one of them (which: bit 0 long rows, bit 1 short ones), with the
 // bitmap and the warps' hashes in dynamic shared memory.
-__global__ void __launch_bounds__(kNoAllocBlock, 4) k_tri(int32_t n, const int32_t* __restrict__ rp,
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, 2048 / kThreads) k_tri(int32_t n, const int32_t* __restrict__ rp,
                                                           const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
                                                           uint32_t* __restrict__ scratch, int which) {
   extern __shared__ uint32_t s_dyn[];
-  __shared__ int32_t s_cnt[kNoAllocBlock / 32][32];
+  __shared__ int32_t s_cnt[kThreads / 32][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   after_previous();
   if (scratch[kOneKernel]) return;
   uint32_t* tables = s_dyn;
   if (which & 1) {
-    long_parts(n, rp, ci, tri, scratch, s_dyn, s_cnt[warp]);
+    long_parts<kThreads>(n, rp, ci, tri, scratch, s_dyn, s_cnt[warp]);
     tables += (n + 31) / 32;
   }
   if (which & 2) {
@@ -598,9 +622,10 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
       if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress");
       if ((e = cudaDeviceGetAttribute(&g_noalloc_sms[dev], cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return cuda_fail(e, "cudaDeviceGetAttribute");
-      if ((e = cudaFuncSetAttribute(k_tri, cudaFuncAttributeMaxDynamicSharedMemorySize, kNoAllocWords * 4)) !=
-          cudaSuccess)
-        return cuda_fail(e, "k_tri");
+      for (auto kernel : {k_tri<kNoAllocBlock>, k_tri<2 * kNoAllocBlock>})
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kNoAllocWords * 4)) !=
+            cudaSuccess)
+          return cuda_fail(e, "k_tri");
       g_noalloc_ptr[dev] = static_cast<uint32_t*>(p);
     }
     scratch = g_noalloc_ptr[dev];
@@ -625,16 +650,20 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
     return cuda_fail(e, "zero counters");
   }
   launch_after(k_rows, grid, kTriBlock, 0, s, n, row_ptr, col_idx, scratch);
-  auto tri = [&](int which, int per_sm, size_t smem) {
-    launch_after(k_tri, sms * per_sm, kNoAllocBlock, smem, s, n, row_ptr, col_idx, tri_out, scratch, which);
+  auto tri = [&](int which, int per_sm, int block, size_t smem) {
+    launch_after(block == kNoAllocBlock ? k_tri<kNoAllocBlock> : k_tri<2 * kNoAllocBlock>, sms * per_sm, block, smem, s,
+                 n, row_ptr, col_idx, tri_out, scratch, which);
   };
   // CTAs an SM: four (2048 threads) while the bitmaps leave room for them in
-  // 227 KB, beside the 11 KB that every CTA takes
+  // 227 KB, beside the 11 KB that every CTA takes; with larger bitmaps fewer, of
+  // twice the threads (R-MAT scale 20: 20.7 ms with 512 and 16.0 with 1024)
   if (n <= kBothMaxN) {
-    tri(3, 4, bitmap + kTables);
+    tri(3, 4, kNoAllocBlock, bitmap + kTables);
   } else {
-    tri(1, (int)std::min<size_t>(4, ((size_t)227 << 10) / (bitmap + ((size_t)13 << 10))), bitmap);
-    tri(2, 4, kTables);
+    auto fit = [&](size_t besides) { return ((size_t)227 << 10) / (bitmap + (besides << 10)); };
+    if (fit(13) >= 4) tri(1, 4, kNoAllocBlock, bitmap);
+    else tri(1, (int)std::min<size_t>(2, fit(15)), 2 * kNoAllocBlock, bitmap);
+    tri(2, 4, kNoAllocBlock, kTables);
   }
   launch_after(k_tri_reverse, grid, kTriBlock, 0, s, n, row_ptr, col_idx, tri_out, scratch);
   launch_after(k_tri_marked, kNoAllocCtas, kNoAllocBlock, 0, s, n, row_ptr, col_idx, tri_out, scratch);

@@ -200,8 +200,7 @@ def test_noalloc_small_call_is_one_kernel_and_can_be_captured():
 
 def test_noalloc_slots_beyond_2_to_the_30():
     # 950 complete graphs on 1100 vertices: 1.15e9 slots, so that the sum of two of
-    # them, as a binary search forms it, passes 2^31; a third of the rows does not
-    # fit the list of parts either
+    # them, as a binary search forms it, passes 2^31
     import torch
     k, copies = 1100, 950
     v = torch.arange(k, dtype=torch.int32, device="cuda")
@@ -213,6 +212,33 @@ def test_noalloc_slots_beyond_2_to_the_30():
     gcb.gc_edge_triangles_noalloc(rp, ci, out)
     assert bool((out == k - 2).all())
     del ci, out
+    torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("n, sizes", [
+    # rows of one more and one less than a warp's and a CTA's, of runs that a lane, a
+    # warp and a CTA reads; the last n of four CTAs an SM and the first of larger ones
+    (358400, [17, 64, 65, 66, 128, 129, 130, 131, 600, 2048, 2049, 2050, 2600]),
+    (358432, [17, 64, 65, 66, 128, 129, 130, 131, 600, 2048, 2049, 2050, 2600]),
+    (1 << 20, [17, 64, 65, 66, 128, 129, 130, 131, 600, 2048, 2049, 2050, 2600]),
+    (131073, [2100] * 62),  # 2^28 entries: more of a part's runs than its CTA can list
+])
+def test_noalloc_long_rows_by_number_of_vertices(n, sizes):
+    # disjoint complete graphs after isolated vertices
+    import torch
+    ks = torch.tensor(sizes, device="cuda")
+    k = torch.cat([torch.zeros(n - sum(sizes), dtype=torch.long, device="cuda"), torch.repeat_interleave(ks, ks)])
+    rp = torch.zeros(n + 1, dtype=torch.int32, device="cuda")
+    rp[1:] = torch.cumsum((k - 1).clamp(min=0), 0)
+    ci, at = [], n - sum(sizes)
+    for s in sizes:
+        v = torch.arange(s, dtype=torch.int32, device="cuda")
+        ci.append(v.repeat(s, 1)[~torch.eye(s, dtype=torch.bool, device="cuda")] + at)
+        at += s
+    out = torch.full((int(rp[-1]),), -1, dtype=torch.int32, device="cuda")
+    gcb.gc_edge_triangles_noalloc(rp, torch.cat(ci), out)
+    assert torch.equal(out, torch.repeat_interleave(k - 2, (k - 1).clamp(min=0)).to(torch.int32))
+    del ci, out, k
     torch.cuda.empty_cache()
 
 

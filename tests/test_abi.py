@@ -330,7 +330,7 @@ print('ok')
 def test_symmetry_check_follows_the_mean_degree(lib):
     """Walking the rows with counters or searching the reverses: the entries of a
     graph of 29 a vertex must not cost several times those of one of 200 a vertex
-    (they did, with searches: four times)."""
+    (they did, with searches: 2.7 to 4 times; now 1.2 to 1.8)."""
     import time
     import graphgen
 
@@ -344,4 +344,4 @@ def test_symmetry_check_follows_the_mean_degree(lib):
 
     skewed, dense = graphgen.rmat(18, 16, 0.57, 0.19, 0.19, 1), graphgen.er(50000, 4e-3, 3)
     assert 20 < len(skewed[1]) / (len(skewed[0]) - 1) < 40 and len(dense[1]) > len(skewed[1])
-    assert took(skewed) < 3 * took(dense)
+    assert took(skewed) < 2.3 * took(dense)

@@ -17,8 +17,8 @@
 // sum min(d_x, d_y) lookups over the edges, where looking up row y in a bitmap
 // of row x for every slot, in global memory, took sum d^2 (Chung-Lu, 100 003
 // vertices, 1 000 003 edges, exponent 2.3: 2.2e9 lookups and 7.9 ms for a
-// pass, 0.50 ms now: 37 us k_rows, 368 k_tri, whose warps wait at barriers for the
-// longest chain of loads among them, 64 k_tri_reverse, which waits on loads).
+// pass, 0.45 ms now: 37 us k_rows, 318 k_tri, whose warps wait at barriers for the
+// longest chain of loads among them, 66 k_tri_reverse, which waits on loads).
 // Up to kOneN vertices one kernel does it all, a CTA per row (k_tri_one). Above,
 // five launches, each waiting for the one before:
 //   k_rows   marks the rows that break the CSR rules (not strictly ascending,

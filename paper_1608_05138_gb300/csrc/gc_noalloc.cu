@@ -25,7 +25,7 @@
 //            a column out of range, a self-loop) and lists the long rows
 //   k_tri    the slots (x, y), y below x in (degree, id): a CTA per part of a
 //            long row with a bitmap of the vertices in shared memory, then a
-//            warp per other row with a hash of at most 128 entries
+//            warp per other row with a hash of at most 128 entries (or 256)
 //   k_tri_reverse   the other slots, from the reverse slot (a binary search);
 //            slots without one, or with an end whose row breaks the rules, are
 //            marked
@@ -57,6 +57,13 @@ constexpr size_t kOffMaps = (size_t)2 * kNoAllocMaxN;
 constexpr size_t kScratchWords = kOffMaps + (size_t)kNoAllocCtas * kNoAllocWords;  // 32 MiB
 static_assert(kScratchWords * 4 == (size_t)32 << 20, "scratch size");
 
+// Up to this many vertices, the bitmap and the warps' hashes leave room for four
+// CTAs an SM, and one kernel takes the long rows and then the short ones.
+constexpr int32_t kBothMaxN = 1 << 17;
+// Up to this many, the bitmap leaves room for four CTAs of 512 threads an SM beside
+// the 13 KB that every CTA takes; beyond, fewer fit, of 1024 threads.
+constexpr int32_t kFourMaxN = 358400;
+
 // Slots of a long row that a warp takes at a time: the runs of that many lower
 // neighbours are a warp's chain of loads. Graphs of fewer entries have fewer
 // warps' worth of slots, and there the longest chain is the kernel's time
@@ -65,21 +72,26 @@ static_assert(kScratchWords * 4 == (size_t)32 << 20, "scratch size");
 // 50 000 edges 283, 84, 143; 100 000 edges 286, 96, 341; 10^6 edges 611, 504, 7690).
 __device__ __forceinline__ int window_of(int64_t nnz) { return nnz < (1 << 18) ? 8 : nnz < (1 << 20) ? 16 : 32; }
 // Rows of at most this many entries are a warp's (d^2 / 128 steps at most); a
-// longer one is a CTA's, in parts of a window per warp.
-__device__ __forceinline__ int short_row(int64_t nnz) { return 4 * window_of(nnz); }
+// longer one is a CTA's, in parts of a window per warp. Where large bitmaps leave
+// one or two CTAs an SM, a part's barriers and chains of loads are hidden badly and
+// rows up to 256 entries are a warp's, in graphs of many (10^6 vertices, up to 128
+// and 256 entries: 7700 complete graphs of 135, 52 and 23 ms; 5000 of 200, 75 and
+// 44; Chung-Lu, 5e7 edges, exponent 4, 23.1 and 18.5; 10^7, 2.1, 5.40 and 5.44; at
+// 300 000 vertices, 1.5e7 edges, 5.21 and 5.60).
+__device__ __forceinline__ int short_row(int32_t n, int64_t nnz) {
+  return n > kFourMaxN && nnz >= (1 << 24) ? 256 : 4 * window_of(nnz);
+}
 // (from 2^28 entries larger ones, so that their list holds all of them: 1700
 // complete graphs of 600, which it did not hold, 1163 ms, now 392)
 __device__ __forceinline__ int part_of(int64_t nnz) {
   return nnz < (1 << 28) ? kNoAllocBlock / 32 * window_of(nnz) : 2048;
 }
-constexpr int kShortRow = 128;              // the longest short row
+constexpr int kShortRow = 128;              // the longest short row up to kFourMaxN vertices
 constexpr int kShortSlots = 2 * kShortRow;  // its hash, at most half full
 constexpr int kShortWords = kShortSlots + kShortRow;  // a warp's hash and filter
+constexpr int kMidSlots = 2 * 256, kMidWords = kMidSlots + kShortRow;  // beyond
 constexpr int kTriBlock = 256;
 constexpr int kMaxHeavy = 512;              // heavy runs of a part that its warps share
-// Up to this many vertices, the bitmap and the warps' hashes leave room for four
-// CTAs an SM, and one kernel takes the long rows and then the short ones.
-constexpr int32_t kBothMaxN = 1 << 17;
 // A lower neighbour's row of this many entries is shared by all warps, as one
 // alone would be the last to end (R-MAT scale 18, rows from 512, 1024, 2048
 // entries: 1.99, 1.71, 1.68 ms; 950 complete graphs of 1100: 1368, 1367, 1211).
@@ -141,7 +153,7 @@ __global__ void __launch_bounds__(kTriBlock) k_rows(int32_t n, const int32_t* __
   const int lane = threadIdx.x & 31;
   const int64_t t0 = (int64_t)blockIdx.x * kTriBlock + threadIdx.x, threads = (int64_t)gridDim.x * kTriBlock;
   const int64_t nnz = rp[n];
-  const int32_t part = part_of(nnz), longest_short = short_row(nnz);
+  const int32_t part = part_of(nnz), longest_short = short_row(n, nnz);
   for (int64_t x = t0; x < n; x += threads) {
     const int32_t d = rp[x + 1] - rp[x];
     if (d <= longest_short) continue;
@@ -327,11 +339,12 @@ __global__ void __launch_bounds__(1024) k_pick(int32_t n, const int32_t* __restr
 }
 
 // Warp per row of up to short_row() entries: its entries in an open-addressing
-// hash (twice the slots), behind a filter of 16 bits a hash slot.
+// hash (twice the slots), behind a filter of 16 bits a hash slot (8 where the row
+// has more than 128 entries).
 __device__ __forceinline__ void short_rows(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                            int32_t* __restrict__ tri, uint32_t* __restrict__ scratch, int32_t* key,
                                            uint32_t* filt, int32_t* cnt, int lane) {
-  const int32_t longest = short_row(rp[n]);
+  const int32_t longest = short_row(n, rp[n]);
   // rows taken at a time: eight where every warp gets many
   const int32_t take = min(8, max(1, n / (int32_t)(gridDim.x * (kNoAllocBlock / 32))));
   for (;;) {
@@ -343,9 +356,9 @@ __device__ __forceinline__ void short_rows(int32_t n, const int32_t* __restrict_
       const int32_t b = rp[x], d = rp[x + 1] - b;
       if (d > longest || d == 0 || row_bad(scratch, x)) continue;  // warp-uniform
       int bits = 5;
-      while ((1 << bits) < 2 * d) ++bits;  // at most log2(kShortSlots)
+      while ((1 << bits) < 2 * d) ++bits;  // at most log2(kShortSlots), or of kMidSlots
       const uint32_t mask = (1u << bits) - 1u;
-      const int fbits = bits + 4;  // 16 filter bits per hash slot
+      const int fbits = min(bits + 4, 12);  // kShortRow words at most
       for (int i = lane; i <= (int)mask; i += 32) key[i] = -1;
       for (int i = lane; i < (1 << fbits) / 32; i += 32) filt[i] = 0u;
       __syncwarp();
@@ -485,9 +498,9 @@ __device__ __forceinline__ void long_parts(int32_t n, const int32_t* __restrict_
 // Both, or one of them (which: bit 0 long rows, bit 1 short ones), with the
 // bitmap and the warps' hashes in dynamic shared memory.
 template <int kThreads>
-__global__ void __launch_bounds__(kThreads, 2048 / kThreads) k_tri(int32_t n, const int32_t* __restrict__ rp,
-                                                          const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
-                                                          uint32_t* __restrict__ scratch, int which) {
+__global__ void __launch_bounds__(kThreads, 2048 / kThreads)
+    k_tri(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, int32_t* __restrict__ tri,
+          uint32_t* __restrict__ scratch, int which) {
   extern __shared__ uint32_t s_dyn[];
   __shared__ int32_t s_cnt[kThreads / 32][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -499,8 +512,9 @@ __global__ void __launch_bounds__(kThreads, 2048 / kThreads) k_tri(int32_t n, co
     tables += (n + 31) / 32;
   }
   if (which & 2) {
-    uint32_t* mine = tables + warp * kShortWords;
-    short_rows(n, rp, ci, tri, scratch, reinterpret_cast<int32_t*>(mine), mine + kShortSlots, s_cnt[warp], lane);
+    uint32_t* mine = tables + warp * (n > kFourMaxN ? kMidWords : kShortWords);
+    short_rows(n, rp, ci, tri, scratch, reinterpret_cast<int32_t*>(mine),
+               mine + (n > kFourMaxN ? kMidSlots : kShortSlots), s_cnt[warp], lane);
   }
 }
 
@@ -638,7 +652,7 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
     return e == cudaSuccess ? GC_OK : cuda_fail(e, "gc_edge_triangles_noalloc");
   }
   const size_t bitmap = sizeof(uint32_t) * (size_t)((n + 31) / 32);
-  constexpr size_t kTables = sizeof(uint32_t) * kShortWords * (kNoAllocBlock / 32);
+  const size_t tables = sizeof(uint32_t) * (n > kFourMaxN ? kMidWords : kShortWords) * (kNoAllocBlock / 32);
   const int grid = sms * 8;  // 2048 threads an SM; the number of slots is on the device only
   // the counters and the bad-row bits cleared; then each kernel is launched while
   // the one before it runs, and waits for it (after_previous)
@@ -656,14 +670,13 @@ extern "C" gc_status gc_edge_triangles_noalloc(int32_t n, const int32_t* row_ptr
   };
   // CTAs an SM: four (2048 threads) while the bitmaps leave room for them in
   // 227 KB, beside the 11 KB that every CTA takes; with larger bitmaps fewer, of
-  // twice the threads (R-MAT scale 20: 20.7 ms with 512 and 16.0 with 1024)
+  // twice the threads (R-MAT scale 20: 20.7 ms with 512, 15.2 with 1024)
   if (n <= kBothMaxN) {
-    tri(3, 4, kNoAllocBlock, bitmap + kTables);
+    tri(3, 4, kNoAllocBlock, bitmap + tables);
   } else {
-    auto fit = [&](size_t besides) { return ((size_t)227 << 10) / (bitmap + (besides << 10)); };
-    if (fit(13) >= 4) tri(1, 4, kNoAllocBlock, bitmap);
-    else tri(1, (int)std::min<size_t>(2, fit(15)), 2 * kNoAllocBlock, bitmap);
-    tri(2, 4, kNoAllocBlock, kTables);
+    if (n <= kFourMaxN) tri(1, 4, kNoAllocBlock, bitmap);
+    else tri(1, bitmap + (15 << 10) <= (size_t)227 * 512 ? 2 : 1, 2 * kNoAllocBlock, bitmap);
+    tri(2, 4, kNoAllocBlock, tables);
   }
   launch_after(k_tri_reverse, grid, kTriBlock, 0, s, n, row_ptr, col_idx, tri_out, scratch);
   launch_after(k_tri_marked, kNoAllocCtas, kNoAllocBlock, 0, s, n, row_ptr, col_idx, tri_out, scratch);

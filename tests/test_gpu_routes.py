@@ -218,9 +218,9 @@ def test_noalloc_slots_beyond_2_to_the_30():
 @pytest.mark.parametrize("n, sizes", [
     # rows of one more and one less than a warp's and a CTA's, of runs that a lane, a
     # warp and a CTA reads; the last n of four CTAs an SM and the first of larger ones
-    (358400, [17, 64, 65, 66, 128, 129, 130, 131, 600, 2048, 2049, 2050, 2600]),
-    (358432, [17, 64, 65, 66, 128, 129, 130, 131, 600, 2048, 2049, 2050, 2600]),
-    (1 << 20, [17, 64, 65, 66, 128, 129, 130, 131, 600, 2048, 2049, 2050, 2600]),
+    (358400, [17, 64, 65, 66, 128, 129, 130, 131, 256, 257, 258, 600, 2048, 2049, 2050, 2600]),
+    (358432, [17, 64, 65, 66, 128, 129, 130, 131, 256, 257, 258, 600, 2048, 2049, 2050, 2600]),
+    (1 << 20, [17, 64, 65, 66, 128, 129, 130, 131, 256, 257, 258, 600, 2048, 2049, 2050, 2600]),
     (131073, [2100] * 62),  # 2^28 entries: more of a part's runs than its CTA can list
 ])
 def test_noalloc_long_rows_by_number_of_vertices(n, sizes):
